@@ -1,0 +1,444 @@
+// GEMM and attention of the fp32 model on the CUDA cores (its 1e-4 tolerance against fp64 rules out TF32, whose operands
+// carry 11 bits).  Both are built on one register-tiled product of two row-major shared-memory tiles, dot_tile():
+//     acc[i][j] += sum_k A[ty + 8 i][k] * B[tx + 16 j][k]        128 threads, ty = tid / 16, tx = tid % 16
+// Products are taken two k at a time with the packed fma.rn.f32x2 (even k in the low half, odd k in the high half, added at the
+// end): operands come out of the tiles in the order they are stored, 16 bytes (four k) per load, with no register shuffling, and
+// the packed form halves the issue slots a multiply-add takes, which leaves room for the loads beside them.
+// Rows are padded to 4 words beyond a multiple of 32, so that the 16 B rows a half-warp reads fall into distinct banks
+// (two wavefronts for 256 bytes, the minimum) and the two A rows of a warp are broadcasts in distinct banks: per four k a
+// warp spends RT + 8 wavefronts of shared-memory bandwidth on RT * 16 clocks of multiply-adds.
+#include <algorithm>
+
+#include "kernels.cuh"
+
+namespace relaygr {
+
+namespace {
+
+constexpr int kThreads = 128;
+
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ float fold(uint64_t v)
+{
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+    return lo + hi;
+}
+// 16-byte (or 4-byte) asynchronous copy into shared memory; `bytes` < the size fills the rest with zeros
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, int bytes)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void *dst, const void *src, int bytes)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+template <int RT, int CT, int K, int LDA, int LDB>
+__device__ __forceinline__ void dot_tile(uint64_t (&acc)[RT][CT], const float *A, const float *B, int ty, int tx)
+{
+#pragma unroll 4
+    for (int k = 0; k < K; k += 4) {
+        ulonglong2 b[CT];
+#pragma unroll
+        for (int j = 0; j < CT; ++j) b[j] = *reinterpret_cast<const ulonglong2 *>(B + (tx + 16 * j) * LDB + k);
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+            const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(A + (ty + 8 * i) * LDA + k);
+#pragma unroll
+            for (int j = 0; j < CT; ++j) acc[i][j] = fma2(a.y, b[j].y, fma2(a.x, b[j].x, acc[i][j]));
+        }
+    }
+}
+
+// ---- GEMM: C[m, n] = sum_k A[m, k] W[n, k] ---------------------------------------------------------------------------
+// Tiles of 8 RT x 64, K in steps of 32 through a three-stage cp.async ring.  kVec: A and W may be read 16 bytes at a time.
+constexpr int kBN = 64, kBK = 32, kStages = 3, kLdk = kBK + 4;
+
+template <int RT> constexpr int gemm_smem() { return kStages * (8 * RT + kBN) * kLdk * 4 + 8 * RT * (8 + 4); }
+
+template <int RT, bool kVec>
+__global__ void __launch_bounds__(kThreads)
+f32_gemm_kernel(const float *__restrict__ A, const float *__restrict__ W, int64_t M, int N, int K, Epilogue e)
+{
+    constexpr int BM = 8 * RT;
+    extern __shared__ __align__(16) uint8_t smem_raw[];
+    float *As = reinterpret_cast<float *>(smem_raw), *Ws = As + kStages * BM * kLdk;
+    int64_t *page_off = reinterpret_cast<int64_t *>(Ws + kStages * kBN * kLdk);    // rows that go to pages: offset of (page, K, slot)
+    int *last_slot = reinterpret_cast<int *>(page_off + BM);                       // ... and of a user's last row: its slot, else -1
+    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+    const int64_t m0 = (int64_t)blockIdx.y * BM;
+    const int n0 = blockIdx.x * kBN;
+    const int n_k = (K + kBK - 1) / kBK;
+
+    auto load = [&](float *dst, const float *src, int64_t row0, int64_t n_rows, int rows, int kb) {
+        if constexpr (kVec) {
+            for (int i = tid; i < rows * (kBK / 4); i += kThreads) {
+                const int r = i / (kBK / 4), k = (i % (kBK / 4)) * 4;
+                const bool in = row0 + r < n_rows && kb * kBK + k < K;             // K is a multiple of 4
+                cp_async16(dst + r * kLdk + k, in ? src + (row0 + r) * K + kb * kBK + k : src, in ? 16 : 0);
+            }
+        } else {
+            for (int i = tid; i < rows * kBK; i += kThreads) {
+                const int r = i / kBK, k = i % kBK;
+                const bool in = row0 + r < n_rows && kb * kBK + k < K;
+                cp_async4(dst + r * kLdk + k, in ? src + (row0 + r) * K + kb * kBK + k : src, in ? 4 : 0);
+            }
+        }
+    };
+    auto load_w = [&](int kb) { load(Ws + (kb % kStages) * kBN * kLdk, W, n0, N, kBN, kb); };
+    auto load_a = [&](int kb) { load(As + (kb % kStages) * BM * kLdk, A, m0, M, BM, kb); };
+
+    // the weights are parameters: the first stages of W are on their way while the previous kernel finishes
+    grid_launch_dependents();
+#pragma unroll
+    for (int s = 0; s < kStages - 1; ++s) if (s < n_k) load_w(s);
+    grid_dependency_wait();
+#pragma unroll
+    for (int s = 0; s < kStages - 1; ++s) { if (s < n_k) load_a(s); cp_commit(); }      // (W of both stages is in the first group)
+
+    const bool to_pages = e.mode == EPI_QKV && e.paged.slab != nullptr && e.col0 + n0 + kBN > e.d_model;
+    if (to_pages && tid < BM) {
+        int64_t off = 0;
+        int last = -1;
+        if (m0 + tid < M) {
+            const int u = find_user(e.row_off, e.n_users, (int)(m0 + tid));
+            const int t = (int)(m0 + tid) - e.row_off[u];
+            off = (int64_t)page_elem_offset(e.paged, e.paged.pt[e.seqs[u].pt_base + (t >> 6)], 0, t & 63);
+            if (t == e.seqs[u].n_q - 1) last = t & 63;
+        }
+        page_off[tid] = off;
+        last_slot[tid] = last;
+    }
+
+    uint64_t acc[RT][4] = {};
+    for (int kb = 0; kb < n_k; ++kb) {
+        cp_wait<kStages - 2>();
+        __syncthreads();                              // stage kb has landed for everybody; stage kb - 1 has been read by everybody
+        if (kb + kStages - 1 < n_k) { load_w(kb + kStages - 1); load_a(kb + kStages - 1); }
+        cp_commit();
+        const int s = kb % kStages;
+        dot_tile<RT, 4, kBK, kLdk, kLdk>(acc, As + s * BM * kLdk, Ws + s * kBN * kLdk, ty, tx);
+    }
+
+#pragma unroll
+    for (int i = 0; i < RT; ++i) {
+        const int64_t m = m0 + ty + 8 * i;
+        if (m >= M) continue;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int n = n0 + tx + 16 * j;
+            if (n >= N) continue;
+            float v = fold(acc[i][j]) + (e.bias ? e.bias[n] : 0.f);
+            if (e.mode == EPI_STORE) {
+                if (e.silu) v = v / (1.f + expf(-v));
+                reinterpret_cast<float *>(e.out)[m * N + n] = v;
+                continue;
+            }
+            if (e.mode == EPI_RESID) { e.out_f32[m * N + n] = e.resid[m * N + n] + v; continue; }
+            const int d = e.d_model, col = e.col0 + n, which = (col >= d) + (col >= 2 * d), c = col - which * d;
+            if (which == 0) { reinterpret_cast<float *>(e.q)[m * d + c] = v; continue; }
+            if (!to_pages) { reinterpret_cast<float *>(which == 1 ? e.k_lin : e.v_lin)[m * d + c] = v; continue; }
+            float *row = reinterpret_cast<float *>(e.paged.slab) + page_off[ty + 8 * i] + (int64_t)(which - 1) * 64 * d + c;
+            *row = v;
+            const int ls = last_slot[ty + 8 * i];     // last row of the prefix: clear the unused slots of its page
+            if (ls >= 0)
+                for (int z = 1; ls + z < 64; ++z) row[(int64_t)z * d] = 0.f;
+        }
+    }
+}
+
+template <int RT>
+cudaError_t launch_gemm(const float *A, const float *W, int64_t M, int N, int K, const Epilogue &epi, cudaStream_t stream)
+{
+    const bool vec = ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(W)) & 15) == 0;
+    auto kernel = vec ? f32_gemm_kernel<RT, true> : f32_gemm_kernel<RT, false>;
+    static PerDeviceValue attr_set;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (!attr_set.get(dev)) {
+        e = cudaFuncSetAttribute(f32_gemm_kernel<RT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem<RT>());
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(f32_gemm_kernel<RT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem<RT>());
+        if (e != cudaSuccess) return e;
+        attr_set.set(dev, 1);
+    }
+    const dim3 grid((unsigned)((N + kBN - 1) / kBN), (unsigned)((M + 8 * RT - 1) / (8 * RT)));
+    return launch_dependent(kernel, grid, dim3(kThreads), (size_t)gemm_smem<RT>(), stream, 1, A, W, M, N, K, epi);
+}
+
+// ---- attention: flash-style over 64-key blocks ------------------------------------------------------------------------
+// A block of 128 threads owns 8 RT query rows of one head of one user.  Thread (ty, tx) holds, of rows ty + 8 i, the logits of
+// keys tx + 16 j, and the output dimensions tx + 16 j; a row belongs to 16 lanes of one warp, so its maximum and its weights
+// need no block-wide exchange.  Per key block: S = Q K^T (dot_tile), online softmax (or SiLU), P through shared memory,
+// O = O * correction + P V (dot_tile again, V transposed in shared memory so that keys are its inner index).  K arrives by
+// cp.async under the softmax and the P V of the block before, V through registers under S (the transposition).
+template <int DH, int RT> struct AttnSmem {
+    static constexpr int kLdq = DH + 4, kLdv = 64 + 4, kLdp = 80;      // P rows 16 words apart (mod 32): its scalar stores do not collide
+    static constexpr int kQ = 0, kK = kQ + 8 * RT * kLdq, kV = kK + 64 * kLdq, kP = kV + DH * kLdv, kFloats = kP + 8 * RT * kLdp;
+    static constexpr int kBytes = kFloats * 4;
+};
+
+template <int DH, int RT, bool kPointwise>
+__global__ void __launch_bounds__(kThreads, RT == 8 ? 3 : 4)
+f32_attention_kernel(const float *__restrict__ q, const float *__restrict__ k_lin, const float *__restrict__ v_lin, PagedKV paged,
+                     const SeqDesc *__restrict__ seqs, const F32Tile *__restrict__ tiles, int n_heads, float *__restrict__ out)
+{
+    using L = AttnSmem<DH, RT>;
+    constexpr int CT = DH / 16, BQ = 8 * RT, kV4 = 64 * DH / 4 / kThreads;      // kV4: 16-byte pieces of V per thread
+    extern __shared__ __align__(16) float smem[];
+    float *Qs = smem + L::kQ, *Ks = smem + L::kK, *Vt = smem + L::kV, *Ps = smem + L::kP;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = tid >> 4, tx = tid & 15;
+    grid_launch_dependents();
+    grid_dependency_wait();
+    const F32Tile tile = tiles[blockIdx.x / n_heads];
+    const int h = blockIdx.x % n_heads, d = n_heads * DH;
+    const SeqDesc sd = seqs[tile.seq];
+    const int n_q = min(BQ, sd.n_q - tile.q0);
+    const int64_t row0 = (int64_t)sd.q_row0 + tile.q0;
+    const int pos0 = sd.q_pos0 + tile.q0;                                       // sequence position of the tile's first row
+
+    // logits in units of log2(e) (softmax), so that a weight is 2^x
+    const float scale = rsqrtf((float)DH) * (kPointwise ? 1.f : 1.4426950408889634f);
+    for (int i = tid; i < BQ * DH / 4; i += kThreads) {
+        const int r = i / (DH / 4), c = (i % (DH / 4)) * 4;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < n_q) v = *reinterpret_cast<const float4 *>(q + (row0 + r) * d + h * DH + c);
+        *reinterpret_cast<float4 *>(Qs + r * L::kLdq + c) = make_float4(v.x * scale, v.y * scale, v.z * scale, v.w * scale);
+    }
+
+    // key blocks: the pages first, then 64-row groups of the call's own rows; only what the tile's last row (or, with a
+    // candidate among them, any row) can see
+    const int last_lim = pos0 + n_q - 1 >= sd.causal_end ? sd.causal_end : pos0 + n_q;     // keys at positions < last_lim are visible
+    const int n_page_keys = min(sd.n_paged, last_lim), n_lin_keys = max(0, min(sd.n_lin, last_lim - sd.lin_pos0));
+    const int n_page_blocks = (n_page_keys + 63) >> 6, n_blocks = n_page_blocks + ((n_lin_keys + 63) >> 6);
+    struct Block { const float *k, *v; int n_valid, pos; };
+    auto block_of = [&](int j) {
+        Block b;
+        if (j < n_page_blocks) {
+            const int page = paged.pt[sd.pt_base + j];
+            const float *slab = reinterpret_cast<const float *>(paged.slab);
+            b.k = slab + page_elem_offset(paged, page, 0, 0) + h * DH;
+            b.v = slab + page_elem_offset(paged, page, 1, 0) + h * DH;
+            b.n_valid = min(64, n_page_keys - j * 64); b.pos = j * 64;
+        } else {
+            const int k0 = (j - n_page_blocks) * 64;
+            const int64_t off = (int64_t)(sd.lin_row0 + k0) * d + h * DH;
+            b.k = k_lin + off; b.v = v_lin + off;
+            b.n_valid = min(64, n_lin_keys - k0); b.pos = sd.lin_pos0 + k0;
+        }
+        return b;
+    };
+    auto load_k = [&](const Block &b) {               // 16 (or 8) lanes per row; rows past n_valid are zeros
+        for (int i = tid; i < 64 * DH / 4; i += kThreads) {
+            const int r = i / (DH / 4), c = (i % (DH / 4)) * 4;
+            const bool in = r < b.n_valid;
+            cp_async16(Ks + r * L::kLdq + c, in ? b.k + (int64_t)r * d + c : b.k, in ? 16 : 0);
+        }
+        cp_commit();
+    };
+    int lim[RT];                                      // of each row: keys at positions < lim are visible
+#pragma unroll
+    for (int i = 0; i < RT; ++i) {
+        const int t = pos0 + ty + 8 * i;
+        lim[i] = t >= sd.causal_end ? sd.causal_end : t + 1;
+    }
+    const int min_lim = pos0 >= sd.causal_end ? sd.causal_end : pos0 + 1;
+
+    float o[RT][CT] = {}, m[RT], l[RT];
+#pragma unroll
+    for (int i = 0; i < RT; ++i) { m[i] = -INFINITY; l[i] = 0.f; }
+    Block cur{};
+    if (n_blocks > 0) { cur = block_of(0); load_k(cur); }
+    for (int j = 0; j < n_blocks; ++j) {
+        float4 vr[kV4];                               // keys lane and lane + 32 of dimensions 4 g .. 4 g + 3
+#pragma unroll
+        for (int i = 0; i < kV4; ++i) {
+            const int key = lane + 32 * (i & 1), g = (i >> 1) * 4 + warp;
+            vr[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (key < cur.n_valid) vr[i] = *reinterpret_cast<const float4 *>(cur.v + (int64_t)key * d + 4 * g);
+        }
+        cp_wait<0>();
+        __syncthreads();                              // K of this block (and, the first time, Q) is there; V of the last one has been read
+        uint64_t s2[RT][4] = {};
+        dot_tile<RT, 4, DH, L::kLdq, L::kLdq>(s2, Qs, Ks, ty, tx);
+#pragma unroll
+        for (int i = 0; i < kV4; ++i) {
+            const int key = lane + 32 * (i & 1), g = (i >> 1) * 4 + warp;
+            Vt[(4 * g) * L::kLdv + key] = vr[i].x; Vt[(4 * g + 1) * L::kLdv + key] = vr[i].y;
+            Vt[(4 * g + 2) * L::kLdv + key] = vr[i].z; Vt[(4 * g + 3) * L::kLdv + key] = vr[i].w;
+        }
+        __syncthreads();                              // V is there; K has been read
+        const bool mask = cur.n_valid < 64 || cur.pos + 64 > min_lim;
+        const int pos = cur.pos;
+        const int end = cur.pos + cur.n_valid;
+        if (j + 1 < n_blocks) { cur = block_of(j + 1); load_k(cur); }
+        float corr[RT];
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+            float s[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) s[c] = fold(s2[i][c]);
+            const int vis = min(lim[i], end) - pos;    // keys tx + 16 c < vis of this block are visible
+            if constexpr (kPointwise) {
+                // the weight of a key is SiLU(logit); the sum is divided by the number of visible keys
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    float p = s[c] / (1.f + expf(-s[c]));
+                    if (mask && tx + 16 * c >= vis) p = 0.f;
+                    Ps[(ty + 8 * i) * L::kLdp + tx + 16 * c] = p;
+                }
+                corr[i] = 1.f;
+            } else {
+                if (mask)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) if (tx + 16 * c >= vis) s[c] = -INFINITY;
+                float mx = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
+#pragma unroll
+                for (int x = 8; x > 0; x >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, x));
+                const float mn = fmaxf(m[i], mx), ref = mn == -INFINITY ? 0.f : mn;
+                corr[i] = exp2f(m[i] - ref);
+                m[i] = mn;
+                float rs = 0.f;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const float p = exp2f(s[c] - ref);
+                    rs += p;
+                    Ps[(ty + 8 * i) * L::kLdp + tx + 16 * c] = p;
+                }
+                l[i] = l[i] * corr[i] + rs;           // of this lane's keys; the 16 lanes are added up at the end
+            }
+        }
+        __syncwarp();                                 // a row's weights come from, and go to, lanes of one warp
+        uint64_t o2[RT][CT] = {};
+        dot_tile<RT, CT, 64, L::kLdp, L::kLdv>(o2, Ps, Vt, ty, tx);
+#pragma unroll
+        for (int i = 0; i < RT; ++i)
+#pragma unroll
+            for (int c = 0; c < CT; ++c) o[i][c] = o[i][c] * corr[i] + fold(o2[i][c]);
+    }
+    if (n_blocks == 0) __syncthreads();               // Q is there
+
+#pragma unroll
+    for (int i = 0; i < RT; ++i) {
+        const int r = ty + 8 * i, t = pos0 + r;
+        if constexpr (kPointwise) {
+            l[i] = (float)lim[i];
+        } else {
+#pragma unroll
+            for (int x = 8; x > 0; x >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], x);
+        }
+        const bool is_cand = t >= sd.causal_end && r < n_q;
+        const int64_t self = (int64_t)(sd.self_row0 + tile.q0 + r) * d + h * DH + tx;
+        float dot = 0.f;
+        if (is_cand)
+#pragma unroll
+            for (int c = 0; c < CT; ++c) dot += Qs[r * L::kLdq + tx + 16 * c] * k_lin[self + 16 * c];
+#pragma unroll
+        for (int x = 8; x > 0; x >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, x);
+        if (is_cand) {                                // a candidate also sees itself
+            float corr = 1.f, p;
+            if constexpr (kPointwise) {
+                p = dot / (1.f + expf(-dot));
+                l[i] += 1.f;
+            } else {
+                const float mn = fmaxf(m[i], dot);
+                corr = exp2f(m[i] - mn);
+                p = exp2f(dot - mn);
+                l[i] = l[i] * corr + p;
+            }
+#pragma unroll
+            for (int c = 0; c < CT; ++c) o[i][c] = o[i][c] * corr + p * v_lin[self + 16 * c];
+        }
+        if (r >= n_q) continue;
+        const float inv = 1.f / l[i];
+#pragma unroll
+        for (int c = 0; c < CT; ++c) out[(row0 + r) * d + h * DH + tx + 16 * c] = o[i][c] * inv;
+    }
+}
+
+template <int DH, int RT>
+cudaError_t launch_attention(const float *q, const float *k_lin, const float *v_lin, PagedKV paged, const SeqDesc *seqs,
+                             const F32Tile *tiles, int n_tiles, int n_heads, int attn_kind, float *out, cudaStream_t stream)
+{
+    constexpr int kBytes = AttnSmem<DH, RT>::kBytes;
+    static PerDeviceValue attr_set;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (!attr_set.get(dev)) {
+        e = cudaFuncSetAttribute(f32_attention_kernel<DH, RT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(f32_attention_kernel<DH, RT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+        if (e != cudaSuccess) return e;
+        attr_set.set(dev, 1);
+    }
+    auto kernel = attn_kind == ATTN_POINTWISE ? f32_attention_kernel<DH, RT, true> : f32_attention_kernel<DH, RT, false>;
+    return launch_dependent(kernel, dim3((unsigned)n_tiles * (unsigned)n_heads), dim3(kThreads), (size_t)kBytes, stream, 1, q, k_lin, v_lin,
+                            paged, seqs, tiles, n_heads, out);
+}
+
+}  // namespace
+
+// Tile heights.  Eight rows per thread make the most of every operand load; fewer rows make more blocks.  The tallest tile
+// that still gives every SM two blocks is taken (a lone block of four warps leaves each scheduler one warp to hide its
+// latencies with), the lowest one when none does.
+static int tile_rows_for(int64_t blocks64, int64_t blocks32, int n_sms)
+{
+    if (blocks64 >= 2 * (int64_t)n_sms) return 64;
+    return blocks32 >= 2 * (int64_t)n_sms ? 32 : 16;
+}
+
+cudaError_t launch_gemm_f32(const float *A, const float *W, int64_t M, int N, int K, const Epilogue &epi, int n_sms, cudaStream_t stream,
+                            int64_t *launches)
+{
+    if (M == 0 || N == 0) return cudaSuccess;
+    *launches += 1;
+    const int64_t cols = (N + kBN - 1) / kBN;
+    switch (tile_rows_for(cols * ((M + 63) / 64), cols * ((M + 31) / 32), n_sms)) {
+        case 64: return launch_gemm<8>(A, W, M, N, K, epi, stream);
+        case 32: return launch_gemm<4>(A, W, M, N, K, epi, stream);
+        default: return launch_gemm<2>(A, W, M, N, K, epi, stream);
+    }
+}
+
+int build_f32_tiles(const std::vector<SeqDesc> &seqs, int n_heads, int n_sms, std::vector<F32Tile> &tiles)
+{
+    int64_t n64 = 0, n32 = 0;
+    for (const SeqDesc &s : seqs) { n64 += (s.n_q + 63) / 64; n32 += (s.n_q + 31) / 32; }
+    const int rows = tile_rows_for(n64 * n_heads, n32 * n_heads, n_sms);
+    tiles.clear();
+    for (int u = 0; u < (int)seqs.size(); ++u)
+        for (int q0 = 0; q0 < seqs[(size_t)u].n_q; q0 += rows) tiles.push_back({u, q0});
+    // most keys first: the longest tiles of a causal pass would otherwise start last
+    auto keys = [&](const F32Tile &t) {
+        const SeqDesc &s = seqs[(size_t)t.seq];
+        return std::min(s.causal_end, s.q_pos0 + std::min(s.n_q, t.q0 + rows));
+    };
+    std::stable_sort(tiles.begin(), tiles.end(), [&](const F32Tile &a, const F32Tile &b) { return keys(a) > keys(b); });
+    return rows;
+}
+
+cudaError_t launch_attention_f32(const float *q, const float *k_lin, const float *v_lin, PagedKV paged, const SeqDesc *seqs,
+                                 const F32Tile *tiles, int n_tiles, int tile_rows, int n_heads, int d_head, int attn_kind, float *out,
+                                 cudaStream_t stream, int64_t *launches)
+{
+    if (n_tiles == 0) return cudaSuccess;
+    *launches += 1;
+#define RELAYGR_ATTN(DH)                                                                                                              \
+    return tile_rows == 64   ? launch_attention<DH, 8>(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, out, stream) \
+           : tile_rows == 32 ? launch_attention<DH, 4>(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, out, stream) \
+                             : launch_attention<DH, 2>(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, out, stream)
+    if (d_head == 32) RELAYGR_ATTN(32);
+    if (d_head == 64) RELAYGR_ATTN(64);
+#undef RELAYGR_ATTN
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace relaygr

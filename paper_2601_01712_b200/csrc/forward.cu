@@ -205,11 +205,9 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     // The last layer of a rank / full-inference call (bf16 model): only the candidates' hidden states are read afterwards, so
     // every other row needs nothing but its K and V there.  The candidate rows are moved together and the layer's query
     // projection, attention, output projection and feed-forward run on those rows alone.
-    const bool compact_last = kTensor && !preinfer;
-
-    auto build_items = [&](const std::vector<SeqDesc> &seqs, std::vector<AttnItem> &items, std::vector<AttnMerge> &merges) {
-        build_attention_worklist(seqs, H, n_sms, kMaxSplitTiles, items, merges);
-    };
+    // (The fp32 model does so in full inference, where the prefix rows it saves are most of the work; the few short-term rows of a
+    // rank call do not pay for the two launches.)
+    const bool compact_last = !preinfer && (kTensor || call.mode == MODE_FULL);
 
     // ---- metadata blob: row_off | seg_off x3 | score_off | SeqDesc[] | page table | attention items [| the same for the last layer]
     std::vector<int32_t> blob;
@@ -227,10 +225,22 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     std::vector<AttnMerge> merges, merges_c;
     std::vector<SeqDesc> seqs_c;                  // the candidates of each user as rows of their own (last layer)
     size_t o_items = 0, o_merges = 0, o_seq_c = 0, o_items_c = 0, o_merges_c = 0;
-    if (kTensor) {
-        build_items(call.seqs, items, merges);
-        if (!items.empty()) o_items = put(reinterpret_cast<const int32_t *>(items.data()), items.size() * (sizeof(AttnItem) / 4));
-        if (!merges.empty()) o_merges = put(reinterpret_cast<const int32_t *>(merges.data()), merges.size() * (sizeof(AttnMerge) / 4));
+    // the work of an attention launch over `seqs`: items and merges (tensor cores), or query tiles (fp32 model)
+    std::vector<F32Tile> tiles, tiles_c;
+    int tile_rows = 0, tile_rows_c = 0;
+    auto put_work = [&](const std::vector<SeqDesc> &seqs, std::vector<AttnItem> &it, std::vector<AttnMerge> &mg, std::vector<F32Tile> &ti,
+                        size_t &o_it, size_t &o_mg, int &rows) {
+        if (kTensor) {
+            build_attention_worklist(seqs, H, n_sms, kMaxSplitTiles, it, mg);
+            if (!it.empty()) o_it = put(reinterpret_cast<const int32_t *>(it.data()), it.size() * (sizeof(AttnItem) / 4));
+            if (!mg.empty()) o_mg = put(reinterpret_cast<const int32_t *>(mg.data()), mg.size() * (sizeof(AttnMerge) / 4));
+        } else {
+            rows = build_f32_tiles(seqs, H, n_sms, ti);
+            if (!ti.empty()) o_it = put(reinterpret_cast<const int32_t *>(ti.data()), ti.size() * (sizeof(F32Tile) / 4));
+        }
+    };
+    {
+        put_work(call.seqs, items, merges, tiles, o_items, o_merges, tile_rows);
         if (compact_last && n_scores > 0) {
             seqs_c = call.seqs;
             for (int u = 0; u < B; ++u) {
@@ -242,9 +252,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
                 c.score_row0 = call.score_off[u];
             }
             o_seq_c = put(reinterpret_cast<const int32_t *>(seqs_c.data()), (size_t)B * (sizeof(SeqDesc) / 4));
-            build_items(seqs_c, items_c, merges_c);
-            if (!items_c.empty()) o_items_c = put(reinterpret_cast<const int32_t *>(items_c.data()), items_c.size() * (sizeof(AttnItem) / 4));
-            if (!merges_c.empty()) o_merges_c = put(reinterpret_cast<const int32_t *>(merges_c.data()), merges_c.size() * (sizeof(AttnMerge) / 4));
+            put_work(seqs_c, items_c, merges_c, tiles_c, o_items_c, o_merges_c, tile_rows_c);
         }
     }
     // one item counter per layer's attention launch (the persistent kernel draws its work from it), zeroed by this upload
@@ -318,7 +326,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         cudaEvent_t pe = prof_begin(stream);
         cudaError_t r;
         if constexpr (kTensor) r = launch_gemm_tc(tmA, *tmW, om, M, N, K, ep, d_status, stream, &launches);
-        else r = launch_gemm_simt<T>(A, W, M, N, K, ep, stream, &launches);
+        else r = launch_gemm_f32(A, W, M, N, K, ep, n_sms, stream, &launches);
         prof_end(KC_GEMM, pe, stream);
         return r;
     };
@@ -337,7 +345,8 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     const SeqDesc *seqs_m = d_seqs;
     const AttnItem *items_m = reinterpret_cast<const AttnItem *>(meta + o_items);
     const AttnMerge *merges_m = reinterpret_cast<const AttnMerge *>(meta + o_merges);
-    int n_items_m = (int)items.size(), n_merges_m = (int)merges.size();
+    const F32Tile *tiles_m = reinterpret_cast<const F32Tile *>(meta + o_items);
+    int n_items_m = (int)(kTensor ? items.size() : tiles.size()), n_merges_m = (int)merges.size();
     bool dead_tail = false;                       // a call without candidates: nothing reads the last layer
 
     for (int l = 0; l < L; ++l) {
@@ -380,7 +389,8 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
             seqs_m = reinterpret_cast<const SeqDesc *>(meta + o_seq_c);
             items_m = reinterpret_cast<const AttnItem *>(meta + o_items_c);
             merges_m = reinterpret_cast<const AttnMerge *>(meta + o_merges_c);
-            n_items_m = (int)items_c.size(); n_merges_m = (int)merges_c.size();
+            tiles_m = reinterpret_cast<const F32Tile *>(meta + o_items_c); tile_rows = tile_rows_c;
+            n_items_m = (int)(kTensor ? items_c.size() : tiles_c.size()); n_merges_m = (int)merges_c.size();
             cudaEvent_t pe = prof_begin(stream);
             e = launch_compact_rows<T>(x, a, seqs_m, B, meta + o_score, n_scores, d, x_c, a_c, stream, &launches);
             prof_end(KC_LAYERNORM, pe, stream);
@@ -403,7 +413,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
                                         l, d, cfg.attn_kind, att, reinterpret_cast<float *>(ws + lay.partial),
                                         reinterpret_cast<int *>(ws + lay.meta) + o_ctr + l, n_sms, d_status, stream, &launches);
             else
-                e = launch_attention_simt<T>(q, kl, vl, paged, d_seqs, d_row_off, B, R, H, cfg.d_head, cfg.attn_kind, att, stream, &launches);
+                e = launch_attention_f32(q, kl, vl, paged, seqs_m, tiles_m, n_items_m, tile_rows, H, cfg.d_head, cfg.attn_kind, att, stream, &launches);
             prof_end(KC_ATTENTION, pe, stream);
         }
         if (!ck("attention")) return RELAYGR_E_CUDA;

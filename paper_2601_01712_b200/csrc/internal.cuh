@@ -57,6 +57,9 @@ struct AttnMerge {
     int32_t slot0, n_splits;
 };
 
+// One query tile of the fp32 attention: rows q0 .. of a user.
+struct F32Tile { int32_t seq, q0; };
+
 // Codes a kernel may record in the status word at the start of the workspace (relaygr_device_status; 0 = healthy).
 // The first code recorded stays.
 enum DeviceStatus : int { STATUS_OK = 0, STATUS_WAIT_TIMEOUT = RELAYGR_DEVSTATUS_WAIT_TIMEOUT, STATUS_BAD_INDEX = RELAYGR_DEVSTATUS_BAD_INDEX };

@@ -6,6 +6,7 @@
 
 #include <atomic>
 #include <utility>
+#include <vector>
 
 #include "internal.cuh"
 
@@ -74,16 +75,16 @@ cudaError_t launch_score(const float *x, int d, const SeqDesc *seqs, int n_users
 
 // ---- CUDA-core GEMM and attention (the fp32 model) ---------------------------------------------
 
-// C[m, n] = sum_k A[m, k] W[n, k], m < M, n < N, then `epi`.
-template <typename T>
-cudaError_t launch_gemm_simt(const T *A, const T *W, int64_t M, int N, int K, const Epilogue &epi,
-                             cudaStream_t stream, int64_t *launches);
+// C[m, n] = sum_k A[m, k] W[n, k], m < M, n < N, then `epi`.  K % 4 == 0, A and W 4-byte aligned (16 is faster).
+cudaError_t launch_gemm_f32(const float *A, const float *W, int64_t M, int N, int K, const Epilogue &epi, int n_sms, cudaStream_t stream,
+                            int64_t *launches);
 
-// One warp per (row, head): attention (softmax, or pointwise SiLU for ATTN_POINTWISE) under the SeqDesc mask.  out [n_rows, d] in T.
-template <typename T>
-cudaError_t launch_attention_simt(const T *q, const T *k_lin, const T *v_lin, PagedKV paged, const SeqDesc *seqs,
-                                  const int32_t *row_off, int n_users, int64_t n_rows, int n_heads, int d_head, int attn_kind,
-                                  T *out, cudaStream_t stream, int64_t *launches);
+// One block per (query tile, head): attention (softmax, or pointwise SiLU for ATTN_POINTWISE) under the SeqDesc mask.
+// build_f32_tiles fills the tiles of a call (host) and returns their height, which the launcher takes with them (device).
+int build_f32_tiles(const std::vector<SeqDesc> &seqs, int n_heads, int n_sms, std::vector<F32Tile> &tiles);
+cudaError_t launch_attention_f32(const float *q, const float *k_lin, const float *v_lin, PagedKV paged, const SeqDesc *seqs,
+                                 const F32Tile *tiles, int n_tiles, int tile_rows, int n_heads, int d_head, int attn_kind, float *out,
+                                 cudaStream_t stream, int64_t *launches);
 
 // ---- tensor-core kernels (the bf16 model) -------------------------------------------------------------
 
