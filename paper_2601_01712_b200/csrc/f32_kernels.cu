@@ -23,6 +23,18 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t dup(float v)
+{
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(v));
+    return d;
+}
 __device__ __forceinline__ float fold(uint64_t v)
 {
     float lo, hi;
@@ -175,27 +187,32 @@ cudaError_t launch_gemm(const float *A, const float *W, int64_t M, int N, int K,
 }
 
 // ---- attention: flash-style over 64-key blocks ------------------------------------------------------------------------
-// A block of 128 threads owns 8 RT query rows of one head of one user.  Thread (ty, tx) holds, of rows ty + 8 i, the logits of
-// keys tx + 16 j, and the output dimensions tx + 16 j; a row belongs to 16 lanes of one warp, so its maximum and its weights
-// need no block-wide exchange.  Per key block: S = Q K^T (dot_tile), online softmax (or SiLU), P through shared memory,
-// O = O * correction + P V (dot_tile again, V transposed in shared memory so that keys are its inner index).  K arrives by
-// cp.async under the softmax and the P V of the block before, V through registers under S (the transposition).
-template <int DH, int RT> struct AttnSmem {
-    static constexpr int kLdq = DH + 4, kLdv = 64 + 4, kLdp = 80;      // P rows 16 words apart (mod 32): its scalar stores do not collide
-    static constexpr int kQ = 0, kK = kQ + 8 * RT * kLdq, kV = kK + 64 * kLdq, kP = kV + DH * kLdv, kFloats = kP + 8 * RT * kLdp;
-    static constexpr int kBytes = kFloats * 4;
+// A block owns 8 RT query rows of one head of one user and splits the key blocks over G groups of 64 threads, each with its own
+// K / V tiles, running maxima and output, merged at the end.  Thread (ty, tx) of a group holds, of rows ty + 8 i, the logits of
+// keys 4 tx .. + 3 and 32 + 4 tx .. + 3 and as many output dimensions: RT x 8 per thread is what shared memory can feed (per
+// multiply-add clock of an SM, 2 / 8 clocks of broadcast row loads and 4 / RT of the other operand's), where 8 x 4 would be
+// bound by it.  S = Q K^T takes two dimensions per fma.rn.f32x2, O += P V two output dimensions (P duplicated in registers),
+// so neither K nor V is transposed and both arrive by cp.async, V under S.  A row belongs to eight lanes of one warp: its maximum
+// and its weights, which overwrite the K tile, need no wider exchange.
+template <int DH, int RT, int G> struct AttnSmem {
+    static constexpr int kLdq = DH + 4, kLdp = 64 + 4;
+    static constexpr int kQ = 8 * RT * kLdq;                                              // floats
+    static constexpr int kK = 64 * kLdq > 8 * RT * kLdp ? 64 * kLdq : 8 * RT * kLdp;      // a group's K tile, then its P tile
+    static constexpr int kV = 64 * DH;
+    static constexpr int kBytes = (kQ + G * (kK + kV)) * 4;
+    static_assert(kK >= 16 * RT && kV >= 8 * RT * DH, "the merge keeps (m, l) in the K tile and O in the V tile");
 };
 
-template <int DH, int RT, bool kPointwise>
-__global__ void __launch_bounds__(kThreads, RT == 8 ? 3 : 4)
+template <int DH, int RT, int G, bool kPointwise>
+__global__ void __launch_bounds__(64 * G, RT == 8 ? 4 / G : 1)
 f32_attention_kernel(const float *__restrict__ q, const float *__restrict__ k_lin, const float *__restrict__ v_lin, PagedKV paged,
                      const SeqDesc *__restrict__ seqs, const F32Tile *__restrict__ tiles, int n_heads, float *__restrict__ out)
 {
-    using L = AttnSmem<DH, RT>;
-    constexpr int CT = DH / 16, BQ = 8 * RT, kV4 = 64 * DH / 4 / kThreads;      // kV4: 16-byte pieces of V per thread
+    using L = AttnSmem<DH, RT, G>;
+    constexpr int CT = DH / 8, BQ = 8 * RT;             // CT: output dimensions per thread
     extern __shared__ __align__(16) float smem[];
-    float *Qs = smem + L::kQ, *Ks = smem + L::kK, *Vt = smem + L::kV, *Ps = smem + L::kP;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = tid >> 4, tx = tid & 15;
+    const int tid = threadIdx.x, grp = tid >> 6, gt = tid & 63, ty = gt >> 3, tx = gt & 7;
+    float *Qs = smem, *Ks = smem + L::kQ + grp * (L::kK + L::kV), *Vs = Ks + L::kK;
     grid_launch_dependents();
     grid_dependency_wait();
     const F32Tile tile = tiles[blockIdx.x / n_heads];
@@ -205,145 +222,172 @@ f32_attention_kernel(const float *__restrict__ q, const float *__restrict__ k_li
     const int64_t row0 = (int64_t)sd.q_row0 + tile.q0;
     const int pos0 = sd.q_pos0 + tile.q0;                                       // sequence position of the tile's first row
 
-    // logits in units of log2(e) (softmax), so that a weight is 2^x
-    const float scale = rsqrtf((float)DH) * (kPointwise ? 1.f : 1.4426950408889634f);
-    for (int i = tid; i < BQ * DH / 4; i += kThreads) {
-        const int r = i / (DH / 4), c = (i % (DH / 4)) * 4;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r < n_q) v = *reinterpret_cast<const float4 *>(q + (row0 + r) * d + h * DH + c);
-        *reinterpret_cast<float4 *>(Qs + r * L::kLdq + c) = make_float4(v.x * scale, v.y * scale, v.z * scale, v.w * scale);
-    }
-
     // key blocks: the pages first, then 64-row groups of the call's own rows; only what the tile's last row (or, with a
     // candidate among them, any row) can see
     const int last_lim = pos0 + n_q - 1 >= sd.causal_end ? sd.causal_end : pos0 + n_q;     // keys at positions < last_lim are visible
     const int n_page_keys = min(sd.n_paged, last_lim), n_lin_keys = max(0, min(sd.n_lin, last_lim - sd.lin_pos0));
     const int n_page_blocks = (n_page_keys + 63) >> 6, n_blocks = n_page_blocks + ((n_lin_keys + 63) >> 6);
-    struct Block { const float *k, *v; int n_valid, pos; };
-    auto block_of = [&](int j) {
-        Block b;
+    auto group_sync = [&] { asm volatile("bar.sync %0, 64;" ::"r"(1 + grp) : "memory"); };
+    int b_pos = 0, b_valid = 0;                         // the current block: position of its first key, number of keys
+    auto load_block = [&](int j) {                      // K and V rows; those past the last key are zeros
+        const float *k, *v;
         if (j < n_page_blocks) {
             const int page = paged.pt[sd.pt_base + j];
             const float *slab = reinterpret_cast<const float *>(paged.slab);
-            b.k = slab + page_elem_offset(paged, page, 0, 0) + h * DH;
-            b.v = slab + page_elem_offset(paged, page, 1, 0) + h * DH;
-            b.n_valid = min(64, n_page_keys - j * 64); b.pos = j * 64;
+            k = slab + page_elem_offset(paged, page, 0, 0);
+            v = slab + page_elem_offset(paged, page, 1, 0);
+            b_valid = min(64, n_page_keys - j * 64); b_pos = j * 64;
         } else {
             const int k0 = (j - n_page_blocks) * 64;
-            const int64_t off = (int64_t)(sd.lin_row0 + k0) * d + h * DH;
-            b.k = k_lin + off; b.v = v_lin + off;
-            b.n_valid = min(64, n_lin_keys - k0); b.pos = sd.lin_pos0 + k0;
+            const int64_t off = (int64_t)(sd.lin_row0 + k0) * d;
+            k = k_lin + off; v = v_lin + off;
+            b_valid = min(64, n_lin_keys - k0); b_pos = sd.lin_pos0 + k0;
         }
-        return b;
-    };
-    auto load_k = [&](const Block &b) {               // 16 (or 8) lanes per row; rows past n_valid are zeros
-        for (int i = tid; i < 64 * DH / 4; i += kThreads) {
-            const int r = i / (DH / 4), c = (i % (DH / 4)) * 4;
-            const bool in = r < b.n_valid;
-            cp_async16(Ks + r * L::kLdq + c, in ? b.k + (int64_t)r * d + c : b.k, in ? 16 : 0);
+        constexpr int kLanes = DH / 4, kStep = 64 / kLanes;                     // lanes per row, rows at a time
+        const int c = (gt % kLanes) * 4, r0 = gt / kLanes;
+#pragma unroll
+        for (int i = 0; i < 64 / kStep; ++i) {
+            // key r of the tile sits in row p: a thread's eight keys are eight rows apart and its neighbours' rows adjacent
+            const int r = r0 + i * kStep, p = (r & 32) + (r & 3) * 8 + ((r >> 2) & 7);
+            const bool in = r < b_valid;
+            cp_async16(Ks + p * L::kLdq + c, in ? k + (int64_t)r * d + h * DH + c : k, in ? 16 : 0);
+        }
+        cp_commit();
+#pragma unroll
+        for (int i = 0; i < 64 / kStep; ++i) {
+            const int r = r0 + i * kStep;
+            const bool in = r < b_valid;
+            cp_async16(Vs + r * DH + c, in ? v + (int64_t)r * d + h * DH + c : v, in ? 16 : 0);
         }
         cp_commit();
     };
-    int lim[RT];                                      // of each row: keys at positions < lim are visible
-#pragma unroll
-    for (int i = 0; i < RT; ++i) {
-        const int t = pos0 + ty + 8 * i;
-        lim[i] = t >= sd.causal_end ? sd.causal_end : t + 1;
-    }
-    const int min_lim = pos0 >= sd.causal_end ? sd.causal_end : pos0 + 1;
+    if (grp < n_blocks) load_block(grp);
 
-    float o[RT][CT] = {}, m[RT], l[RT];
+    // logits in units of log2(e) (softmax), so that a weight is 2^x
+    const float scale = rsqrtf((float)DH) * (kPointwise ? 1.f : 1.4426950408889634f);
+    for (int i = tid; i < BQ * DH / 4; i += 64 * G) {
+        const int r = i / (DH / 4), c = (i % (DH / 4)) * 4;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < n_q) v = *reinterpret_cast<const float4 *>(q + (row0 + r) * d + h * DH + c);
+        *reinterpret_cast<float4 *>(Qs + r * L::kLdq + c) = make_float4(v.x * scale, v.y * scale, v.z * scale, v.w * scale);
+    }
+    __syncthreads();
+    const int min_lim = pos0 >= sd.causal_end ? sd.causal_end : pos0 + 1;
+    auto lim_of = [&](int r) { return pos0 + r >= sd.causal_end ? sd.causal_end : pos0 + r + 1; };   // row r sees keys at positions < this
+
+    uint64_t o[RT][CT / 2] = {};
+    float m[RT], l[RT];
 #pragma unroll
-    for (int i = 0; i < RT; ++i) { m[i] = -INFINITY; l[i] = 0.f; }
-    Block cur{};
-    if (n_blocks > 0) { cur = block_of(0); load_k(cur); }
-    for (int j = 0; j < n_blocks; ++j) {
-        float4 vr[kV4];                               // keys lane and lane + 32 of dimensions 4 g .. 4 g + 3
+    for (int i = 0; i < RT; ++i) { m[i] = kPointwise ? 0.f : -INFINITY; l[i] = 0.f; }
+    for (int j = grp; j < n_blocks; j += G) {
+        const int end = b_pos + b_valid;
+        const bool mask = b_valid < 64 || b_pos + 64 > min_lim;
+        cp_wait<1>();
+        group_sync();                                   // K of this block is there
+        float s[RT][8];
+        {
+            uint64_t s2[RT][8] = {};
+            const float *A = Qs + ty * L::kLdq, *B = Ks + tx * L::kLdq;
+#pragma unroll 4
+            for (int k = 0; k < DH; k += 2) {
+                uint64_t b[8];
 #pragma unroll
-        for (int i = 0; i < kV4; ++i) {
-            const int key = lane + 32 * (i & 1), g = (i >> 1) * 4 + warp;
-            vr[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (key < cur.n_valid) vr[i] = *reinterpret_cast<const float4 *>(cur.v + (int64_t)key * d + 4 * g);
+                for (int c = 0; c < 8; ++c) b[c] = *reinterpret_cast<const uint64_t *>(B + 8 * c * L::kLdq + k);
+#pragma unroll
+                for (int i = 0; i < RT; ++i) {
+                    const uint64_t a = *reinterpret_cast<const uint64_t *>(A + 8 * i * L::kLdq + k);
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) s2[i][c] = fma2(a, b[c], s2[i][c]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < RT; ++i)
+#pragma unroll
+                for (int c = 0; c < 8; ++c) s[i][c] = fold(s2[i][c]);
         }
         cp_wait<0>();
-        __syncthreads();                              // K of this block (and, the first time, Q) is there; V of the last one has been read
-        uint64_t s2[RT][4] = {};
-        dot_tile<RT, 4, DH, L::kLdq, L::kLdq>(s2, Qs, Ks, ty, tx);
-#pragma unroll
-        for (int i = 0; i < kV4; ++i) {
-            const int key = lane + 32 * (i & 1), g = (i >> 1) * 4 + warp;
-            Vt[(4 * g) * L::kLdv + key] = vr[i].x; Vt[(4 * g + 1) * L::kLdv + key] = vr[i].y;
-            Vt[(4 * g + 2) * L::kLdv + key] = vr[i].z; Vt[(4 * g + 3) * L::kLdv + key] = vr[i].w;
-        }
-        __syncthreads();                              // V is there; K has been read
-        const bool mask = cur.n_valid < 64 || cur.pos + 64 > min_lim;
-        const int pos = cur.pos;
-        const int end = cur.pos + cur.n_valid;
-        if (j + 1 < n_blocks) { cur = block_of(j + 1); load_k(cur); }
-        float corr[RT];
+        group_sync();                                   // V is there, K has been read
 #pragma unroll
         for (int i = 0; i < RT; ++i) {
-            float s[4];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) s[c] = fold(s2[i][c]);
-            const int vis = min(lim[i], end) - pos;    // keys tx + 16 c < vis of this block are visible
+            // row ty + 8 i, keys 4 tx + c (c < 4) and 32 + 4 tx + c - 4
+            const int vis = min(lim_of(ty + 8 * i), end) - b_pos - 4 * tx;
             if constexpr (kPointwise) {
                 // the weight of a key is SiLU(logit); the sum is divided by the number of visible keys
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    float p = s[c] / (1.f + expf(-s[c]));
-                    if (mask && tx + 16 * c >= vis) p = 0.f;
-                    Ps[(ty + 8 * i) * L::kLdp + tx + 16 * c] = p;
+                for (int c = 0; c < 8; ++c) {
+                    s[i][c] = s[i][c] / (1.f + expf(-s[i][c]));
+                    if (mask && (c < 4 ? c : 28 + c) >= vis) s[i][c] = 0.f;
                 }
-                corr[i] = 1.f;
             } else {
                 if (mask)
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) if (tx + 16 * c >= vis) s[c] = -INFINITY;
-                float mx = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
+                    for (int c = 0; c < 8; ++c) if ((c < 4 ? c : 28 + c) >= vis) s[i][c] = -INFINITY;
+                float mx = fmaxf(fmaxf(fmaxf(s[i][0], s[i][1]), fmaxf(s[i][2], s[i][3])), fmaxf(fmaxf(s[i][4], s[i][5]), fmaxf(s[i][6], s[i][7])));
 #pragma unroll
-                for (int x = 8; x > 0; x >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, x));
-                const float mn = fmaxf(m[i], mx), ref = mn == -INFINITY ? 0.f : mn;
-                corr[i] = exp2f(m[i] - ref);
+                for (int x = 4; x > 0; x >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, x));
+                const float mn = fmaxf(m[i], mx), ref = mn == -INFINITY ? 0.f : mn, corr = exp2f(m[i] - ref);
                 m[i] = mn;
                 float rs = 0.f;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const float p = exp2f(s[c] - ref);
-                    rs += p;
-                    Ps[(ty + 8 * i) * L::kLdp + tx + 16 * c] = p;
+                for (int c = 0; c < 8; ++c) { s[i][c] = exp2f(s[i][c] - ref); rs += s[i][c]; }
+                l[i] = l[i] * corr + rs;                // of this lane's keys; the eight lanes are added up at the end
+                const uint64_t corr2 = dup(corr);
+#pragma unroll
+                for (int c = 0; c < CT / 2; ++c) o[i][c] = mul2(o[i][c], corr2);
+            }
+            float *P = Ks + (ty + 8 * i) * L::kLdp + 4 * tx;
+            *reinterpret_cast<float4 *>(P) = make_float4(s[i][0], s[i][1], s[i][2], s[i][3]);
+            *reinterpret_cast<float4 *>(P + 32) = make_float4(s[i][4], s[i][5], s[i][6], s[i][7]);
+        }
+        __syncwarp();                                   // a row's weights come from, and go to, lanes of one warp
+#pragma unroll 2
+        for (int k = 0; k < 64; k += 4) {
+            float4 p[RT];
+#pragma unroll
+            for (int i = 0; i < RT; ++i) p[i] = *reinterpret_cast<const float4 *>(Ks + (ty + 8 * i) * L::kLdp + k);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                uint64_t v[CT / 2];
+#pragma unroll
+                for (int c = 0; c < CT / 4; ++c) {
+                    const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(Vs + (k + kk) * DH + 4 * tx + 32 * c);
+                    v[2 * c] = w.x; v[2 * c + 1] = w.y;
                 }
-                l[i] = l[i] * corr[i] + rs;           // of this lane's keys; the 16 lanes are added up at the end
+#pragma unroll
+                for (int i = 0; i < RT; ++i) {
+                    const uint64_t pp = dup(kk == 0 ? p[i].x : kk == 1 ? p[i].y : kk == 2 ? p[i].z : p[i].w);
+#pragma unroll
+                    for (int c = 0; c < CT / 2; ++c) o[i][c] = fma2(pp, v[c], o[i][c]);
+                }
             }
         }
-        __syncwarp();                                 // a row's weights come from, and go to, lanes of one warp
-        uint64_t o2[RT][CT] = {};
-        dot_tile<RT, CT, 64, L::kLdp, L::kLdv>(o2, Ps, Vt, ty, tx);
-#pragma unroll
-        for (int i = 0; i < RT; ++i)
-#pragma unroll
-            for (int c = 0; c < CT; ++c) o[i][c] = o[i][c] * corr[i] + fold(o2[i][c]);
+        group_sync();                                   // P and V have been read
+        if (j + G < n_blocks) load_block(j + G);
     }
-    if (n_blocks == 0) __syncthreads();               // Q is there
 
+    // a candidate also sees itself: its own key goes to the first group
 #pragma unroll
     for (int i = 0; i < RT; ++i) {
-        const int r = ty + 8 * i, t = pos0 + r;
-        if constexpr (kPointwise) {
-            l[i] = (float)lim[i];
+        const int r = ty + 8 * i;
+        if constexpr (!kPointwise) {
+#pragma unroll
+            for (int x = 4; x > 0; x >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], x);
         } else {
-#pragma unroll
-            for (int x = 8; x > 0; x >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], x);
+            l[i] = grp == 0 ? (float)lim_of(r) : 0.f;
         }
-        const bool is_cand = t >= sd.causal_end && r < n_q;
-        const int64_t self = (int64_t)(sd.self_row0 + tile.q0 + r) * d + h * DH + tx;
+        const bool own = grp == 0 && r < n_q && pos0 + r >= sd.causal_end;
+        const int64_t self = (int64_t)(sd.self_row0 + tile.q0 + r) * d + h * DH + 4 * tx;
         float dot = 0.f;
-        if (is_cand)
+        if (own)
 #pragma unroll
-            for (int c = 0; c < CT; ++c) dot += Qs[r * L::kLdq + tx + 16 * c] * k_lin[self + 16 * c];
+            for (int c = 0; c < CT / 4; ++c) {
+                const float4 a = *reinterpret_cast<const float4 *>(Qs + r * L::kLdq + 4 * tx + 32 * c);
+                const float4 b = *reinterpret_cast<const float4 *>(k_lin + self + 32 * c);
+                dot += (a.x * b.x + a.y * b.y) + (a.z * b.z + a.w * b.w);
+            }
 #pragma unroll
-        for (int x = 8; x > 0; x >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, x);
-        if (is_cand) {                                // a candidate also sees itself
+        for (int x = 4; x > 0; x >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, x);
+        if (own) {
             float corr = 1.f, p;
             if constexpr (kPointwise) {
                 p = dot / (1.f + expf(-dot));
@@ -353,34 +397,57 @@ f32_attention_kernel(const float *__restrict__ q, const float *__restrict__ k_li
                 corr = exp2f(m[i] - mn);
                 p = exp2f(dot - mn);
                 l[i] = l[i] * corr + p;
+                m[i] = mn;
             }
 #pragma unroll
-            for (int c = 0; c < CT; ++c) o[i][c] = o[i][c] * corr + p * v_lin[self + 16 * c];
+            for (int c = 0; c < CT / 4; ++c) {
+                const ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(v_lin + self + 32 * c);
+                o[i][2 * c] = fma2(dup(p), b.x, mul2(o[i][2 * c], dup(corr)));
+                o[i][2 * c + 1] = fma2(dup(p), b.y, mul2(o[i][2 * c + 1], dup(corr)));
+            }
         }
-        if (r >= n_q) continue;
-        const float inv = 1.f / l[i];
+        // this group's part of the row, in its own tiles
+        if (tx == 0) { Ks[r] = m[i]; Ks[BQ + r] = l[i]; }
 #pragma unroll
-        for (int c = 0; c < CT; ++c) out[(row0 + r) * d + h * DH + tx + 16 * c] = o[i][c] * inv;
+        for (int c = 0; c < CT / 4; ++c) *reinterpret_cast<ulonglong2 *>(Vs + r * DH + 4 * tx + 32 * c) = make_ulonglong2(o[i][2 * c], o[i][2 * c + 1]);
+    }
+    __syncthreads();
+    for (int i = tid; i < n_q * (DH / 4); i += 64 * G) {
+        const int r = i / (DH / 4), c = (i % (DH / 4)) * 4;
+        float M = -INFINITY, lsum = 0.f;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int g = 0; g < G; ++g) M = fmaxf(M, smem[L::kQ + g * (L::kK + L::kV) + r]);
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const float *part = smem + L::kQ + g * (L::kK + L::kV);
+            const float w = exp2f(part[r] - M);
+            const float4 v = *reinterpret_cast<const float4 *>(part + L::kK + r * DH + c);
+            lsum = fmaf(part[BQ + r], w, lsum);
+            acc.x = fmaf(v.x, w, acc.x); acc.y = fmaf(v.y, w, acc.y); acc.z = fmaf(v.z, w, acc.z); acc.w = fmaf(v.w, w, acc.w);
+        }
+        const float inv = 1.f / lsum;
+        *reinterpret_cast<float4 *>(out + (row0 + r) * d + h * DH + c) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
     }
 }
 
-template <int DH, int RT>
+template <int DH, int RT, int G>
 cudaError_t launch_attention(const float *q, const float *k_lin, const float *v_lin, PagedKV paged, const SeqDesc *seqs,
                              const F32Tile *tiles, int n_tiles, int n_heads, int attn_kind, float *out, cudaStream_t stream)
 {
-    constexpr int kBytes = AttnSmem<DH, RT>::kBytes;
+    constexpr int kBytes = AttnSmem<DH, RT, G>::kBytes;
     static PerDeviceValue attr_set;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (!attr_set.get(dev)) {
-        e = cudaFuncSetAttribute(f32_attention_kernel<DH, RT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(f32_attention_kernel<DH, RT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+        e = cudaFuncSetAttribute(f32_attention_kernel<DH, RT, G, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(f32_attention_kernel<DH, RT, G, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
         if (e != cudaSuccess) return e;
         attr_set.set(dev, 1);
     }
-    auto kernel = attn_kind == ATTN_POINTWISE ? f32_attention_kernel<DH, RT, true> : f32_attention_kernel<DH, RT, false>;
-    return launch_dependent(kernel, dim3((unsigned)n_tiles * (unsigned)n_heads), dim3(kThreads), (size_t)kBytes, stream, 1, q, k_lin, v_lin,
+    auto kernel = attn_kind == ATTN_POINTWISE ? f32_attention_kernel<DH, RT, G, true> : f32_attention_kernel<DH, RT, G, false>;
+    return launch_dependent(kernel, dim3((unsigned)n_tiles * (unsigned)n_heads), dim3(64 * G), (size_t)kBytes, stream, 1, q, k_lin, v_lin,
                             paged, seqs, tiles, n_heads, out);
 }
 
@@ -391,8 +458,8 @@ cudaError_t launch_attention(const float *q, const float *k_lin, const float *v_
 // latencies with), the lowest one when none does.
 static int tile_rows_for(int64_t blocks64, int64_t blocks32, int n_sms)
 {
-    if (blocks64 >= 2 * (int64_t)n_sms) return 64;
-    return blocks32 >= 2 * (int64_t)n_sms ? 32 : 16;
+    if (2 * blocks64 >= 3 * (int64_t)n_sms) return 64;
+    return 2 * blocks32 >= 3 * (int64_t)n_sms ? 32 : 16;
 }
 
 cudaError_t launch_gemm_f32(const float *A, const float *W, int64_t M, int N, int K, const Epilogue &epi, int n_sms, cudaStream_t stream,
@@ -432,9 +499,9 @@ cudaError_t launch_attention_f32(const float *q, const float *k_lin, const float
     if (n_tiles == 0) return cudaSuccess;
     *launches += 1;
 #define RELAYGR_ATTN(DH)                                                                                                              \
-    return tile_rows == 64   ? launch_attention<DH, 8>(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, out, stream) \
-           : tile_rows == 32 ? launch_attention<DH, 4>(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, out, stream) \
-                             : launch_attention<DH, 2>(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, out, stream)
+    return tile_rows == 64   ? launch_attention<DH, 8, 2>(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, out, stream) \
+           : tile_rows == 32 ? launch_attention<DH, 4, 4>(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, out, stream) \
+                             : launch_attention<DH, 2, 4>(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, out, stream)
     if (d_head == 32) RELAYGR_ATTN(32);
     if (d_head == 64) RELAYGR_ATTN(64);
 #undef RELAYGR_ATTN
