@@ -37,6 +37,11 @@ namespace relaygr {
 
 namespace {
 
+using tc::add2;
+using tc::fma2;
+using tc::pack2;
+using tc::unpack2;
+
 constexpr int kQTile = 128, kKeys = 64, kDh = 64;
 constexpr int kQBytes = kQTile * kDh * 2;           // 16 KB
 constexpr int kKVBytes = kKeys * kDh * 2;           // 8 KB per K or V tile
@@ -66,26 +71,6 @@ __device__ __forceinline__ float ex2(float x)
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
-}
-// Packed pairs of fp32 (sm_100 executes fma / add on two lanes of a 64-bit register per instruction).
-__device__ __forceinline__ uint64_t pack2(float lo, float hi)
-{
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
-{
-    uint64_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
 }
 // 2^x for a packed pair WITHOUT the XU pipe: x is rounded to the nearest integer n by adding 1.5 * 2^23 (n then sits in
 // the low mantissa bits), a cubic gives 2^(x - n) on [-0.5, 0.5] (relative error 7.5e-5, far below the bf16 rounding of P

@@ -10,6 +10,7 @@
 #include <algorithm>
 
 #include "kernels.cuh"
+#include "tc_common.cuh"
 
 namespace relaygr {
 
@@ -17,28 +18,13 @@ namespace {
 
 constexpr int kThreads = 128;
 
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
-{
-    uint64_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t dup(float v)
-{
-    uint64_t d;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(v));
-    return d;
-}
+using tc::fma2;
+using tc::mul2;
+__device__ __forceinline__ uint64_t dup(float v) { return tc::pack2(v, v); }
 __device__ __forceinline__ float fold(uint64_t v)
 {
     float lo, hi;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+    tc::unpack2(v, lo, hi);
     return lo + hi;
 }
 // 16-byte (or 4-byte) asynchronous copy into shared memory; `bytes` < the size fills the rest with zeros

@@ -80,12 +80,13 @@ int Forward::init_device(int dev, std::string &err)
             int rc = make_tmap_2d_bf16(&wmaps[(size_t)l].qkv, wq, 3 * d, d, d, (uint32_t)kGemmWeightBoxRows, 64);
             rc |= make_tmap_2d_bf16(&wmaps[(size_t)l].kv, wq + d * d, 2 * d, d, d, (uint32_t)kGemmWeightBoxRows, 64);
             rc |= make_tmap_2d_bf16(&wmaps[(size_t)l].wq, wq, d, d, d, (uint32_t)kGemmWeightBoxRows, 64);
-            rc |= make_tmap_2d_bf16(&wmaps[(size_t)l].wo, (const __nv_bfloat16 *)w.w_o + (size_t)l * d * d, d, d, d, (uint32_t)kGemmWeightBoxRows, 64);
-            rc |= make_tmap_2d_bf16(&wmaps[(size_t)l].w1, (const __nv_bfloat16 *)w.w1 + (size_t)l * F * d, F, d, d, (uint32_t)kGemmWeightBoxRows, 64);
-            rc |= make_tmap_2d_bf16(&wmaps[(size_t)l].w2, (const __nv_bfloat16 *)w.w2 + (size_t)l * d * F, d, F, F, (uint32_t)kGemmWeightBoxRows, 64);
+            rc |= make_tmap_2d_bf16(&wmaps[(size_t)l].ffn.wo, (const __nv_bfloat16 *)w.w_o + (size_t)l * d * d, d, d, d, (uint32_t)kGemmWeightBoxRows, 64);
+            rc |= make_tmap_2d_bf16(&wmaps[(size_t)l].ffn.w1, (const __nv_bfloat16 *)w.w1 + (size_t)l * F * d, F, d, d, (uint32_t)kGemmWeightBoxRows, 64);
+            rc |= make_tmap_2d_bf16(&wmaps[(size_t)l].ffn.w2, (const __nv_bfloat16 *)w.w2 + (size_t)l * d * F, d, F, F, (uint32_t)kGemmWeightBoxRows, 64);
             if (ffn_fused_supported((int)d, (int)F)) {
-                rc |= make_tmap_2d_bf16(&wmaps[(size_t)l].w2_wide, (const __nv_bfloat16 *)w.w2 + (size_t)l * d * F, d, F, F, 256, 64);
-                rc |= make_tmap_2d_bf16(&wmaps[(size_t)l].wo_wide, (const __nv_bfloat16 *)w.w_o + (size_t)l * d * d, d, d, d, 256, 64);
+                rc |= make_tmap_2d_bf16(&wmaps[(size_t)l].ffn.w1_half, (const __nv_bfloat16 *)w.w1 + (size_t)l * F * d, F, d, d, 64, 64);
+                rc |= make_tmap_2d_bf16(&wmaps[(size_t)l].ffn.w2_wide, (const __nv_bfloat16 *)w.w2 + (size_t)l * d * F, d, F, F, 256, 64);
+                rc |= make_tmap_2d_bf16(&wmaps[(size_t)l].ffn.wo_wide, (const __nv_bfloat16 *)w.w_o + (size_t)l * d * d, d, d, d, 256, 64);
             }
             if (rc != 0) { err = "tensor-map encoding of the weights failed (pointers must be 16-byte aligned)"; return RELAYGR_E_CUDA; }
         }
@@ -421,16 +422,16 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         if (kTensor && ffn_fused_supported((int)d, (int)F)) {
             // output projection + residual, LayerNorm 2, both feed-forward GEMMs, SiLU and the second residual add in one kernel
             cudaEvent_t pe = prof_begin(stream);
-            e = launch_ffn_fused(lm->w1, lm->w2_wide, om_xm->o[0], xm, w.ln2_g + (size_t)l * d, w.ln2_b + (size_t)l * d,
-                                 w.b1 ? w.b1 + (size_t)l * F : nullptr, w.b2 ? w.b2 + (size_t)l * d : nullptr, &tm_att, &lm->wo_wide,
-                                 w.b_o ? w.b_o + (size_t)l * d : nullptr, M, (int)F, cfg.ln_eps, d_status, stream, &launches);
+            e = launch_ffn_fused(lm->ffn, om_xm->o[0], xm, w.ln2_g + (size_t)l * d, w.ln2_b + (size_t)l * d, w.b1 ? w.b1 + (size_t)l * F : nullptr,
+                                 w.b2 ? w.b2 + (size_t)l * d : nullptr, tm_att, w.b_o ? w.b_o + (size_t)l * d : nullptr, M, (int)F, cfg.ln_eps,
+                                 d_status, stream, &launches);
             prof_end(KC_GEMM, pe, stream);
             if (!ck("output projection + feed-forward")) return RELAYGR_E_CUDA;
             continue;
         }
         Epilogue eo{};
         eo.mode = EPI_RESID; eo.bias = w.b_o ? w.b_o + (size_t)l * d : nullptr; eo.resid = xm; eo.out_f32 = xm;
-        e = gemm(M, att, tm_att, (const T *)w.w_o + (size_t)l * d * d, lm ? &lm->wo : nullptr, *om_xm, d, d, eo);
+        e = gemm(M, att, tm_att, (const T *)w.w_o + (size_t)l * d * d, lm ? &lm->ffn.wo : nullptr, *om_xm, d, d, eo);
         if (!ck("output projection")) return RELAYGR_E_CUDA;
 
         e = layernorm(xm, M, w.ln2_g + (size_t)l * d, w.ln2_b + (size_t)l * d);
@@ -438,12 +439,12 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
 
         Epilogue e1{};
         e1.mode = EPI_STORE; e1.silu = 1; e1.bias = w.b1 ? w.b1 + (size_t)l * F : nullptr; e1.out = hid;
-        e = gemm(M, a, tm_a, (const T *)w.w1 + (size_t)l * F * d, lm ? &lm->w1 : nullptr, om_hid, F, d, e1);
+        e = gemm(M, a, tm_a, (const T *)w.w1 + (size_t)l * F * d, lm ? &lm->ffn.w1 : nullptr, om_hid, F, d, e1);
         if (!ck("FFN 1")) return RELAYGR_E_CUDA;
 
         Epilogue e2{};
         e2.mode = EPI_RESID; e2.bias = w.b2 ? w.b2 + (size_t)l * d : nullptr; e2.resid = xm; e2.out_f32 = xm;
-        e = gemm(M, hid, tm_hid, (const T *)w.w2 + (size_t)l * d * F, lm ? &lm->w2 : nullptr, *om_xm, d, F, e2);
+        e = gemm(M, hid, tm_hid, (const T *)w.w2 + (size_t)l * d * F, lm ? &lm->ffn.w2 : nullptr, *om_xm, d, F, e2);
         if (!ck("FFN 2")) return RELAYGR_E_CUDA;
     }
 

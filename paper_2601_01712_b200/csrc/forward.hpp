@@ -48,7 +48,7 @@ struct Forward {
     int n_sms = 148;
 
     // tensor maps of the weights (bf16 model), one set per layer
-    struct LayerMaps { CUtensorMap qkv, kv, wq, wo, w1, w2, w2_wide, wo_wide; };      // *_wide: boxes of 256 rows (fused out-proj + feed-forward)
+    struct LayerMaps { CUtensorMap qkv, kv, wq; FfnMaps ffn; };
     std::vector<LayerMaps> wmaps;
 
     // tensor maps of the activations (bf16 model): a function of the workspace, the row counts and the pool slab alone, so

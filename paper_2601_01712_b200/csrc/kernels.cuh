@@ -110,19 +110,22 @@ struct GemmOutMaps { CUtensorMap o[3]; CUtensorMap pool; };
 cudaError_t launch_gemm_tc(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmOutMaps &om, int64_t M, int N, int K,
                            const Epilogue &epi, int *err, cudaStream_t stream, int64_t *launches);
 
-// The feed-forward half of a block in one kernel, x <- x + W2 SiLU(W1 LN(x; g, b) + b1) + b2, for the shapes
-// ffn_fused_supported() accepts (d_model = 256, d_ff a multiple of 128 up to 2048): LayerNorm, both GEMMs, SiLU and the
-// residual add without a round trip of the normalised or hidden activations through global memory.  tmW1: W1 [d_ff, 256]
-// in boxes of 128 rows x 64 columns; tmW2: W2 [256, d_ff] in boxes of 256 rows x 64 columns; tmX: the fp32 residual stream
-// [M, 256] in boxes of 32 rows x 32 columns (read by the LayerNorm of the projection form, target of the add-reduction);
-// all with the 128-byte swizzle.
-// With tmAtt / tmWo (both or neither) the attention block's output projection runs first in the same kernel:
-// mid = x + att Wo^T + bo, x <- mid + W2 SiLU(W1 LN(mid) + b1) + b2.  tmAtt: att [M, 256] bf16 in boxes of 128 rows x 64
-// columns; tmWo: Wo [256, 256] in boxes of 256 rows x 64 columns.
+// Everything of a block after the attention in one kernel, for the shapes ffn_fused_supported() accepts (d_model = 256, d_ff a
+// multiple of 128 up to 2048):  mid = x + att Wo^T + bo,  x <- mid + W2 SiLU(W1 LN(mid; g, b) + b1) + b2  on M rows, without a
+// round trip of mid, the normalised or the hidden activations through global memory.  tmAtt: att [M, 256] bf16 in boxes of 128 rows x
+// 64 columns; tmX: the fp32 residual stream x [M, 256] (room for M rounded up to 128 rows) in boxes of 32 rows x 32 columns; all
+// maps with the 128-byte swizzle.
+struct FfnMaps {                                  // one layer's weights, boxes 64 columns wide
+    CUtensorMap w1, w1_half;                      // W1 [d_ff, 256], boxes of 128 and of 64 rows
+    CUtensorMap w2, w2_wide, wo, wo_wide;         // W2 [256, d_ff] and Wo [256, 256], boxes of 128 and (wide) of 256 rows
+};
 bool ffn_fused_supported(int d_model, int d_ff);
-cudaError_t launch_ffn_fused(const CUtensorMap &tmW1, const CUtensorMap &tmW2, const CUtensorMap &tmX, const float *x, const float *g,
-                             const float *b, const float *b1, const float *b2, const CUtensorMap *tmAtt, const CUtensorMap *tmWo,
-                             const float *bo, int64_t M, int d_ff, float eps, int *err, cudaStream_t stream, int64_t *launches);
+cudaError_t launch_ffn_fused(const FfnMaps &w, const CUtensorMap &tmX, float *x, const float *g, const float *b, const float *b1,
+                             const float *b2, const CUtensorMap &tmAtt, const float *bo, int64_t M, int d_ff, float eps, int *err,
+                             cudaStream_t stream, int64_t *launches);
+// (the form for many rows, called by the launcher above)
+cudaError_t launch_ffn_pair(const FfnMaps &w, const CUtensorMap &tmX, const float *x, const float *g, const float *b, const float *b1, const float *b2,
+                            const CUtensorMap &tmAtt, const float *bo, int64_t M, int d_ff, float eps, int *err, cudaStream_t stream);
 
 // Flash-style attention on tcgen05 (d_head = 64) over the work items, then the merge of split items.  attn_kind: ATTN_SOFTMAX, or
 // ATTN_POINTWISE (weights SiLU(q.k / sqrt(d_h)) divided by the number of visible keys).
