@@ -56,12 +56,20 @@ constexpr uint32_t kColS = 0, kColP = 128, kColO = 192;
 constexpr int kPartStride = kDh + 4;                // floats per row of a split partial: m, l, two unused, then O (16-byte aligned rows)
 constexpr float kRowSumLimit = 256.f;               // a block's row sum above this: some p may exceed 2^8 -> redo against a raised maximum
 
+// A work item as the producer hands it to the other warps (nb_keys < 0: no more).
+struct ItemInfo {
+    int nb_keys, n_diag, d0;     // key blocks; blocks of the candidates' own keys, the first of their 64-row groups
+    int blk0, n_q, head, partial_slot;
+    int pos0, row0;              // sequence position and row of the tile's first query
+    int causal_end, n_paged, n_lin, lin_pos0;
+};
+
 struct Bars {
     uint64_t q_full, q_empty;
     uint64_t k_full[kStagesKV], k_empty[kStagesKV], v_full[kStagesKV], v_empty[kStagesKV];
     uint64_t s_full[2], p_full[2], p_free[2];
     uint64_t item_full[2], item_empty[2];
-    int ring[2];                 // item indices on their way from the producer to the other warps (-1: no more)
+    ItemInfo ring[2];            // items on their way from the producer to the other warps
     uint32_t tmem_slot;
     int abort_flag;
 };
@@ -135,7 +143,7 @@ __global__ void __launch_bounds__(192, 2)
 attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKlin,
                     const __grid_constant__ CUtensorMap tmVlin, const __grid_constant__ CUtensorMap tmPool,
                     const AttnItem *__restrict__ items, int n_items, int *__restrict__ next_item, const SeqDesc *__restrict__ seqs,
-                    const int32_t *__restrict__ pt, int n_layers, int layer, int d_model, __nv_bfloat16 *__restrict__ out,
+                    const int32_t *__restrict__ pt, int n_layers, int layer, int d_model, bool early_pages, __nv_bfloat16 *__restrict__ out,
                     float *__restrict__ partial, int *err)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -165,6 +173,62 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         tc::tmem_alloc(&bars->tmem_slot, kTmemCols);
         tc::tmem_relinquish();
     }
+    // The producer (thread 0).  Its item, the item's user and the page table are metadata that was on the device before the call's
+    // first kernel ran to its end, and a rank call only reads its pages: the first item, and there its first K / V tiles, are
+    // fetched while the previous kernel is still running (early_pages; the pages of a pre-infer call are that kernel's output).
+    AttnItem it{};
+    SeqDesc sd{};
+    int nb = 0, d0 = 0, n_diag = 0, n_page_blocks = 0, g = 0, j0 = 0;      // of the item: key blocks in all, its own-key blocks, the user's pages
+    auto draw_item = [&](int n) {                     // this CTA's n-th item into ring slot n & 1; false: no more
+        const int slot = n & 1;
+        const int idx = n == 0 ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(next_item, 1);
+        ItemInfo &info = bars->ring[slot];
+        const bool more = idx < n_items;
+        if (more) {
+            it = items[idx];
+            sd = seqs[it.seq];
+            own_key_blocks(it, sd, d0, n_diag);
+            nb = it.blk1 - it.blk0 + n_diag;
+            n_page_blocks = (sd.n_paged + kKeys - 1) / kKeys;
+            info = ItemInfo{it.blk1 - it.blk0, n_diag, d0, it.blk0, it.n_q, it.head, it.partial_slot, sd.q_pos0 + it.q0, sd.q_row0 + it.q0,
+                            sd.causal_end, sd.n_paged, sd.n_lin, sd.lin_pos0};
+        } else {
+            info.nb_keys = -1;
+        }
+        tc::mbar_arrive(&bars->item_full[slot]);
+        return more;
+    };
+    auto load_kv = [&](int j) {                       // K and V of the item's block j into the next stage
+        const int b = it.blk0 + j, s = g % kStagesKV;
+        const uint32_t par = ((g / kStagesKV) & 1) ^ 1;
+        int ky, vy;
+        const CUtensorMap *mk, *mv;
+        if (j >= nb - n_diag) {                       // the candidates' own rows
+            ky = vy = sd.self_row0 + it.q0 + (d0 + j - (nb - n_diag)) * kKeys;
+            mk = &tmKlin; mv = &tmVlin;
+        } else if (b < n_page_blocks) {
+            const int page = pt[sd.pt_base + b];
+            ky = ((page * n_layers + layer) * 2) * 64; vy = ky + 64;
+            mk = &tmPool; mv = &tmPool;
+        } else {
+            ky = vy = sd.lin_row0 + (b - n_page_blocks) * kKeys;
+            mk = &tmKlin; mv = &tmVlin;
+        }
+        if (!tc::mbar_wait(&bars->k_empty[s], par, err)) return false;
+        tc::mbar_expect_tx(&bars->k_full[s], kKVBytes);
+        tc::tma_load_2d(sK + s * kKVBytes, mk, it.head * kDh, ky, &bars->k_full[s]);
+        if (!tc::mbar_wait(&bars->v_empty[s], par, err)) return false;
+        tc::mbar_expect_tx(&bars->v_full[s], kKVBytes);
+        tc::tma_load_2d(sV + s * kKVBytes, mv, it.head * kDh, vy, &bars->v_full[s]);
+        ++g;
+        return true;
+    };
+    bool more = false;
+    if (threadIdx.x == 0) {
+        more = draw_item(0);
+        if (more && early_pages)
+            for (; j0 < min(kStagesKV, min(nb - n_diag, n_page_blocks - it.blk0)) && load_kv(j0);) ++j0;
+    }
     grid_launch_dependents();
     grid_dependency_wait();                                       // from here on: data of earlier kernels
     if (threadIdx.x == 0) bars->abort_flag = *reinterpret_cast<volatile int *>(err);
@@ -174,67 +238,35 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     const uint32_t tmem_base = bars->tmem_slot;
     const bool live = bars->abort_flag == 0;                      // an earlier kernel gave up: do not pile on
 
-    // Every role walks the same sequence of items: the producer draws an index from the launch's counter and passes it on
-    // through a two-slot ring.  `n` counts this CTA's items, `g` its key blocks since the kernel began: the stage of a K / V
-    // tile, the S / P buffer of a block and the phase of every barrier follow from g, so the pipelines run on across items.
-    // take_item(n): the index of this CTA's n-th item, or -1 when the list is exhausted (consumer side of the ring).
+    // Every role walks the same sequence of items: the producer draws an index (the first is the CTA's own number, the others come from
+    // the launch's counter) and passes the item on through a two-slot ring in shared memory, so that the other warps do not repeat its
+    // chain of look-ups.  `n` counts this CTA's items, `g` its key blocks since the kernel began: the stage of a K / V tile, the S / P
+    // buffer of a block and the phase of every barrier follow from g, so the pipelines run on across items.
+    // take_item(n): this CTA's n-th item (consumer side of the ring; nb_keys < 0: the list is exhausted, or a wait ran out).
     auto take_item = [&](int n, bool &ok) {
         const int slot = n & 1;
         ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->item_full[slot], (n >> 1) & 1, err));
-        const int idx = ok ? bars->ring[slot] : -1;
+        ItemInfo info = bars->ring[slot];
+        if (!ok) info.nb_keys = -1;
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(&bars->item_empty[slot]);
-        return idx;
+        return info;
     };
 
     if (!live) {
+        if (threadIdx.x == 0)                                     // what was requested above lands before the CTA ends
+            for (int s = 0; s < j0; ++s) { tc::mbar_wait(&bars->k_full[s], 0, err); tc::mbar_wait(&bars->v_full[s], 0, err); }
     } else if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer
         if (lane == 0) {
-            int g = 0;
-            for (int n = 0;; ++n) {
-                const int slot = n & 1;
-                if (!tc::mbar_wait(&bars->item_empty[slot], ((n >> 1) & 1) ^ 1, err)) break;
-                int idx = atomicAdd(next_item, 1);
-                if (idx >= n_items) idx = -1;
-                bars->ring[slot] = idx;
-                tc::mbar_arrive(&bars->item_full[slot]);
-                if (idx < 0) break;
-                const AttnItem it = items[idx];
-                const SeqDesc sd = seqs[it.seq];
-                const int nb = it.blk1 - it.blk0;
-                int d0, n_diag;
-                own_key_blocks(it, sd, d0, n_diag);
-                const int n_paged_blocks = (sd.n_paged + kKeys - 1) / kKeys;      // = the user's page count
+            for (int n = 0; more; ++n) {
                 if (!tc::mbar_wait(&bars->q_empty, (n & 1) ^ 1, err)) break;       // the previous item's last Q K^T has read Q
                 tc::mbar_expect_tx(&bars->q_full, kQBytes);
                 tc::tma_load_2d(sQ, &tmQ, it.head * kDh, sd.q_row0 + it.q0, &bars->q_full);
-                bool ok = true;
-                for (int j = 0; j < nb + n_diag; ++j, ++g) {
-                    const int b = it.blk0 + j;
-                    const int s = g % kStagesKV;
-                    const uint32_t par = ((g / kStagesKV) & 1) ^ 1;
-                    int ky, vy;
-                    const CUtensorMap *mk, *mv;
-                    if (j >= nb) {                                       // the candidates' own rows
-                        ky = vy = sd.self_row0 + it.q0 + (d0 + j - nb) * kKeys;
-                        mk = &tmKlin; mv = &tmVlin;
-                    } else if (b < n_paged_blocks) {
-                        const int page = pt[sd.pt_base + b];
-                        ky = ((page * n_layers + layer) * 2) * 64; vy = ky + 64;
-                        mk = &tmPool; mv = &tmPool;
-                    } else {
-                        ky = vy = sd.lin_row0 + (b - n_paged_blocks) * kKeys;
-                        mk = &tmKlin; mv = &tmVlin;
-                    }
-                    if (!(ok = tc::mbar_wait(&bars->k_empty[s], par, err))) break;
-                    tc::mbar_expect_tx(&bars->k_full[s], kKVBytes);
-                    tc::tma_load_2d(sK + s * kKVBytes, mk, it.head * kDh, ky, &bars->k_full[s]);
-                    if (!(ok = tc::mbar_wait(&bars->v_empty[s], par, err))) break;
-                    tc::mbar_expect_tx(&bars->v_full[s], kKVBytes);
-                    tc::tma_load_2d(sV + s * kKVBytes, mv, it.head * kDh, vy, &bars->v_full[s]);
-                }
-                if (!ok) break;
+                int j = n == 0 ? j0 : 0;
+                while (j < nb && load_kv(j)) ++j;
+                if (j < nb || !tc::mbar_wait(&bars->item_empty[(n + 1) & 1], (((n + 1) >> 1) & 1) ^ 1, err)) break;
+                more = draw_item(n + 1);
             }
         }
     } else if (warp == 1) {
@@ -243,15 +275,11 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         constexpr uint32_t idesc_qk = tc::make_idesc(128, kKeys, 0, 0);   // Q, K both K-major
         constexpr uint32_t idesc_pv = tc::make_idesc(128, kDh, 0, 1);     // P from TMEM, V MN-major
         const uint64_t qdesc = tc::smem_desc_sw128(tc::smem_u32(sQ));
-        int g = 0;
         bool ok = true;
         for (int n = 0; ok; ++n) {
-            const int idx = take_item(n, ok);
-            if (idx < 0) break;
-            const AttnItem it = items[idx];
-            int d0, n_diag;
-            own_key_blocks(it, seqs[it.seq], d0, n_diag);
-            const int nb = it.blk1 - it.blk0 + n_diag;         // key blocks of the item, the candidates' own included
+            const ItemInfo info = take_item(n, ok);
+            if (info.nb_keys < 0) break;
+            const int nb = info.nb_keys + info.n_diag;         // key blocks of the item, the candidates' own included
             ok = tc::mbar_wait(&bars->q_full, n & 1, err);
             if (!ok) break;
             auto issue_qk = [&](int j) {        // S[(g + j) & 1] = Q K(j)^T; the item's last one also hands Q back
@@ -306,27 +334,22 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         const int quad = warp & 3;
         const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
         const float c = 0.125f * 1.4426950408889634f;        // 1/sqrt(64) * log2(e)
-        int g = 0;
         bool ok = true;
         for (int n = 0; ok; ++n) {
-        const int idx = take_item(n, ok);
-        if (idx < 0) break;
-        const AttnItem it = items[idx];
-        const SeqDesc sd = seqs[it.seq];
-        int d0, n_diag;
-        own_key_blocks(it, sd, d0, n_diag);
-        const int nb_keys = it.blk1 - it.blk0, nb = nb_keys + n_diag;     // the candidates' own keys come last
-        const int n_paged_blocks = (sd.n_paged + kKeys - 1) / kKeys;      // = the user's page count
+        const ItemInfo it = take_item(n, ok);
+        if (it.nb_keys < 0) break;
+        const int nb_keys = it.nb_keys, nb = nb_keys + it.n_diag;     // the candidates' own keys come last
+        const int n_paged_blocks = (it.n_paged + kKeys - 1) / kKeys;      // = the user's page count
         const int r = quad * 32 + lane;                      // row of the tile this thread owns
-        const int tpos = sd.q_pos0 + it.q0 + r;              // sequence position of the row
-        const bool is_cand = tpos >= sd.causal_end;
-        const int lim = is_cand ? sd.causal_end - 1 : tpos;  // last visible key position
-        const int tile_min_lim = (sd.q_pos0 + it.q0 >= sd.causal_end) ? sd.causal_end - 1 : sd.q_pos0 + it.q0;
+        const int tpos = it.pos0 + r;                        // sequence position of the row
+        const bool is_cand = tpos >= it.causal_end;
+        const int lim = is_cand ? it.causal_end - 1 : tpos;  // last visible key position
+        const int tile_min_lim = it.pos0 >= it.causal_end ? it.causal_end - 1 : it.pos0;
         // Blocks [0, n_clean) of the user are complete (64 keys) and visible to every row of the tile: no mask, and none of
         // the per-block position arithmetic, which otherwise sits as a dependent chain between publishing P(j) and polling
         // for S(j + 1).  Pages come first in the block order, then the 64-row groups of linear keys.
-        int n_clean = min(sd.n_paged / kKeys, (tile_min_lim + 1) / kKeys);
-        if (n_clean == n_paged_blocks && tile_min_lim >= sd.lin_pos0) n_clean += min(sd.n_lin, tile_min_lim + 1 - sd.lin_pos0) / kKeys;
+        int n_clean = min(it.n_paged / kKeys, (tile_min_lim + 1) / kKeys);
+        if (n_clean == n_paged_blocks && tile_min_lim >= it.lin_pos0) n_clean += min(it.n_lin, tile_min_lim + 1 - it.lin_pos0) / kKeys;
         n_clean -= it.blk0;                                   // relative to the item's first block
         float m = -INFINITY, l = 0.f;
         // a warp whose 32 rows all lie past the tile's last row keeps the hand-shakes going but takes no exponentials:
@@ -342,8 +365,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 const int blk = it.blk0 + j;
                 const bool paged = blk < n_paged_blocks;
                 const int kidx0 = paged ? blk * kKeys : (blk - n_paged_blocks) * kKeys;    // index of the block's first key in its source
-                const int kpos0 = paged ? kidx0 : sd.lin_pos0 + kidx0;                     // its sequence position
-                const int n_valid = min(kKeys, (paged ? sd.n_paged : sd.n_lin) - kidx0);
+                const int kpos0 = paged ? kidx0 : it.lin_pos0 + kidx0;                     // its sequence position
+                const int n_valid = min(kKeys, (paged ? it.n_paged : it.n_lin) - kidx0);
                 need_mask = (n_valid < kKeys) || (kpos0 + kKeys - 1 > tile_min_lim);
                 jmax = min(n_valid, lim - kpos0 + 1);
             }
@@ -372,7 +395,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             if (own_keys) {
                 // a candidate row of this 64-row group sees its own key (the diagonal of the block) and nothing else;
                 // every other row of the tile sees nothing here
-                const int own = is_cand ? r - (d0 + j - nb_keys) * kKeys : -1;
+                const int own = is_cand ? r - (it.d0 + j - nb_keys) * kKeys : -1;
 #pragma unroll
                 for (int i = 0; i < 32; ++i) {
                     s0[i] = select_eq(i, own, s0[i], kPointwise ? 0u : 0xff800000u);
@@ -492,39 +515,37 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         if (ok && warp_live) {
             float o[kDh];
             if (nb > 0) {
+                uint32_t ov[2][32];
+                tc::tmem_ld32(lane_addr + kColO, ov[0]);
+                tc::tmem_ld32(lane_addr + kColO + 32, ov[1]);
+                tc::tmem_ld_wait();
 #pragma unroll
-                for (int cc = 0; cc < kDh; cc += 16) {
-                    uint32_t ov[16];
-                    tc::tmem_ld16(lane_addr + kColO + cc, ov);
-                    tc::tmem_ld_wait();
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) o[cc + i] = __uint_as_float(ov[i]);
-                }
+                for (int i = 0; i < kDh; ++i) o[i] = __uint_as_float(ov[i / 32][i % 32]);
             } else {
 #pragma unroll
                 for (int i = 0; i < kDh; ++i) o[i] = 0.f;
             }
             const bool row_ok = r < it.n_q;
-            const int64_t row = (int64_t)sd.q_row0 + it.q0 + r;
+            const int64_t row = (int64_t)it.row0 + r;
             if constexpr (kPointwise) {
                 // the normaliser is the number of keys the row may see (every key position below its limit, plus itself for
                 // a candidate); a split item hands it over as l with m = 0, so that the merge of partials needs no change
-                const float n_seen = (float)(is_cand ? sd.causal_end + 1 : tpos + 1);
+                const float n_seen = (float)(is_cand ? it.causal_end + 1 : tpos + 1);
                 m = 0.f;
                 l = (it.partial_slot < 0 || it.blk0 == 0) ? n_seen : 0.f;
             }
             if (row_ok) {
                 if (it.partial_slot < 0) {
                     const float inv = 1.f / l;
-                    uint4 *dst = reinterpret_cast<uint4 *>(out + row * d_model + it.head * kDh);
+                    // 32 bytes a store, one whole sector: a lane owns a row, so every store of a warp touches 32 lines
+                    __nv_bfloat16 *dst = out + row * d_model + it.head * kDh;
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        uint4 w4;
-                        w4.x = tc::pack_bf16(o[8 * i] * inv, o[8 * i + 1] * inv);
-                        w4.y = tc::pack_bf16(o[8 * i + 2] * inv, o[8 * i + 3] * inv);
-                        w4.z = tc::pack_bf16(o[8 * i + 4] * inv, o[8 * i + 5] * inv);
-                        w4.w = tc::pack_bf16(o[8 * i + 6] * inv, o[8 * i + 7] * inv);
-                        dst[i] = w4;
+                    for (int i = 0; i < 4; ++i) {
+                        uint32_t w[8];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) w[e] = tc::pack_bf16(o[16 * i + 2 * e] * inv, o[16 * i + 2 * e + 1] * inv);
+                        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + 16 * i), "r"(w[0]), "r"(w[1]),
+                                     "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
                     }
                 } else {
                     float4 *dst = reinterpret_cast<float4 *>(partial + ((size_t)it.partial_slot * kQTile + r) * kPartStride);
@@ -578,7 +599,7 @@ attention_merge_kernel(const AttnMerge *__restrict__ merges, const SeqDesc *__re
 
 cudaError_t launch_attention_tc(const CUtensorMap &tmQ, const CUtensorMap &tmK, const CUtensorMap &tmV, const CUtensorMap &tmPool,
                                 const AttnItem *items, int n_items, const AttnMerge *merges, int n_merges, const SeqDesc *seqs,
-                                const int32_t *pt, int n_layers, int layer, int d_model, int attn_kind, __nv_bfloat16 *out,
+                                const int32_t *pt, int n_layers, int layer, int d_model, int attn_kind, bool early_pages, __nv_bfloat16 *out,
                                 float *partial, int *next_item, int n_sms, int *err, cudaStream_t stream, int64_t *launches)
 {
     if (n_items == 0) return cudaSuccess;
@@ -596,7 +617,7 @@ cudaError_t launch_attention_tc(const CUtensorMap &tmQ, const CUtensorMap &tmK, 
     auto kernel = attn_kind == ATTN_POINTWISE ? attention_tc_kernel<true> : attention_tc_kernel<false>;
     const int grid = std::min(n_items, 2 * std::max(1, n_sms));       // two CTAs per SM, each drawing items until none is left
     cudaError_t e = launch_dependent(kernel, dim3(grid), dim3(192), (size_t)kSmemBytes, stream, 1, tmQ, tmK, tmV, tmPool, items,
-                                     n_items, next_item, seqs, pt, n_layers, layer, d_model, out, partial, err);
+                                     n_items, next_item, seqs, pt, n_layers, layer, d_model, early_pages, out, partial, err);
     if (e != cudaSuccess || n_merges == 0) return e;
     *launches += 1;
     return launch_dependent(attention_merge_kernel, dim3(n_merges, kQTile / 8), dim3(256), 0, stream, 1, merges, seqs, partial, d_model, out);

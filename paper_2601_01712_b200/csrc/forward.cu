@@ -203,12 +203,13 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     constexpr bool kTensor = sizeof(T) == 2;      // bf16 model: GEMMs and attention run on the tensor cores
     const bool preinfer = call.mode == MODE_PREINFER;
     const int64_t n_scores = (!preinfer && call.score_off) ? call.score_off[B] : 0;
-    // The last layer of a rank / full-inference call (bf16 model): only the candidates' hidden states are read afterwards, so
-    // every other row needs nothing but its K and V there.  The candidate rows are moved together and the layer's query
-    // projection, attention, output projection and feed-forward run on those rows alone.
-    // (The fp32 model does so in full inference, where the prefix rows it saves are most of the work; the few short-term rows of a
-    // rank call do not pay for the two launches.)
-    const bool compact_last = !preinfer && (kTensor || call.mode == MODE_FULL);
+    // In the last layer of a rank / full-inference call only the candidates' hidden states are read afterwards: its attention runs on
+    // their rows alone.  What follows may run on them alone too, once they have been moved together (and their query projection
+    // made a launch of its own): worth it when the other rows' share of the linear maps (4 d^2 + 4 d F FLOPs a row at about
+    // 0.6 PFLOP/s) costs more than two more launches (10 us) and the copy (12 d bytes a candidate at about 4 TB/s) - full
+    // inference with its prefix rows, not a rank call with its few short-term rows.
+    const bool cand_last = !preinfer && n_scores > 0;
+    const bool compact_last = cand_last && (double)(R - n_scores) * (4.0 * d * d + 4.0 * d * F) / 0.6e15 > 10e-6 + (double)n_scores * 12.0 * d / 4e12;
 
     // ---- metadata blob: row_off | seg_off x3 | score_off | SeqDesc[] | page table | attention items [| the same for the last layer]
     std::vector<int32_t> blob;
@@ -242,15 +243,14 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     };
     {
         put_work(call.seqs, items, merges, tiles, o_items, o_merges, tile_rows);
-        if (compact_last && n_scores > 0) {
+        if (cand_last) {
             seqs_c = call.seqs;
             for (int u = 0; u < B; ++u) {
                 SeqDesc &c = seqs_c[(size_t)u];
-                c.self_row0 = c.score_row0;           // where the candidates' own K / V rows (and their x, a rows) are
-                c.q_row0 = call.score_off[u];         // where their rows are once moved together
+                c.self_row0 = c.q_row0 = c.score_row0;      // where the candidates' rows are: their own K / V, and x, a, q, att
+                if (compact_last) c.q_row0 = c.score_row0 = call.score_off[u];      // ... of those, x, a, q and att are moved together
                 c.n_q = c.n_score;
                 c.q_pos0 = c.causal_end;              // every row is a candidate
-                c.score_row0 = call.score_off[u];
             }
             o_seq_c = put(reinterpret_cast<const int32_t *>(seqs_c.data()), (size_t)B * (sizeof(SeqDesc) / 4));
             put_work(seqs_c, items_c, merges_c, tiles_c, o_items_c, o_merges_c, tile_rows_c);
@@ -314,7 +314,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
             om_qkv.pool = om_qkv.o[0];
         om_hid.o[1] = om_hid.o[2] = om_hid.pool = om_hid.o[0];
         om_x.o[1] = om_x.o[2] = om_x.pool = om_x.o[0];
-        if (compact_last && n_scores > 0) {
+        if (compact_last) {
             trc |= make_tmap_2d_bf16(&tm_a_c, a_c, (uint64_t)n_scores, (uint64_t)d, (uint64_t)d, 128, 64);
             trc |= make_tmap_2d_f32(&om_x_c.o[0], x_c, (uint64_t)n_scores, (uint64_t)d, (uint64_t)d, 32, 32);
             om_x_c.o[1] = om_x_c.o[2] = om_x_c.pool = om_x_c.o[0];
@@ -384,14 +384,16 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         if (!ck("QKV projection")) return RELAYGR_E_CUDA;
         if (preinfer && last) break;
 
-        if (last && compact_last) {
-            // move the candidates' rows of x and of LN1(x) together, then project their queries
-            M = n_scores; xm = x_c; om_xm = &om_x_c;
+        if (last && cand_last) {
             seqs_m = reinterpret_cast<const SeqDesc *>(meta + o_seq_c);
             items_m = reinterpret_cast<const AttnItem *>(meta + o_items_c);
             merges_m = reinterpret_cast<const AttnMerge *>(meta + o_merges_c);
             tiles_m = reinterpret_cast<const F32Tile *>(meta + o_items_c); tile_rows = tile_rows_c;
             n_items_m = (int)(kTensor ? items_c.size() : tiles_c.size()); n_merges_m = (int)merges_c.size();
+        }
+        if (last && compact_last) {
+            // move the candidates' rows of x and of LN1(x) together, then project their queries
+            M = n_scores; xm = x_c; om_xm = &om_x_c;
             cudaEvent_t pe = prof_begin(stream);
             e = launch_compact_rows<T>(x, a, seqs_m, B, meta + o_score, n_scores, d, x_c, a_c, stream, &launches);
             prof_end(KC_LAYERNORM, pe, stream);
@@ -411,7 +413,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
             cudaEvent_t pe = prof_begin(stream);
             if constexpr (kTensor)
                 e = launch_attention_tc(tm_q, tm_k, tm_v, tm_pool, items_m, n_items_m, merges_m, n_merges_m, seqs_m, meta + o_pt, L,
-                                        l, d, cfg.attn_kind, att, reinterpret_cast<float *>(ws + lay.partial),
+                                        l, d, cfg.attn_kind, call.mode == MODE_RANK, att, reinterpret_cast<float *>(ws + lay.partial),
                                         reinterpret_cast<int *>(ws + lay.meta) + o_ctr + l, n_sms, d_status, stream, &launches);
             else
                 e = launch_attention_f32(q, kl, vl, paged, seqs_m, tiles_m, n_items_m, tile_rows, H, cfg.d_head, cfg.attn_kind, att, stream, &launches);

@@ -131,11 +131,13 @@ cudaError_t launch_ffn_pair(const FfnMaps &w, const CUtensorMap &tmX, const floa
 // ATTN_POINTWISE (weights SiLU(q.k / sqrt(d_h)) divided by the number of visible keys).
 // tmQ: [rows, d] box 128 x 64; tmK / tmV: the call's transient K / V rows, box 64 x 64; tmPool: the pool
 // slab viewed as [pages * L * 2 * 64, d], box 64 x 64 (pass tmK when the call has no pool).
-// The kernel is persistent: min(n_items, 2 x n_sms) CTAs draw item indices from *next_item, a device counter that must be
-// zero when the kernel starts and belongs to this launch alone (the kernel leaves it non-zero).
+// The kernel is persistent: min(n_items, 2 x n_sms) CTAs start with the item of their own number and draw the others from *next_item,
+// a device counter that must be zero when the kernel starts and belongs to this launch alone (the kernel leaves it non-zero).
+// items, seqs, pt and the counter must be in place when the kernel BEFORE this one on the stream starts; early_pages: so are the
+// pages (the call does not write them).
 cudaError_t launch_attention_tc(const CUtensorMap &tmQ, const CUtensorMap &tmK, const CUtensorMap &tmV, const CUtensorMap &tmPool,
                                 const AttnItem *items, int n_items, const AttnMerge *merges, int n_merges, const SeqDesc *seqs,
-                                const int32_t *pt, int n_layers, int layer, int d_model, int attn_kind, __nv_bfloat16 *out,
+                                const int32_t *pt, int n_layers, int layer, int d_model, int attn_kind, bool early_pages, __nv_bfloat16 *out,
                                 float *partial, int *next_item, int n_sms, int *err, cudaStream_t stream, int64_t *launches);
 
 }  // namespace relaygr

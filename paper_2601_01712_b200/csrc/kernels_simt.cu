@@ -119,8 +119,10 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 gather_ln_kernel(const T *__restrict__ emb, int64_t vocab, int d, RowSource src, int64_t n_rows,
                  const float *__restrict__ g, const float *__restrict__ b, float eps, float *__restrict__ x, T *__restrict__ a, int *err)
 {
-    grid_launch_dependents();
+    // The first kernel of a call lets the next one start only after its own wait: the call's metadata (uploaded before it) and the
+    // pool pages a rank call reads are then in place for every later kernel, which may fetch them before its own wait.
     grid_dependency_wait();
+    grid_launch_dependents();
     const int64_t row0 = ((int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5)) * ROWS;
     const int lane = threadIdx.x & 31;
     if (row0 >= n_rows) return;
