@@ -136,7 +136,7 @@ WorkspaceLayout Forward::layout(int64_t rows, int64_t users, int64_t pages) cons
     l.partial = take(l.partial_bytes);
     const size_t n_items = (size_t)cfg.n_heads * ((size_t)rows / 128 + (size_t)users + 1) + 2 * (size_t)kMaxSplitTiles;
     // two descriptor arrays and two work lists: all rows, and the candidate rows of the last layer
-    l.meta_bytes = 4 * (((size_t)users + 1) * 5 + 2 * (size_t)users * (sizeof(SeqDesc) / 4) + (size_t)pages + 2 * n_items * (sizeof(AttnItem) / 4) + (size_t)cfg.n_layers + 64);
+    l.meta_bytes = 4 * (((size_t)users + 1) * 5 + 2 * (size_t)users * (sizeof(SeqDesc) / 4) + (size_t)pages + 2 * n_items * (sizeof(AttnItem) / 4) + (size_t)rows / 32 + 1 + (size_t)cfg.n_layers + 64);
     l.meta = take(l.meta_bytes);
     l.total = at;
     return l;
@@ -223,6 +223,18 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     const size_t o_score = call.score_off ? put(call.score_off, (size_t)B + 1) : 0;
     const size_t o_seq = put(reinterpret_cast<const int32_t *>(call.seqs.data()), (size_t)B * (sizeof(SeqDesc) / 4));
     const size_t o_pt = call.page_table.empty() ? 0 : put(call.page_table.data(), call.page_table.size());
+    size_t o_runs = 0;
+    if (kTensor && preinfer) {                    // see Epilogue::page_runs
+        std::vector<int32_t> runs((size_t)((R + 31) / 32), -1);
+        for (int u = 0; u < B; ++u) {
+            const SeqDesc &sd = call.seqs[(size_t)u];
+            for (int64_t g = (sd.q_row0 + 31) / 32; g * 32 + 32 <= (int64_t)sd.q_row0 + sd.n_q; ++g) {
+                const int t = (int)(g * 32 - sd.q_row0), slot = t & 63;
+                if (slot <= 32 && (t + 32 < sd.n_q || slot == 32)) runs[(size_t)g] = call.page_table[(size_t)(sd.pt_base + (t >> 6))] * 64 + slot;
+            }
+        }
+        o_runs = put(runs.data(), runs.size());
+    }
     std::vector<AttnItem> items, items_c;
     std::vector<AttnMerge> merges, merges_c;
     std::vector<SeqDesc> seqs_c;                  // the candidates of each user as rows of their own (last layer)
@@ -377,7 +389,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         if (call.pool_slab) {
             paged.slab = call.pool_slab; paged.pt = meta + o_pt; paged.n_layers = L; paged.d_model = d; paged.layer = l;
         }
-        if (preinfer) ep.paged = paged;
+        if (preinfer) { ep.paged = paged; ep.page_runs = meta + o_runs; }
         const T *Wqkv = (const T *)w.w_qkv + ((size_t)l * 3 * d + ep.col0) * d;
         lm = kTensor ? &wmaps[(size_t)l] : nullptr;
         e = gemm(R, a, tm_a, Wqkv, lm ? (kv_only ? &lm->kv : &lm->qkv) : nullptr, om_qkv, 3 * d - ep.col0, d, ep);

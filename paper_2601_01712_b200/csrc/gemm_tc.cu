@@ -33,6 +33,7 @@ constexpr int kThreads = 32 * (2 + kEpiWarps);
 constexpr int kABytes = BM * BK * 2;
 constexpr int kPatchBytes = 32 * 128;                                // one staged store: 32 rows x 128 bytes
 constexpr int kPatches = 1;                                          // per warp (a store has read its patch long before the next is packed)
+constexpr int kMaxBias = 4096;                                       // output columns whose bias fits the shared copy
 
 // A tile is 128 x BN per CTA.  CTAS = 1: BN = 128 (or 256), the CTA loads all of A and B.  CTAS = 2: a pair of CTAs works on
 // 256 x 256 with one tcgen05 cta_group::2 MMA stream issued by the even CTA; each CTA loads its 128 rows of A and half
@@ -44,8 +45,8 @@ template <int BN, int CTAS> struct Cfg {
     static constexpr int kStage = kABytes + kBBytes;
     static constexpr int kStages = (CTAS == 1 && BN == 256) ? 3 : 5;
     static constexpr int kOffPatch = kStages * kStage;                                    // 1024-byte aligned: stages are
-    static constexpr int kOffBias = kOffPatch + kEpiWarps * kPatches * kPatchBytes;       // per warp BN / 2 floats
-    static constexpr int kOffRowOff = kOffBias + kEpiWarps * (BN / 2) * 4;                // per warp 32 x int64
+    static constexpr int kOffBias = kOffPatch + kEpiWarps * kPatches * kPatchBytes;       // kMaxBias floats
+    static constexpr int kOffRowOff = kOffBias + kMaxBias * 4;                            // per warp 32 x int64
     static constexpr int kOffBars = kOffRowOff + kEpiWarps * 32 * 8;
     static constexpr int kSmemBytes = kOffBars + 256 /*barriers*/ + 1024 /*alignment slack*/;
     static constexpr uint32_t kTmemCols = 2 * BN;
@@ -93,9 +94,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int kblocks = K / BK;
     const int n_tiles_n = N / BN;
-    const int64_t n_tiles = ((M + BM * CTAS - 1) / (BM * CTAS)) * n_tiles_n;       // tiles of the CTA (or the pair)
+    const int n_tiles = (int)((M + BM * CTAS - 1) / (BM * CTAS)) * n_tiles_n;      // tiles of the CTA (or the pair)
     const uint32_t rank = CTAS == 2 ? tc::cluster_ctarank() : 0;                     // this CTA's half of a pair tile
-    const int64_t worker = blockIdx.x / CTAS, n_workers = gridDim.x / CTAS;
+    const int worker = blockIdx.x / CTAS, n_workers = gridDim.x / CTAS;
     const bool leader = rank == 0;                                                   // issues the MMAs, owns full / acc_empty
 
     // set-up that touches nothing earlier kernels wrote; it may run while the previous kernel is still finishing
@@ -126,9 +127,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (lane == 0) {
             uint32_t it = 0;
             bool ok = true;
-            for (int64_t t = worker; t < n_tiles && ok; t += n_workers) {
-                const int m0 = (int)(t / n_tiles_n) * (BM * CTAS) + (int)rank * BM;
-                const int n0 = (int)(t % n_tiles_n) * BN + (int)rank * (BN / CTAS);
+            for (int t = worker; t < n_tiles && ok; t += n_workers) {
+                const int m0 = (t / n_tiles_n) * (BM * CTAS) + (int)rank * BM;
+                const int n0 = (t % n_tiles_n) * BN + (int)rank * (BN / CTAS);
                 for (int kb = 0; kb < kblocks; ++kb, ++it) {
                     const int s = it % STAGES;
                     ok = tc::mbar_wait(&bars->empty[s], ((it / STAGES) & 1) ^ 1, err);
@@ -155,7 +156,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             constexpr uint32_t idesc = tc::make_idesc(BM * CTAS, BN, 0, 0);
             uint32_t it = 0, ti = 0;
             bool ok = true;
-            for (int64_t t = worker; t < n_tiles && ok; t += n_workers, ++ti) {
+            for (int t = worker; t < n_tiles && ok; t += n_workers, ++ti) {
                 const uint32_t as = ti & 1;
                 ok = tc::mbar_wait(&bars->acc_empty[as], ((ti >> 1) & 1) ^ 1, err);     // the epilogue has drained this accumulator
                 if (!ok) break;
@@ -195,7 +196,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int half = ew >> 2;                           // columns (BN/2)*half .. +BN/2-1 of the tile, 64 at a time
         constexpr int kColsPerWarp = BN / 2;
         uint8_t *patches = smem + C::kOffPatch + ew * (kPatches * kPatchBytes);
-        float *bias_s = reinterpret_cast<float *>(smem + C::kOffBias) + ew * kColsPerWarp;
+        // the whole bias once, under the first tile's loads: a look-up per tile would be on the epilogue's path
+        float *bias_s = reinterpret_cast<float *>(smem + C::kOffBias);
+        const bool bias_staged = epi.bias && N <= kMaxBias;
+        if (bias_staged) {
+            for (int i = threadIdx.x - 64; i < N; i += 32 * kEpiWarps) bias_s[i] = epi.bias[i];
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
+        }
         int64_t *rowoff = reinterpret_cast<int64_t *>(smem + C::kOffRowOff) + ew * 32;
         const bool scatter = epi.mode == EPI_QKV && epi.paged.slab != nullptr;
         uint32_t pp = 0;                                    // the patch the next staged store fills
@@ -219,37 +226,40 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         uint32_t ti = 0;
         bool ok = true;
         const uint32_t acc_empty_bar = CTAS == 2 ? tc::cluster_addr(&bars->acc_empty[0], 0) : tc::smem_u32(&bars->acc_empty[0]);
-        for (int64_t t = worker; t < n_tiles && ok; t += n_workers, ++ti) {
-            const int64_t m0 = (t / n_tiles_n) * (BM * CTAS) + rank * BM;
-            const int n_w = (int)(t % n_tiles_n) * BN + half * kColsPerWarp;      // first column of this warp's part
+        for (int t = worker; t < n_tiles && ok; t += n_workers, ++ti) {
+            const int64_t m0 = (int64_t)(t / n_tiles_n) * (BM * CTAS) + rank * BM;
+            const int n_w = (t % n_tiles_n) * BN + half * kColsPerWarp;      // first column of this warp's part
             const uint32_t as = ti & 1;
             const int64_t m_base = m0 + quad * 32;
             const int64_t m = m_base + lane;
-            // before the accumulator is ready: this warp's slice of the bias, and for K / V rows of a pre-infer call
-            // (they go straight into the user's pages) the offset of (page, K, slot) per row
-            if (epi.bias) {
+            float *bias_w = bias_s + (bias_staged ? n_w : ew * kColsPerWarp);      // this warp's slice of the bias
+            if (epi.bias && !bias_staged) {
 #pragma unroll
-                for (int c = 0; c < kColsPerWarp; c += 32) bias_s[c + lane] = epi.bias[n_w + c + lane];
+                for (int c = 0; c < kColsPerWarp; c += 32) bias_w[c + lane] = epi.bias[n_w + c + lane];
             }
+            // before the accumulator is ready, for K / V rows of a pre-infer call (they go straight into the user's pages): where in
+            // the pool the warp's 32 rows are, if they are 32 consecutive slots of one page (the table says so), else the offset
+            // of (page, K, slot) row by row
             int last_slot = -1, page = 0;
             const bool paged_tile = scatter && epi.col0 + n_w + kColsPerWarp - 1 >= epi.d_model;
-            bool run = false;                               // the warp's 32 rows are 32 consecutive slots of one page
-            int pool_row0 = 0;                              // row of (page, K, first slot) in the pool map; V is 64 rows on
-            if (paged_tile) {
-                int64_t off = 0;
-                int u = -1, tt = 0;
-                if (m < M) {
-                    u = find_user(epi.row_off, epi.n_users, (int)m);
-                    tt = (int)m - epi.row_off[u];
-                    page = epi.paged.pt[epi.seqs[u].pt_base + (tt >> 6)];
-                    off = (int64_t)page_elem_offset(epi.paged, page, 0, tt & 63);
-                    if (tt == epi.seqs[u].n_q - 1) last_slot = tt & 63;
+            int pool_row0 = -1;                             // row of (page, K, first slot) in the pool map; V is 64 rows on
+            if (paged_tile && m_base < M) {
+                const int g = epi.page_runs[m_base >> 5];
+                if (g >= 0) {
+                    pool_row0 = ((g >> 6) * epi.paged.n_layers + epi.paged.layer) * 128 + (g & 63);
+                } else {
+                    int64_t off = 0;
+                    if (m < M) {
+                        const int u = find_user(epi.row_off, epi.n_users, (int)m);
+                        const int tt = (int)m - epi.row_off[u];
+                        page = epi.paged.pt[epi.seqs[u].pt_base + (tt >> 6)];
+                        off = (int64_t)page_elem_offset(epi.paged, page, 0, tt & 63);
+                        if (tt == epi.seqs[u].n_q - 1) last_slot = tt & 63;
+                    }
+                    rowoff[lane] = off;
                 }
-                rowoff[lane] = off;
-                const int u0 = __shfl_sync(0xffffffffu, u, 0), tt0 = __shfl_sync(0xffffffffu, tt, 0), page0 = __shfl_sync(0xffffffffu, page, 0);
-                run = __all_sync(0xffffffffu, u >= 0 && u == u0 && tt == tt0 + lane && (tt0 & 63) <= 32);
-                pool_row0 = ((page0 * epi.paged.n_layers + epi.paged.layer) * 2) * 64 + (tt0 & 63);
             }
+            const bool run = pool_row0 >= 0;
             __syncwarp();
             ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->acc_full[as], (ti >> 1) & 1, err));
             if (!ok) break;
@@ -272,7 +282,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 if (m_base >= M) continue;                                       // the whole row group lies past the last row
                 const int n = n_w + pass * 64;                                   // first output column of these 64
                 if (epi.bias) {
-                    const float4 *b4 = reinterpret_cast<const float4 *>(bias_s + pass * 64);
+                    const float4 *b4 = reinterpret_cast<const float4 *>(bias_w + pass * 64);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         const float4 b = b4[i], c = b4[8 + i];

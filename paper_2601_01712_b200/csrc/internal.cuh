@@ -83,6 +83,9 @@ struct Epilogue {
     void *q;                      // [M, d]
     void *k_lin, *v_lin;          // [M, d] transient K/V (used when paged.slab == nullptr)
     PagedKV paged;                // else K/V rows are scattered into pages
+    // Per group of 32 rows of a paged scatter: page * 64 + first slot if the rows are 32 consecutive slots of one page of a user whose
+    // prefix ends in none of them but the page's last slot; else -1 (look the rows up one by one).
+    const int32_t *page_runs;
     const SeqDesc *seqs;          // per-user descriptors (paged scatter needs row -> user -> page)
     const int32_t *row_off;
     int32_t n_users;
