@@ -45,10 +45,11 @@ using tc::unpack2;
 constexpr int kQTile = 128, kKeys = 64, kDh = 64;
 constexpr int kQBytes = kQTile * kDh * 2;           // 16 KB
 constexpr int kKVBytes = kKeys * kDh * 2;           // 8 KB per K or V tile
-#ifndef RELAYGR_ATTN_OFFLOAD
-#define RELAYGR_ATTN_OFFLOAD 1
+#ifndef RELAYGR_OFFP
+#define RELAYGR_OFFP 4
 #endif
-constexpr bool kOffload = RELAYGR_ATTN_OFFLOAD != 0;                       // a quarter of the exponentials runs on the FMA pipe (exp2_fma_pipe)
+constexpr int kOffloadPairs = RELAYGR_OFFP;         // of every 16 pairs of exponentials, evenly spread, run on the FMA pipe (exp2_fma_pipe)
+constexpr bool offloaded(int pair) { return (pair + 1) * kOffloadPairs / 16 != pair * kOffloadPairs / 16; }
 constexpr int kStagesKV = 4;
 constexpr int kSmemBytes = kQBytes + 2 * kStagesKV * kKVBytes + 1024 + 512;
 constexpr uint32_t kTmemCols = 256;                 // S[2]: 0..127, P[2]: 128..191, O: 192..255
@@ -80,21 +81,21 @@ __device__ __forceinline__ float ex2(float x)
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-// 2^x for a packed pair WITHOUT the XU pipe: x is rounded to the nearest integer n by adding 1.5 * 2^23 (n then sits in
-// the low mantissa bits), a cubic gives 2^(x - n) on [-0.5, 0.5] (relative error 7.5e-5, far below the bf16 rounding of P
-// that follows) and n is added to the exponent field as an integer.  x is clamped to [-126, 126] first: below that the
-// result is ~1e-38 instead of 0 (a masked key's -inf included: its weight stays negligible), above it the row-sum check
-// of the caller fails and the block is redone against a true maximum.
-__device__ __forceinline__ void exp2_fma_pipe(uint64_t x2, float &p0, float &p1)
+// 2^x, x = s * c - mc, for a pair WITHOUT the XU pipe: x is rounded to the nearest integer n by adding 1.5 * 2^23 (n then sits
+// in the low mantissa bits), a cubic gives 2^(x - n) on [-0.5, 0.5] (relative error 7.5e-5, far below the bf16 rounding of P that
+// follows) and n is added to the exponent field as an integer.  x has to lie in [-126, 127]: below, the result is ~1e-38 instead
+// of 0 (a masked key's -inf included: its weight stays negligible), above, the row-sum check of the caller fails and the block is
+// redone against a true maximum.  The multiply-add that scales s clamps for nothing: it computes t = (x + 126) / 253 saturated to
+// [0, 1] (x is then off by at most 8e-6).  ct = c / 253, mt = (126 - mc) / 253.
+constexpr float kExpLo = 126.f, kExpSpan = 253.f;
+__device__ __forceinline__ void exp2_fma_pipe(float s0, float s1, float ct, float mt, float &p0, float &p1)
 {
-    float x0, x1;
-    unpack2(x2, x0, x1);
-    x0 = fminf(fmaxf(x0, -126.f), 126.f);
-    x1 = fminf(fmaxf(x1, -126.f), 126.f);
-    const uint64_t xc = pack2(x0, x1);
-    const uint64_t r2 = add2(xc, pack2(12582912.f, 12582912.f));
-    const uint64_t n2 = add2(r2, pack2(-12582912.f, -12582912.f));
-    const uint64_t f2 = fma2(n2, pack2(-1.f, -1.f), xc);
+    float t0, t1;
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(t0) : "f"(s0), "f"(ct), "f"(mt));
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(t1) : "f"(s1), "f"(ct), "f"(mt));
+    const uint64_t t2 = pack2(t0, t1), span2 = pack2(kExpSpan, kExpSpan);
+    const uint64_t r2 = fma2(t2, span2, pack2(12582912.f - kExpLo, 12582912.f - kExpLo));
+    const uint64_t f2 = fma2(t2, span2, fma2(r2, pack2(-1.f, -1.f), pack2(12582912.f - kExpLo, 12582912.f - kExpLo)));
     uint64_t q2 = fma2(pack2(0.0551716685f, 0.0551716685f), f2, pack2(0.2426111251f, 0.2426111251f));
     q2 = fma2(q2, f2, pack2(0.6932609677f, 0.6932609677f));
     q2 = fma2(q2, f2, pack2(0.9999280572f, 0.9999280572f));
@@ -163,7 +164,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         }
         for (int b = 0; b < 2; ++b) {
             tc::mbar_init(&bars->s_full[b], 1);
-            tc::mbar_init(&bars->p_full[b], 128); tc::mbar_init(&bars->p_free[b], 1);
+            tc::mbar_init(&bars->p_full[b], 4); tc::mbar_init(&bars->p_free[b], 1);
             tc::mbar_init(&bars->item_full[b], 1); tc::mbar_init(&bars->item_empty[b], 5);     // MMA warp + four softmax warps
         }
         tc::fence_mbar_init();
@@ -308,8 +309,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             if (ok && nb > 1) ok = issue_qk(1);
             for (int j = 0; j < nb && ok; ++j) {
                 const int gb = g + j, s = gb % kStagesKV, b = gb & 1;
+                if (!(ok = tc::mbar_wait(&bars->v_full[s], (gb / kStagesKV) & 1, err))) break;       // (long there)
                 if (!(ok = tc::mbar_wait(&bars->p_full[b], (gb >> 1) & 1, err))) break;
-                if (!(ok = tc::mbar_wait(&bars->v_full[s], (gb / kStagesKV) & 1, err))) break;
                 tc::tc_fence_after();
                 const uint64_t vdesc = tc::smem_desc_sw128(tc::smem_u32(sV + s * kKVBytes));
                 if (tc::elect_one()) {
@@ -335,6 +336,12 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
         const float c = 0.125f * 1.4426950408889634f;        // 1/sqrt(64) * log2(e)
         bool ok = true;
+        // one arrival per warp: 32 lanes arriving one after the other cost 100 clocks of every block
+        auto publish_p = [&](int b) {
+            tc::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&bars->p_full[b]);
+        };
         for (int n = 0; ok; ++n) {
         const ItemInfo it = take_item(n, ok);
         if (it.nb_keys < 0) break;
@@ -375,8 +382,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             if (!ok) break;
             tc::tc_fence_after();
             if (!warp_live) {
-                tc::tc_fence_before();
-                tc::mbar_arrive(&bars->p_full[b]);
+                publish_p(b);
                 continue;
             }
 
@@ -422,8 +428,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     tc::tmem_st16(lane_addr + kColP + b * (kKeys / 2) + 16 * half, pk);
                 }
                 tc::tmem_st_wait();
-                tc::tc_fence_before();
-                tc::mbar_arrive(&bars->p_full[b]);
+                publish_p(b);
                 continue;
             }
             // p = 2^(s c - m c), bf16 P into TMEM (P[b] is free: see the MMA issuer), row sum in fp32.  The exponentials
@@ -435,32 +440,28 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             // the unrolled block cost more than the off-loading gains.)
             auto exp_block = [&](float mc) {
                 const uint64_t c2 = pack2(c, c), nmc2 = pack2(-mc, -mc);
-                uint64_t ra = pack2(0.f, 0.f), rb = ra;
+                const float mt = (kExpLo - mc) * (1.f / kExpSpan);
+                uint64_t rs2[2] = {0, 0};
                 uint32_t pk[16];
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
 #pragma unroll
-                    for (int i = 0; i < 16; i += 2) {
-                        const uint32_t a0 = half == 0 ? s0[2 * i] : s1[2 * i], a1 = half == 0 ? s0[2 * i + 1] : s1[2 * i + 1];
-                        const uint32_t a2 = half == 0 ? s0[2 * i + 2] : s1[2 * i + 2], a3 = half == 0 ? s0[2 * i + 3] : s1[2 * i + 3];
-                        const uint64_t xa = fma2(pack2(__uint_as_float(a0), __uint_as_float(a1)), c2, nmc2);
-                        const uint64_t xb = fma2(pack2(__uint_as_float(a2), __uint_as_float(a3)), c2, nmc2);
-                        float p0, p1, p2, p3, x0, x1, x2, x3;
-                        unpack2(xb, x2, x3);
-                        p2 = ex2(x2); p3 = ex2(x3);
-                        if (kOffload && (i & 2) != 0) {
-                            exp2_fma_pipe(xa, p0, p1);
+                    for (int i = 0; i < 16; ++i) {
+                        const float a0 = __uint_as_float(half == 0 ? s0[2 * i] : s1[2 * i]), a1 = __uint_as_float(half == 0 ? s0[2 * i + 1] : s1[2 * i + 1]);
+                        float p0, p1;
+                        if (offloaded(i)) {
+                            exp2_fma_pipe(a0, a1, c * (1.f / kExpSpan), mt, p0, p1);
                         } else {
-                            unpack2(xa, x0, x1);
-                            p0 = ex2(x0); p1 = ex2(x1);
+                            unpack2(fma2(pack2(a0, a1), c2, nmc2), p0, p1);
+                            p0 = ex2(p0); p1 = ex2(p1);
                         }
-                        ra = add2(ra, pack2(p0, p1)); rb = add2(rb, pack2(p2, p3));
-                        pk[i] = tc::pack_bf16(p0, p1); pk[i + 1] = tc::pack_bf16(p2, p3);
+                        rs2[i & 1] = add2(rs2[i & 1], pack2(p0, p1));
+                        pk[i] = tc::pack_bf16(p0, p1);
                     }
                     tc::tmem_st16(lane_addr + kColP + b * (kKeys / 2) + 16 * half, pk);
                 }
                 float r0, r1;
-                unpack2(add2(ra, rb), r0, r1);
+                unpack2(add2(rs2[0], rs2[1]), r0, r1);
                 return r0 + r1;
             };
             float rs = 0.f, alpha = 1.f;
@@ -503,8 +504,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             }
             l = fmaf(l, alpha, rs);
             tc::tmem_st_wait();
-            tc::tc_fence_before();
-            tc::mbar_arrive(&bars->p_full[b]);     // P(j) (and any correction of O) is in TMEM
+            publish_p(b);                          // P(j) (and any correction of O) is in TMEM
         }
 
         if (!ok) break;
