@@ -8,17 +8,18 @@
 namespace relaygr {
 
 // ---- tensor-core attention work items: one per (user, head, 128-row tile[, KV split]) of the rows in `seqs` ------------------
-// The kernel runs one item per CTA, two CTAs per SM, handed out in list order as CTAs retire.  The list is therefore
+// Items are taken in list order by whichever of the machine's slots is free (bf16: two CTAs per SM; fp32: one).  The list is therefore
 // ordered costliest first, and the plan decides how finely to split the key ranges so that the last wave is not a few
 // whole items running on an otherwise idle GPU.  Cost model, in units of one 64-key block of one tile (about 0.7 us):
-// an item costs kItemFixed (launch, Q and first K loads, first S, epilogue) plus its key blocks; `slots` items run at a
+// an item costs item_fixed (launch, Q and first K loads, first S, epilogue) plus its key blocks; `slots` items run at a
 // time.  Every item is split `ns` ways; the items left over after the last full wave (the cheapest ones, at the end of
 // the list) are split `nst` times finer still, so that their pieces spread over all slots.  ns is the value with the
 // smallest estimated makespan; a split piece keeps at least kMinSplitBlocks key blocks.
-void build_attention_worklist(const std::vector<SeqDesc> &seqs, int n_heads, int n_sms, int64_t max_split_tiles,
+void build_attention_worklist(const std::vector<SeqDesc> &seqs, int n_heads, const AttnMachine &machine, int64_t max_split_tiles,
                               std::vector<AttnItem> &items, std::vector<AttnMerge> &merges)
 {
-    constexpr double kItemFixed = 8.0, kMergeCost = 5.0;
+    constexpr double kMergeCost = 5.0;
+    const double item_fixed = machine.item_fixed;
     constexpr int kMinSplitBlocks = 4, kMaxSplit = 16;
     items.clear();
     merges.clear();
@@ -52,7 +53,7 @@ void build_attention_worklist(const std::vector<SeqDesc> &seqs, int n_heads, int
         return x.q0 < y.q0;
     });
 
-    const int64_t slots = 2 * (int64_t)std::max(1, n_sms);
+    const int64_t slots = machine.slots;
     const int64_t base = (int64_t)tiles.size() * n_heads;
     const double mean_nb = (double)sum_nb / (double)tiles.size();
     // tail_of(ns): how many items (of the unsplit list) do not fit the full waves, and how much finer they are split
@@ -75,8 +76,8 @@ void build_attention_worklist(const std::vector<SeqDesc> &seqs, int n_heads, int
         int64_t tail_items;
         int nst;
         const int64_t waves = tail_of(ns, tail_items, nst);
-        double est = (double)waves * (kItemFixed + mean_nb / ns);
-        if (tail_items > 0) est += kItemFixed + mean_nb / (ns * nst);
+        double est = (double)waves * (item_fixed + mean_nb / ns);
+        if (tail_items > 0) est += item_fixed + mean_nb / (ns * nst);
         if (ns * nst > 1) est += kMergeCost;
         if (ns == 1 || est < best_est) { best_est = est; best_ns = ns; }
     }

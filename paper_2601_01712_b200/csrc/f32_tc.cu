@@ -1,0 +1,772 @@
+// GEMM and attention of the fp32 model on the 5th-generation tensor cores, without giving up fp32 precision.
+//
+// An fp32 number is the exact sum of three bf16 numbers, x = x1 + x2 + x3 (24 significand bits = 3 x 8, every part rounded to
+// nearest, so |x2| <= 2^-8 |x|, |x3| <= 2^-16 |x|), and a product is
+//     x y = x1 y1 + (x1 y2 + x2 y1) + (x2 y2 + x1 y3 + x3 y1)
+//           (+ x2 y3 + x3 y2 + x3 y3: left out, at most 2^-23 |x y| and 2^-26 on average, where a fp32 multiply-add rounds at 2^-24)
+// - six bf16 products with fp32 accumulation.  (TF32 parts carry 11 bits: two of them miss two bits of x, three would cost twice as
+// much.)  The leading product and the small ones are summed apart, or the small ones first, so that the small ones are not added
+// into a large accumulator again and again.  The tensor core does not round its sums to nearest, so a chain of leading products is
+// kept short (16 steps in the GEMM, 4 in the attention) and the chains are added up in registers: the error against fp64 measured
+// the same as the CUDA-core kernels' at d_model 256 and below it at 1024, where one chain over K = 4096 had four times that.
+#include "kernels.cuh"
+#include "tc_common.cuh"
+
+namespace relaygr {
+
+namespace {
+
+// the three parts of a pair, one bf16x2 word each: nine instructions
+__device__ __forceinline__ void split2(uint64_t x, uint32_t (&w)[3])
+{
+    const uint64_t minus1 = tc::pack2(-1.f, -1.f);
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        w[p] = tc::pack_bf16(x);
+        if (p < 2) x = tc::fma2(tc::pack2(w[p] << 16, w[p] & 0xffff0000u), minus1, x);      // exact
+    }
+}
+// four floats: 8 bytes of each plane, at `dst` and every `plane` bytes from there
+__device__ __forceinline__ void split_store(uint8_t *dst, int plane, float4 v)
+{
+    uint32_t lo[3], hi[3];
+    split2(tc::pack2(v.x, v.y), lo);
+    split2(tc::pack2(v.z, v.w), hi);
+#pragma unroll
+    for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2 *>(dst + p * plane) = make_uint2(lo[p], hi[p]);
+}
+
+// 16-byte chunk j of row r in a tile of 128-byte rows with the 128-byte swizzle
+__device__ __forceinline__ uint8_t *chunk_at(uint8_t *tile, int r, int j) { return tile + r * 128 + ((j ^ (r & 7)) << 4); }
+
+__device__ __forceinline__ float max3(float a, float b, float c)
+{
+    float d;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+// 2^x; results below 2^-126 are zero (exp2f scales around that, with the same error otherwise)
+__device__ __forceinline__ float ex2(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// ---- GEMM: C[m, n] = sum_k A[m, k] W[n, k] ---------------------------------------------------------------------------
+// Persistent CTAs, one per SM, 128 x 64 tiles, 64 columns of K at a time.  Warp 13 loads fp32 by TMA (three stages of 48 KB);
+// warps 0-7 split it, the parts of A into TMEM (a row per thread), those of W into shared memory, two stages each; warp 8 owns TMEM
+// and issues the MMAs; warps 9-12 add up and store the tile before, under the next one's products.
+// What bounds it: shared memory at 128 B / clk.  Per K block the fp32 tiles are written and read once (96 KB), W's parts written
+// (24 KB) and read by the 24 products (48 KB): 1312 clocks, where the MMAs need 768 and the loads 768 at the 64 B / clk an SM gets
+// from L2.  With A's parts in shared memory as well it was 2460, with the loads through registers 2550 and the epilogue behind them.
+constexpr int kGroup = 4;                             // K blocks of one accumulator of leading products; two take turns
+constexpr int kBM = 128, kBN = 64, kBK = 64, kStages = 2, kSlots = 3;
+constexpr int kWorkers = 256, kEpiWarps = 4, kGemmThreads = kWorkers + 32 + 32 * kEpiWarps + 32;
+constexpr int kWPlane = kBN * 128, kStage = 3 * kWPlane;                        // W's parts: three planes of 64 rows x 64 columns
+constexpr int kSlotA = kBM * 128, kSlotW = kBN * 128, kSlot = 2 * (kSlotA + kSlotW);      // fp32: two tiles of 32 columns of A, two of W
+constexpr int kOffSlots = kStages * kStage, kOffPatch = kOffSlots + kSlots * kSlot, kOffGBars = kOffPatch + kEpiWarps * 4096;
+constexpr int kGemmSmem = kOffGBars + 256 + 1024;
+static_assert(kGemmSmem <= 227 * 1024, "shared memory budget");
+constexpr uint32_t kColLead = 0, kColSmall = 2 * kBN, kColA = 4 * kBN, kColAStage = 96, kGemmCols = 512;      // A's parts: 3 x 32 columns a stage
+
+struct GemmBars {
+    uint64_t full[kStages], empty[kStages], acc_full[2], acc_empty[2], slot_full[kSlots], slot_empty[kSlots];
+    uint32_t tmem_slot;
+    int abort_flag;
+};
+static_assert(sizeof(GemmBars) <= 256, "barrier block");
+
+__global__ void __launch_bounds__(kGemmThreads, 1)
+f32_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, int64_t M, int N, int K, Epilogue e, int *err)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    GemmBars *bars = reinterpret_cast<GemmBars *>(smem + kOffGBars);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tiles_n = (N + kBN - 1) / kBN, n_tiles = (int)((M + kBM - 1) / kBM) * tiles_n;
+    const int n_k = (K + kBK - 1) / kBK, n_groups = (n_k + kGroup - 1) / kGroup;
+
+    if (tid == 0) {
+        for (int s = 0; s < kStages; ++s) { tc::mbar_init(&bars->full[s], kWorkers / 32); tc::mbar_init(&bars->empty[s], 1); }
+        for (int i = 0; i < 2; ++i) { tc::mbar_init(&bars->acc_full[i], 1); tc::mbar_init(&bars->acc_empty[i], kEpiWarps); }
+        for (int i = 0; i < kSlots; ++i) { tc::mbar_init(&bars->slot_full[i], 1); tc::mbar_init(&bars->slot_empty[i], kWorkers / 32); }
+        tc::fence_mbar_init();
+        tc::tma_prefetch_desc(&tmA); tc::tma_prefetch_desc(&tmW);
+    }
+    if (warp == 8) {
+        tc::tmem_alloc(&bars->tmem_slot, kGemmCols);
+        tc::tmem_relinquish();
+    }
+    grid_launch_dependents();
+    grid_dependency_wait();
+    if (tid == 0) bars->abort_flag = *reinterpret_cast<volatile int *>(err);
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    const uint32_t tmem_base = bars->tmem_slot;
+    const bool live = bars->abort_flag == 0;
+
+    if (!live) {
+    } else if (warp < 8) {
+        // ---------------------------------------------------------------- splits: warp (quad, half) takes columns 32 half .. + 31 of a K
+        // block: of A rows 32 quad .. + 31, one per lane; of W pieces of four floats, eight lanes to a row, rows 0, 4, 1, 5 (or 2, 6, 3,
+        // 7) of eight at a time, whose halves of the planes' rows lie in different banks
+        const int quad = warp & 3, half = warp >> 2, r = quad * 32 + lane;
+        const int pj = lane & 7, g = lane >> 3, pr = quad * 8 + (g & 1) * 4 + (g >> 1);
+        const uint32_t a_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + kColA + half * 16;
+        int it = 0, slot = 0, sphase = 0;              // K blocks so far; position in the ring
+        bool ok = true;
+        for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+            for (int kb = 0; kb < n_k; ++kb, ++it) {
+                const int s = it & 1;
+                uint8_t *src = smem + kOffSlots + slot * kSlot, *src_w = src + 2 * kSlotA + half * kSlotW;
+                src += half * kSlotA;
+                ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->slot_full[slot], sphase, err) &&
+                                             tc::mbar_wait(&bars->empty[s], ((it >> 1) & 1) ^ 1, err));
+                if (!ok) break;
+                tc::tc_fence_after();
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h) {          // 16 columns = 8 words per plane (rolled loops: cold code costs its fetch)
+                    uint32_t w[3][8], part[3];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(chunk_at(src, r, 4 * h + i));
+                        split2(x.x, part);
+                        w[0][2 * i] = part[0]; w[1][2 * i] = part[1]; w[2][2 * i] = part[2];
+                        split2(x.y, part);
+                        w[0][2 * i + 1] = part[0]; w[1][2 * i + 1] = part[1]; w[2][2 * i + 1] = part[2];
+                    }
+#pragma unroll
+                    for (int p = 0; p < 3; ++p) tc::tmem_st8(a_addr + s * kColAStage + p * 32 + 8 * h, w[p]);
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const int row = pr + 2 * i + 32 * h;
+                        split_store(chunk_at(smem + s * kStage, row, 4 * half + (pj >> 1)) + (pj & 1) * 8, kWPlane,
+                                    *reinterpret_cast<const float4 *>(chunk_at(src_w, row, pj)));
+                    }
+                }
+                tc::tmem_st_wait();
+                tc::fence_proxy_async();
+                tc::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) { tc::mbar_arrive(&bars->slot_empty[slot]); tc::mbar_arrive(&bars->full[s]); }
+                if (++slot == kSlots) { slot = 0; sphase ^= 1; }
+            }
+        }
+    } else if (warp == 13) {
+        // ---------------------------------------------------------------- TMA producer
+        if (lane == 0) {
+            int slot = 0, phase = 1;
+            bool ok = true;
+            for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+                const int m0 = (tile / tiles_n) * kBM, n0 = (tile % tiles_n) * kBN;
+                for (int x = 0; x < n_k * kBK; x += kBK) {
+                    ok = tc::mbar_wait(&bars->slot_empty[slot], phase, err);
+                    if (!ok) break;
+                    uint8_t *dst = smem + kOffSlots + slot * kSlot;
+                    tc::mbar_expect_tx(&bars->slot_full[slot], kSlot);
+                    for (int h = 0; h < 2; ++h) {      // (rows and columns past the last are zeros)
+                        tc::tma_load_2d(dst + h * kSlotA, &tmA, x + 32 * h, m0, &bars->slot_full[slot]);
+                        tc::tma_load_2d(dst + 2 * kSlotA + h * kSlotW, &tmW, x + 32 * h, n0, &bars->slot_full[slot]);
+                    }
+                    if (++slot == kSlots) { slot = 0; phase ^= 1; }
+                }
+            }
+        }
+    } else if (warp == 8) {
+        // ---------------------------------------------------------------- MMA issuer
+        constexpr uint32_t idesc = tc::make_idesc(kBM, kBN, 0, 0);
+        bool ok = true;
+        int it = 0, grp = 0, nt = 0;
+        for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++nt) {
+            const uint32_t small = tmem_base + kColSmall + (nt & 1) * kBN;
+            for (int kb = 0; kb < n_k; ++kb, ++it) {
+                const int s = it % kStages;
+                const bool first = kb % kGroup == 0, last = kb % kGroup == kGroup - 1 || kb == n_k - 1;
+                // the accumulator's group before has been added up (and with it the small products of the tile before the last)
+                if (first) ok = tc::mbar_wait(&bars->acc_empty[grp & 1], ((grp >> 1) & 1) ^ 1, err);
+                if (ok) ok = tc::mbar_wait(&bars->full[s], (it / kStages) & 1, err);
+                if (!ok) break;
+                tc::tc_fence_after();
+                const uint64_t wdesc = tc::smem_desc_sw128(tc::smem_u32(smem + s * kStage));
+                const uint32_t lead = tmem_base + kColLead + (grp & 1) * kBN, a = tmem_base + kColA + s * kColAStage;
+                if (tc::elect_one()) {
+                    auto product = [&](int pa, int pw, uint32_t acc, bool clear) {
+#pragma unroll
+                        for (int k = 0; k < kBK / 16; ++k)
+                            tc::mma_ts(acc, a + pa * 32 + 8 * k, wdesc + pw * (kWPlane >> 4) + 2 * k, idesc, !(clear && k == 0));
+                    };
+                    product(0, 0, lead, first);
+                    product(2, 0, small, kb == 0); product(0, 2, small, false); product(1, 1, small, false);
+                    product(1, 0, small, false); product(0, 1, small, false);
+                    tc::mma_commit(&bars->empty[s]);
+                    if (last) tc::mma_commit(&bars->acc_full[grp & 1]);
+                }
+                __syncwarp();
+                if (last) ++grp;
+            }
+        }
+    } else {
+        // ---------------------------------------------------------------- epilogue: warp w has TMEM lanes 32 (w % 4) .. + 31
+        const int quad = warp & 3;
+        const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
+        uint8_t *patch = smem + kOffPatch + quad * 4096;
+        const int pj = lane & 7, prow = lane >> 3, d = e.d_model;      // when a patch is stored: this lane's chunk of a row, first row
+        bool ok = true;
+        int grp = 0, nt = 0;
+        for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++nt) {
+            const int64_t m0 = (int64_t)(tile / tiles_n) * kBM + quad * 32;
+            const int n0 = (tile % tiles_n) * kBN;
+            // where rows go that belong in pages: offset of (page, K, slot); of a user's last row its slot
+            const bool to_pages = e.mode == EPI_QKV && e.paged.slab != nullptr && e.col0 + n0 + kBN > e.d_model;
+            int64_t page_off = 0;
+            int last_slot = -1;
+            if (to_pages && m0 + lane < M) {
+                const int u = find_user(e.row_off, e.n_users, (int)(m0 + lane));
+                const int t = (int)(m0 + lane) - e.row_off[u];
+                page_off = (int64_t)page_elem_offset(e.paged, e.paged.pt[e.seqs[u].pt_base + (t >> 6)], 0, t & 63);
+                if (t == e.seqs[u].n_q - 1) last_slot = t & 63;
+            }
+            float acc[2][32];
+            for (int g = 0; g < n_groups; ++g, ++grp) {
+                ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->acc_full[grp & 1], (grp >> 1) & 1, err));
+                if (!ok) break;
+                tc::tc_fence_after();
+                auto add = [&](uint32_t col, bool set) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        uint32_t r[32];
+                        tc::tmem_ld32(lane_addr + col + h * 32, r);
+                        tc::tmem_ld_wait();
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) acc[h][i] = set ? __uint_as_float(r[i]) : acc[h][i] + __uint_as_float(r[i]);
+                    }
+                };
+                add(kColLead + (grp & 1) * kBN, g == 0);
+                if (g == n_groups - 1) add(kColSmall + (nt & 1) * kBN, false);
+                tc::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&bars->acc_empty[grp & 1]);
+            }
+            if (!ok) break;
+            // one row per thread so far; 32 rows x 32 columns at a time are turned around in shared memory, so that global memory sees
+            // whole rows of 128 bytes
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int n = n0 + h * 32 + pj * 4;    // this lane's four columns (N is a multiple of 4)
+                const bool in_n = n < N;
+                float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (e.bias && in_n) bias = make_float4(e.bias[n], e.bias[n + 1], e.bias[n + 2], e.bias[n + 3]);
+                // where column n goes: the output (or residual stream), q, or K / V (rows of pages: added per row)
+                float *out = e.mode == EPI_STORE ? reinterpret_cast<float *>(e.out) : e.out_f32;
+                int64_t pitch = N, off0 = n;
+                bool paged = false;
+                if (e.mode == EPI_QKV) {
+                    const int qcol = e.col0 + n, which = (qcol >= d) + (qcol >= 2 * d);
+                    paged = to_pages && which > 0;
+                    out = reinterpret_cast<float *>(paged ? e.paged.slab : which == 0 ? e.q : which == 1 ? e.k_lin : e.v_lin);
+                    pitch = d;
+                    off0 = qcol - which * d + (paged ? (int64_t)(which - 1) * 64 * d : 0);
+                }
+                float4 x[8];                           // the residual, of rows prow, prow + 4, ...: all on their way before any is used
+                if (e.mode == EPI_RESID) {
+                    const float *p = e.resid + (m0 + prow) * N + n;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i, p += (int64_t)4 * N) {
+                        x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (in_n && m0 + 4 * i + prow < M) x[i] = *reinterpret_cast<const float4 *>(p);
+                    }
+                }
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    *reinterpret_cast<float4 *>(chunk_at(patch, lane, j)) = make_float4(acc[h][4 * j], acc[h][4 * j + 1], acc[h][4 * j + 2], acc[h][4 * j + 3]);
+                __syncwarp();
+                auto value = [&](int i) {
+                    const float4 v = *reinterpret_cast<const float4 *>(chunk_at(patch, 4 * i + prow, pj));
+                    return make_float4(v.x + bias.x, v.y + bias.y, v.z + bias.z, v.w + bias.w);
+                };
+                float *dst = out + off0 + (m0 + prow) * pitch;
+                if (e.mode == EPI_RESID) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i, dst += 4 * pitch) {
+                        const float4 v = value(i);
+                        if (in_n && m0 + 4 * i + prow < M) *reinterpret_cast<float4 *>(dst) = make_float4(x[i].x + v.x, x[i].y + v.y, x[i].z + v.z, x[i].w + v.w);
+                    }
+                } else if (!to_pages) {
+                    const bool silu = e.mode == EPI_STORE && e.silu;
+#pragma unroll 2
+                    for (int i = 0; i < 8; ++i, dst += 4 * pitch) {
+                        float4 v = value(i);
+                        if (silu) { v.x /= 1.f + expf(-v.x); v.y /= 1.f + expf(-v.y); v.z /= 1.f + expf(-v.z); v.w /= 1.f + expf(-v.w); }
+                        if (in_n && m0 + 4 * i + prow < M) *reinterpret_cast<float4 *>(dst) = v;
+                    }
+                } else {
+#pragma unroll 1
+                    for (int i = 0; i < 8; ++i) {
+                        const int rr = 4 * i + prow;
+                        const float4 v = value(i);
+                        const int64_t row_off = __shfl_sync(0xffffffffu, page_off, rr);
+                        const int ls = __shfl_sync(0xffffffffu, last_slot, rr);
+                        float *q = out + off0 + (paged ? row_off : (m0 + rr) * pitch);
+                        if (in_n && m0 + rr < M) {
+                            *reinterpret_cast<float4 *>(q) = v;
+                            if (paged && ls >= 0)      // last row of the prefix: clear the unused slots of its page
+                                for (int z = 1; ls + z < 64; ++z) *reinterpret_cast<float4 *>(q + (int64_t)z * d) = make_float4(0.f, 0.f, 0.f, 0.f);
+                        }
+                    }
+                }
+            }
+        }
+    }
+    tc::tc_fence_before();
+    __syncthreads();
+    if (warp == 8) tc::tmem_dealloc(tmem_base, kGemmCols);
+}
+
+// ---- attention ----------------------------------------------------------------------------------------------------------
+// A CTA runs one work item (attn_plan.cpp): a 128-row query tile of one head of one user against a range of its 64-key blocks, the
+// candidates' own keys as one or two more blocks with a diagonal mask.  Per block:
+//     S = Q K^T          six products, the small ones first; Q's parts in TMEM, K's in shared memory
+//     P = softmax(S)     online, fp32, against the running maximum; its parts take the place of S
+//     O += P V           six products per block into a fresh accumulator, added up in registers: the sum over the blocks is fp32
+//                        round-to-nearest whatever the tensor core does inside a block, and a raised maximum rescales registers
+// Warps 0-7: softmax, two threads per row (warp w: TMEM lanes 32 (w % 4) .., half w / 4 of the keys and of the output
+// dimensions); the two exchange the block maximum through shared memory.  Warps 8-15: load K and V, split, store the planes - K one
+// block ahead of V: K of block j + 2 may come when Q K(j)^T is done, V only after P V(j) - and before that of Q.  Warp 16: TMEM and
+// MMAs.  K and V planes and S / P and O are double-buffered, each with barriers of its own.
+// What bounds it: per block the MMAs take 48 x 32 = 1536 clocks; the softmax warps' chain (scores, maximum, exchange, weights, split,
+// output of the block before) takes about 2500 beside the splitting warps.
+constexpr int kQRows = 128, kKeys = 64;
+constexpr int kSoftThreads = 256, kConvThreads = 256, kAttnThreads = kSoftThreads + kConvThreads + 32;
+constexpr int kQPlane = kQRows * 128, kKVPlane = kKeys * 128, kKVStage = 6 * kKVPlane;      // a buffer: three planes of K, three of V
+constexpr int kOffKV = 3 * kQPlane, kOffStat = kOffKV + 2 * kKVStage, kOffABars = kOffStat + 2 * 2 * kQRows * 4;
+constexpr int kAttnSmem = kOffABars + 256 + 1024;
+static_assert(kAttnSmem <= 227 * 1024, "shared memory budget");
+constexpr uint32_t kColS = 0, kSP = 96, kColO = 192, kColQ = 320, kAttnCols = 512;      // S (64) / P (3 x 32) buffers, O buffers (64), Q (3 x 32)
+
+struct AttnBars {
+    uint64_t q_full, q_tmem, k_full[2], v_full[2], k_empty[2], v_empty[2], s_full[2], p_full[2], o_full[2];
+    uint32_t tmem_slot;
+    int abort_flag;
+};
+static_assert(sizeof(AttnBars) <= 256, "barrier block");
+
+template <int DH, bool kPointwise>
+__global__ void __launch_bounds__(kAttnThreads, 1)
+f32_attention_tc_kernel(const float *__restrict__ q, const float *__restrict__ k_lin, const float *__restrict__ v_lin, PagedKV paged,
+                        const SeqDesc *__restrict__ seqs, const AttnItem *__restrict__ items, int n_heads, float *__restrict__ out,
+                        float *__restrict__ partial, int *err)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    float *stat = reinterpret_cast<float *>(smem + kOffStat);
+    AttnBars *bars = reinterpret_cast<AttnBars *>(smem + kOffABars);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, d = n_heads * DH;
+
+    if (tid == 0) {
+        tc::mbar_init(&bars->q_full, kConvThreads / 32); tc::mbar_init(&bars->q_tmem, kSoftThreads / 32);
+        for (int i = 0; i < 2; ++i) {
+            tc::mbar_init(&bars->k_full[i], kConvThreads / 32); tc::mbar_init(&bars->v_full[i], kConvThreads / 32);
+            tc::mbar_init(&bars->k_empty[i], 1); tc::mbar_init(&bars->v_empty[i], 1);
+            tc::mbar_init(&bars->s_full[i], 1); tc::mbar_init(&bars->p_full[i], kSoftThreads / 32); tc::mbar_init(&bars->o_full[i], 1);
+        }
+        tc::fence_mbar_init();
+    }
+    if (warp == 16) {
+        tc::tmem_alloc(&bars->tmem_slot, kAttnCols);
+        tc::tmem_relinquish();
+    }
+    grid_launch_dependents();
+    grid_dependency_wait();
+    if (tid == 0) bars->abort_flag = *reinterpret_cast<volatile int *>(err);
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    const uint32_t tmem_base = bars->tmem_slot;
+    const bool live = bars->abort_flag == 0;
+
+    const AttnItem it = items[blockIdx.x];
+    const SeqDesc sd = seqs[it.seq];
+    const int n_page_blocks = (sd.n_paged + 63) >> 6, nb_keys = it.blk1 - it.blk0;
+    const int pos0 = sd.q_pos0 + it.q0;                              // sequence position of the tile's first row
+    // the 64-row groups of the tile that hold candidates: their own keys, a diagonal block each
+    const int first_cand = max(0, sd.causal_end - pos0);
+    const bool own = it.with_self && first_cand < it.n_q;
+    const int d0 = own ? first_cand >> 6 : 0, nb = nb_keys + (own ? ((it.n_q + 63) >> 6) - d0 : 0);
+
+    if (!live) {
+    } else if (warp == 16) {
+        // ---------------------------------------------------------------- MMA issuer
+        constexpr uint32_t idesc_qk = tc::make_idesc(kQRows, kKeys, 0, 0), idesc_pv = tc::make_idesc(kQRows, DH, 0, 1);
+        bool ok = tc::mbar_wait(&bars->q_tmem, 0, err);
+        const uint32_t kv0 = tc::smem_u32(smem + kOffKV);
+        auto issue_qk = [&](int j) {
+            const int b = j & 1;
+            if (!(ok = tc::mbar_wait(&bars->k_full[b], (j >> 1) & 1, err))) return;
+            tc::tc_fence_after();
+            const uint64_t kd = tc::smem_desc_sw128(kv0 + b * kKVStage);
+            const uint32_t acc = tmem_base + kColS + b * kSP, qa = tmem_base + kColQ;
+            if (tc::elect_one()) {
+                auto product = [&](int pq, int pk, bool first) {
+#pragma unroll
+                    for (int k = 0; k < DH / 16; ++k) tc::mma_ts(acc, qa + pq * 32 + 8 * k, kd + pk * (kKVPlane >> 4) + 2 * k, idesc_qk, !(first && k == 0));
+                };
+                product(2, 0, true); product(0, 2, false); product(1, 1, false); product(1, 0, false); product(0, 1, false); product(0, 0, false);
+                tc::mma_commit(&bars->s_full[b]);
+                tc::mma_commit(&bars->k_empty[b]);
+            }
+            __syncwarp();
+        };
+        if (ok && nb > 0) issue_qk(0);
+        if (ok && nb > 1) issue_qk(1);
+        for (int j = 0; j < nb && ok; ++j) {
+            const int b = j & 1;
+            // P(j) in TMEM, where S(j) was; O(j - 2), whose buffer this block's products overwrite, is in registers by then
+            if (!(ok = tc::mbar_wait(&bars->v_full[b], (j >> 1) & 1, err))) break;
+            if (!(ok = tc::mbar_wait(&bars->p_full[b], (j >> 1) & 1, err))) break;
+            tc::tc_fence_after();
+            const uint64_t vd = tc::smem_desc_sw128(kv0 + b * kKVStage + 3 * kKVPlane);
+            const uint32_t acc = tmem_base + kColO + b * 64, pa = tmem_base + kColS + b * kSP;
+            if (tc::elect_one()) {
+                auto product = [&](int pp, int pv, bool first) {
+#pragma unroll
+                    for (int k = 0; k < kKeys / 16; ++k)      // 16 keys: 8 columns of P, 2048 bytes of V
+                        tc::mma_ts(acc, pa + pp * 32 + 8 * k, vd + pv * (kKVPlane >> 4) + 128 * k, idesc_pv, !(first && k == 0));
+                };
+                product(2, 0, true); product(0, 2, false); product(1, 1, false); product(1, 0, false); product(0, 1, false); product(0, 0, false);
+                tc::mma_commit(&bars->o_full[b]);
+                tc::mma_commit(&bars->v_empty[b]);
+            }
+            __syncwarp();
+            if (j + 2 < nb) issue_qk(j + 2);                   // over P(j), behind the products that read it
+        }
+    } else if (warp >= 8) {
+        // ---------------------------------------------------------------- loads and splits: pieces of four floats, DH / 4 lanes to a row
+        constexpr int kLanes = DH / 4, kStep = kConvThreads / kLanes, kPer = kKeys / kStep;      // lanes per row, rows at a time, pieces per thread
+        const int ct = tid - kSoftThreads, pr = ct / kLanes, pc = ct % kLanes;
+        const int64_t piece_off = (int64_t)pr * d + it.head * DH + 4 * pc, step_off = (int64_t)kStep * d;
+        uint8_t *piece_dst = chunk_at(smem, pr, pc >> 1) + (pc & 1) * 8;      // rows kStep on: kStep * 128 bytes on (kStep % 8 == 0)
+        float4 rk[kPer], rv[kPer];
+        int page_next = 0;                                 // of the next block that K is loaded for: its look-up is off the loads' path
+        auto look_up = [&](int j) { if (j < nb_keys && it.blk0 + j < n_page_blocks) page_next = paged.pt[sd.pt_base + it.blk0 + j]; };
+        const float *v_src = nullptr;
+        int v_rows = 0;
+        auto load_rows = [&](const float *p, int n, float4 (&v)[kPer]) {      // n rows exist; the others are zeros
+            p += piece_off;
+#pragma unroll
+            for (int i = 0; i < kPer; ++i, p += step_off) {
+                v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (pr + i * kStep < n) v[i] = *reinterpret_cast<const float4 *>(p);
+            }
+        };
+        auto load_k = [&](int j) {                         // also notes where the block's V is
+            const float *k;
+            if (j >= nb_keys) {
+                const int r0 = (d0 + j - nb_keys) * 64;
+                const int64_t off = (int64_t)(sd.self_row0 + it.q0 + r0) * d;
+                k = k_lin + off; v_src = v_lin + off; v_rows = it.n_q - r0;
+            } else if (it.blk0 + j < n_page_blocks) {
+                const float *slab = reinterpret_cast<const float *>(paged.slab);
+                k = slab + page_elem_offset(paged, page_next, 0, 0); v_src = slab + page_elem_offset(paged, page_next, 1, 0);
+                v_rows = sd.n_paged - (it.blk0 + j) * 64;
+            } else {
+                const int r0 = (it.blk0 + j - n_page_blocks) * 64;
+                const int64_t off = (int64_t)(sd.lin_row0 + r0) * d;
+                k = k_lin + off; v_src = v_lin + off; v_rows = sd.n_lin - r0;
+            }
+            load_rows(k, v_rows, rk);
+            look_up(j + 1);
+        };
+        auto store_planes = [&](uint32_t off, const float4 (&v)[kPer], uint64_t *full) {
+#pragma unroll
+            for (int i = 0; i < kPer; ++i) split_store(piece_dst + off + i * (kStep * 128), kKVPlane, v[i]);
+            tc::fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(full);
+        };
+        look_up(0);
+        if (nb > 0) load_k(0);
+        {
+            // logits in units of log2(e) (softmax), so that a weight is 2^x
+            const float scale = rsqrtf((float)DH) * (kPointwise ? 1.f : 1.4426950408889634f);
+            const float *src = q + ((int64_t)sd.q_row0 + it.q0) * d + piece_off;
+#pragma unroll
+            for (int i = 0; i < kQRows / kStep; ++i, src += step_off) {
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (pr + i * kStep < it.n_q) v = *reinterpret_cast<const float4 *>(src);
+                split_store(piece_dst + i * (kStep * 128), kQPlane, make_float4(v.x * scale, v.y * scale, v.z * scale, v.w * scale));
+            }
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&bars->q_full);      // (read by the softmax warps)
+        }
+        // K(0); then K(j + 1) before V(j): the scores of the next block do not wait for the products that hold this V's buffer.  What
+        // is stored next is on its way already: K two blocks ahead, V one.
+        auto buffer = [&](int j) { return (uint32_t)(kOffKV + (j & 1) * kKVStage); };
+        if (nb > 0) {
+            load_rows(v_src, v_rows, rv);
+            store_planes(buffer(0), rk, &bars->k_full[0]);
+            if (nb > 1) load_k(1);
+        }
+        for (int j = 0; j < nb; ++j) {
+            bool ok = true;
+            const float *v_next = v_src;                   // of block j + 1, if there is one
+            const int v_next_rows = v_rows;
+            if (j + 1 < nb) {
+                ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->k_empty[(j + 1) & 1], ((j + 1) >> 1 & 1) ^ 1, err));
+                if (!ok) break;
+                store_planes(buffer(j + 1), rk, &bars->k_full[(j + 1) & 1]);
+                if (j + 2 < nb) load_k(j + 2);
+            }
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->v_empty[j & 1], ((j >> 1) & 1) ^ 1, err));
+            if (!ok) break;
+            store_planes(buffer(j) + 3 * kKVPlane, rv, &bars->v_full[j & 1]);
+            if (j + 1 < nb) load_rows(v_next, v_next_rows, rv);
+        }
+    } else {
+        // ---------------------------------------------------------------- softmax
+        const int quad = warp & 3, half = warp >> 2;
+        const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
+        const int r = quad * 32 + lane;
+        const int tpos = pos0 + r;
+        const bool is_cand = tpos >= sd.causal_end;
+        const int lim = is_cand ? sd.causal_end : tpos + 1;              // this row sees keys at positions < lim
+        const int min_lim = pos0 >= sd.causal_end ? sd.causal_end : pos0 + 1;
+        constexpr int kOD = DH / 2;                                      // output dimensions of this thread, in pairs
+        uint64_t o[kOD / 2];
+        float m = -INFINITY, l = 0.f, corr = 1.f;
+#pragma unroll
+        for (int i = 0; i < kOD / 2; ++i) o[i] = 0;
+        // Q's planes, from shared memory into TMEM: this thread's half of its row
+        bool ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->q_full, 0, err));
+        if (ok) {
+#pragma unroll
+            for (int p = 0; p < 3; ++p)
+#pragma unroll
+                for (int g = 0; g < DH / 32; ++g) {        // two 16-byte chunks = 16 dimensions = 8 words
+                    const int j = half * (DH / 16) + 2 * g;
+                    const uint4 x = *reinterpret_cast<const uint4 *>(chunk_at(smem + p * kQPlane, r, j));
+                    const uint4 y = *reinterpret_cast<const uint4 *>(chunk_at(smem + p * kQPlane, r, j + 1));
+                    const uint32_t w[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+                    tc::tmem_st8(lane_addr + kColQ + p * 32 + 4 * j, w);
+                }
+            tc::tmem_st_wait();
+            tc::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&bars->q_tmem);
+        }
+        // o = o * corr + (block j's product)
+        auto take_o = [&](int j) {
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->o_full[j & 1], (j >> 1) & 1, err));
+            if (!ok) return;
+            tc::tc_fence_after();
+            const uint64_t corr2 = tc::pack2(corr, corr);
+#pragma unroll
+            for (int g = 0; g < kOD / 16; ++g) {
+                uint32_t t[16];
+                tc::tmem_ld16(lane_addr + kColO + (j & 1) * 64 + half * kOD + 16 * g, t);
+                tc::tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 8; ++i) o[8 * g + i] = tc::fma2(o[8 * g + i], corr2, tc::pack2(t[2 * i], t[2 * i + 1]));
+            }
+        };
+        for (int j = 0; j < nb && ok; ++j) {
+            const int b = j & 1;
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->s_full[b], (j >> 1) & 1, err));
+            if (!ok) break;
+            tc::tc_fence_after();
+            float s[32];
+            {
+                uint32_t t[32];
+                tc::tmem_ld32(lane_addr + kColS + b * kSP + half * 32, t);
+                tc::tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 32; ++i) s[i] = __uint_as_float(t[i]);
+            }
+            // visible: keys jlo <= key < jhi of the block
+            int jlo = 0, jhi = 64;
+            bool mask = false;
+            if (j >= nb_keys) {                            // own keys: the diagonal
+                jlo = r - (d0 + j - nb_keys) * 64;
+                jhi = is_cand ? jlo + 1 : jlo;
+                mask = true;
+            } else {
+                const int blk = it.blk0 + j;
+                const bool in_pages = blk < n_page_blocks;
+                const int idx = in_pages ? blk * 64 : (blk - n_page_blocks) * 64, pos = in_pages ? idx : sd.lin_pos0 + idx;
+                const int n_valid = (in_pages ? sd.n_paged : sd.n_lin) - idx;
+                jhi = min(n_valid, lim - pos);
+                mask = n_valid < 64 || pos + 64 > min_lim;
+            }
+            if (mask) {
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    const int key = half * 32 + i;
+                    if (key < jlo || key >= jhi) s[i] = kPointwise ? 0.f : -INFINITY;      // a logit of 0: SiLU(0) = 0
+                }
+            }
+            float c_new = 1.f;
+            if constexpr (kPointwise) {
+#pragma unroll
+                for (int i = 0; i < 32; ++i) s[i] = s[i] / (1.f + expf(-s[i]));
+                asm volatile("bar.sync %0, 64;" ::"r"(1 + quad) : "memory");      // both halves of S are in registers: P may take its place
+            } else {
+                float mx = fmaxf(s[0], s[1]), mx1 = fmaxf(s[2], s[3]);
+#pragma unroll
+                for (int i = 4; i < 32; i += 4) { mx = max3(mx, s[i], s[i + 1]); mx1 = max3(mx1, s[i + 2], s[i + 3]); }
+                mx = fmaxf(mx, mx1);
+                stat[(b * 2 + half) * kQRows + r] = mx;
+                asm volatile("bar.sync %0, 64;" ::"r"(1 + quad) : "memory");      // the two warps of these 32 rows (and: both have S in registers)
+                mx = fmaxf(mx, stat[(b * 2 + (half ^ 1)) * kQRows + r]);
+                const float mn = fmaxf(m, mx), ref = mn == -INFINITY ? 0.f : mn;
+                c_new = ex2(m - ref);
+                m = mn;
+                const uint64_t nref2 = tc::pack2(-ref, -ref);
+                uint64_t rs2 = 0;
+#pragma unroll
+                for (int i = 0; i < 32; i += 2) {
+                    tc::unpack2(tc::add2(tc::pack2(s[i], s[i + 1]), nref2), s[i], s[i + 1]);
+                    s[i] = ex2(s[i]); s[i + 1] = ex2(s[i + 1]);
+                    rs2 = tc::add2(rs2, tc::pack2(s[i], s[i + 1]));
+                }
+                float r0, r1;
+                tc::unpack2(rs2, r0, r1);
+                l = l * c_new + (r0 + r1);                 // of this thread's keys
+            }
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {                  // 16 keys = 8 words per plane
+                uint32_t w[3][8], part[3];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    split2(tc::pack2(s[16 * g + 2 * i], s[16 * g + 2 * i + 1]), part);
+                    w[0][i] = part[0]; w[1][i] = part[1]; w[2][i] = part[2];
+                }
+#pragma unroll
+                for (int p = 0; p < 3; ++p) tc::tmem_st8(lane_addr + kColS + b * kSP + p * 32 + half * 16 + 8 * g, w[p]);
+            }
+            tc::tmem_st_wait();
+            tc::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&bars->p_full[b]);
+            if (j > 0) take_o(j - 1);                      // while this block's products run
+            corr = c_new;
+        }
+        if (ok && nb > 0) take_o(nb - 1);
+        if constexpr (kPointwise) {
+            // divided by the number of visible keys; a split item hands it over as l with m = 0
+            m = 0.f;
+            l = (it.partial_slot < 0 || it.blk0 == 0) ? 0.5f * (float)(is_cand ? sd.causal_end + 1 : tpos + 1) : 0.f;
+        }
+        // l of the row: both threads' parts
+        stat[half * kQRows + r] = l;
+        asm volatile("bar.sync %0, 64;" ::"r"(1 + quad) : "memory");
+        l += stat[(half ^ 1) * kQRows + r];
+        if (ok && r < it.n_q) {
+            float *dst;
+            float inv = 1.f;
+            if (it.partial_slot < 0) {
+                dst = out + ((int64_t)sd.q_row0 + it.q0 + r) * d + it.head * DH + half * kOD;
+                inv = 1.f / l;
+            } else {
+                float *row = partial + ((size_t)it.partial_slot * kQRows + r) * (DH + 4);
+                if (half == 0) *reinterpret_cast<float4 *>(row) = make_float4(m, l, 0.f, 0.f);
+                dst = row + 4 + half * kOD;
+            }
+            const uint64_t inv2 = tc::pack2(inv, inv);
+#pragma unroll
+            for (int i = 0; i < kOD / 2; i += 2)
+                *reinterpret_cast<ulonglong2 *>(dst + 2 * i) = make_ulonglong2(tc::mul2(o[i], inv2), tc::mul2(o[i + 1], inv2));
+        }
+    }
+    tc::tc_fence_before();
+    __syncthreads();
+    if (warp == 16) tc::tmem_dealloc(tmem_base, kAttnCols);
+}
+
+// The partial results of split items (maxima in units of log2): a warp per row, coalesced.
+template <int DH>
+__global__ void __launch_bounds__(256)
+f32_merge_kernel(const AttnMerge *__restrict__ merges, const SeqDesc *__restrict__ seqs, const float *__restrict__ partial, int d_model,
+                 float *__restrict__ out)
+{
+    grid_launch_dependents();
+    grid_dependency_wait();
+    const AttnMerge mg = merges[blockIdx.x];
+    const int r = blockIdx.y * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (r >= mg.n_q) return;
+    const float *p0 = partial + ((size_t)mg.slot0 * kQRows + r) * (DH + 4);
+    constexpr size_t kStep = (size_t)kQRows * (DH + 4);
+    float M = -INFINITY, l = 0.f, o[DH / 32];
+    for (int i = 0; i < mg.n_splits; ++i) M = fmaxf(M, p0[i * kStep]);
+#pragma unroll
+    for (int c = 0; c < DH / 32; ++c) o[c] = 0.f;
+    for (int i = 0; i < mg.n_splits; ++i) {
+        const float *p = p0 + i * kStep;
+        const float w = p[0] == -INFINITY ? 0.f : ex2(p[0] - M);
+        l = fmaf(p[1], w, l);
+#pragma unroll
+        for (int c = 0; c < DH / 32; ++c) o[c] = fmaf(p[4 + lane + 32 * c], w, o[c]);
+    }
+    const float inv = 1.f / l;
+    float *dst = out + ((int64_t)seqs[mg.seq].q_row0 + mg.q0 + r) * d_model + mg.head * DH + lane;
+#pragma unroll
+    for (int c = 0; c < DH / 32; ++c) dst[32 * c] = o[c] * inv;
+}
+
+template <int DH>
+cudaError_t launch_attention(const float *q, const float *k_lin, const float *v_lin, PagedKV paged, const SeqDesc *seqs, const AttnItem *items,
+                             int n_items, const AttnMerge *merges, int n_merges, int n_heads, int attn_kind, float *out, float *partial, int *err,
+                             cudaStream_t stream, int64_t *launches)
+{
+    static PerDeviceValue attr_set;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (!attr_set.get(dev)) {
+        e = cudaFuncSetAttribute(f32_attention_tc_kernel<DH, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(f32_attention_tc_kernel<DH, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem);
+        if (e != cudaSuccess) return e;
+        attr_set.set(dev, 1);
+    }
+    auto kernel = attn_kind == ATTN_POINTWISE ? f32_attention_tc_kernel<DH, true> : f32_attention_tc_kernel<DH, false>;
+    *launches += 1;
+    e = launch_dependent(kernel, dim3((unsigned)n_items), dim3(kAttnThreads), (size_t)kAttnSmem, stream, 1, q, k_lin, v_lin, paged, seqs, items,
+                         n_heads, out, partial, err);
+    if (e != cudaSuccess || n_merges == 0) return e;
+    *launches += 1;
+    return launch_dependent(f32_merge_kernel<DH>, dim3((unsigned)n_merges, kQRows / 8), dim3(256), 0, stream, 1, merges, seqs, partial, n_heads * DH, out);
+}
+
+}  // namespace
+
+cudaError_t launch_gemm_f32_tc(const CUtensorMap &tmA, const CUtensorMap &tmW, int64_t M, int N, int K, const Epilogue &epi, int n_sms, int *err,
+                               cudaStream_t stream, int64_t *launches)
+{
+    if (M == 0 || N == 0) return cudaSuccess;
+    *launches += 1;
+    static PerDeviceValue attr_set;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (!attr_set.get(dev)) {
+        e = cudaFuncSetAttribute(f32_gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
+        if (e != cudaSuccess) return e;
+        attr_set.set(dev, 1);
+    }
+    const int64_t tiles = ((M + kBM - 1) / kBM) * ((N + kBN - 1) / kBN);
+    return launch_dependent(f32_gemm_tc_kernel, dim3((unsigned)(tiles < n_sms ? tiles : n_sms)), dim3(kGemmThreads), (size_t)kGemmSmem, stream, 1,
+                            tmA, tmW, M, N, K, epi, err);
+}
+
+cudaError_t launch_attention_f32_tc(const float *q, const float *k_lin, const float *v_lin, PagedKV paged, const SeqDesc *seqs, const AttnItem *items,
+                                    int n_items, const AttnMerge *merges, int n_merges, int n_heads, int d_head, int attn_kind, float *out,
+                                    float *partial, int *err, cudaStream_t stream, int64_t *launches)
+{
+    if (n_items == 0) return cudaSuccess;
+    if (d_head == 32) return launch_attention<32>(q, k_lin, v_lin, paged, seqs, items, n_items, merges, n_merges, n_heads, attn_kind, out, partial, err, stream, launches);
+    if (d_head == 64) return launch_attention<64>(q, k_lin, v_lin, paged, seqs, items, n_items, merges, n_merges, n_heads, attn_kind, out, partial, err, stream, launches);
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace relaygr

@@ -9,6 +9,12 @@
 namespace relaygr {
 
 namespace {
+// Whether a call of the fp32 model runs on the tensor cores or on the CUDA cores: by the values of an activation tensor.  The
+// tensor-core kernels have the longer start-up (tile loads, splits, turning accumulators around: 9 us at least, 7 us on the CUDA
+// cores) and 128-row tiles where those have 16-row ones.  Measured, a call on the CUDA cores / the tensor cores in us: 384 rows x 64
+// columns 94 / 127, 300 x 256 949 / 563, 576 x 256 1655 / 725, 4352 x 64 209 / 145, 4608 x 256 4910 / 1570.
+constexpr int64_t kF32TensorValues = 49152;
+inline bool f32_on_tensor_cores(int64_t rows, int d) { return rows * d >= kF32TensorValues; }
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 std::string cuda_msg(const char *what, cudaError_t e) { return std::string(what) + ": " + cudaGetErrorString(e); }
 }  // namespace
@@ -90,6 +96,24 @@ int Forward::init_device(int dev, std::string &err)
             }
             if (rc != 0) { err = "tensor-map encoding of the weights failed (pointers must be 16-byte aligned)"; return RELAYGR_E_CUDA; }
         }
+        wmaps_ok = true;
+    } else if (cfg.d_model >= 32 && cfg.d_ff >= 32) {
+        const uint64_t d = (uint64_t)cfg.d_model, F = (uint64_t)cfg.d_ff;
+        wmaps.resize((size_t)cfg.n_layers);
+        int rc = 0;
+        for (int l = 0; l < cfg.n_layers; ++l) {
+            LayerMaps &m = wmaps[(size_t)l];
+            auto map = [&](CUtensorMap &out, const void *base, size_t first, uint64_t rows, uint64_t cols) {
+                rc |= make_tmap_2d_f32(&out, (const float *)base + first, rows, cols, cols, (uint32_t)kF32WeightBoxRows, 32);
+            };
+            map(m.qkv, w.w_qkv, (size_t)l * 3 * d * d, 3 * d, d);
+            map(m.kv, w.w_qkv, ((size_t)l * 3 + 1) * d * d, 2 * d, d);
+            map(m.wq, w.w_qkv, (size_t)l * 3 * d * d, d, d);
+            map(m.ffn.wo, w.w_o, (size_t)l * d * d, d, d);
+            map(m.ffn.w1, w.w1, (size_t)l * F * d, F, d);
+            map(m.ffn.w2, w.w2, (size_t)l * d * F, d, F);
+        }
+        wmaps_ok = rc == 0;
     }
     return RELAYGR_OK;
 }
@@ -202,6 +226,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     const WorkspaceLayout lay = layout(R, B, (int64_t)call.page_table.size());
     constexpr bool kTensor = sizeof(T) == 2;      // bf16 model: GEMMs and attention run on the tensor cores
     const bool preinfer = call.mode == MODE_PREINFER;
+    const bool tensor32 = !kTensor && wmaps_ok && f32_on_tensor_cores(R, d);
     const int64_t n_scores = (!preinfer && call.score_off) ? call.score_off[B] : 0;
     // In the last layer of a rank / full-inference call only the candidates' hidden states are read afterwards: its attention runs on
     // their rows alone.  What follows may run on them alone too, once they have been moved together (and their query projection
@@ -239,13 +264,13 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     std::vector<AttnMerge> merges, merges_c;
     std::vector<SeqDesc> seqs_c;                  // the candidates of each user as rows of their own (last layer)
     size_t o_items = 0, o_merges = 0, o_seq_c = 0, o_items_c = 0, o_merges_c = 0;
-    // the work of an attention launch over `seqs`: items and merges (tensor cores), or query tiles (fp32 model)
+    // the work of an attention launch over `seqs`: items and merges (tensor cores), or query tiles (CUDA cores)
     std::vector<F32Tile> tiles, tiles_c;
     int tile_rows = 0, tile_rows_c = 0;
     auto put_work = [&](const std::vector<SeqDesc> &seqs, std::vector<AttnItem> &it, std::vector<AttnMerge> &mg, std::vector<F32Tile> &ti,
                         size_t &o_it, size_t &o_mg, int &rows) {
-        if (kTensor) {
-            build_attention_worklist(seqs, H, n_sms, kMaxSplitTiles, it, mg);
+        if (kTensor || tensor32) {
+            build_attention_worklist(seqs, H, kTensor ? attn_machine_bf16(n_sms) : attn_machine_f32(n_sms), kMaxSplitTiles, it, mg);
             if (!it.empty()) o_it = put(reinterpret_cast<const int32_t *>(it.data()), it.size() * (sizeof(AttnItem) / 4));
             if (!mg.empty()) o_mg = put(reinterpret_cast<const int32_t *>(mg.data()), mg.size() * (sizeof(AttnMerge) / 4));
         } else {
@@ -334,11 +359,21 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         if (trc != 0) { err = "tensor-map encoding of the activations failed"; return RELAYGR_E_CUDA; }
         act.ws = ws; act.rows = R; act.cand_rows = cand_rows; act.slab = call.pool_slab; act.pages = call.pool_pages;
     }
+    if (tensor32 && !maps_cached) {
+        act.ws = nullptr;
+        int trc = make_tmap_2d_f32(&tm_a, a, (uint64_t)R, (uint64_t)d, (uint64_t)d, 128, 32);
+        trc |= make_tmap_2d_f32(&tm_att, att, (uint64_t)R, (uint64_t)d, (uint64_t)d, 128, 32);
+        trc |= make_tmap_2d_f32(&tm_hid, hid, (uint64_t)R, (uint64_t)F, (uint64_t)F, 128, 32);
+        if (compact_last) trc |= make_tmap_2d_f32(&tm_a_c, a_c, (uint64_t)n_scores, (uint64_t)d, (uint64_t)d, 128, 32);
+        if (trc != 0) { err = "tensor-map encoding of the activations failed"; return RELAYGR_E_CUDA; }
+        act.ws = ws; act.rows = R; act.cand_rows = cand_rows; act.slab = call.pool_slab; act.pages = call.pool_pages;
+    }
     auto gemm = [&](int64_t M, const T *A, const CUtensorMap &tmA, const T *W, const CUtensorMap *tmW, const GemmOutMaps &om, int N, int K,
                     const Epilogue &ep) {
         cudaEvent_t pe = prof_begin(stream);
         cudaError_t r;
         if constexpr (kTensor) r = launch_gemm_tc(tmA, *tmW, om, M, N, K, ep, d_status, stream, &launches);
+        else if (tensor32) r = launch_gemm_f32_tc(tmA, *tmW, M, N, K, ep, n_sms, d_status, stream, &launches);
         else r = launch_gemm_f32(A, W, M, N, K, ep, n_sms, stream, &launches);
         prof_end(KC_GEMM, pe, stream);
         return r;
@@ -359,7 +394,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     const AttnItem *items_m = reinterpret_cast<const AttnItem *>(meta + o_items);
     const AttnMerge *merges_m = reinterpret_cast<const AttnMerge *>(meta + o_merges);
     const F32Tile *tiles_m = reinterpret_cast<const F32Tile *>(meta + o_items);
-    int n_items_m = (int)(kTensor ? items.size() : tiles.size()), n_merges_m = (int)merges.size();
+    int n_items_m = (int)(kTensor || tensor32 ? items.size() : tiles.size()), n_merges_m = (int)merges.size();
     bool dead_tail = false;                       // a call without candidates: nothing reads the last layer
 
     for (int l = 0; l < L; ++l) {
@@ -391,7 +426,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         }
         if (preinfer) { ep.paged = paged; ep.page_runs = meta + o_runs; }
         const T *Wqkv = (const T *)w.w_qkv + ((size_t)l * 3 * d + ep.col0) * d;
-        lm = kTensor ? &wmaps[(size_t)l] : nullptr;
+        lm = wmaps_ok ? &wmaps[(size_t)l] : nullptr;
         e = gemm(R, a, tm_a, Wqkv, lm ? (kv_only ? &lm->kv : &lm->qkv) : nullptr, om_qkv, 3 * d - ep.col0, d, ep);
         if (!ck("QKV projection")) return RELAYGR_E_CUDA;
         if (preinfer && last) break;
@@ -401,7 +436,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
             items_m = reinterpret_cast<const AttnItem *>(meta + o_items_c);
             merges_m = reinterpret_cast<const AttnMerge *>(meta + o_merges_c);
             tiles_m = reinterpret_cast<const F32Tile *>(meta + o_items_c); tile_rows = tile_rows_c;
-            n_items_m = (int)(kTensor ? items_c.size() : tiles_c.size()); n_merges_m = (int)merges_c.size();
+            n_items_m = (int)(kTensor || tensor32 ? items_c.size() : tiles_c.size()); n_merges_m = (int)merges_c.size();
         }
         if (last && compact_last) {
             // move the candidates' rows of x and of LN1(x) together, then project their queries
@@ -427,6 +462,9 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
                 e = launch_attention_tc(tm_q, tm_k, tm_v, tm_pool, items_m, n_items_m, merges_m, n_merges_m, seqs_m, meta + o_pt, L,
                                         l, d, cfg.attn_kind, call.mode == MODE_RANK, att, reinterpret_cast<float *>(ws + lay.partial),
                                         reinterpret_cast<int *>(ws + lay.meta) + o_ctr + l, n_sms, d_status, stream, &launches);
+            else if (tensor32)
+                e = launch_attention_f32_tc(q, kl, vl, paged, seqs_m, items_m, n_items_m, merges_m, n_merges_m, H, cfg.d_head, cfg.attn_kind, att,
+                                            reinterpret_cast<float *>(ws + lay.partial), d_status, stream, &launches);
             else
                 e = launch_attention_f32(q, kl, vl, paged, seqs_m, tiles_m, n_items_m, tile_rows, H, cfg.d_head, cfg.attn_kind, att, stream, &launches);
             prof_end(KC_ATTENTION, pe, stream);

@@ -17,8 +17,12 @@ namespace relaygr {
 
 enum CallMode { MODE_PREINFER = 0, MODE_RANK = 1, MODE_FULL = 2 };
 
-// The attention work list of one call (host only): items in launch order, and the merges of split items.
-void build_attention_worklist(const std::vector<SeqDesc> &seqs, int n_heads, int n_sms, int64_t max_split_tiles,
+// The attention work list of one call (host only): items in launch order, and the merges of split items.  `slots` items run at a
+// time; item_fixed = what an item costs beside its key blocks, in key blocks.
+struct AttnMachine { int64_t slots; double item_fixed; };
+inline AttnMachine attn_machine_bf16(int n_sms) { return {2 * (int64_t)(n_sms < 1 ? 1 : n_sms), 8.0}; }      // two CTAs per SM
+inline AttnMachine attn_machine_f32(int n_sms) { return {(int64_t)(n_sms < 1 ? 1 : n_sms), 4.0}; }           // one CTA per SM, blocks of about 1.5 us
+void build_attention_worklist(const std::vector<SeqDesc> &seqs, int n_heads, const AttnMachine &machine, int64_t max_split_tiles,
                               std::vector<AttnItem> &items, std::vector<AttnMerge> &merges);
 
 struct CallDesc {
@@ -47,11 +51,12 @@ struct Forward {
     int device = 0;
     int n_sms = 148;
 
-    // tensor maps of the weights (bf16 model), one set per layer
+    // tensor maps of the weights, one set per layer
     struct LayerMaps { CUtensorMap qkv, kv, wq; FfnMaps ffn; };
     std::vector<LayerMaps> wmaps;
+    bool wmaps_ok = false;       // false (fp32 model only): a weight pointer is not 16-byte aligned and cannot have a map
 
-    // tensor maps of the activations (bf16 model): a function of the workspace, the row counts and the pool slab alone, so
+    // tensor maps of the activations: a function of the workspace, the row counts and the pool slab alone, so
     // calls of the same shape - the usual case in serving - reuse them instead of encoding some twenty maps per call
     struct ActMaps {
         const char *ws = nullptr; int64_t rows = -1, cand_rows = -1; const void *slab = nullptr; int64_t pages = -1;

@@ -86,6 +86,16 @@ cudaError_t launch_attention_f32(const float *q, const float *k_lin, const float
                                  const F32Tile *tiles, int n_tiles, int tile_rows, int n_heads, int d_head, int attn_kind, float *out,
                                  cudaStream_t stream, int64_t *launches);
 
+// The same two on the tensor cores, every fp32 operand as three bf16 parts.  tmA / tmW: A [M, K] in boxes of 128 rows x 32 columns, W
+// [N, K] in boxes of kF32WeightBoxRows rows x 32 columns, 128-byte swizzle; N and K multiples of 4.  partial: split results of the
+// attention, rows of d_head + 4 floats.
+constexpr int kF32WeightBoxRows = 64;
+cudaError_t launch_gemm_f32_tc(const CUtensorMap &tmA, const CUtensorMap &tmW, int64_t M, int N, int K, const Epilogue &epi, int n_sms, int *err,
+                               cudaStream_t stream, int64_t *launches);
+cudaError_t launch_attention_f32_tc(const float *q, const float *k_lin, const float *v_lin, PagedKV paged, const SeqDesc *seqs, const AttnItem *items,
+                                    int n_items, const AttnMerge *merges, int n_merges, int n_heads, int d_head, int attn_kind, float *out,
+                                    float *partial, int *err, cudaStream_t stream, int64_t *launches);
+
 // ---- tensor-core kernels (the bf16 model) -------------------------------------------------------------
 
 // The tensor-core GEMM for [M, K] x [N, K]^T (N % 128 == 0) runs on CTA pairs (256 x 256 tiles, tcgen05 cta_group::2)

@@ -166,7 +166,7 @@ int32_t relaygr_attention_plan(int32_t mode, int32_t n_users, const int32_t *pre
     }
     std::vector<AttnItem> it;
     std::vector<AttnMerge> mg;
-    build_attention_worklist(seqs, n_heads, n_sms, Forward::kMaxSplitTiles, it, mg);
+    build_attention_worklist(seqs, n_heads, attn_machine_bf16(n_sms), Forward::kMaxSplitTiles, it, mg);
     *n_items = (int32_t)it.size();
     *n_merges = (int32_t)mg.size();
     if ((int64_t)it.size() > cap_items || (int64_t)mg.size() > cap_merges) return fail(RELAYGR_E_NOSPACE, "plan larger than the arrays given");
