@@ -65,7 +65,8 @@ constexpr int kBM = 128, kBN = 64, kBK = 64, kStages = 2, kSlots = 3;
 constexpr int kWorkers = 256, kEpiWarps = 4, kGemmThreads = kWorkers + 32 + 32 * kEpiWarps + 32;
 constexpr int kWPlane = kBN * 128, kStage = 3 * kWPlane;                        // W's parts: three planes of 64 rows x 64 columns
 constexpr int kSlotA = kBM * 128, kSlotW = kBN * 128, kSlot = 2 * (kSlotA + kSlotW);      // fp32: two tiles of 32 columns of A, two of W
-constexpr int kOffSlots = kStages * kStage, kOffPatch = kOffSlots + kSlots * kSlot, kOffGBars = kOffPatch + kEpiWarps * 4096;
+constexpr int kOffSlots = kStages * kStage, kOffPatch = kOffSlots + kSlots * kSlot, kOffBias = kOffPatch + kEpiWarps * 2 * 4096,
+              kOffGBars = kOffBias + kEpiWarps * kBN * 4;
 constexpr int kGemmSmem = kOffGBars + 256 + 1024;
 static_assert(kGemmSmem <= 227 * 1024, "shared memory budget");
 constexpr uint32_t kColLead = 0, kColSmall = 2 * kBN, kColA = 4 * kBN, kColAStage = 96, kGemmCols = 512;      // A's parts: 3 x 32 columns a stage
@@ -78,7 +79,8 @@ struct GemmBars {
 static_assert(sizeof(GemmBars) <= 256, "barrier block");
 
 __global__ void __launch_bounds__(kGemmThreads, 1)
-f32_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, int64_t M, int N, int K, Epilogue e, int *err)
+f32_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, const __grid_constant__ GemmOutMaps om, int64_t M,
+                   int N, int K, Epilogue e, int *err)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -126,8 +128,8 @@ f32_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                                              tc::mbar_wait(&bars->empty[s], ((it >> 1) & 1) ^ 1, err));
                 if (!ok) break;
                 tc::tc_fence_after();
-#pragma unroll 1
-                for (int h = 0; h < 2; ++h) {          // 16 columns = 8 words per plane (rolled loops: cold code costs its fetch)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {          // 16 columns = 8 words per plane
                     uint32_t w[3][8], part[3];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
@@ -211,23 +213,33 @@ f32_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         // ---------------------------------------------------------------- epilogue: warp w has TMEM lanes 32 (w % 4) .. + 31
         const int quad = warp & 3;
         const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
-        uint8_t *patch = smem + kOffPatch + quad * 4096;
-        const int pj = lane & 7, prow = lane >> 3, d = e.d_model;      // when a patch is stored: this lane's chunk of a row, first row
+        uint8_t *patches = smem + kOffPatch + quad * (2 * 4096);
+        float *bias_s = reinterpret_cast<float *>(smem + kOffBias) + quad * kBN;
+        const int d = e.d_model;
         bool ok = true;
         int grp = 0, nt = 0;
         for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++nt) {
             const int64_t m0 = (int64_t)(tile / tiles_n) * kBM + quad * 32;
             const int n0 = (tile % tiles_n) * kBN;
-            // where rows go that belong in pages: offset of (page, K, slot); of a user's last row its slot
-            const bool to_pages = e.mode == EPI_QKV && e.paged.slab != nullptr && e.col0 + n0 + kBN > e.d_model;
+#pragma unroll
+            for (int c = 0; c < kBN; c += 32) bias_s[c + lane] = e.bias && n0 + c + lane < N ? e.bias[n0 + c + lane] : 0.f;
+            // K / V rows of a pre-infer call go into pages: where in the pool the warp's 32 rows are, if they are 32 consecutive slots of
+            // one page, else the offset of (page, K, slot) of this lane's row, and of a user's last row its slot
+            const bool to_pages = e.mode == EPI_QKV && e.paged.slab != nullptr && e.col0 + n0 + kBN > d;
+            int pool_row0 = -1, last_slot = -1;
             int64_t page_off = 0;
-            int last_slot = -1;
-            if (to_pages && m0 + lane < M) {
-                const int u = find_user(e.row_off, e.n_users, (int)(m0 + lane));
-                const int t = (int)(m0 + lane) - e.row_off[u];
-                page_off = (int64_t)page_elem_offset(e.paged, e.paged.pt[e.seqs[u].pt_base + (t >> 6)], 0, t & 63);
-                if (t == e.seqs[u].n_q - 1) last_slot = t & 63;
+            if (to_pages && m0 < M) {
+                const int g = e.page_runs[m0 >> 5];
+                if (g >= 0) {
+                    pool_row0 = ((g >> 6) * e.paged.n_layers + e.paged.layer) * 128 + (g & 63);
+                } else if (m0 + lane < M) {
+                    const int u = find_user(e.row_off, e.n_users, (int)(m0 + lane));
+                    const int t = (int)(m0 + lane) - e.row_off[u];
+                    page_off = (int64_t)page_elem_offset(e.paged, e.paged.pt[e.seqs[u].pt_base + (t >> 6)], 0, t & 63);
+                    if (t == e.seqs[u].n_q - 1) last_slot = t & 63;
+                }
             }
+            __syncwarp();
             float acc[2][32];
             for (int g = 0; g < n_groups; ++g, ++grp) {
                 ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->acc_full[grp & 1], (grp >> 1) & 1, err));
@@ -250,75 +262,61 @@ f32_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                 if (lane == 0) tc::mbar_arrive(&bars->acc_empty[grp & 1]);
             }
             if (!ok) break;
-            // one row per thread so far; 32 rows x 32 columns at a time are turned around in shared memory, so that global memory sees
-            // whole rows of 128 bytes
+            // 32 rows x 32 columns at a time are staged (a row per thread) and handed to the TMA unit: a store, or for the residual stream
+            // an fp32 add-reduction in L2.  (Plain loads and stores queue behind the other warps' shared-memory traffic: 3500 clocks a patch.)
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const int n = n0 + h * 32 + pj * 4;    // this lane's four columns (N is a multiple of 4)
-                const bool in_n = n < N;
-                float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (e.bias && in_n) bias = make_float4(e.bias[n], e.bias[n + 1], e.bias[n + 2], e.bias[n + 3]);
-                // where column n goes: the output (or residual stream), q, or K / V (rows of pages: added per row)
-                float *out = e.mode == EPI_STORE ? reinterpret_cast<float *>(e.out) : e.out_f32;
-                int64_t pitch = N, off0 = n;
-                bool paged = false;
-                if (e.mode == EPI_QKV) {
-                    const int qcol = e.col0 + n, which = (qcol >= d) + (qcol >= 2 * d);
-                    paged = to_pages && which > 0;
-                    out = reinterpret_cast<float *>(paged ? e.paged.slab : which == 0 ? e.q : which == 1 ? e.k_lin : e.v_lin);
-                    pitch = d;
-                    off0 = qcol - which * d + (paged ? (int64_t)(which - 1) * 64 * d : 0);
-                }
-                float4 x[8];                           // the residual, of rows prow, prow + 4, ...: all on their way before any is used
-                if (e.mode == EPI_RESID) {
-                    const float *p = e.resid + (m0 + prow) * N + n;
-#pragma unroll
-                    for (int i = 0; i < 8; ++i, p += (int64_t)4 * N) {
-                        x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (in_n && m0 + 4 * i + prow < M) x[i] = *reinterpret_cast<const float4 *>(p);
-                    }
-                }
+                const int n = n0 + 32 * h;             // 32 columns lie in one of q, K, V: d_model is a multiple of 32
+                if (n >= N || m0 >= M) continue;
+                uint8_t *patch = patches + h * 4096;
+                if (lane == 0) tc::bulk_wait_read<1>();      // the patch's last store but the other's has read it
                 __syncwarp();
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    *reinterpret_cast<float4 *>(chunk_at(patch, lane, j)) = make_float4(acc[h][4 * j], acc[h][4 * j + 1], acc[h][4 * j + 2], acc[h][4 * j + 3]);
-                __syncwarp();
-                auto value = [&](int i) {
-                    const float4 v = *reinterpret_cast<const float4 *>(chunk_at(patch, 4 * i + prow, pj));
-                    return make_float4(v.x + bias.x, v.y + bias.y, v.z + bias.z, v.w + bias.w);
-                };
-                float *dst = out + off0 + (m0 + prow) * pitch;
-                if (e.mode == EPI_RESID) {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i, dst += 4 * pitch) {
-                        const float4 v = value(i);
-                        if (in_n && m0 + 4 * i + prow < M) *reinterpret_cast<float4 *>(dst) = make_float4(x[i].x + v.x, x[i].y + v.y, x[i].z + v.z, x[i].w + v.w);
-                    }
-                } else if (!to_pages) {
-                    const bool silu = e.mode == EPI_STORE && e.silu;
+                for (int j = 0; j < 8; ++j) {
+                    const float4 b = *reinterpret_cast<const float4 *>(bias_s + 32 * h + 4 * j);
+                    *reinterpret_cast<float4 *>(chunk_at(patch, lane, j)) = make_float4(acc[h][4 * j] + b.x, acc[h][4 * j + 1] + b.y, acc[h][4 * j + 2] + b.z, acc[h][4 * j + 3] + b.w);
+                }
+                if (e.mode == EPI_STORE && e.silu) {
 #pragma unroll 2
-                    for (int i = 0; i < 8; ++i, dst += 4 * pitch) {
-                        float4 v = value(i);
-                        if (silu) { v.x /= 1.f + expf(-v.x); v.y /= 1.f + expf(-v.y); v.z /= 1.f + expf(-v.z); v.w /= 1.f + expf(-v.w); }
-                        if (in_n && m0 + 4 * i + prow < M) *reinterpret_cast<float4 *>(dst) = v;
-                    }
-                } else {
-#pragma unroll 1
-                    for (int i = 0; i < 8; ++i) {
-                        const int rr = 4 * i + prow;
-                        const float4 v = value(i);
-                        const int64_t row_off = __shfl_sync(0xffffffffu, page_off, rr);
-                        const int ls = __shfl_sync(0xffffffffu, last_slot, rr);
-                        float *q = out + off0 + (paged ? row_off : (m0 + rr) * pitch);
-                        if (in_n && m0 + rr < M) {
-                            *reinterpret_cast<float4 *>(q) = v;
-                            if (paged && ls >= 0)      // last row of the prefix: clear the unused slots of its page
-                                for (int z = 1; ls + z < 64; ++z) *reinterpret_cast<float4 *>(q + (int64_t)z * d) = make_float4(0.f, 0.f, 0.f, 0.f);
-                        }
+                    for (int j = 0; j < 8; ++j) {
+                        float4 *p = reinterpret_cast<float4 *>(chunk_at(patch, lane, j));
+                        const float4 v = *p;
+                        *p = make_float4(v.x / (1.f + expf(-v.x)), v.y / (1.f + expf(-v.y)), v.z / (1.f + expf(-v.z)), v.w / (1.f + expf(-v.w)));
                     }
                 }
+                int which = 0, c = n;                  // destination tensor and its column
+                if (e.mode == EPI_QKV) { const int col = e.col0 + n; which = (col >= d) + (col >= 2 * d); c = col - which * d; }
+                const bool paged = to_pages && which > 0;
+                tc::fence_proxy_async();
+                __syncwarp();
+                if (!paged || pool_row0 >= 0) {
+                    if (lane == 0) {
+                        if (e.mode == EPI_RESID) tc::tma_reduce_add_2d(&om.o[0], patch, c, (int)m0);
+                        else if (paged) tc::tma_store_2d(&om.pool, patch, c, pool_row0 + (which - 1) * 64);
+                        else tc::tma_store_2d(&om.o[which], patch, c, (int)m0);
+                        tc::bulk_commit();
+                    }
+                    continue;
+                }
+                if (lane == 0) tc::bulk_commit();      // (an empty group: the count above stays one per patch)
+                const int pj = lane & 7, prow = lane >> 3;
+#pragma unroll 1
+                for (int i = 0; i < 8; ++i) {
+                    const int rr = 4 * i + prow;
+                    const float4 v = *reinterpret_cast<const float4 *>(chunk_at(patch, rr, pj));
+                    const int64_t row_off = __shfl_sync(0xffffffffu, page_off, rr);
+                    const int ls = __shfl_sync(0xffffffffu, last_slot, rr);
+                    float *q = reinterpret_cast<float *>(e.paged.slab) + row_off + (int64_t)(which - 1) * 64 * d + c + 4 * pj;
+                    if (m0 + rr < M) {
+                        *reinterpret_cast<float4 *>(q) = v;
+                        if (ls >= 0)                   // last row of the prefix: clear the unused slots of its page
+                            for (int z = 1; ls + z < 64; ++z) *reinterpret_cast<float4 *>(q + (int64_t)z * d) = make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+                }
+                __syncwarp();
             }
         }
+        if (lane == 0) tc::bulk_wait_read<0>();        // the patches have been read; the grid's completion covers the global writes
     }
     tc::tc_fence_before();
     __syncthreads();
@@ -740,8 +738,8 @@ cudaError_t launch_attention(const float *q, const float *k_lin, const float *v_
 
 }  // namespace
 
-cudaError_t launch_gemm_f32_tc(const CUtensorMap &tmA, const CUtensorMap &tmW, int64_t M, int N, int K, const Epilogue &epi, int n_sms, int *err,
-                               cudaStream_t stream, int64_t *launches)
+cudaError_t launch_gemm_f32_tc(const CUtensorMap &tmA, const CUtensorMap &tmW, const GemmOutMaps &om, int64_t M, int N, int K, const Epilogue &epi,
+                               int n_sms, int *err, cudaStream_t stream, int64_t *launches)
 {
     if (M == 0 || N == 0) return cudaSuccess;
     *launches += 1;
@@ -756,7 +754,7 @@ cudaError_t launch_gemm_f32_tc(const CUtensorMap &tmA, const CUtensorMap &tmW, i
     }
     const int64_t tiles = ((M + kBM - 1) / kBM) * ((N + kBN - 1) / kBN);
     return launch_dependent(f32_gemm_tc_kernel, dim3((unsigned)(tiles < n_sms ? tiles : n_sms)), dim3(kGemmThreads), (size_t)kGemmSmem, stream, 1,
-                            tmA, tmW, M, N, K, epi, err);
+                            tmA, tmW, om, M, N, K, epi, err);
 }
 
 cudaError_t launch_attention_f32_tc(const float *q, const float *k_lin, const float *v_lin, PagedKV paged, const SeqDesc *seqs, const AttnItem *items,

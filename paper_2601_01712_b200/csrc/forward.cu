@@ -10,9 +10,9 @@ namespace relaygr {
 
 namespace {
 // Whether a call of the fp32 model runs on the tensor cores or on the CUDA cores: by the values of an activation tensor.  The
-// tensor-core kernels have the longer start-up (tile loads, splits, turning accumulators around: 9 us at least, 7 us on the CUDA
-// cores) and 128-row tiles where those have 16-row ones.  Measured, a call on the CUDA cores / the tensor cores in us: 384 rows x 64
-// columns 94 / 127, 300 x 256 949 / 563, 576 x 256 1655 / 725, 4352 x 64 209 / 145, 4608 x 256 4910 / 1570.
+// tensor-core kernels have the longer start-up (tile loads, splits, turning accumulators around) and 128-row tiles where those have
+// 16-row ones.  Measured, a call on the CUDA cores / the tensor cores in us: rank, 384 rows x 64 columns 93 / 110, 768 x 64 117 / 110,
+// 1536 x 64 134 / 114, 100 x 256 1015 / 605; pre-infer, 700 x 64 62 / 69, 1400 x 64 79 / 75, 700 x 256 1307 / 575.
 constexpr int64_t kF32TensorValues = 49152;
 inline bool f32_on_tensor_cores(int64_t rows, int d) { return rows * d >= kF32TensorValues; }
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -249,7 +249,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     const size_t o_seq = put(reinterpret_cast<const int32_t *>(call.seqs.data()), (size_t)B * (sizeof(SeqDesc) / 4));
     const size_t o_pt = call.page_table.empty() ? 0 : put(call.page_table.data(), call.page_table.size());
     size_t o_runs = 0;
-    if (kTensor && preinfer) {                    // see Epilogue::page_runs
+    if ((kTensor || tensor32) && preinfer) {      // see Epilogue::page_runs
         std::vector<int32_t> runs((size_t)((R + 31) / 32), -1);
         for (int u = 0; u < B; ++u) {
             const SeqDesc &sd = call.seqs[(size_t)u];
@@ -364,7 +364,20 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         int trc = make_tmap_2d_f32(&tm_a, a, (uint64_t)R, (uint64_t)d, (uint64_t)d, 128, 32);
         trc |= make_tmap_2d_f32(&tm_att, att, (uint64_t)R, (uint64_t)d, (uint64_t)d, 128, 32);
         trc |= make_tmap_2d_f32(&tm_hid, hid, (uint64_t)R, (uint64_t)F, (uint64_t)F, 128, 32);
-        if (compact_last) trc |= make_tmap_2d_f32(&tm_a_c, a_c, (uint64_t)n_scores, (uint64_t)d, (uint64_t)d, 128, 32);
+        trc |= make_tmap_2d_f32(&om_qkv.o[0], q, (uint64_t)R, (uint64_t)d, (uint64_t)d, 32, 32);
+        trc |= make_tmap_2d_f32(&om_qkv.o[1], kl, (uint64_t)R, (uint64_t)d, (uint64_t)d, 32, 32);
+        trc |= make_tmap_2d_f32(&om_qkv.o[2], vl, (uint64_t)R, (uint64_t)d, (uint64_t)d, 32, 32);
+        trc |= make_tmap_2d_f32(&om_hid.o[0], hid, (uint64_t)R, (uint64_t)F, (uint64_t)F, 32, 32);
+        trc |= make_tmap_2d_f32(&om_x.o[0], x, (uint64_t)R, (uint64_t)d, (uint64_t)d, 32, 32);
+        om_qkv.pool = om_qkv.o[0];
+        if (call.pool_slab) trc |= make_tmap_2d_f32(&om_qkv.pool, call.pool_slab, (uint64_t)call.pool_pages * L * 2 * 64, (uint64_t)d, (uint64_t)d, 32, 32);
+        om_hid.o[1] = om_hid.o[2] = om_hid.pool = om_hid.o[0];
+        om_x.o[1] = om_x.o[2] = om_x.pool = om_x.o[0];
+        if (compact_last) {
+            trc |= make_tmap_2d_f32(&tm_a_c, a_c, (uint64_t)n_scores, (uint64_t)d, (uint64_t)d, 128, 32);
+            trc |= make_tmap_2d_f32(&om_x_c.o[0], x_c, (uint64_t)n_scores, (uint64_t)d, (uint64_t)d, 32, 32);
+            om_x_c.o[1] = om_x_c.o[2] = om_x_c.pool = om_x_c.o[0];
+        }
         if (trc != 0) { err = "tensor-map encoding of the activations failed"; return RELAYGR_E_CUDA; }
         act.ws = ws; act.rows = R; act.cand_rows = cand_rows; act.slab = call.pool_slab; act.pages = call.pool_pages;
     }
@@ -373,7 +386,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         cudaEvent_t pe = prof_begin(stream);
         cudaError_t r;
         if constexpr (kTensor) r = launch_gemm_tc(tmA, *tmW, om, M, N, K, ep, d_status, stream, &launches);
-        else if (tensor32) r = launch_gemm_f32_tc(tmA, *tmW, M, N, K, ep, n_sms, d_status, stream, &launches);
+        else if (tensor32) r = launch_gemm_f32_tc(tmA, *tmW, om, M, N, K, ep, n_sms, d_status, stream, &launches);
         else r = launch_gemm_f32(A, W, M, N, K, ep, n_sms, stream, &launches);
         prof_end(KC_GEMM, pe, stream);
         return r;

@@ -86,12 +86,18 @@ cudaError_t launch_attention_f32(const float *q, const float *k_lin, const float
                                  const F32Tile *tiles, int n_tiles, int tile_rows, int n_heads, int d_head, int attn_kind, float *out,
                                  cudaStream_t stream, int64_t *launches);
 
+// Where a GEMM's epilogue stores: tensor maps with a 32-row box of 128 bytes and the 128-byte swizzle, in the model's type.
+// EPI_STORE: o[0] = out [M, N].  EPI_RESID: o[0] = the fp32 residual stream [M, N] (tile added in place).
+// EPI_QKV: o[0] = q, o[1] = k_lin, o[2] = v_lin, each [M, d] (o[1], o[2] are not used when K / V go to pages);
+// pool = the pool slab viewed as [pages * L * 2 * 64, d] (used when K / V go to pages, else any valid map).
+struct GemmOutMaps { CUtensorMap o[3]; CUtensorMap pool; };
+
 // The same two on the tensor cores, every fp32 operand as three bf16 parts.  tmA / tmW: A [M, K] in boxes of 128 rows x 32 columns, W
 // [N, K] in boxes of kF32WeightBoxRows rows x 32 columns, 128-byte swizzle; N and K multiples of 4.  partial: split results of the
 // attention, rows of d_head + 4 floats.
 constexpr int kF32WeightBoxRows = 64;
-cudaError_t launch_gemm_f32_tc(const CUtensorMap &tmA, const CUtensorMap &tmW, int64_t M, int N, int K, const Epilogue &epi, int n_sms, int *err,
-                               cudaStream_t stream, int64_t *launches);
+cudaError_t launch_gemm_f32_tc(const CUtensorMap &tmA, const CUtensorMap &tmW, const GemmOutMaps &om, int64_t M, int N, int K, const Epilogue &epi,
+                               int n_sms, int *err, cudaStream_t stream, int64_t *launches);
 cudaError_t launch_attention_f32_tc(const float *q, const float *k_lin, const float *v_lin, PagedKV paged, const SeqDesc *seqs, const AttnItem *items,
                                     int n_items, const AttnMerge *merges, int n_merges, int n_heads, int d_head, int attn_kind, float *out,
                                     float *partial, int *err, cudaStream_t stream, int64_t *launches);
@@ -107,12 +113,6 @@ inline bool gemm_pair(int64_t M, int N, int K)
     return N % 256 == 0 && (K >= 512 || ((M + 255) / 256) * (N / 256) >= 4 * 74);
 }
 constexpr int kGemmWeightBoxRows = 128;
-
-// Where a GEMM's epilogue stores: tensor maps with a 32-row box of 128 bytes and the 128-byte swizzle.
-// EPI_STORE: o[0] = out [M, N] bf16.  EPI_RESID: o[0] = the fp32 residual stream [M, N] (tile added in place).
-// EPI_QKV: o[0] = q, o[1] = k_lin, o[2] = v_lin, each [M, d] bf16 (o[1], o[2] are not used when K / V go to pages);
-// pool = the pool slab viewed as [pages * L * 2 * 64, d] (used when K / V go to pages, else any valid map).
-struct GemmOutMaps { CUtensorMap o[3]; CUtensorMap pool; };
 
 // C[m, n] = sum_k A[m, k] W[n, k] on tcgen05; tmA covers A [M, K] with a 128-row box, tmB covers W [N, K]
 // with a box of kGemmWeightBoxRows rows, both 64 columns wide with the 128-byte swizzle.  N % 128 == 0, K % 64 == 0.
