@@ -7,7 +7,8 @@
 //     A = LN(mid)             bf16 into shared memory where the attention tile was
 //     per chunk:              S = A W1c^T (fp32 in TMEM), H = SiLU(S + b1c) (bf16 over S's own columns), O += H W2c^T
 // The partial O (only the first CTA's holds mid) are added up through distributed shared memory in rank order - one
-// fixed order of the fp32 sums, so results do not vary from run to run - and each CTA finishes its share of the tile's rows.
+// fixed order of the fp32 sums, so results do not vary from run to run - and each CTA finishes its share of the tile's rows, the
+// next layer's LayerNorm (or the final one and the scoring head) included: a launch less in a chain of short ones.
 //
 // What bounds it: a serial chain - loads, projection, LayerNorm, chunk products, exchange.  With one CTA per tile the chain of a
 // 1024-unit feed-forward took 27 us while most SMs were idle; every split of the chunks shortens it.
@@ -49,6 +50,12 @@ struct Bars {
 };
 static_assert(sizeof(Bars) <= 256, "barrier block");
 
+__device__ __forceinline__ float warp_sum(float v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
 __device__ __forceinline__ float4 load_cluster4(uint32_t addr)
 {
     float4 v;
@@ -61,7 +68,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2,
                  const __grid_constant__ CUtensorMap tmAtt, const __grid_constant__ CUtensorMap tmWo,
                  float *__restrict__ x, const float *__restrict__ g, const float *__restrict__ b, const float *__restrict__ b1,
-                 const float *__restrict__ b2, const float *__restrict__ bo, int64_t M, int F, float eps, int *err)
+                 const float *__restrict__ b2, const float *__restrict__ bo, int64_t M, int F, float eps, FfnTail tail, int *err)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -317,33 +324,83 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant
         } while (false);
     }
     __syncwarp();
-    // The cluster's partial sums, added in rank order.  Everybody takes both barriers, whatever happened before: after the first
-    // all partial O are in shared memory (and nobody still reads x), after the second nobody reads a peer's memory any more.
+    // The cluster's partial sums, added in rank order, by whole rows (128 / CS of them per CTA, a warp for 16 / CS): a row that is
+    // complete in one warp goes on to the next layer's LayerNorm, or to the scoring head, right here (FfnTail).
+    constexpr int kRowsPerWarp = 16 / CS, kBatch = kRowsPerWarp / 2;
+    const int row_first = rank * (kRows / CS) + (warp - 4) * kRowsPerWarp, c0 = 4 * lane;      // columns c0 .. + 3 and 128 + c0 .. + 3
+    float4 tg[2], tb[2], tw[2];
+    int score_at = -1;                                // lane i < kRowsPerWarp: where the score of the warp's row i goes (-1: not a candidate's)
+    if (live && warp >= 4 && tail.kind != FFN_TAIL_NONE) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            tg[h] = *reinterpret_cast<const float4 *>(tail.g + c0 + 128 * h); tb[h] = *reinterpret_cast<const float4 *>(tail.b + c0 + 128 * h);
+            if (tail.kind == FFN_TAIL_SCORE) tw[h] = *reinterpret_cast<const float4 *>(tail.w + c0 + 128 * h);
+        }
+        const int64_t row = (int64_t)tile * kRows + row_first + lane;
+        if (tail.kind == FFN_TAIL_SCORE && lane < kRowsPerWarp && row < M) {
+            const int u = find_user(tail.row_off, tail.n_users, (int)row), i = (int)row - tail.seqs[u].score_row0;
+            if (i >= 0 && i < tail.seqs[u].n_score) score_at = tail.score_off[u] + i;
+        }
+    }
+    // Everybody takes both barriers, whatever happened before: after the first all partial O are in shared memory (and nobody still
+    // reads x), after the second nobody reads a peer's memory any more.
     tc::cluster_sync();
     if (live && warp >= 4 && o_ready) {
-        // 32 * 256 / CS 16-byte pieces of the tile are this CTA's to finish: two batches per thread, each with sixteen loads in flight
-        constexpr int kBatch = 16 / CS;
 #pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-            float4 t[kBatch][CS];
-            const int e0 = rank * (32 * 256 / CS) + h * (kBatch * kEpiThreads) + (int)threadIdx.x - 128;
+        for (int hb = 0; hb < 2; ++hb) {              // two batches of rows, each with sixteen loads in flight
+            float4 t[kBatch][2][CS];
 #pragma unroll
             for (int i = 0; i < kBatch; ++i) {
-                const int e = e0 + i * kEpiThreads, r = (e >> 3) & 31, j = e & 7;               // piece j of row r of patch e >> 8
-                const uint8_t *src = sW + (e >> 8) * 4096 + r * 128 + ((j ^ (r & 7)) << 4);
+                const int rt = row_first + hb * kBatch + i, r = rt & 31;                    // row of the tile, of its patches
+                const uint8_t *src = sW + ((rt >> 5) * 8 + (lane >> 3)) * 4096 + r * 128 + (((lane & 7) ^ (r & 7)) << 4);
 #pragma unroll
-                for (int k = 0; k < CS; ++k) t[i][k] = load_cluster4(tc::cluster_addr(src, k));
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int k = 0; k < CS; ++k) t[i][h][k] = load_cluster4(tc::cluster_addr(src + h * (4 * 4096), k));
             }
 #pragma unroll
             for (int i = 0; i < kBatch; ++i) {
-                const int e = e0 + i * kEpiThreads, p = e >> 8, r = (e >> 3) & 31, j = e & 7;
-                const int64_t row = (int64_t)tile * kRows + (p >> 3) * 32 + r;
-                const int col = (p & 7) * 32 + j * 4;
-                float4 sum = t[i][0];
+                const int64_t row = (int64_t)tile * kRows + row_first + hb * kBatch + i;
+                float4 v[2];
+                float sum = 0.f;
 #pragma unroll
-                for (int k = 1; k < CS; ++k) { sum.x += t[i][k].x; sum.y += t[i][k].y; sum.z += t[i][k].z; sum.w += t[i][k].w; }
-                const float4 q = *reinterpret_cast<const float4 *>(b2s + col);
-                if (row < M) *reinterpret_cast<float4 *>(x + row * kD + col) = make_float4(sum.x + q.x, sum.y + q.y, sum.z + q.z, sum.w + q.w);
+                for (int h = 0; h < 2; ++h) {
+                    v[h] = t[i][h][0];
+#pragma unroll
+                    for (int k = 1; k < CS; ++k) { v[h].x += t[i][h][k].x; v[h].y += t[i][h][k].y; v[h].z += t[i][h][k].z; v[h].w += t[i][h][k].w; }
+                    const float4 q = *reinterpret_cast<const float4 *>(b2s + c0 + 128 * h);
+                    v[h].x += q.x; v[h].y += q.y; v[h].z += q.z; v[h].w += q.w;
+                    sum += (v[h].x + v[h].y) + (v[h].z + v[h].w);
+                }
+                if (tail.kind != FFN_TAIL_SCORE && row < M) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) *reinterpret_cast<float4 *>(x + row * kD + c0 + 128 * h) = v[h];
+                }
+                if (tail.kind == FFN_TAIL_NONE) continue;
+                const float mean = warp_sum(sum) * (1.f / kD);
+                float sq = 0.f;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    v[h].x -= mean; v[h].y -= mean; v[h].z -= mean; v[h].w -= mean;
+                    sq += v[h].x * v[h].x + v[h].y * v[h].y + v[h].z * v[h].z + v[h].w * v[h].w;
+                }
+                const float rstd = rsqrtf(warp_sum(sq) * (1.f / kD) + eps);
+                float acc = 0.f;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float4 y = make_float4(v[h].x * rstd * tg[h].x + tb[h].x, v[h].y * rstd * tg[h].y + tb[h].y,
+                                                 v[h].z * rstd * tg[h].z + tb[h].z, v[h].w * rstd * tg[h].w + tb[h].w);
+                    if (tail.kind == FFN_TAIL_LN) {
+                        if (row < M) *reinterpret_cast<uint2 *>(tail.a + row * kD + c0 + 128 * h) = make_uint2(tc::pack_bf16(y.x, y.y), tc::pack_bf16(y.z, y.w));
+                    } else {
+                        acc += y.x * tw[h].x + y.y * tw[h].y + y.z * tw[h].z + y.w * tw[h].w;
+                    }
+                }
+                if (tail.kind == FFN_TAIL_SCORE) {
+                    acc = warp_sum(acc);
+                    const int at = __shfl_sync(0xffffffffu, score_at, hb * kBatch + i);
+                    if (lane == 0 && at >= 0) tail.scores[at] = acc + (tail.bias ? tail.bias[0] : 0.f);
+                }
             }
         }
     }
@@ -380,9 +437,10 @@ cudaError_t ffn_resident(int dev, int *out)
 bool ffn_fused_supported(int d_model, int d_ff) { return d_model == kD && d_ff % kChunk == 0 && d_ff >= kChunk && d_ff <= kMaxF; }
 
 cudaError_t launch_ffn_fused(const FfnMaps &w, const CUtensorMap &tmX, float *x, const float *g, const float *b, const float *b1,
-                             const float *b2, const CUtensorMap &tmAtt, const float *bo, int64_t M, int d_ff, float eps, int *err,
-                             cudaStream_t stream, int64_t *launches)
+                             const float *b2, const CUtensorMap &tmAtt, const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail,
+                             bool *tail_done, int *err, cudaStream_t stream, int64_t *launches)
 {
+    *tail_done = false;
     if (M == 0) return cudaSuccess;
     int dev = 0, n2 = 0, n4 = 0, n8 = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -396,8 +454,9 @@ cudaError_t launch_ffn_fused(const FfnMaps &w, const CUtensorMap &tmX, float *x,
     const int64_t tiles = (M + kRows - 1) / kRows;
     const int chunks = d_ff / kChunk;
     auto launch = [&](auto kernel, int cs) {
+        *tail_done = true;
         return launch_dependent(kernel, dim3((unsigned)(tiles * cs)), dim3(kThreads), (size_t)kSmemBytes, stream, cs, w.w1, w.w2_wide, tmAtt,
-                                w.wo_wide, x, g, b, b1, b2, bo, M, d_ff, eps, err);
+                                w.wo_wide, x, g, b, b1, b2, bo, M, d_ff, eps, tail, err);
     };
     if (tiles <= n8 && chunks >= 8) return launch(ffn_fused_kernel<8>, 8);
     if (tiles <= n4 && chunks >= 4) return launch(ffn_fused_kernel<4>, 4);

@@ -409,6 +409,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     const F32Tile *tiles_m = reinterpret_cast<const F32Tile *>(meta + o_items);
     int n_items_m = (int)(kTensor || tensor32 ? items.size() : tiles.size()), n_merges_m = (int)merges.size();
     bool dead_tail = false;                       // a call without candidates: nothing reads the last layer
+    bool ln_done = false, scored = false;         // the fused kernel of the layer before has taken this layer's LayerNorm 1 / the scores
 
     for (int l = 0; l < L; ++l) {
         const bool last = l == L - 1;
@@ -418,7 +419,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
             cudaEvent_t pe = prof_begin(stream);
             e = launch_gather_ln<T>((const T *)w.emb, cfg.vocab, d, src, R, g1, b1n, cfg.ln_eps, x, a, d_status, stream, &launches);
             prof_end(KC_GATHER_LN, pe, stream);
-        } else {
+        } else if (!ln_done) {
             e = layernorm(x, R, g1, b1n);
         }
         if (!ck("LayerNorm 1")) return RELAYGR_E_CUDA;
@@ -487,9 +488,22 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         if (kTensor && ffn_fused_supported((int)d, (int)F)) {
             // output projection + residual, LayerNorm 2, both feed-forward GEMMs, SiLU and the second residual add in one kernel
             cudaEvent_t pe = prof_begin(stream);
+            FfnTail tail{};
+            if (!last) {
+                tail.kind = FFN_TAIL_LN;
+                tail.g = w.ln1_g + (size_t)(l + 1) * d; tail.b = w.ln1_b + (size_t)(l + 1) * d; tail.a = reinterpret_cast<__nv_bfloat16 *>(a);
+            } else {
+                tail.kind = FFN_TAIL_SCORE;
+                tail.g = w.lnf_g; tail.b = w.lnf_b; tail.w = w.w_score; tail.bias = w.b_score; tail.scores = scores;
+                tail.row_off = compact_last ? meta + o_score : d_row_off; tail.seqs = compact_last ? seqs_m : d_seqs;
+                tail.score_off = meta + o_score; tail.n_users = B;
+            }
+            bool tail_done = false;
             e = launch_ffn_fused(lm->ffn, om_xm->o[0], xm, w.ln2_g + (size_t)l * d, w.ln2_b + (size_t)l * d, w.b1 ? w.b1 + (size_t)l * F : nullptr,
                                  w.b2 ? w.b2 + (size_t)l * d : nullptr, tm_att, w.b_o ? w.b_o + (size_t)l * d : nullptr, M, (int)F, cfg.ln_eps,
-                                 d_status, stream, &launches);
+                                 tail, &tail_done, d_status, stream, &launches);
+            ln_done = tail_done && !last;
+            scored = tail_done && last;
             prof_end(KC_GEMM, pe, stream);
             if (!ck("output projection + feed-forward")) return RELAYGR_E_CUDA;
             continue;
@@ -513,7 +527,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         if (!ck("FFN 2")) return RELAYGR_E_CUDA;
     }
 
-    if (!dead_tail && n_scores > 0) {
+    if (!dead_tail && n_scores > 0 && !scored) {
         cudaEvent_t pe = prof_begin(stream);
         e = launch_score(xm, d, seqs_m, B, n_scores, meta + o_score, w.lnf_g, w.lnf_b, cfg.ln_eps, w.w_score, w.b_score,
                          scores, stream, &launches);

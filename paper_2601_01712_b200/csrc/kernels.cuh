@@ -129,11 +129,25 @@ struct FfnMaps {                                  // one layer's weights, boxes 
     CUtensorMap w1, w1_half;                      // W1 [d_ff, 256], boxes of 128 and of 64 rows
     CUtensorMap w2, w2_wide, wo, wo_wide;         // W2 [256, d_ff] and Wo [256, 256], boxes of 128 and (wide) of 256 rows
 };
+// What the kernel does with finished rows beside storing them to x: nothing; the next layer's a = LN(x; g, b); or, instead of storing
+// them, the scores of the candidates' rows, w . LN(x; g, b) + bias (users by row_off and seqs, as in launch_score).
+enum FfnTailKind : int { FFN_TAIL_NONE = 0, FFN_TAIL_LN, FFN_TAIL_SCORE };
+struct FfnTail {
+    int kind;
+    const float *g, *b;
+    __nv_bfloat16 *a;
+    const float *w, *bias;
+    float *scores;
+    const int32_t *row_off;       // [n_users + 1] rows of this launch
+    const SeqDesc *seqs;          // score_row0, n_score: rows of this launch
+    const int32_t *score_off;
+    int n_users;
+};
 bool ffn_fused_supported(int d_model, int d_ff);
 cudaError_t launch_ffn_fused(const FfnMaps &w, const CUtensorMap &tmX, float *x, const float *g, const float *b, const float *b1,
-                             const float *b2, const CUtensorMap &tmAtt, const float *bo, int64_t M, int d_ff, float eps, int *err,
-                             cudaStream_t stream, int64_t *launches);
-// (the form for many rows, called by the launcher above)
+                             const float *b2, const CUtensorMap &tmAtt, const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail,
+                             bool *tail_done, int *err, cudaStream_t stream, int64_t *launches);
+// (the form for many rows, called by the launcher above: it leaves the tail to the caller, *tail_done = false)
 cudaError_t launch_ffn_pair(const FfnMaps &w, const CUtensorMap &tmX, const float *x, const float *g, const float *b, const float *b1, const float *b2,
                             const CUtensorMap &tmAtt, const float *bo, int64_t M, int d_ff, float eps, int *err, cudaStream_t stream);
 
