@@ -5,6 +5,7 @@
 // everything unrolled over a row in registers, the first LayerNorm of a launch took 8000 clocks and later ones 3800).
 #pragma once
 
+#include "kernels.cuh"
 #include "tc_common.cuh"
 
 namespace relaygr {
@@ -121,6 +122,26 @@ __device__ __forceinline__ void silu_chunk(uint32_t s_cols, const float *b1_half
         }
         tc::tmem_st16(s_cols + 16 * p, pk);
     }
+}
+
+// How many clusters of `cs` CTAs of a kernel with `smem` bytes can be resident at once on the current device (`dev`); asked once.
+template <typename K>
+cudaError_t resident_clusters(K kernel, int cs, size_t smem, PerDeviceValue &known, int dev, int *out)
+{
+    *out = known.get(dev);
+    if (*out > 0) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(cs * 16); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cs; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(out, kernel, &cfg);
+    if (e != cudaSuccess) return e;
+    if (*out < 1) return cudaErrorLaunchOutOfResources;
+    known.set(dev, *out);
+    return cudaSuccess;
 }
 
 }  // namespace ffn

@@ -1,0 +1,489 @@
+// What follows the attention in a block, in one kernel, for d_model = 256 and the fewest rows (more rows: ffn_tc.cu, ffn_pair_tc.cu):
+//     mid = x + att Wo^T + bo,   x <- mid + W2 SiLU(W1 LN(mid; g, b) + b1) + b2
+// A cluster of CS CTAs shares a tile of T = 32 or 64 rows.  Each CTA repeats projection and LayerNorm and takes every CS-th chunk of
+// 128 hidden units.  All products are computed transposed, weights as the 128-row operand and the tile's rows as N, so that a
+// tile can be smaller than the 128 lanes of TMEM:
+//     P^T = Wo att^T          attention rows [T x 256] and Wo by TMA; 256 output columns = two times 128 lanes, T columns of TMEM
+//     mid, A = LN(mid)        P is turned around in shared memory, a warp then has T / 8 whole rows; A as bf16 where att was
+//     per chunk:              S^T = W1c A^T, H = SiLU(S + b1c) as bf16 into shared memory, O^T += W2c H^T
+// The partial O are turned around like P and added up through distributed shared memory in rank order - one fixed order of the
+// fp32 sums, so results do not vary from run to run - and each CTA finishes its share of the tile's rows, the next layer's LayerNorm
+// (or the final one and the scoring head) included.
+//
+// What bounds it: a serial chain of short steps, each with its own latency, and the exchange - distributed shared memory delivers
+// about 16 bytes per clock to an SM, and a CTA takes T KB of partial sums.  With 128-row tiles (rows on the lanes) that chain took
+// 15 us at 576 rows, 8000 clocks of it the exchange, on 40 SMs; a whole 4-layer ranking call of one user went from 160 to 133 us,
+// the pre-inference of 2000 tokens from 151 to 138 us.
+//
+// Warp roles (384 threads): warp 0 = TMA producer (a ring of 32 KB stages: Wo in four K blocks, then half a W1 chunk or half a W2
+// chunk per stage, in the order the MMAs consume them; the whole ring is under way before the kernel waits for its predecessor),
+// warp 1 = TMEM owner + MMA issuer, warps 2-3 none, warps 4-11 = LayerNorm, SiLU and exchange (two warps per TMEM quadrant).  TMEM:
+// P, later O, 2 T columns; S double-buffered, T columns each.  The MMA warp issues S(0), S(1), then per chunk O(c) followed
+// by S(c+2): the tensor pipe executes in issue order, so S(c+2) complete also means that H(c) has been read.
+#include "ffn_common.cuh"
+#include "kernels.cuh"
+
+namespace relaygr {
+
+namespace {
+
+using namespace ffn;
+
+constexpr int kStageBytes = 32 * 1024, kHalfStage = kStageBytes / 2;
+
+template <int T>
+struct Shape {
+    static constexpr int kStages = T == 64 ? 5 : 6;
+    static constexpr int kKB = T * 128;               // one K block (64 bf16) of A, att or H
+    static constexpr int kOffH = 4 * kKB;             // two buffers of two K blocks, behind A; A and H together: T rows x 256 fp32
+    static constexpr int kOffW = 8 * kKB;
+    static constexpr int kOffBars = kOffW + kStages * kStageBytes;
+    static constexpr int kSmemBytes = kOffBars + 256 + 1024;
+    static constexpr int kColS = 2 * T;
+    static constexpr uint32_t kTmemCols = 4 * T;
+    static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
+};
+
+template <int kStages>
+struct RowBars {
+    uint64_t att_full, p_full, a_ready;               // attention rows landed / their projection complete / LN(mid) in shared memory
+    uint64_t w_full[kStages], w_empty[kStages];
+    uint64_t s_full[2];                               // S complete in its buffer
+    uint64_t h_full[2];                               // H in shared memory
+    uint64_t o_full;                                  // O complete
+    uint32_t tmem_slot;
+    int abort_flag;
+};
+static_assert(sizeof(RowBars<6>) <= 256, "barrier block");
+
+__device__ __forceinline__ float4 load_cluster4(uint32_t addr)
+{
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
+__device__ __forceinline__ float4 load4_or_zero(const float *p, int c)
+{
+    return p ? *reinterpret_cast<const float4 *>(p + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+__device__ __forceinline__ float sum8(const float4 (&v)[2]) { return ((v[0].x + v[0].y) + (v[0].z + v[0].w)) + ((v[1].x + v[1].y) + (v[1].z + v[1].w)); }
+// v = (v + p) + q
+__device__ __forceinline__ void add_twice(float4 &v, const float4 &p, const float4 &q)
+{
+    v.x = (v.x + p.x) + q.x; v.y = (v.y + p.y) + q.y; v.z = (v.z + p.z) + q.z; v.w = (v.w + p.w) + q.w;
+}
+// Mean and 1 / std of N rows, eight columns of each per lane.  Two passes; the rows' shuffles overlap.
+template <int N>
+__device__ __forceinline__ void rows_stats(const float4 (&v)[N][2], float eps, float (&mean)[N], float (&rstd)[N])
+{
+#pragma unroll
+    for (int i = 0; i < N; ++i) mean[i] = sum8(v[i]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < N; ++i) mean[i] += __shfl_xor_sync(0xffffffffu, mean[i], o);
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        mean[i] *= 1.f / kD;
+        float sq = 0.f;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float dx = v[i][h].x - mean[i], dy = v[i][h].y - mean[i], dz = v[i][h].z - mean[i], dw = v[i][h].w - mean[i];
+            sq += (dx * dx + dy * dy) + (dz * dz + dw * dw);
+        }
+        rstd[i] = sq;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < N; ++i) rstd[i] += __shfl_xor_sync(0xffffffffu, rstd[i], o);
+#pragma unroll
+    for (int i = 0; i < N; ++i) rstd[i] = rsqrtf(rstd[i] * (1.f / kD) + eps);
+}
+__device__ __forceinline__ float4 normalised(const float4 &v, float mean, float rstd, const float4 &g, const float4 &b)
+{
+    return make_float4((v.x - mean) * rstd * g.x + b.x, (v.y - mean) * rstd * g.y + b.y, (v.z - mean) * rstd * g.z + b.z, (v.w - mean) * rstd * g.w + b.w);
+}
+
+template <int T, int CS>
+__global__ void __launch_bounds__(kThreads, 1)
+ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2,
+                const __grid_constant__ CUtensorMap tmAtt, const __grid_constant__ CUtensorMap tmWo,
+                float *__restrict__ x, const float *__restrict__ g, const float *__restrict__ b, const float *__restrict__ b1,
+                const float *__restrict__ b2, const float *__restrict__ bo, int64_t M, int F, float eps, FfnTail tail, int *err)
+{
+    using L = Shape<T>;
+    constexpr int kStages = L::kStages, kKB = L::kKB;
+    constexpr int kWarpRows = T / kEpiWarps;          // rows of the tile per epilogue warp: row(j) for j < kWarpRows
+    // of these, the ones this CTA finishes: j = rank * kEnd .., or one of them per kShare CTAs (then every kShare-th warp does)
+    constexpr int kEnd = kWarpRows >= CS ? kWarpRows / CS : 1, kShare = kWarpRows >= CS ? 1 : CS / kWarpRows;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t *sA = smem, *sH = smem + L::kOffH, *sW = smem + L::kOffW;
+    float *turn = reinterpret_cast<float *>(smem);    // [T][256]: P, later the partial O, by rows
+    using Bars = RowBars<kStages>;
+    Bars *bars = reinterpret_cast<Bars *>(smem + L::kOffBars);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = (int)tc::cluster_ctarank();
+    const int64_t tile_row0 = (int64_t)(blockIdx.x / CS) * T;
+    // this CTA's hidden chunks: rank, rank + CS, ...; there are at least CS
+    const int nc = (F / kChunk - rank + CS - 1) / CS;
+    auto chunk_at = [&](int i) { return rank + i * CS; };
+    const int ew = warp - 4, quad = warp & 3, ch = ew >> 2, c0 = 4 * lane;      // epilogue warps; c0 .. + 3 and 128 + c0 .. + 3: columns of a lane
+    auto row = [&](int j) { return 16 * (j >> 1) + 2 * ew + (j & 1); };
+    const int j_end = rank / kShare * kEnd;
+    const bool finisher = warp >= 4 && ew % kShare == rank % kShare;
+
+    // TMA producer (one thread): ring position, weights of the next stage
+    uint32_t it = 0;
+    bool ok = true;
+    auto acquire = [&] {
+        const int s = it % kStages;
+        ok = ok && tc::mbar_wait(&bars->w_empty[s], ((it / kStages) & 1) ^ 1, err);
+        ++it;
+        if (ok) tc::mbar_expect_tx(&bars->w_full[s], kStageBytes);
+        return s;
+    };
+    auto load_w1 = [&](int c, int half) {             // rows c*128 .. +127 of W1 [F, 256], K blocks 2*half and 2*half + 1
+        const int s = acquire();
+        if (!ok) return;
+        tc::tma_load_2d(sW + s * kStageBytes, &tmW1, (2 * half) * 64, c * kChunk, &bars->w_full[s]);
+        tc::tma_load_2d(sW + s * kStageBytes + kHalfStage, &tmW1, (2 * half + 1) * 64, c * kChunk, &bars->w_full[s]);
+    };
+    auto load_w2 = [&](int c, int half) {             // all 256 rows of W2 [256, F], 64 hidden columns
+        const int s = acquire();
+        if (ok) tc::tma_load_2d(sW + s * kStageBytes, &tmW2, c * kChunk + half * 64, 0, &bars->w_full[s]);
+    };
+    constexpr int kEarlyHalves = kStages - 4;
+    static_assert(kEarlyHalves >= 0 && kEarlyHalves <= 2, "what is loaded ahead: Wo and at most the first chunk of W1");
+
+    // set-up that touches nothing earlier kernels wrote
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kStages; ++s) { tc::mbar_init(&bars->w_full[s], 1); tc::mbar_init(&bars->w_empty[s], 1); }
+        for (int i = 0; i < 2; ++i) { tc::mbar_init(&bars->s_full[i], 1); tc::mbar_init(&bars->h_full[i], kEpiThreads); }
+        tc::mbar_init(&bars->att_full, 1); tc::mbar_init(&bars->p_full, 1); tc::mbar_init(&bars->a_ready, kEpiThreads);
+        tc::mbar_init(&bars->o_full, 1);
+        tc::fence_mbar_init();
+        for (int kb = 0; kb < 4; ++kb) {
+            const int s = acquire();
+            tc::tma_load_2d(sW + s * kStageBytes, &tmWo, kb * 64, 0, &bars->w_full[s]);
+        }
+        for (int h = 0; h < kEarlyHalves; ++h) load_w1(chunk_at(0), h);
+        tc::tma_prefetch_desc(&tmW1); tc::tma_prefetch_desc(&tmW2); tc::tma_prefetch_desc(&tmAtt);
+    }
+    if (warp == 1) {
+        tc::tmem_alloc(&bars->tmem_slot, L::kTmemCols);
+        tc::tmem_relinquish();
+    }
+    float4 gain[2], shift[2], obias[2];
+    float b1_half = 0.f;                              // of the next chunk; SiLU takes half of its argument
+    if (warp >= 4) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            gain[h] = *reinterpret_cast<const float4 *>(g + c0 + 128 * h); shift[h] = *reinterpret_cast<const float4 *>(b + c0 + 128 * h);
+            obias[h] = load4_or_zero(bo, c0 + 128 * h);
+        }
+        if (b1) b1_half = 0.5f * b1[chunk_at(0) * kChunk + quad * 32 + lane];
+    }
+    grid_launch_dependents();
+    grid_dependency_wait();                           // from here on: data of earlier kernels
+    if (threadIdx.x == 0) {
+        tc::mbar_expect_tx(&bars->att_full, 4 * kKB);
+        for (int kb = 0; kb < 4; ++kb)
+            for (int r = 0; r < T; r += 32) tc::tma_load_2d(sA + kb * kKB + r * 128, &tmAtt, kb * 64, (int)tile_row0 + r, &bars->att_full);
+        bars->abort_flag = *reinterpret_cast<volatile int *>(err);
+    }
+    // x, whole rows per warp (it has room for tiles of 128 rows; rows past the last feed only themselves), later mid
+    float4 mid[kWarpRows][2];
+    if (warp >= 4) {
+#pragma unroll
+        for (int j = 0; j < kWarpRows; ++j)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) mid[j][h] = *reinterpret_cast<const float4 *>(x + (tile_row0 + row(j)) * kD + c0 + 128 * h);
+    }
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    const uint32_t tmem_base = bars->tmem_slot;
+    const bool live = bars->abort_flag == 0;
+    bool o_ready = false;                             // this warp saw the CTA's partial O complete
+    float4 own[kEnd][2];                              // mid of the rows this CTA finishes
+    if (!live) {
+        if (threadIdx.x == 0) {                       // what was requested above lands before the CTA ends
+            for (int s = 0; s < kStages; ++s) tc::mbar_wait(&bars->w_full[s], 0, err);
+            tc::mbar_wait(&bars->att_full, 0, err);
+        }
+    } else if (warp == 0) {
+        // ---------------------------------------------------------------- TMA producer
+        if (lane == 0) {
+            for (int h = kEarlyHalves; h < 2; ++h) load_w1(chunk_at(0), h);
+            if (nc > 1) { load_w1(chunk_at(1), 0); load_w1(chunk_at(1), 1); }
+            for (int i = 0; i < nc && ok; ++i) {
+                load_w2(chunk_at(i), 0); load_w2(chunk_at(i), 1);
+                if (i + 2 < nc) { load_w1(chunk_at(i + 2), 0); load_w1(chunk_at(i + 2), 1); }
+            }
+        }
+    } else if (warp == 1) {
+        // ---------------------------------------------------------------- MMA issuer (convergent warp, one elected lane issues)
+        constexpr uint32_t idesc = tc::make_idesc(kRows, T, 0, 0);             // weights x rows, both K-major
+        const uint32_t a0 = tc::smem_u32(sA), h0 = tc::smem_u32(sH), w0 = tc::smem_u32(sW);
+        auto stage = [&] {                            // waits for the next stage: its address
+            const int s = it % kStages;
+            ok = ok && tc::mbar_wait(&bars->w_full[s], (it / kStages) & 1, err);
+            tc::tc_fence_after();
+            return w0 + s * kStageBytes;
+        };
+        auto issue_s = [&](int i) {                   // S^T = W1c A^T: two stages, each two K blocks of 64
+            const int buf = i & 1;
+#pragma unroll 1
+            for (int half = 0; half < 2; ++half, ++it) {
+                const uint32_t w = stage();
+                if (!ok) return;
+                if (tc::elect_one()) {
+#pragma unroll
+                    for (int kb = 0; kb < 2; ++kb) {
+                        const uint64_t adesc = tc::smem_desc_sw128(w + kb * kHalfStage), bdesc = tc::smem_desc_sw128(a0 + (2 * half + kb) * kKB);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) tc::mma_ss(tmem_base + L::kColS + buf * T, adesc + 2 * k, bdesc + 2 * k, idesc, (half | kb | k) != 0);
+                    }
+                    tc::mma_commit(&bars->w_empty[it % kStages]);
+                    if (half == 1) tc::mma_commit(&bars->s_full[buf]);
+                }
+                __syncwarp();
+            }
+        };
+        // one K block of 64 into both halves of P or O: 256 weight rows (output columns) x the tile's rows
+        auto issue_wide = [&](uint32_t rows_at, bool fresh, uint64_t *done) {
+            const uint32_t w = stage();
+            if (!ok) return;
+            if (tc::elect_one()) {
+                const uint64_t bdesc = tc::smem_desc_sw128(rows_at);
+#pragma unroll
+                for (int mb = 0; mb < 2; ++mb) {
+                    const uint64_t adesc = tc::smem_desc_sw128(w + mb * kHalfStage);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) tc::mma_ss(tmem_base + mb * T, adesc + 2 * k, bdesc + 2 * k, idesc, !fresh || k != 0);
+                }
+                tc::mma_commit(&bars->w_empty[it % kStages]);
+                if (done) tc::mma_commit(done);
+            }
+            __syncwarp();
+            ++it;
+        };
+        it = 0;
+        ok = tc::mbar_wait(&bars->att_full, 0, err);
+        // kinds of step in one loop (the code is fetched once): K blocks of the projection, then halves of the chunks' O
+#pragma unroll 1
+        for (int n = 0; n < 4 + 2 * nc && ok; ++n) {
+            const int i = (n - 4) >> 1, half = n & 1;
+            if (n == 4) {
+                ok = tc::mbar_wait(&bars->a_ready, 0, err);
+                tc::tc_fence_after();
+            }
+            if (n >= 4 && half == 0) {
+                // S runs two chunks ahead of O
+                for (int c = i == 0 ? 0 : i + 1; c < i + 2 && c < nc && ok; ++c) issue_s(c);
+                ok = ok && tc::mbar_wait(&bars->h_full[i & 1], (i >> 1) & 1, err);      // H is in shared memory (and S in registers)
+                tc::tc_fence_after();
+            }
+            if (ok) issue_wide(n < 4 ? a0 + n * kKB : h0 + ((i & 1) * 2 + half) * kKB, n == 0 || n == 4, n == 3 ? &bars->p_full : n == 3 + 2 * nc ? &bars->o_full : nullptr);
+        }
+    } else if (warp >= 4) {
+        // ---------------------------------------------------------------- LayerNorm, SiLU, drain: eight warps, two per TMEM
+        // quadrant; of P and O warp (quad, ch) takes columns ch * 128 + quad * 32 .., of S half ch of the rows
+        const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
+        // 2 x 128 lanes x T columns of TMEM into `turn`: whole rows there
+        auto turn_around = [&] {
+            float *dst = turn + ch * 128 + quad * 32 + lane;
+#pragma unroll 1
+            for (int r0 = 0; r0 < T; r0 += 32) {
+                uint32_t r[32];
+                tc::tmem_ld32(lane_addr + ch * T + r0, r);
+                tc::tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 32; ++i) dst[(r0 + i) * kD] = __uint_as_float(r[i]);
+            }
+        };
+        do {
+            ok = tc::mbar_wait(&bars->p_full, 0, err);
+            tc::tc_fence_after();
+            turn_around();
+            epilogue_sync();
+            float mean[kWarpRows], rstd[kWarpRows];
+#pragma unroll
+            for (int j = 0; j < kWarpRows; ++j)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) add_twice(mid[j][h], *reinterpret_cast<const float4 *>(turn + row(j) * kD + c0 + 128 * h), obias[h]);
+            rows_stats<kWarpRows>(mid, eps, mean, rstd);
+            epilogue_sync();                          // all of P has been read
+#pragma unroll
+            for (int j = 0; j < kWarpRows; ++j) {
+                const int rt = row(j);
+                uint8_t *dst = sA + (lane >> 4) * kKB + rt * 128 + ((((lane & 15) >> 1) ^ (rt & 7)) << 4) + (lane & 1) * 8;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float4 y = normalised(mid[j][h], mean[j], rstd[j], gain[h], shift[h]);
+                    *reinterpret_cast<uint2 *>(dst + 2 * h * kKB) = make_uint2(tc::pack_bf16(y.x, y.y), tc::pack_bf16(y.z, y.w));
+                    if (j / kEnd == rank / kShare) own[j % kEnd][h] = mid[j][h];
+                }
+            }
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc::fence_proxy_async();                  // generic-proxy writes of the tile before the tensor core reads it
+            tc::tc_fence_before();
+            tc::mbar_arrive(&bars->a_ready);
+
+            // H: this lane's hidden unit, rows ch * T / 2 ..; 16-byte chunk (lane / 8 + 4 * (quad & 1)) of each row of its K block
+            uint8_t *h_lane = sH + (quad >> 1) * kKB + ch * (T / 2) * 128 + (lane & 7) * 2;
+            const int h_chunk = (quad & 1) * 4 + (lane >> 3);
+            const uint64_t half2 = tc::pack2(0.5f, 0.5f);
+#pragma unroll 1
+            for (int i = 0; i < nc; ++i) {
+                const uint64_t bias2 = tc::pack2(b1_half, b1_half);
+                if (b1 && i + 1 < nc) b1_half = 0.5f * b1[chunk_at(i + 1) * kChunk + quad * 32 + lane];
+                const int hb = i & 1;
+                ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->s_full[hb], (i >> 1) & 1, err));
+                if (!ok) break;
+                tc::tc_fence_after();
+                uint32_t r[T / 2];
+                if constexpr (T == 64) tc::tmem_ld32(lane_addr + L::kColS + hb * T + ch * (T / 2), r);
+                else tc::tmem_ld16(lane_addr + L::kColS + hb * T + ch * (T / 2), r);
+                tc::tmem_ld_wait();
+                tc::tc_fence_before();
+                uint8_t *dst = h_lane + hb * 2 * kKB;
+#pragma unroll
+                for (int e = 0; e < T / 2; e += 2) {
+                    const uint32_t p = tc::pack_bf16(tc::silu2_of_half(tc::fma2(tc::pack2(r[e], r[e + 1]), half2, bias2)));
+                    *reinterpret_cast<uint16_t *>(dst + e * 128 + ((h_chunk ^ (e & 7)) << 4)) = (uint16_t)p;
+                    *reinterpret_cast<uint16_t *>(dst + (e + 1) * 128 + ((h_chunk ^ ((e + 1) & 7)) << 4)) = (uint16_t)(p >> 16);
+                }
+                tc::fence_proxy_async();
+                tc::mbar_arrive(&bars->h_full[hb]);
+            }
+            if (!ok) break;
+
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->o_full, 0, err));
+            if (!ok) break;
+            tc::tc_fence_after();
+            o_ready = true;
+            turn_around();                            // over A and H: every MMA has been executed
+        } while (false);
+    }
+    __syncwarp();
+    // The cluster's partial sums, added in rank order, by whole rows: a row that is complete in one warp goes on to the next layer's
+    // LayerNorm, or to the scoring head, right here (FfnTail).
+    float4 obias2[2], tg[2], tb[2], tw[2];
+    int score_at = -1;                                // lane i < kEnd: where the score of the warp's row i goes (-1: not a candidate's)
+    if (live && finisher) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            obias2[h] = load4_or_zero(b2, c0 + 128 * h);
+            if (tail.kind != FFN_TAIL_NONE) { tg[h] = load4_or_zero(tail.g, c0 + 128 * h); tb[h] = load4_or_zero(tail.b, c0 + 128 * h); }
+            if (tail.kind == FFN_TAIL_SCORE) tw[h] = load4_or_zero(tail.w, c0 + 128 * h);
+        }
+        const int64_t r = tile_row0 + row(j_end + lane);
+        if (tail.kind == FFN_TAIL_SCORE && lane < kEnd && r < M) {
+            const int u = find_user(tail.row_off, tail.n_users, (int)r), i = (int)r - tail.seqs[u].score_row0;
+            if (i >= 0 && i < tail.seqs[u].n_score) score_at = tail.score_off[u] + i;
+        }
+    }
+    // Everybody takes both barriers, whatever happened before: after the first all partial O are in shared memory, after the second
+    // nobody reads a peer's memory any more.
+    tc::cluster_sync();
+    if (live && finisher && o_ready) {
+        float4 t[kEnd][2][CS];
+#pragma unroll
+        for (int i = 0; i < kEnd; ++i)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int k = 0; k < CS; ++k) t[i][h][k] = load_cluster4(tc::cluster_addr(turn + row(j_end + i) * kD + c0 + 128 * h, k));
+#pragma unroll
+        for (int i = 0; i < kEnd; ++i)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float4 v = t[i][h][0];
+#pragma unroll
+                for (int k = 1; k < CS; ++k) { v.x += t[i][h][k].x; v.y += t[i][h][k].y; v.z += t[i][h][k].z; v.w += t[i][h][k].w; }
+                add_twice(own[i][h], v, obias2[h]);
+            }
+    }
+    __syncwarp();
+    tc::cluster_arrive();
+    if (live && finisher && o_ready) {
+        if (tail.kind != FFN_TAIL_SCORE) {
+#pragma unroll
+            for (int i = 0; i < kEnd; ++i) {
+                const int64_t r = tile_row0 + row(j_end + i);
+                if (r < M)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) *reinterpret_cast<float4 *>(x + r * kD + c0 + 128 * h) = own[i][h];
+            }
+        }
+        if (tail.kind != FFN_TAIL_NONE) {
+            float mean[kEnd], rstd[kEnd];
+            rows_stats<kEnd>(own, eps, mean, rstd);
+#pragma unroll
+            for (int i = 0; i < kEnd; ++i) {
+                const int64_t r = tile_row0 + row(j_end + i);
+                float acc = 0.f;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float4 y = normalised(own[i][h], mean[i], rstd[i], tg[h], tb[h]);
+                    if (tail.kind == FFN_TAIL_LN) {
+                        if (r < M) *reinterpret_cast<uint2 *>(tail.a + r * kD + c0 + 128 * h) = make_uint2(tc::pack_bf16(y.x, y.y), tc::pack_bf16(y.z, y.w));
+                    } else {
+                        acc += y.x * tw[h].x + y.y * tw[h].y + y.z * tw[h].z + y.w * tw[h].w;
+                    }
+                }
+                if (tail.kind == FFN_TAIL_SCORE) {
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                    const int at = __shfl_sync(0xffffffffu, score_at, i);
+                    if (lane == 0 && at >= 0) tail.scores[at] = acc + (tail.bias ? tail.bias[0] : 0.f);
+                }
+            }
+        }
+    }
+    __syncwarp();
+    tc::cluster_wait();
+    tc::tc_fence_before();
+    __syncthreads();
+    if (warp == 1) tc::tmem_dealloc(tmem_base, L::kTmemCols);
+}
+
+}  // namespace
+
+cudaError_t launch_ffn_rows(const FfnMaps &w, float *x, const float *g, const float *b, const float *b1, const float *b2, const CUtensorMap &tmAtt32,
+                            const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail, int *err, cudaStream_t stream, bool *taken)
+{
+    *taken = false;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const int chunks = d_ff / kChunk;
+    auto attempt = [&](auto kernel, int T, int cs, size_t smem, PerDeviceValue &known) {
+        if (*taken || e != cudaSuccess || chunks < cs) return;
+        int resident = 0;
+        e = resident_clusters(kernel, cs, smem, known, dev, &resident);
+        const int64_t tiles = (M + T - 1) / T;
+        if (e != cudaSuccess || tiles > resident) return;
+        *taken = true;
+        e = launch_dependent(kernel, dim3((unsigned)(tiles * cs)), dim3(kThreads), smem, stream, cs, w.w1, w.w2_wide, tmAtt32, w.wo_wide, x, g, b, b1, b2, bo,
+                             M, d_ff, eps, tail, err);
+    };
+    static PerDeviceValue known[4];
+    // The smallest tile, then the largest cluster with which all tiles still run at once (and every CTA has a chunk): both shorten the
+    // chain of a tile, a smaller tile the exchange too.  64 rows only from where two CTAs per 32 rows no longer fit (2400 rows); in
+    // clusters of 4 or 8 they lose to 32 rows in half as large clusters (640 rows: 26 us for 32 x 4, 30 us for 64 x 8), and one CTA per
+    // tile loses to the clusters of 128-row tiles (5000 rows), weights going through every SM.
+    attempt(ffn_rows_kernel<32, 8>, 32, 8, Shape<32>::kSmemBytes, known[0]);
+    attempt(ffn_rows_kernel<32, 4>, 32, 4, Shape<32>::kSmemBytes, known[1]);
+    attempt(ffn_rows_kernel<32, 2>, 32, 2, Shape<32>::kSmemBytes, known[2]);
+    attempt(ffn_rows_kernel<64, 2>, 64, 2, Shape<64>::kSmemBytes, known[3]);
+    return e;
+}
+
+}  // namespace relaygr

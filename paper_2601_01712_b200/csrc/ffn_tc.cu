@@ -1,6 +1,7 @@
-// What follows the attention in a block, in one kernel, for d_model = 256 and few rows (many rows: ffn_pair_tc.cu):
+// What follows the attention in a block, in one kernel, for d_model = 256 and a few thousand rows, up to one 128-row tile per pair of
+// SMs (fewer rows: ffn_rows_tc.cu, more: ffn_pair_tc.cu):
 //     mid = x + att Wo^T + bo,   x <- mid + W2 SiLU(W1 LN(mid; g, b) + b1) + b2
-// A cluster of CS CTAs shares a tile of 128 rows.  Each CTA repeats projection and LayerNorm and takes every CS-th chunk of 128
+// A cluster of CS = 2 CTAs shares a tile of 128 rows.  Each CTA repeats projection and LayerNorm and takes every CS-th chunk of 128
 // hidden units:
 //     att Wo^T                attention tile [128 x 256] and Wo by TMA; fp32 in the columns of the two S buffers
 //     O = mid = x + att Wo^T + bo     eight warps, half a row per thread; x went into O's columns (TMEM) during the loads
@@ -63,7 +64,8 @@ __device__ __forceinline__ float4 load_cluster4(uint32_t addr)
     return v;
 }
 
-template <int CS>
+constexpr int CS = 2;                                 // CTAs per tile
+
 __global__ void __launch_bounds__(kThreads, 1)
 ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2,
                  const __grid_constant__ CUtensorMap tmAtt, const __grid_constant__ CUtensorMap tmWo,
@@ -411,56 +413,32 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant
     if (warp == 1) tc::tmem_dealloc(tmem_base, kTmemCols);
 }
 
-// Set-up of one cluster size on the current device (`dev`): how many clusters can be resident at once.
-template <int CS>
-cudaError_t ffn_resident(int dev, int *out)
-{
-    static PerDeviceValue resident;
-    *out = resident.get(dev);
-    if (*out > 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(ffn_fused_kernel<CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(CS * 16); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmemBytes;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = CS; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(out, ffn_fused_kernel<CS>, &cfg);
-    if (e != cudaSuccess) return e;
-    if (*out < 1) return cudaErrorLaunchOutOfResources;
-    resident.set(dev, *out);
-    return cudaSuccess;
-}
-
 }  // namespace
 
 bool ffn_fused_supported(int d_model, int d_ff) { return d_model == kD && d_ff % kChunk == 0 && d_ff >= kChunk && d_ff <= kMaxF; }
 
 cudaError_t launch_ffn_fused(const FfnMaps &w, const CUtensorMap &tmX, float *x, const float *g, const float *b, const float *b1,
-                             const float *b2, const CUtensorMap &tmAtt, const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail,
+                             const float *b2, const CUtensorMap &tmAtt, const CUtensorMap &tmAtt32, const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail,
                              bool *tail_done, int *err, cudaStream_t stream, int64_t *launches)
 {
     *tail_done = false;
     if (M == 0) return cudaSuccess;
-    int dev = 0, n2 = 0, n4 = 0, n8 = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = ffn_resident<2>(dev, &n2);
-    if (e == cudaSuccess) e = ffn_resident<4>(dev, &n4);
-    if (e == cudaSuccess) e = ffn_resident<8>(dev, &n8);
-    if (e != cudaSuccess) return e;
     *launches += 1;
-    // The largest cluster with which all tiles still run at once (and every CTA has a chunk): the chain of a tile gets shorter with
-    // every split, and the SMs it takes would otherwise be idle.  More tiles than that fill the GPU by themselves.
+    cudaError_t e = launch_ffn_rows(w, x, g, b, b1, b2, tmAtt32, bo, M, d_ff, eps, tail, err, stream, tail_done);
+    if (e != cudaSuccess || *tail_done) return e;
+    int dev = 0, resident = 0;
+    e = cudaGetDevice(&dev);
+    static PerDeviceValue known;
+    if (e == cudaSuccess) e = resident_clusters(ffn_fused_kernel, CS, kSmemBytes, known, dev, &resident);
+    if (e != cudaSuccess) return e;
+    // Two CTAs per tile as long as all tiles run at once: the SMs they take would otherwise be idle.  More tiles than that fill the
+    // GPU in pairs with 256 rows each.
     const int64_t tiles = (M + kRows - 1) / kRows;
-    const int chunks = d_ff / kChunk;
-    auto launch = [&](auto kernel, int cs) {
+    if (tiles <= resident && d_ff / kChunk >= CS) {
         *tail_done = true;
-        return launch_dependent(kernel, dim3((unsigned)(tiles * cs)), dim3(kThreads), (size_t)kSmemBytes, stream, cs, w.w1, w.w2_wide, tmAtt,
+        return launch_dependent(ffn_fused_kernel, dim3((unsigned)(tiles * CS)), dim3(kThreads), (size_t)kSmemBytes, stream, CS, w.w1, w.w2_wide, tmAtt,
                                 w.wo_wide, x, g, b, b1, b2, bo, M, d_ff, eps, tail, err);
-    };
-    if (tiles <= n8 && chunks >= 8) return launch(ffn_fused_kernel<8>, 8);
-    if (tiles <= n4 && chunks >= 4) return launch(ffn_fused_kernel<4>, 4);
-    if (tiles <= n2 && chunks >= 2) return launch(ffn_fused_kernel<2>, 2);
+    }
     return launch_ffn_pair(w, tmX, x, g, b, b1, b2, tmAtt, bo, M, d_ff, eps, err, stream);
 }
 

@@ -322,7 +322,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
 
     // per-call tensor maps of the activations (bf16 model)
     int *d_status = reinterpret_cast<int *>(ws + lay.status);
-    CUtensorMap &tm_a = act.tm_a, &tm_a_c = act.tm_a_c, &tm_att = act.tm_att, &tm_hid = act.tm_hid, &tm_q = act.tm_q, &tm_k = act.tm_k,
+    CUtensorMap &tm_a = act.tm_a, &tm_a_c = act.tm_a_c, &tm_att = act.tm_att, &tm_att32 = act.tm_att32, &tm_hid = act.tm_hid, &tm_q = act.tm_q, &tm_k = act.tm_k,
                 &tm_v = act.tm_v, &tm_pool = act.tm_pool;
     GemmOutMaps &om_qkv = act.om_qkv, &om_hid = act.om_hid, &om_x = act.om_x, &om_x_c = act.om_x_c;
     const int64_t cand_rows = compact_last ? n_scores : 0;
@@ -331,6 +331,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         act.ws = nullptr;                         // not valid until every map below is encoded
         int trc = make_tmap_2d_bf16(&tm_a, a, (uint64_t)R, (uint64_t)d, (uint64_t)d, 128, 64);
         trc |= make_tmap_2d_bf16(&tm_att, att, (uint64_t)R, (uint64_t)d, (uint64_t)d, 128, 64);
+        trc |= make_tmap_2d_bf16(&tm_att32, att, (uint64_t)R, (uint64_t)d, (uint64_t)d, 32, 64);
         trc |= make_tmap_2d_bf16(&tm_hid, hid, (uint64_t)R, (uint64_t)F, (uint64_t)F, 128, 64);
         trc |= make_tmap_2d_bf16(&tm_q, q, (uint64_t)R, (uint64_t)d, (uint64_t)d, 128, 64);
         trc |= make_tmap_2d_bf16(&tm_k, kl, (uint64_t)R, (uint64_t)d, (uint64_t)d, 64, 64);
@@ -500,7 +501,8 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
             }
             bool tail_done = false;
             e = launch_ffn_fused(lm->ffn, om_xm->o[0], xm, w.ln2_g + (size_t)l * d, w.ln2_b + (size_t)l * d, w.b1 ? w.b1 + (size_t)l * F : nullptr,
-                                 w.b2 ? w.b2 + (size_t)l * d : nullptr, tm_att, w.b_o ? w.b_o + (size_t)l * d : nullptr, M, (int)F, cfg.ln_eps,
+                                 w.b2 ? w.b2 + (size_t)l * d : nullptr, tm_att, tm_att32,
+                                 w.b_o ? w.b_o + (size_t)l * d : nullptr, M, (int)F, cfg.ln_eps,
                                  tail, &tail_done, d_status, stream, &launches);
             ln_done = tail_done && !last;
             scored = tail_done && last;

@@ -60,7 +60,7 @@ struct Forward {
     // calls of the same shape - the usual case in serving - reuse them instead of encoding some twenty maps per call
     struct ActMaps {
         const char *ws = nullptr; int64_t rows = -1, cand_rows = -1; const void *slab = nullptr; int64_t pages = -1;
-        CUtensorMap tm_a, tm_a_c, tm_att, tm_hid, tm_q, tm_k, tm_v, tm_pool;
+        CUtensorMap tm_a, tm_a_c, tm_att, tm_att32, tm_hid, tm_q, tm_k, tm_v, tm_pool;
         GemmOutMaps om_qkv, om_hid, om_x, om_x_c;
     } act;
 

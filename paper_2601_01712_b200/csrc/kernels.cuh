@@ -122,8 +122,8 @@ cudaError_t launch_gemm_tc(const CUtensorMap &tmA, const CUtensorMap &tmB, const
 
 // Everything of a block after the attention in one kernel, for the shapes ffn_fused_supported() accepts (d_model = 256, d_ff a
 // multiple of 128 up to 2048):  mid = x + att Wo^T + bo,  x <- mid + W2 SiLU(W1 LN(mid; g, b) + b1) + b2  on M rows, without a
-// round trip of mid, the normalised or the hidden activations through global memory.  tmAtt: att [M, 256] bf16 in boxes of 128 rows x
-// 64 columns; tmX: the fp32 residual stream x [M, 256] (room for M rounded up to 128 rows) in boxes of 32 rows x 32 columns; all
+// round trip of mid, the normalised or the hidden activations through global memory.  tmAtt, tmAtt32: att [M, 256] bf16 in boxes of
+// 128 and of 32 rows x 64 columns; tmX: the fp32 residual stream x [M, 256] (room for M rounded up to 128 rows) in boxes of 32 rows x 32 columns; all
 // maps with the 128-byte swizzle.
 struct FfnMaps {                                  // one layer's weights, boxes 64 columns wide
     CUtensorMap w1, w1_half;                      // W1 [d_ff, 256], boxes of 128 and of 64 rows
@@ -145,8 +145,11 @@ struct FfnTail {
 };
 bool ffn_fused_supported(int d_model, int d_ff);
 cudaError_t launch_ffn_fused(const FfnMaps &w, const CUtensorMap &tmX, float *x, const float *g, const float *b, const float *b1,
-                             const float *b2, const CUtensorMap &tmAtt, const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail,
+                             const float *b2, const CUtensorMap &tmAtt, const CUtensorMap &tmAtt32, const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail,
                              bool *tail_done, int *err, cudaStream_t stream, int64_t *launches);
+// (the form for the fewest rows: *taken tells whether there was one)
+cudaError_t launch_ffn_rows(const FfnMaps &w, float *x, const float *g, const float *b, const float *b1, const float *b2, const CUtensorMap &tmAtt32,
+                            const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail, int *err, cudaStream_t stream, bool *taken);
 // (the form for many rows, called by the launcher above: it leaves the tail to the caller, *tail_done = false)
 cudaError_t launch_ffn_pair(const FfnMaps &w, const CUtensorMap &tmX, const float *x, const float *g, const float *b, const float *b1, const float *b2,
                             const CUtensorMap &tmAtt, const float *bo, int64_t M, int d_ff, float eps, int *err, cudaStream_t stream);
