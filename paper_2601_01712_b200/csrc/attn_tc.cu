@@ -565,31 +565,55 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 
 // Combine the (m, l, O) partials of a split work item:  O = sum_i 2^((m_i - M) c) O_i / sum_i 2^((m_i - M) c) l_i.
 // blockIdx.x = item, blockIdx.y = group of 8 rows; one warp per row, a lane per pair of output columns: every load is a
-// coalesced row segment and all rows are in flight at once (the kernel is a chain of two memory round trips).
+// coalesced row segment and all rows are in flight at once.  The kernel is one memory round trip: what says where to read is call
+// metadata, on the device before the attention kernel began, and a row's partials are all requested before the first is used (as
+// three round trips - metadata, maxima, sums - it cost 3 us of every layer of a small call).
+template <int kBatch>
+__device__ __forceinline__ void merge_row(const float *p, int n, int lane, float &o0, float &o1, float &l)
+{
+    const float c = 0.125f * 1.4426950408889634f;
+    float M = -INFINITY;
+    o0 = o1 = l = 0.f;
+    for (int i0 = 0; i0 < n; i0 += kBatch) {
+        float2 ml[kBatch], v[kBatch];
+        float Mb = M;
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) {
+            const float *q = p + (size_t)(i0 + i) * (kQTile * kPartStride);
+            ml[i] = i0 + i < n ? *reinterpret_cast<const float2 *>(q) : make_float2(-INFINITY, 0.f);
+            v[i] = i0 + i < n ? *reinterpret_cast<const float2 *>(q + 4 + 2 * lane) : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) Mb = fmaxf(Mb, ml[i].x);
+        const float alpha = M == -INFINITY ? 0.f : ex2((M - Mb) * c);
+        M = Mb;
+        l *= alpha; o0 *= alpha; o1 *= alpha;
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) {
+            const float wgt = (ml[i].x == -INFINITY) ? 0.f : ex2((ml[i].x - M) * c);
+            l = fmaf(ml[i].y, wgt, l);
+            o0 = fmaf(v[i].x, wgt, o0);
+            o1 = fmaf(v[i].y, wgt, o1);
+        }
+    }
+}
+
+// kBatch: partials of a row in flight.
+template <int kBatch>
 __global__ void __launch_bounds__(256)
 attention_merge_kernel(const AttnMerge *__restrict__ merges, const SeqDesc *__restrict__ seqs, const float *__restrict__ partial,
                        int d_model, __nv_bfloat16 *__restrict__ out)
 {
-    grid_launch_dependents();
-    grid_dependency_wait();
     const AttnMerge mg = merges[blockIdx.x];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const float c = 0.125f * 1.4426950408889634f;
     const int64_t row0 = (int64_t)seqs[mg.seq].q_row0 + mg.q0;
     const int r = blockIdx.y * 8 + warp;
+    grid_launch_dependents();
+    grid_dependency_wait();
     if (r < mg.n_q) {
-        float M = -INFINITY;
-        for (int i = 0; i < mg.n_splits; ++i) M = fmaxf(M, partial[((size_t)(mg.slot0 + i) * kQTile + r) * kPartStride]);
-        float o0 = 0.f, o1 = 0.f, l = 0.f;
-        for (int i = 0; i < mg.n_splits; ++i) {
-            const float *p = partial + ((size_t)(mg.slot0 + i) * kQTile + r) * kPartStride;
-            const float mi = p[0];
-            const float wgt = (mi == -INFINITY) ? 0.f : ex2((mi - M) * c);
-            const float2 v = *reinterpret_cast<const float2 *>(p + 4 + 2 * lane);
-            l = fmaf(p[1], wgt, l);
-            o0 = fmaf(v.x, wgt, o0);
-            o1 = fmaf(v.y, wgt, o1);
-        }
+        const float *p = partial + ((size_t)mg.slot0 * kQTile + r) * kPartStride;
+        float o0, o1, l;
+        merge_row<kBatch>(p, mg.n_splits, lane, o0, o1, l);
         const float inv = 1.f / l;
         *reinterpret_cast<uint32_t *>(out + (row0 + r) * d_model + mg.head * kDh + 2 * lane) = tc::pack_bf16(o0 * inv, o1 * inv);
     }
@@ -620,7 +644,9 @@ cudaError_t launch_attention_tc(const CUtensorMap &tmQ, const CUtensorMap &tmK, 
                                      n_items, next_item, seqs, pt, n_layers, layer, d_model, early_pages, out, partial, err);
     if (e != cudaSuccess || n_merges == 0) return e;
     *launches += 1;
-    return launch_dependent(attention_merge_kernel, dim3(n_merges, kQTile / 8), dim3(256), 0, stream, 1, merges, seqs, partial, d_model, out);
+    // few rows to merge have many partials each, and registers for all of them; with many rows the occupancy counts
+    auto merge = n_merges * (kQTile / 8) <= 3 * n_sms ? attention_merge_kernel<16> : attention_merge_kernel<8>;
+    return launch_dependent(merge, dim3(n_merges, kQTile / 8), dim3(256), 0, stream, 1, merges, seqs, partial, d_model, out);
 }
 
 }  // namespace relaygr

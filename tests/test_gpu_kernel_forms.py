@@ -35,3 +35,18 @@ def test_feed_forward_forms(rows, ff):
     if len(err) >= 100:                                 # (a handful of errors is no sample of their size)
         assert np.sqrt(np.mean(err ** 2)) <= rms_bound
     pool.close(); model.close()
+
+
+# The merge of split attention items: more partials than one batch of loads (17 per tile), and many tiles with few (the form for occupancy).
+@pytest.mark.parametrize("prefix,cand,kind", [([4500], [40], 0), ([4500], [40], 1), ([1024] * 12, [60] * 12, 0)])
+def test_attention_merge_forms(prefix, cand, kind):
+    shape = small_bf16_shape(vocab=3000, attn_kind=kind)
+    batch = _tiny_batch(shape, 7 + len(prefix), prefix, [3] * len(prefix), cand)
+    w, model, pool, db = _setup(shape, 62, batch)
+    pool.preinfer(db)
+    scores = pool.rank(db).cpu().numpy()
+    assert model.device_status() == 0
+    want = oracle_scores(oracle_model(shape, w), batch, users=sorted({0, len(prefix) - 1}))
+    max_bound, _, _ = bf16_noise_bounds(shape, w, batch, want)
+    assert max_abs_err(scores, batch, want) <= max_bound
+    pool.close(); model.close()
