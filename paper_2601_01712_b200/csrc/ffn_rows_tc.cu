@@ -193,8 +193,8 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
         tc::mbar_expect_tx(&bars->att_full, 4 * kKB);
         for (int kb = 0; kb < 4; ++kb)
             for (int r = 0; r < T; r += 32) tc::tma_load_2d(sA + kb * kKB + r * 128, &tmAtt, kb * 64, (int)tile_row0 + r, &bars->att_full);
-        bars->abort_flag = *reinterpret_cast<volatile int *>(err);
     }
+    if (threadIdx.x == 64) bars->abort_flag = *reinterpret_cast<volatile int *>(err);
     // x, whole rows per warp (it has room for tiles of 128 rows; rows past the last feed only themselves), later mid
     float4 mid[kWarpRows][2];
     if (warp >= 4) {
@@ -210,6 +210,8 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
     const bool live = bars->abort_flag == 0;
     bool o_ready = false;                             // this warp saw the CTA's partial O complete
     float4 own[kEnd][2];                              // mid of the rows this CTA finishes
+    float4 obias2[2], tg[2], tb[2], tw[2];            // of the end of the block
+    int score_at = -1;                                // lane i < kEnd: where the score of the warp's row i goes (-1: not a candidate's)
     if (!live) {
         if (threadIdx.x == 0) {                       // what was requested above lands before the CTA ends
             for (int s = 0; s < kStages; ++s) tc::mbar_wait(&bars->w_full[s], 0, err);
@@ -227,68 +229,67 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer (convergent warp, one elected lane issues)
+        // The chain's pace: an MMA of 128 x T x 16 takes some 50 clocks, what surrounds a stage's eight must not take as long again
+        // (it did, 350 clocks, with one loop for all kinds of stage and divisions for the ring position).
         constexpr uint32_t idesc = tc::make_idesc(kRows, T, 0, 0);             // weights x rows, both K-major
-        const uint32_t a0 = tc::smem_u32(sA), h0 = tc::smem_u32(sH), w0 = tc::smem_u32(sW);
-        auto stage = [&] {                            // waits for the next stage: its address
-            const int s = it % kStages;
-            ok = ok && tc::mbar_wait(&bars->w_full[s], (it / kStages) & 1, err);
+        const uint64_t adesc0 = tc::smem_desc_sw128(tc::smem_u32(sA)), hdesc0 = tc::smem_desc_sw128(tc::smem_u32(sH)), wdesc0 = tc::smem_desc_sw128(tc::smem_u32(sW));
+        uint32_t s = 0, phase = 0;                    // of the ring
+        auto stage = [&] {
+            ok = ok && tc::mbar_wait(&bars->w_full[s], phase, err);
             tc::tc_fence_after();
-            return w0 + s * kStageBytes;
+            return ok;
+        };
+        auto next_stage = [&] {
+            if (++s == kStages) { s = 0; phase ^= 1; }
         };
         auto issue_s = [&](int i) {                   // S^T = W1c A^T: two stages, each two K blocks of 64
-            const int buf = i & 1;
-#pragma unroll 1
-            for (int half = 0; half < 2; ++half, ++it) {
-                const uint32_t w = stage();
-                if (!ok) return;
+            const uint32_t d = tmem_base + L::kColS + (i & 1) * T;
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                if (!stage()) return;
+                const uint64_t wdesc = wdesc0 + s * (kStageBytes / 16);
                 if (tc::elect_one()) {
 #pragma unroll
-                    for (int kb = 0; kb < 2; ++kb) {
-                        const uint64_t adesc = tc::smem_desc_sw128(w + kb * kHalfStage), bdesc = tc::smem_desc_sw128(a0 + (2 * half + kb) * kKB);
+                    for (int kb = 0; kb < 2; ++kb)
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) tc::mma_ss(tmem_base + L::kColS + buf * T, adesc + 2 * k, bdesc + 2 * k, idesc, (half | kb | k) != 0);
-                    }
-                    tc::mma_commit(&bars->w_empty[it % kStages]);
-                    if (half == 1) tc::mma_commit(&bars->s_full[buf]);
+                        for (int k = 0; k < 4; ++k)
+                            tc::mma_ss(d, wdesc + kb * (kHalfStage / 16) + 2 * k, adesc0 + (2 * half + kb) * (kKB / 16) + 2 * k, idesc, (half | kb | k) != 0);
+                    tc::mma_commit(&bars->w_empty[s]);
+                    if (half == 1) tc::mma_commit(&bars->s_full[i & 1]);
                 }
                 __syncwarp();
+                next_stage();
             }
         };
         // one K block of 64 into both halves of P or O: 256 weight rows (output columns) x the tile's rows
-        auto issue_wide = [&](uint32_t rows_at, bool fresh, uint64_t *done) {
-            const uint32_t w = stage();
-            if (!ok) return;
+        auto issue_wide = [&](uint64_t rdesc, bool fresh, uint64_t *done) {
+            if (!stage()) return;
+            const uint64_t wdesc = wdesc0 + s * (kStageBytes / 16);
             if (tc::elect_one()) {
-                const uint64_t bdesc = tc::smem_desc_sw128(rows_at);
 #pragma unroll
-                for (int mb = 0; mb < 2; ++mb) {
-                    const uint64_t adesc = tc::smem_desc_sw128(w + mb * kHalfStage);
+                for (int mb = 0; mb < 2; ++mb)
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) tc::mma_ss(tmem_base + mb * T, adesc + 2 * k, bdesc + 2 * k, idesc, !fresh || k != 0);
-                }
-                tc::mma_commit(&bars->w_empty[it % kStages]);
+                    for (int k = 0; k < 4; ++k) tc::mma_ss(tmem_base + mb * T, wdesc + mb * (kHalfStage / 16) + 2 * k, rdesc + 2 * k, idesc, !fresh || k != 0);
+                tc::mma_commit(&bars->w_empty[s]);
                 if (done) tc::mma_commit(done);
             }
             __syncwarp();
-            ++it;
+            next_stage();
         };
-        it = 0;
         ok = tc::mbar_wait(&bars->att_full, 0, err);
-        // kinds of step in one loop (the code is fetched once): K blocks of the projection, then halves of the chunks' O
+#pragma unroll
+        for (int kb = 0; kb < 4; ++kb) issue_wide(adesc0 + kb * (kKB / 16), kb == 0, kb == 3 ? &bars->p_full : nullptr);
+        ok = ok && tc::mbar_wait(&bars->a_ready, 0, err);
+        tc::tc_fence_after();
+        if (ok) issue_s(0);
 #pragma unroll 1
-        for (int n = 0; n < 4 + 2 * nc && ok; ++n) {
-            const int i = (n - 4) >> 1, half = n & 1;
-            if (n == 4) {
-                ok = tc::mbar_wait(&bars->a_ready, 0, err);
-                tc::tc_fence_after();
-            }
-            if (n >= 4 && half == 0) {
-                // S runs two chunks ahead of O
-                for (int c = i == 0 ? 0 : i + 1; c < i + 2 && c < nc && ok; ++c) issue_s(c);
-                ok = ok && tc::mbar_wait(&bars->h_full[i & 1], (i >> 1) & 1, err);      // H is in shared memory (and S in registers)
-                tc::tc_fence_after();
-            }
-            if (ok) issue_wide(n < 4 ? a0 + n * kKB : h0 + ((i & 1) * 2 + half) * kKB, n == 0 || n == 4, n == 3 ? &bars->p_full : n == 3 + 2 * nc ? &bars->o_full : nullptr);
+        for (int i = 0; i < nc && ok; ++i) {
+            if (i + 1 < nc) issue_s(i + 1);           // S runs ahead of O; its buffer's H has been taken into shared memory
+            ok = ok && tc::mbar_wait(&bars->h_full[i & 1], (i >> 1) & 1, err);      // H is in shared memory (and S in registers)
+            tc::tc_fence_after();
+#pragma unroll
+            for (int half = 0; half < 2; ++half)
+                issue_wide(hdesc0 + ((i & 1) * 2 + half) * (kKB / 16), i == 0 && half == 0, half == 1 && i == nc - 1 ? &bars->o_full : nullptr);
         }
     } else if (warp >= 4) {
         // ---------------------------------------------------------------- LayerNorm, SiLU, drain: eight warps, two per TMEM
@@ -364,6 +365,20 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
             }
             if (!ok) break;
 
+            // what the end of the block needs, while O is on its way
+            if (finisher) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    obias2[h] = load4_or_zero(b2, c0 + 128 * h);
+                    if (tail.kind != FFN_TAIL_NONE) { tg[h] = load4_or_zero(tail.g, c0 + 128 * h); tb[h] = load4_or_zero(tail.b, c0 + 128 * h); }
+                    if (tail.kind == FFN_TAIL_SCORE) tw[h] = load4_or_zero(tail.w, c0 + 128 * h);
+                }
+                const int64_t r = tile_row0 + row(j_end + lane);
+                if (tail.kind == FFN_TAIL_SCORE && lane < kEnd && r < M) {
+                    const int u = find_user(tail.row_off, tail.n_users, (int)r), i = (int)r - tail.seqs[u].score_row0;
+                    if (i >= 0 && i < tail.seqs[u].n_score) score_at = tail.score_off[u] + i;
+                }
+            }
             ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->o_full, 0, err));
             if (!ok) break;
             tc::tc_fence_after();
@@ -374,21 +389,6 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
     __syncwarp();
     // The cluster's partial sums, added in rank order, by whole rows: a row that is complete in one warp goes on to the next layer's
     // LayerNorm, or to the scoring head, right here (FfnTail).
-    float4 obias2[2], tg[2], tb[2], tw[2];
-    int score_at = -1;                                // lane i < kEnd: where the score of the warp's row i goes (-1: not a candidate's)
-    if (live && finisher) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            obias2[h] = load4_or_zero(b2, c0 + 128 * h);
-            if (tail.kind != FFN_TAIL_NONE) { tg[h] = load4_or_zero(tail.g, c0 + 128 * h); tb[h] = load4_or_zero(tail.b, c0 + 128 * h); }
-            if (tail.kind == FFN_TAIL_SCORE) tw[h] = load4_or_zero(tail.w, c0 + 128 * h);
-        }
-        const int64_t r = tile_row0 + row(j_end + lane);
-        if (tail.kind == FFN_TAIL_SCORE && lane < kEnd && r < M) {
-            const int u = find_user(tail.row_off, tail.n_users, (int)r), i = (int)r - tail.seqs[u].score_row0;
-            if (i >= 0 && i < tail.seqs[u].n_score) score_at = tail.score_off[u] + i;
-        }
-    }
     // Everybody takes both barriers, whatever happened before: after the first all partial O are in shared memory, after the second
     // nobody reads a peer's memory any more.
     tc::cluster_sync();
@@ -408,10 +408,11 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
 #pragma unroll
                 for (int k = 1; k < CS; ++k) { v.x += t[i][h][k].x; v.y += t[i][h][k].y; v.z += t[i][h][k].z; v.w += t[i][h][k].w; }
                 add_twice(own[i][h], v, obias2[h]);
+                asm volatile("" ::"f"(own[i][h].x), "f"(own[i][h].y), "f"(own[i][h].z), "f"(own[i][h].w));      // the peers' memory has been read
             }
     }
     __syncwarp();
-    tc::cluster_arrive();
+    tc::cluster_arrive_relaxed();                     // (nothing was written for the peers: a release would wait for nothing, 1100 clocks)
     if (live && finisher && o_ready) {
         if (tail.kind != FFN_TAIL_SCORE) {
 #pragma unroll
