@@ -230,14 +230,16 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         if (more && early_pages)
             for (; j0 < min(kStagesKV, min(nb - n_diag, n_page_blocks - it.blk0)) && load_kv(j0);) ++j0;
     }
-    grid_launch_dependents();
-    grid_dependency_wait();                                       // from here on: data of earlier kernels
-    if (threadIdx.x == 0) bars->abort_flag = *reinterpret_cast<volatile int *>(err);
+    // An earlier kernel gave up: do not pile on.  (Read ahead of the wait: a failure of the kernel just before is seen by the next one.
+    // Behind the wait the word would cost a trip to L2 and a block-wide barrier, 1000 clocks, before the first load.)
+    if (threadIdx.x == 64) bars->abort_flag = *reinterpret_cast<volatile int *>(err);
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem_base = bars->tmem_slot;
-    const bool live = bars->abort_flag == 0;                      // an earlier kernel gave up: do not pile on
+    const bool live = bars->abort_flag == 0;
+    grid_launch_dependents();
+    grid_dependency_wait();                                       // from here on: data of earlier kernels
 
     // Every role walks the same sequence of items: the producer draws an index (the first is the CTA's own number, the others come from
     // the launch's counter) and passes the item on through a two-slot ring in shared memory, so that the other warps do not repeat its

@@ -6,8 +6,8 @@
 //     P^T = Wo att^T          attention rows [T x 256] and Wo by TMA; 256 output columns = two times 128 lanes, T columns of TMEM
 //     mid, A = LN(mid)        P is turned around in shared memory, a warp then has T / 8 whole rows; A as bf16 where att was
 //     per chunk:              S^T = W1c A^T, H = SiLU(S + b1c) as bf16 into shared memory, O^T += W2c H^T
-// The partial O are turned around like P and added up through distributed shared memory in rank order - one fixed order of the
-// fp32 sums, so results do not vary from run to run - and each CTA finishes its share of the tile's rows, the next layer's LayerNorm
+// The partial O are turned around like P and added up through distributed shared memory, the CTA's own first, then in rank order - for
+// every row one fixed order of the fp32 sums, so results do not vary from run to run - and each CTA finishes its share of the tile's rows, the next layer's LayerNorm
 // (or the final one and the scoring head) included.
 //
 // What bounds it: a serial chain of short steps, each with its own latency, and the exchange - distributed shared memory delivers
@@ -52,7 +52,6 @@ struct RowBars {
     uint64_t h_full[2];                               // H in shared memory
     uint64_t o_full;                                  // O complete
     uint32_t tmem_slot;
-    int abort_flag;
 };
 static_assert(sizeof(RowBars<6>) <= 256, "barrier block");
 
@@ -162,8 +161,8 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
     // set-up that touches nothing earlier kernels wrote
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) { tc::mbar_init(&bars->w_full[s], 1); tc::mbar_init(&bars->w_empty[s], 1); }
-        for (int i = 0; i < 2; ++i) { tc::mbar_init(&bars->s_full[i], 1); tc::mbar_init(&bars->h_full[i], kEpiThreads); }
-        tc::mbar_init(&bars->att_full, 1); tc::mbar_init(&bars->p_full, 1); tc::mbar_init(&bars->a_ready, kEpiThreads);
+        for (int i = 0; i < 2; ++i) { tc::mbar_init(&bars->s_full[i], 1); tc::mbar_init(&bars->h_full[i], kEpiWarps); }
+        tc::mbar_init(&bars->att_full, 1); tc::mbar_init(&bars->p_full, 1); tc::mbar_init(&bars->a_ready, kEpiWarps);
         tc::mbar_init(&bars->o_full, 1);
         tc::fence_mbar_init();
         for (int kb = 0; kb < 4; ++kb) {
@@ -187,6 +186,10 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
         }
         if (b1) b1_half = 0.5f * b1[chunk_at(0) * kChunk + quad * 32 + lane];
     }
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    const uint32_t tmem_base = bars->tmem_slot;
     grid_launch_dependents();
     grid_dependency_wait();                           // from here on: data of earlier kernels
     if (threadIdx.x == 0) {
@@ -194,30 +197,21 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
         for (int kb = 0; kb < 4; ++kb)
             for (int r = 0; r < T; r += 32) tc::tma_load_2d(sA + kb * kKB + r * 128, &tmAtt, kb * 64, (int)tile_row0 + r, &bars->att_full);
     }
-    if (threadIdx.x == 64) bars->abort_flag = *reinterpret_cast<volatile int *>(err);
     // x, whole rows per warp (it has room for tiles of 128 rows; rows past the last feed only themselves), later mid
     float4 mid[kWarpRows][2];
+    bool stopped = false;                             // an earlier kernel gave up: everything runs as ever, but nothing is stored
     if (warp >= 4) {
 #pragma unroll
         for (int j = 0; j < kWarpRows; ++j)
 #pragma unroll
             for (int h = 0; h < 2; ++h) mid[j][h] = *reinterpret_cast<const float4 *>(x + (tile_row0 + row(j)) * kD + c0 + 128 * h);
+        stopped = *reinterpret_cast<volatile int *>(err) != 0;
     }
-    tc::tc_fence_before();
-    __syncthreads();
-    tc::tc_fence_after();
-    const uint32_t tmem_base = bars->tmem_slot;
-    const bool live = bars->abort_flag == 0;
     bool o_ready = false;                             // this warp saw the CTA's partial O complete
     float4 own[kEnd][2];                              // mid of the rows this CTA finishes
     float4 obias2[2], tg[2], tb[2], tw[2];            // of the end of the block
     int score_at = -1;                                // lane i < kEnd: where the score of the warp's row i goes (-1: not a candidate's)
-    if (!live) {
-        if (threadIdx.x == 0) {                       // what was requested above lands before the CTA ends
-            for (int s = 0; s < kStages; ++s) tc::mbar_wait(&bars->w_full[s], 0, err);
-            tc::mbar_wait(&bars->att_full, 0, err);
-        }
-    } else if (warp == 0) {
+    if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer
         if (lane == 0) {
             for (int h = kEarlyHalves; h < 2; ++h) load_w1(chunk_at(0), h);
@@ -332,9 +326,14 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
             }
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
-            tc::fence_proxy_async();                  // generic-proxy writes of the tile before the tensor core reads it
-            tc::tc_fence_before();
-            tc::mbar_arrive(&bars->a_ready);
+            // one arrival per warp, when every lane's generic-proxy writes are visible to the tensor core
+            auto publish = [&](uint64_t *bar) {
+                tc::fence_proxy_async();
+                tc::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(bar);
+            };
+            publish(&bars->a_ready);
 
             // H: this lane's hidden unit, rows ch * T / 2 ..; 16-byte chunk (lane / 8 + 4 * (quad & 1)) of each row of its K block
             uint8_t *h_lane = sH + (quad >> 1) * kKB + ch * (T / 2) * 128 + (lane & 7) * 2;
@@ -352,7 +351,6 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
                 if constexpr (T == 64) tc::tmem_ld32(lane_addr + L::kColS + hb * T + ch * (T / 2), r);
                 else tc::tmem_ld16(lane_addr + L::kColS + hb * T + ch * (T / 2), r);
                 tc::tmem_ld_wait();
-                tc::tc_fence_before();
                 uint8_t *dst = h_lane + hb * 2 * kKB;
 #pragma unroll
                 for (int e = 0; e < T / 2; e += 2) {
@@ -360,8 +358,7 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
                     *reinterpret_cast<uint16_t *>(dst + e * 128 + ((h_chunk ^ (e & 7)) << 4)) = (uint16_t)p;
                     *reinterpret_cast<uint16_t *>(dst + (e + 1) * 128 + ((h_chunk ^ ((e + 1) & 7)) << 4)) = (uint16_t)(p >> 16);
                 }
-                tc::fence_proxy_async();
-                tc::mbar_arrive(&bars->h_full[hb]);
+                publish(&bars->h_full[hb]);
             }
             if (!ok) break;
 
@@ -387,19 +384,22 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
         } while (false);
     }
     __syncwarp();
-    // The cluster's partial sums, added in rank order, by whole rows: a row that is complete in one warp goes on to the next layer's
+    // The cluster's partial sums, added up by whole rows: a row that is complete in one warp goes on to the next layer's
     // LayerNorm, or to the scoring head, right here (FfnTail).
     // Everybody takes both barriers, whatever happened before: after the first all partial O are in shared memory, after the second
     // nobody reads a peer's memory any more.
     tc::cluster_sync();
-    if (live && finisher && o_ready) {
+    if (finisher && o_ready) {
         float4 t[kEnd][2][CS];
 #pragma unroll
         for (int i = 0; i < kEnd; ++i)
 #pragma unroll
             for (int h = 0; h < 2; ++h)
 #pragma unroll
-                for (int k = 0; k < CS; ++k) t[i][h][k] = load_cluster4(tc::cluster_addr(turn + row(j_end + i) * kD + c0 + 128 * h, k));
+                for (int k = 0; k < CS; ++k) {
+                    const float *p = turn + row(j_end + i) * kD + c0 + 128 * h;
+                    t[i][h][k] = k == 0 ? *reinterpret_cast<const float4 *>(p) : load_cluster4(tc::cluster_addr(p, (rank + k) & (CS - 1)));
+                }
 #pragma unroll
         for (int i = 0; i < kEnd; ++i)
 #pragma unroll
@@ -413,7 +413,7 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
     }
     __syncwarp();
     tc::cluster_arrive_relaxed();                     // (nothing was written for the peers: a release would wait for nothing, 1100 clocks)
-    if (live && finisher && o_ready) {
+    if (finisher && o_ready && !stopped) {
         if (tail.kind != FFN_TAIL_SCORE) {
 #pragma unroll
             for (int i = 0; i < kEnd; ++i) {

@@ -58,7 +58,6 @@ struct GemmBars {
     uint64_t full[kMaxStages], empty[kMaxStages];
     uint64_t acc_full[2], acc_empty[2];
     uint32_t tmem_slot;
-    int abort_flag;
 };
 static_assert(sizeof(GemmBars) <= 256, "barrier block");
 
@@ -112,17 +111,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         else { tc::tmem_alloc(&bars->tmem_slot, kTmemCols); tc::tmem_relinquish(); }
     }
     if constexpr (CTAS == 2) tc::cluster_sync();                  // the peer's barriers exist before anything signals them
-    grid_launch_dependents();
-    grid_dependency_wait();                                       // from here on: data of earlier kernels
-    if (threadIdx.x == 0) bars->abort_flag = *reinterpret_cast<volatile int *>(err);
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem_base = bars->tmem_slot;
-    const bool live = bars->abort_flag == 0;                      // an earlier kernel gave up: do not pile on
+    grid_launch_dependents();
+    grid_dependency_wait();                                       // from here on: data of earlier kernels
 
-    if (!live) {
-    } else if (warp == 0) {
+    if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer: this CTA's rows of A and of B
         if (lane == 0) {
             uint32_t it = 0;
@@ -196,6 +192,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int half = ew >> 2;                           // columns (BN/2)*half .. +BN/2-1 of the tile, 64 at a time
         constexpr int kColsPerWarp = BN / 2;
         uint8_t *patches = smem + C::kOffPatch + ew * (kPatches * kPatchBytes);
+        // An earlier kernel gave up: nothing is stored.  (The loads and products go on as ever: to wait for this word before them would
+        // put a trip to L2 and a block-wide barrier, 1000 clocks, between the predecessor's end and the first load.)
+        const bool stopped = *reinterpret_cast<volatile int *>(err) != 0;
         // the whole bias once, under the first tile's loads: a look-up per tile would be on the epilogue's path
         float *bias_s = reinterpret_cast<float *>(smem + C::kOffBias);
         const bool bias_staged = epi.bias && N <= kMaxBias;
@@ -279,7 +278,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                         else tc::mbar_arrive(&bars->acc_empty[as]);
                     }
                 }
-                if (m_base >= M) continue;                                       // the whole row group lies past the last row
+                if (m_base >= M || stopped) continue;                            // the whole row group lies past the last row
                 const int n = n_w + pass * 64;                                   // first output column of these 64
                 if (epi.bias) {
                     const float4 *b4 = reinterpret_cast<const float4 *>(bias_w + pass * 64);
