@@ -100,14 +100,16 @@ f32_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         tc::tmem_alloc(&bars->tmem_slot, kGemmCols);
         tc::tmem_relinquish();
     }
-    grid_launch_dependents();
-    grid_dependency_wait();
+    // An earlier kernel gave up: do not pile on.  (Read ahead of the wait: a failure of the kernel just before is seen by the next one.
+    // Behind the wait the word would cost a trip to L2 and a block-wide barrier, 1000 clocks, before the first load.)
     if (tid == 0) bars->abort_flag = *reinterpret_cast<volatile int *>(err);
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem_base = bars->tmem_slot;
     const bool live = bars->abort_flag == 0;
+    grid_launch_dependents();
+    grid_dependency_wait();
 
     if (!live) {
     } else if (warp < 8) {
@@ -376,14 +378,16 @@ f32_attention_tc_kernel(const float *__restrict__ q, const float *__restrict__ k
         tc::tmem_alloc(&bars->tmem_slot, kAttnCols);
         tc::tmem_relinquish();
     }
-    grid_launch_dependents();
-    grid_dependency_wait();
+    // An earlier kernel gave up: do not pile on.  (Read ahead of the wait: a failure of the kernel just before is seen by the next one.
+    // Behind the wait the word would cost a trip to L2 and a block-wide barrier, 1000 clocks, before the first load.)
     if (tid == 0) bars->abort_flag = *reinterpret_cast<volatile int *>(err);
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem_base = bars->tmem_slot;
     const bool live = bars->abort_flag == 0;
+    grid_launch_dependents();
+    grid_dependency_wait();
 
     const AttnItem it = items[blockIdx.x];
     const SeqDesc sd = seqs[it.seq];
