@@ -130,12 +130,12 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
             // ------------------------------------------------------------ weights, in the order of consumption: Wo in four K blocks,
             // W1(0), W1(1), then per chunk c: W2(c), W1(c+2); and the attention rows
             if (lane == 0) {
-                uint32_t it = 4;                      // ring position; the first tile's Wo is on its way
+                int next = 4, phase = 0;              // of the ring; the first tile's Wo is on its way
                 bool ok = true;
                 auto acquire = [&] {
-                    const int s = it % kStages;
-                    ok = ok && tc::mbar_wait(&bars->w_empty[s], ((it / kStages) & 1) ^ 1, err);
-                    ++it;
+                    const int s = next;
+                    ok = ok && tc::mbar_wait(&bars->w_empty[s], phase ^ 1, err);
+                    if (++next == kStages) { next = 0; phase ^= 1; }
                     return s;
                 };
                 auto load = [&](bool second, int c) {
@@ -182,14 +182,14 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
             constexpr uint32_t idesc_s = tc::make_idesc(2 * kRows, kChunk, 0, 0);      // A and W1 both K-major
             constexpr uint32_t idesc_o = tc::make_idesc(2 * kRows, kD, 0, 0);          // att (or H from TMEM), Wo / W2 K-major
             const uint32_t a0 = tc::smem_u32(sA);
-            uint32_t it = 0;
+            int next = 0, phase = 0;                  // of the ring
             int gc = 0;
             bool ok = true;
             auto stage = [&] {                        // the next stage, complete in both CTAs
-                const int s = it % kStages;
-                ok = tc::mbar_wait(&bars->w_full[s], (it / kStages) & 1, err);
+                const int s = next;
+                ok = tc::mbar_wait(&bars->w_full[s], phase, err);
                 tc::tc_fence_after();
-                ++it;
+                if (++next == kStages) { next = 0; phase ^= 1; }
                 return s;
             };
             for (int tile = tile0, n = 0; tile < n_tiles && ok; tile += tile_step, ++n) {
