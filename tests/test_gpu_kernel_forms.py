@@ -4,7 +4,7 @@ import pytest
 import torch
 
 from paper_2601_01712_b200 import synth
-from tests.helpers import TOL_BF16, bf16_noise_bounds, max_abs_err, oracle_model, oracle_scores, small_bf16_shape
+from tests.helpers import TOL_F32, bf16_noise_bounds, max_abs_err, oracle_model, oracle_scores, small_bf16_shape
 from tests.test_gpu_parity import _setup, _tiny_batch
 
 pytestmark = pytest.mark.gpu
@@ -49,4 +49,117 @@ def test_attention_merge_forms(prefix, cand, kind):
     want = oracle_scores(oracle_model(shape, w), batch, users=sorted({0, len(prefix) - 1}))
     max_bound, _, _ = bf16_noise_bounds(shape, w, batch, want)
     assert max_abs_err(scores, batch, want) <= max_bound
+    pool.close(); model.close()
+
+
+def _check_f32(shape, batch, seed, model_of=None, users=None):
+    w, model, pool, db = _setup(shape, seed, batch)
+    if model_of is not None:
+        pool.close()
+        model = model_of(model, batch)
+        from paper_2601_01712_b200 import runtime as rt
+        pool = rt.KvPool(model, sum(synth.pages_for(batch.prefix_off[i + 1] - batch.prefix_off[i]) for i in range(batch.n_users)))
+        for i in range(batch.n_users):
+            pool.alloc(batch.users[i], batch.prefix_off[i + 1] - batch.prefix_off[i])
+    om = oracle_model(shape, w)
+    users = list(range(batch.n_users)) if users is None else users
+    pool.preinfer(db)
+    scores = pool.rank(db).cpu().numpy()
+    full = model.rank_full(db).cpu().numpy()
+    assert model.device_status() == 0
+    for i in users:
+        K, V = om.preinfer(batch.user_slices(i)[0])
+        gK, gV = pool.read_kv(batch.users[i], len(batch.user_slices(i)[0]))
+        assert np.max(np.abs(gK.cpu().numpy().astype(np.float64) - K)) <= TOL_F32
+        assert np.max(np.abs(gV.cpu().numpy().astype(np.float64) - V)) <= TOL_F32
+    want = oracle_scores(om, batch, users=users)
+    assert max_abs_err(scores, batch, want) <= TOL_F32
+    assert max_abs_err(full, batch, want) <= TOL_F32
+    pool.close(); model.close()
+
+
+# fp32 model.  A call runs on the tensor cores from rows x d_model = 49152 on: ranking calls just below and at that, both head
+# widths, widths that are no multiple of the 64-column tiles, users whose rows start inside a group of 32, one user whose key
+# blocks are split over several CTAs (merge), pointwise attention; and calls of a few rows, where the CUDA-core tiles are lowest.
+F32 = [
+    # d, heads, ff, kind, prefix, short, cand
+    (96, 3, 200, 0, [130, 77, 300], [5, 0, 40], [200, 97, 169]),           # 511 rows
+    (96, 3, 200, 0, [130, 77, 300], [5, 0, 40], [200, 97, 170]),           # 512 rows
+    (64, 1, 100, 0, [500, 65], [3, 64], [600, 130]),                       # 797 rows, d_head 64
+    (256, 4, 1024, 0, [1500], [12], [180]),                                # 192 rows: split over the keys
+    (128, 4, 256, 1, [700, 33], [0, 9], [385, 64]),                        # pointwise, d_head 32
+    (128, 2, 260, 1, [900], [1], [400]),                                   # pointwise, d_head 64, split
+    (64, 2, 128, 0, [1, 70], [0, 1], [1, 14]),
+    (64, 2, 128, 0, [64, 200, 90], [7, 0, 1], [100, 33, 60]),
+]
+
+
+@pytest.mark.parametrize("case", range(len(F32)))
+def test_f32_forms(case):
+    d, heads, ff, kind, p, s, c = F32[case]
+    shape = synth.ModelShape(2, d, heads, d // heads, ff, 2000, synth.DTYPE_F32, attn_kind=kind)
+    _check_f32(shape, _tiny_batch(shape, 300 + case, p, s, c), 63)
+
+
+def test_f32_weights_off_16_bytes_stay_on_the_cuda_cores():
+    """Matrices of weights at no multiple of 16 bytes can have no tensor map: a call of any size takes the other kernels.  (The
+    embedding table and the vectors are read 16 bytes at a time in every form, and stay where they are.)"""
+    shape = synth.ModelShape(2, 128, 2, 64, 256, 2000, synth.DTYPE_F32)
+    batch = _tiny_batch(shape, 320, [600, 100], [3, 0], [300, 130])
+
+    def off_by_four(model, batch):
+        from paper_2601_01712_b200 import binding as B
+        weights = B.Weights()
+        for name in B.WEIGHT_FIELDS:
+            t = model._t[name]
+            if name not in ("w_qkv", "w_o", "w1", "w2"):
+                setattr(weights, name, t.data_ptr())
+                continue
+            raw = torch.empty(t.numel() + 1, dtype=t.dtype, device=t.device)
+            raw[1:].copy_(t.flatten())
+            model._t[name] = raw[1:].view(t.shape)
+            setattr(weights, name, model._t[name].data_ptr())
+        model._w = weights
+        other = model.new_slot()
+        other.reserve(int(batch.prefix_off[-1] + batch.short_off[-1] + batch.cand_off[-1]), batch.n_users, 64)
+        return other
+
+    _check_f32(shape, batch, 64, off_by_four)
+
+
+# Full inference moves the candidates together for the end of the last layer when the other rows cost more than that (here from some
+# 4700 rows on); the ranking calls of the tests above never do.
+@pytest.mark.parametrize("dtype", [synth.DTYPE_BF16, synth.DTYPE_F32])
+@pytest.mark.parametrize("users", [2, 9])
+def test_candidates_moved_together_or_not(dtype, users):
+    shape = synth.ModelShape(2, 256, 4, 64, 1024, 2000, dtype)
+    batch = _tiny_batch(shape, 330 + users, [600] * users, [33] * users, [70] * users)
+    sample = [0, users - 1]
+    if dtype == synth.DTYPE_F32:
+        _check_f32(shape, batch, 65, users=sample)
+        return
+    w, model, pool, db = _setup(shape, 65, batch)
+    full = model.rank_full(db).cpu().numpy()
+    assert model.device_status() == 0
+    want = oracle_scores(oracle_model(shape, w), batch, users=sample)
+    max_bound, _, _ = bf16_noise_bounds(shape, w, batch, want)
+    assert max_abs_err(full, batch, want) <= max_bound
+    pool.close(); model.close()
+
+
+# Pre-inference writes K / V rows into pages: 32 rows of the call that are 32 slots of one page leave together, others row by row.
+# Users start at every kind of offset in a group of 32, and end inside, at and behind a page's last slot.
+def test_preinfer_rows_in_and_across_pages():
+    shape = small_bf16_shape(vocab=3000)
+    batch = _tiny_batch(shape, 340, [32, 96, 1, 63, 64, 128, 31, 33, 200], [0] * 9, [4] * 9)
+    w, model, pool, db = _setup(shape, 66, batch)
+    pool.preinfer(db)
+    assert model.device_status() == 0
+    om = oracle_model(shape, w)
+    for i in range(batch.n_users):
+        p = batch.user_slices(i)[0]
+        K, V = om.preinfer(p)
+        gK, gV = pool.read_kv(batch.users[i], len(p))
+        assert np.max(np.abs(gK.float().cpu().numpy() - K)) <= 5e-2      # bf16 rows of magnitude ~1-4, as in test_gpu_parity.py
+        assert np.max(np.abs(gV.float().cpu().numpy() - V)) <= 5e-2
     pool.close(); model.close()
