@@ -47,7 +47,6 @@ struct Bars {
     uint64_t h_full[2];                               // H in TMEM
     uint64_t o_full;                                  // O complete
     uint32_t tmem_slot;
-    int abort_flag;
 };
 static_assert(sizeof(Bars) <= 256, "barrier block");
 
@@ -94,8 +93,8 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant
     // set-up that touches nothing earlier kernels wrote
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) { tc::mbar_init(&bars->w_full[s], 1); tc::mbar_init(&bars->w_empty[s], 1); }
-        for (int i = 0; i < 2; ++i) { tc::mbar_init(&bars->s_full[i], 1); tc::mbar_init(&bars->h_full[i], kEpiThreads); }
-        tc::mbar_init(&bars->att_full, 1); tc::mbar_init(&bars->o1_full, 1); tc::mbar_init(&bars->a_ready, kEpiThreads);
+        for (int i = 0; i < 2; ++i) { tc::mbar_init(&bars->s_full[i], 1); tc::mbar_init(&bars->h_full[i], kEpiWarps); }
+        tc::mbar_init(&bars->att_full, 1); tc::mbar_init(&bars->o1_full, 1); tc::mbar_init(&bars->a_ready, kEpiWarps);
         tc::mbar_init(&bars->o_full, 1);
         tc::fence_mbar_init();
         for (int kb = 0; kb < kStages; ++kb) load_wo(kb);      // parameters, as the biases below
@@ -112,19 +111,21 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant
             gs[i] = g[i]; bs[i] = b[i]; bos[i] = bo ? bo[i] : 0.f;
         }
     }
-    grid_launch_dependents();
-    grid_dependency_wait();                           // from here on: data of earlier kernels
-    if (threadIdx.x == 0) bars->abort_flag = *reinterpret_cast<volatile int *>(err);
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem_base = bars->tmem_slot;
-    const bool live = bars->abort_flag == 0;
+    grid_launch_dependents();
+    grid_dependency_wait();                           // from here on: data of earlier kernels
+    bool stopped = false;                             // an earlier kernel gave up: everything runs as ever, but nothing is stored
     bool o_ready = false;                             // this warp saw the CTA's partial O complete
-    if (!live) {
-        if (threadIdx.x == 0)                         // what was requested above lands before the CTA ends
-            for (int kb = 0; kb < kStages; ++kb) tc::mbar_wait(&bars->w_full[kb], 0, err);
-    } else if (warp == 0) {
+    // the end of the block, by whole rows: kRowsPerWarp of them per warp, from row_first of the tile; columns c0 .. + 3 and 128 + c0 .. + 3
+    // of each per lane
+    constexpr int kRowsPerWarp = 16 / CS, kBatch = kRowsPerWarp / 2;
+    const int row_first = rank * (kRows / CS) + (warp - 4) * kRowsPerWarp, c0 = 4 * lane;
+    float4 tg[2], tb[2], tw[2];
+    int score_at = -1;                                // lane i < kRowsPerWarp: where the score of the warp's row i goes (-1: not a candidate's)
+    if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer
         if (lane == 0) {
             uint32_t it = kStages;                    // ring position; Wo is on its way
@@ -238,6 +239,13 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant
         const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
         const int rr = quad * 32 + lane;
         bool ok = true;
+        stopped = *reinterpret_cast<volatile int *>(err) != 0;
+        // one arrival per warp, when every lane's part is done
+        auto publish = [&](uint64_t *bar) {
+            tc::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(bar);
+        };
         const uint32_t o_cols = lane_addr + kColO + ch * 128;
         do {
             // x into O's columns while the loads and the projection are on their way.  Row-per-lane loads would touch 32 lines each
@@ -294,8 +302,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant
             tc::tmem_st_wait();
             normalise(o_cols, gs, bs, mean, rstd, sA, ch, rr);
             tc::fence_proxy_async();                  // generic-proxy writes of the tile before the tensor core reads it
-            tc::tc_fence_before();
-            tc::mbar_arrive(&bars->a_ready);
+            publish(&bars->a_ready);
 
             for (int i = 0; i < nc; ++i) {
                 const int hb = i & 1;
@@ -304,11 +311,23 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant
                 tc::tc_fence_after();
                 silu_chunk(lane_addr + kColS + hb * kChunk + ch * 64, b1s + chunk_at(i) * kChunk + ch * 64);
                 tc::tmem_st_wait();
-                tc::tc_fence_before();
-                tc::mbar_arrive(&bars->h_full[hb]);
+                publish(&bars->h_full[hb]);
             }
             if (!ok) break;
 
+            // what the end of the block needs, while O is on its way
+            if (tail.kind != FFN_TAIL_NONE) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    tg[h] = *reinterpret_cast<const float4 *>(tail.g + c0 + 128 * h); tb[h] = *reinterpret_cast<const float4 *>(tail.b + c0 + 128 * h);
+                    if (tail.kind == FFN_TAIL_SCORE) tw[h] = *reinterpret_cast<const float4 *>(tail.w + c0 + 128 * h);
+                }
+                const int64_t row = (int64_t)tile * kRows + row_first + lane;
+                if (tail.kind == FFN_TAIL_SCORE && lane < kRowsPerWarp && row < M) {
+                    const int u = find_user(tail.row_off, tail.n_users, (int)row), i = (int)row - tail.seqs[u].score_row0;
+                    if (i >= 0 && i < tail.seqs[u].n_score) score_at = tail.score_off[u] + i;
+                }
+            }
             ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->o_full, 0, err));
             if (!ok) break;
             tc::tc_fence_after();
@@ -326,28 +345,12 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant
         } while (false);
     }
     __syncwarp();
-    // The cluster's partial sums, added in rank order, by whole rows (128 / CS of them per CTA, a warp for 16 / CS): a row that is
-    // complete in one warp goes on to the next layer's LayerNorm, or to the scoring head, right here (FfnTail).
-    constexpr int kRowsPerWarp = 16 / CS, kBatch = kRowsPerWarp / 2;
-    const int row_first = rank * (kRows / CS) + (warp - 4) * kRowsPerWarp, c0 = 4 * lane;      // columns c0 .. + 3 and 128 + c0 .. + 3
-    float4 tg[2], tb[2], tw[2];
-    int score_at = -1;                                // lane i < kRowsPerWarp: where the score of the warp's row i goes (-1: not a candidate's)
-    if (live && warp >= 4 && tail.kind != FFN_TAIL_NONE) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            tg[h] = *reinterpret_cast<const float4 *>(tail.g + c0 + 128 * h); tb[h] = *reinterpret_cast<const float4 *>(tail.b + c0 + 128 * h);
-            if (tail.kind == FFN_TAIL_SCORE) tw[h] = *reinterpret_cast<const float4 *>(tail.w + c0 + 128 * h);
-        }
-        const int64_t row = (int64_t)tile * kRows + row_first + lane;
-        if (tail.kind == FFN_TAIL_SCORE && lane < kRowsPerWarp && row < M) {
-            const int u = find_user(tail.row_off, tail.n_users, (int)row), i = (int)row - tail.seqs[u].score_row0;
-            if (i >= 0 && i < tail.seqs[u].n_score) score_at = tail.score_off[u] + i;
-        }
-    }
+    // The cluster's partial sums, added up by whole rows: a row that is complete in one warp goes on to the next layer's LayerNorm, or to
+    // the scoring head, right here (FfnTail).
     // Everybody takes both barriers, whatever happened before: after the first all partial O are in shared memory (and nobody still
     // reads x), after the second nobody reads a peer's memory any more.
     tc::cluster_sync();
-    if (live && warp >= 4 && o_ready) {
+    if (warp >= 4 && o_ready) {
 #pragma unroll 1
         for (int hb = 0; hb < 2; ++hb) {              // two batches of rows, each with sixteen loads in flight
             float4 t[kBatch][2][CS];
@@ -374,7 +377,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant
                     v[h].x += q.x; v[h].y += q.y; v[h].z += q.z; v[h].w += q.w;
                     sum += (v[h].x + v[h].y) + (v[h].z + v[h].w);
                 }
-                if (tail.kind != FFN_TAIL_SCORE && row < M) {
+                if (tail.kind != FFN_TAIL_SCORE && row < M && !stopped) {
 #pragma unroll
                     for (int h = 0; h < 2; ++h) *reinterpret_cast<float4 *>(x + row * kD + c0 + 128 * h) = v[h];
                 }
@@ -393,7 +396,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant
                     const float4 y = make_float4(v[h].x * rstd * tg[h].x + tb[h].x, v[h].y * rstd * tg[h].y + tb[h].y,
                                                  v[h].z * rstd * tg[h].z + tb[h].z, v[h].w * rstd * tg[h].w + tb[h].w);
                     if (tail.kind == FFN_TAIL_LN) {
-                        if (row < M) *reinterpret_cast<uint2 *>(tail.a + row * kD + c0 + 128 * h) = make_uint2(tc::pack_bf16(y.x, y.y), tc::pack_bf16(y.z, y.w));
+                        if (row < M && !stopped) *reinterpret_cast<uint2 *>(tail.a + row * kD + c0 + 128 * h) = make_uint2(tc::pack_bf16(y.x, y.y), tc::pack_bf16(y.z, y.w));
                     } else {
                         acc += y.x * tw[h].x + y.y * tw[h].y + y.z * tw[h].z + y.w * tw[h].w;
                     }
@@ -401,7 +404,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant
                 if (tail.kind == FFN_TAIL_SCORE) {
                     acc = warp_sum(acc);
                     const int at = __shfl_sync(0xffffffffu, score_at, hb * kBatch + i);
-                    if (lane == 0 && at >= 0) tail.scores[at] = acc + (tail.bias ? tail.bias[0] : 0.f);
+                    if (lane == 0 && at >= 0 && !stopped) tail.scores[at] = acc + (tail.bias ? tail.bias[0] : 0.f);
                 }
             }
         }
