@@ -163,3 +163,11 @@ def test_preinfer_rows_in_and_across_pages():
         assert np.max(np.abs(gK.float().cpu().numpy() - K)) <= 5e-2      # bf16 rows of magnitude ~1-4, as in test_gpu_parity.py
         assert np.max(np.abs(gV.float().cpu().numpy() - V)) <= 5e-2
     pool.close(); model.close()
+
+
+# Few rows of the fp32 model: K in steps of 128 over four groups of threads, with K below one step, no multiple of it and beyond three,
+# as long as every 16 x 64 tile has an SM to itself (the last two cases: just not).
+@pytest.mark.parametrize("d,heads,ff,cand", [(64, 1, 20, 9), (96, 3, 420, 33), (256, 8, 1028, 70), (32, 1, 4, 17), (64, 2, 260, 470), (256, 4, 516, 150)])
+def test_f32_few_rows(d, heads, ff, cand):
+    shape = synth.ModelShape(2, d, heads, d // heads, ff, 2000, synth.DTYPE_F32)
+    _check_f32(shape, _tiny_batch(shape, 350 + d + ff, [20], [3], [cand]), 67)
