@@ -101,6 +101,17 @@ f32_gemm_kernel(const float *__restrict__ A, const float *__restrict__ W, int64_
     auto load_w = [&](int ks) { load(w_at(ks), W, n0, N, kBN, ks); };
     auto load_a = [&](int ks) { load(a_at(ks), A, m0, M, BM, ks); };
 
+    // LayerNorm of A on the way (gemm_f32_takes_ln): a warp per row, 32 columns at a time per lane
+    constexpr int kLnParts = G > 1 ? (kStages - 1) * G : 1;
+    float gain[kLnParts], shift[kLnParts];
+    if (G > 1 && e.ln_g) {
+#pragma unroll
+        for (int i = 0; i < kLnParts; ++i) {
+            const int k = i * kBK + (tid & 31);
+            gain[i] = k < K ? e.ln_g[k] : 0.f;
+            shift[i] = k < K ? e.ln_b[k] : 0.f;
+        }
+    }
     // the weights are parameters: the first stages of W are on their way while the previous kernel finishes
     grid_launch_dependents();
 #pragma unroll
@@ -121,6 +132,32 @@ f32_gemm_kernel(const float *__restrict__ A, const float *__restrict__ W, int64_
         }
         page_off[tid] = off;
         last_slot[tid] = last;
+    }
+
+    if (G > 1 && e.ln_g) {
+        static_assert(G == 1 || kThreads * G == 32 * BM, "a warp per row");
+        cp_wait<0>();
+        __syncthreads();
+        float *row = As + (tid >> 5) * kLdk + (tid & 31), v[kLnParts], s = 0.f, sq = 0.f;
+#pragma unroll
+        for (int i = 0; i < kLnParts; ++i) {
+            v[i] = i * kBK < K ? row[i * BM * kLdk] : 0.f;      // (zeros behind the last column)
+            s += v[i];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        const float mean = s / (float)K;
+#pragma unroll
+        for (int i = 0; i < kLnParts; ++i) {
+            v[i] = i * kBK + (tid & 31) < K ? v[i] - mean : 0.f;
+            sq += v[i] * v[i];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        const float rstd = rsqrtf(sq / (float)K + e.ln_eps);
+#pragma unroll
+        for (int i = 0; i < kLnParts; ++i)
+            if (i * kBK < K) row[i * BM * kLdk] = v[i] * rstd * gain[i] + shift[i];
     }
 
     uint64_t acc[RT][4] = {};
@@ -472,6 +509,13 @@ static int tile_rows_for(int64_t blocks64, int64_t blocks32, int n_sms)
     return 2 * blocks32 >= 3 * (int64_t)n_sms ? 32 : 16;
 }
 
+// Every 16 x 64 tile has an SM to itself.
+static bool f32_gemm_grouped(int64_t M, int N, int n_sms) { return (int64_t)((N + kBN - 1) / kBN) * ((M + 15) / 16) <= n_sms; }
+
+// All of A's columns are in shared memory at once (two stages of 128): every tile can normalise its 16 rows itself, and the LayerNorm's
+// launch of 4 us in a chain of short ones is gone.
+bool gemm_f32_takes_ln(int64_t M, int N, int K, int n_sms) { return K <= (kStages - 1) * 4 * kBK && f32_gemm_grouped(M, N, n_sms); }
+
 cudaError_t launch_gemm_f32(const float *A, const float *W, int64_t M, int N, int K, const Epilogue &epi, int n_sms, cudaStream_t stream,
                             int64_t *launches)
 {
@@ -483,7 +527,7 @@ cudaError_t launch_gemm_f32(const float *A, const float *W, int64_t M, int N, in
         case 32: return launch_gemm<4, 1>(A, W, M, N, K, epi, stream);
     }
     // as long as every block has an SM to itself, with four groups (f32_gemm_kernel)
-    return cols * ((M + 15) / 16) <= n_sms ? launch_gemm<2, 4>(A, W, M, N, K, epi, stream) : launch_gemm<2, 1>(A, W, M, N, K, epi, stream);
+    return f32_gemm_grouped(M, N, n_sms) ? launch_gemm<2, 4>(A, W, M, N, K, epi, stream) : launch_gemm<2, 1>(A, W, M, N, K, epi, stream);
 }
 
 int build_f32_tiles(const std::vector<SeqDesc> &seqs, int n_heads, int n_sms, std::vector<F32Tile> &tiles)

@@ -412,24 +412,31 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     bool dead_tail = false;                       // a call without candidates: nothing reads the last layer
     bool ln_done = false, scored = false;         // the fused kernel of the layer before has taken this layer's LayerNorm 1 / the scores
 
+    // fp32 model, few rows: the GEMM behind a LayerNorm normalises its rows itself
+    auto ln_in_gemm = [&](int64_t M, int N) { return !kTensor && !tensor32 && gemm_f32_takes_ln(M, N, d, n_sms); };
+    auto with_ln = [&](Epilogue &ep, const float *g, const float *b) { ep.ln_g = g; ep.ln_b = b; ep.ln_eps = cfg.ln_eps; };
+
     for (int l = 0; l < L; ++l) {
         const bool last = l == L - 1;
         if (last && !preinfer && n_scores == 0) { dead_tail = true; break; }
         const float *g1 = w.ln1_g + (size_t)l * d, *b1n = w.ln1_b + (size_t)l * d;
+        // K and V only in the last pre-infer layer (psi is K/V alone) and in the last layer of a call whose candidates are moved together
+        // (their queries follow below, on their rows alone)
+        const bool kv_only = last && (preinfer || compact_last);
+        const bool ln1_in_gemm = l > 0 && !(last && compact_last) && ln_in_gemm(R, kv_only ? 2 * d : 3 * d);
         if (l == 0) {
             cudaEvent_t pe = prof_begin(stream);
             e = launch_gather_ln<T>((const T *)w.emb, cfg.vocab, d, src, R, g1, b1n, cfg.ln_eps, x, a, d_status, stream, &launches);
             prof_end(KC_GATHER_LN, pe, stream);
-        } else if (!ln_done) {
+        } else if (!ln_done && !ln1_in_gemm) {
             e = layernorm(x, R, g1, b1n);
         }
         if (!ck("LayerNorm 1")) return RELAYGR_E_CUDA;
 
-        // fused QKV projection over all rows; K and V only in the last pre-infer layer (psi is K/V alone) and in the last
-        // layer of a rank call (the queries of the candidates follow below, on their rows alone)
-        const bool kv_only = last && (preinfer || compact_last);
+        // fused QKV projection over all rows
         Epilogue ep{};
         ep.mode = EPI_QKV;
+        if (ln1_in_gemm) with_ln(ep, g1, b1n);
         ep.col0 = kv_only ? d : 0;
         ep.bias = w.b_qkv ? w.b_qkv + (size_t)l * 3 * d + ep.col0 : nullptr;
         ep.d_model = d;
@@ -442,7 +449,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         if (preinfer) { ep.paged = paged; ep.page_runs = meta + o_runs; }
         const T *Wqkv = (const T *)w.w_qkv + ((size_t)l * 3 * d + ep.col0) * d;
         lm = wmaps_ok ? &wmaps[(size_t)l] : nullptr;
-        e = gemm(R, a, tm_a, Wqkv, lm ? (kv_only ? &lm->kv : &lm->qkv) : nullptr, om_qkv, 3 * d - ep.col0, d, ep);
+        e = gemm(R, ln1_in_gemm ? reinterpret_cast<const T *>(x) : a, tm_a, Wqkv, lm ? (kv_only ? &lm->kv : &lm->qkv) : nullptr, om_qkv, 3 * d - ep.col0, d, ep);
         if (!ck("QKV projection")) return RELAYGR_E_CUDA;
         if (preinfer && last) break;
 
@@ -515,12 +522,15 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         e = gemm(M, att, tm_att, (const T *)w.w_o + (size_t)l * d * d, lm ? &lm->ffn.wo : nullptr, *om_xm, d, d, eo);
         if (!ck("output projection")) return RELAYGR_E_CUDA;
 
-        e = layernorm(xm, M, w.ln2_g + (size_t)l * d, w.ln2_b + (size_t)l * d);
+        const float *g2 = w.ln2_g + (size_t)l * d, *b2n = w.ln2_b + (size_t)l * d;
+        const bool ln2_in_gemm = ln_in_gemm(M, (int)F);
+        if (!ln2_in_gemm) e = layernorm(xm, M, g2, b2n);
         if (!ck("LayerNorm 2")) return RELAYGR_E_CUDA;
 
         Epilogue e1{};
+        if (ln2_in_gemm) with_ln(e1, g2, b2n);
         e1.mode = EPI_STORE; e1.silu = 1; e1.bias = w.b1 ? w.b1 + (size_t)l * F : nullptr; e1.out = hid;
-        e = gemm(M, a, tm_a, (const T *)w.w1 + (size_t)l * F * d, lm ? &lm->ffn.w1 : nullptr, om_hid, F, d, e1);
+        e = gemm(M, ln2_in_gemm ? reinterpret_cast<const T *>(xm) : a, tm_a, (const T *)w.w1 + (size_t)l * F * d, lm ? &lm->ffn.w1 : nullptr, om_hid, F, d, e1);
         if (!ck("FFN 1")) return RELAYGR_E_CUDA;
 
         Epilogue e2{};

@@ -89,6 +89,8 @@ struct Epilogue {
     const SeqDesc *seqs;          // per-user descriptors (paged scatter needs row -> user -> page)
     const int32_t *row_off;
     int32_t n_users;
+    const float *ln_g, *ln_b;     // fp32 GEMM on the CUDA cores, where gemm_f32_takes_ln(): A is LN(A; ln_g, ln_b); else nullptr
+    float ln_eps;
 };
 
 // Programmatic dependent launch: a kernel launched with launch_dependent() may start while the kernel before it on

@@ -75,7 +75,9 @@ cudaError_t launch_score(const float *x, int d, const SeqDesc *seqs, int n_users
 
 // ---- CUDA-core GEMM and attention (the fp32 model) ---------------------------------------------
 
-// C[m, n] = sum_k A[m, k] W[n, k], m < M, n < N, then `epi`.  K % 4 == 0, A and W 4-byte aligned (16 is faster).
+// C[m, n] = sum_k A[m, k] W[n, k], m < M, n < N, then `epi`.  K % 4 == 0, A and W 4-byte aligned (16 is faster).  Where
+// gemm_f32_takes_ln() it can take LN(A) instead of A (epi.ln_g, ln_b, ln_eps).
+bool gemm_f32_takes_ln(int64_t M, int N, int K, int n_sms);
 cudaError_t launch_gemm_f32(const float *A, const float *W, int64_t M, int N, int K, const Epilogue &epi, int n_sms, cudaStream_t stream,
                             int64_t *launches);
 
