@@ -134,6 +134,23 @@ f32_gemm_kernel(const float *__restrict__ A, const float *__restrict__ W, int64_
         last_slot[tid] = last;
     }
 
+    // What the epilogue adds, under the loads (small tiles; a tall tile has no registers to spare for it).  x is read and written in
+    // place, so a load left in the store loop waits for the store before it: one trip to L2 per value (the call above: 80 us with
+    // that, 67 without).
+    constexpr bool kEarly = RT == 2;
+    float bias[4], resid[kEarly ? RT : 1][4];
+    if (kEarly && group == 0) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int n = n0 + tx + 16 * j;
+            bias[j] = e.bias && n < N ? e.bias[n] : 0.f;
+#pragma unroll
+            for (int i = 0; i < RT; ++i) {
+                const int64_t m = m0 + ty + 8 * i;
+                if constexpr (kEarly) resid[i][j] = e.mode == EPI_RESID && n < N && m < M ? e.resid[m * N + n] : 0.f;
+            }
+        }
+    }
     if (G > 1 && e.ln_g) {
         static_assert(G == 1 || kThreads * G == 32 * BM, "a warp per row");
         cp_wait<0>();
@@ -195,13 +212,13 @@ f32_gemm_kernel(const float *__restrict__ A, const float *__restrict__ W, int64_
         for (int j = 0; j < 4; ++j) {
             const int n = n0 + tx + 16 * j;
             if (n >= N) continue;
-            float v = sum[i][j] + (e.bias ? e.bias[n] : 0.f);
+            float v = sum[i][j] + (kEarly ? bias[j] : e.bias ? e.bias[n] : 0.f);
             if (e.mode == EPI_STORE) {
                 if (e.silu) v = v / (1.f + expf(-v));
                 reinterpret_cast<float *>(e.out)[m * N + n] = v;
                 continue;
             }
-            if (e.mode == EPI_RESID) { e.out_f32[m * N + n] = e.resid[m * N + n] + v; continue; }
+            if (e.mode == EPI_RESID) { e.out_f32[m * N + n] = (kEarly ? resid[kEarly ? i : 0][j] : e.resid[m * N + n]) + v; continue; }
             const int d = e.d_model, col = e.col0 + n, which = (col >= d) + (col >= 2 * d), c = col - which * d;
             if (which == 0) { reinterpret_cast<float *>(e.q)[m * d + c] = v; continue; }
             if (!to_pages) { reinterpret_cast<float *>(which == 1 ? e.k_lin : e.v_lin)[m * d + c] = v; continue; }
