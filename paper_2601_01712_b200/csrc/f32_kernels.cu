@@ -278,7 +278,7 @@ f32_attention_kernel(const float *__restrict__ q, const float *__restrict__ k_li
     const int tid = threadIdx.x, grp = tid >> 6, gt = tid & 63, ty = gt >> 3, tx = gt & 7;
     float *Qs = smem, *Ks = smem + L::kQ + grp * (L::kK + L::kV), *Vs = Ks + L::kK;
     grid_launch_dependents();
-    grid_dependency_wait();
+    // call metadata, on the device before the call's first kernel ran to its end: three trips to L2, one after the other
     const F32Tile tile = tiles[blockIdx.x / n_heads];
     const int h = blockIdx.x % n_heads, d = n_heads * DH;
     const SeqDesc sd = seqs[tile.seq];
@@ -292,11 +292,13 @@ f32_attention_kernel(const float *__restrict__ q, const float *__restrict__ k_li
     const int n_page_keys = min(sd.n_paged, last_lim), n_lin_keys = max(0, min(sd.n_lin, last_lim - sd.lin_pos0));
     const int n_page_blocks = (n_page_keys + 63) >> 6, n_blocks = n_page_blocks + ((n_lin_keys + 63) >> 6);
     auto group_sync = [&] { asm volatile("bar.sync %0, 64;" ::"r"(1 + grp) : "memory"); };
+    const int page_first = grp < n_page_blocks ? paged.pt[sd.pt_base + grp] : 0;      // of the group's first block
+    grid_dependency_wait();
     int b_pos = 0, b_valid = 0;                         // the current block: position of its first key, number of keys
     auto load_block = [&](int j) {                      // K and V rows; those past the last key are zeros
         const float *k, *v;
         if (j < n_page_blocks) {
-            const int page = paged.pt[sd.pt_base + j];
+            const int page = j == grp ? page_first : paged.pt[sd.pt_base + j];
             const float *slab = reinterpret_cast<const float *>(paged.slab);
             k = slab + page_elem_offset(paged, page, 0, 0);
             v = slab + page_elem_offset(paged, page, 1, 0);
