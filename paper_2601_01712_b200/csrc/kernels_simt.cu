@@ -163,12 +163,15 @@ compact_rows_kernel(const float *__restrict__ x, const T *__restrict__ a, const 
                     const int32_t *__restrict__ score_off, int64_t n_total, int d, float *__restrict__ x_c, T *__restrict__ a_c)
 {
     grid_launch_dependents();
-    grid_dependency_wait();
     const int64_t i = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
+    int64_t src = 0;
+    if (i < n_total) {                                // call metadata, on the device before the call's first kernel ran to its end
+        const int u = find_user(score_off, n_users, (int)i);
+        src = (int64_t)seqs[u].self_row0 + (i - score_off[u]);
+    }
+    grid_dependency_wait();
     if (i >= n_total) return;
-    const int u = find_user(score_off, n_users, (int)i);
-    const int64_t src = (int64_t)seqs[u].self_row0 + (i - score_off[u]);
     const uint4 *xs = reinterpret_cast<const uint4 *>(x + src * d);
     uint4 *xd = reinterpret_cast<uint4 *>(x_c + i * d);
     for (int j = lane; j < d / 4; j += 32) xd[j] = xs[j];
@@ -210,16 +213,16 @@ score_kernel(const float *__restrict__ x, int d, const SeqDesc *__restrict__ seq
              const float *__restrict__ w, const float *__restrict__ bias, float *__restrict__ scores)
 {
     grid_launch_dependents();
-    grid_dependency_wait();
     const int64_t idx0 = ((int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5)) * ROWS;
     const int lane = threadIdx.x & 31;
-    if (idx0 >= n_total) return;
     long long my_row = 0;
-    if (lane < ROWS && idx0 + lane < n_total) {
+    if (lane < ROWS && idx0 + lane < n_total) {       // call metadata, on the device before the call's first kernel ran to its end
         const int idx = (int)(idx0 + lane);
         const int u = find_user(score_off, n_users, idx);
         my_row = (long long)seqs[u].score_row0 + (idx - score_off[u]);
     }
+    grid_dependency_wait();
+    if (idx0 >= n_total) return;
     float4 v[ROWS][NC];
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
