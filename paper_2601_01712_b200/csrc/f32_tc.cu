@@ -269,9 +269,14 @@ f32_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int n = n0 + 32 * h;             // 32 columns lie in one of q, K, V: d_model is a multiple of 32
-                if (n >= N || m0 >= M) continue;
+                if (n >= N || m0 >= M) {               // (past the last column or row: an empty group, for the count below)
+                    if (lane == 0) tc::bulk_commit();
+                    continue;
+                }
                 uint8_t *patch = patches + h * 4096;
-                if (lane == 0) tc::bulk_wait_read<1>();      // the patch's last store but the other's has read it
+                // One bulk group per patch and tile, an empty one where nothing is stored by TMA: with all but the last complete, this
+                // patch's store has read it, and only the other's may be under way.
+                if (lane == 0) tc::bulk_wait_read<1>();
                 __syncwarp();
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
@@ -300,7 +305,7 @@ f32_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                     }
                     continue;
                 }
-                if (lane == 0) tc::bulk_commit();      // (an empty group: the count above stays one per patch)
+                if (lane == 0) tc::bulk_commit();      // (the empty group)
                 const int pj = lane & 7, prow = lane >> 3;
 #pragma unroll 1
                 for (int i = 0; i < 8; ++i) {

@@ -101,6 +101,15 @@ def test_f32_forms(case):
     _check_f32(shape, _tiny_batch(shape, 300 + case, p, s, c), 63)
 
 
+# Widths whose last 64-column tile holds 32 columns or fewer, with so many rows that a CTA goes on from such a tile to another one: the
+# tile's second staging patch is skipped, and the first must not be refilled while its store still reads it.
+@pytest.mark.parametrize("d,heads,ff,n", [(96, 3, 200, 10000), (32, 1, 100, 19200)])
+def test_f32_narrow_last_tile(d, heads, ff, n):
+    shape = synth.ModelShape(2, d, heads, d // heads, ff, 2000, synth.DTYPE_F32)
+    users = n // 200
+    _check_f32(shape, _tiny_batch(shape, 310 + d, [200] * users, [3] * users, [197] * users), 68)
+
+
 def test_f32_weights_off_16_bytes_stay_on_the_cuda_cores():
     """Matrices of weights at no multiple of 16 bytes can have no tensor map: a call of any size takes the other kernels.  (The
     embedding table and the vectors are read 16 bytes at a time in every form, and stay where they are.)"""
