@@ -17,9 +17,10 @@
 //
 // Warp roles (384 threads): warp 0 = TMA producer (a ring of 32 KB stages: Wo in four K blocks, then half a W1 chunk or half a W2
 // chunk per stage, in the order the MMAs consume them; the whole ring is under way before the kernel waits for its predecessor),
-// warp 1 = TMEM owner + MMA issuer, warps 2-3 none, warps 4-11 = LayerNorm, SiLU and exchange (two warps per TMEM quadrant).  TMEM:
-// P, later O, 2 T columns; S double-buffered, T columns each.  The MMA warp issues S(0), S(1), then per chunk O(c) followed
-// by S(c+2): the tensor pipe executes in issue order, so S(c+2) complete also means that H(c) has been read.
+// warp 1 = TMEM owner + MMA issuer, warp 2 none, warp 3 = arrival at the last cluster barrier, warps 4-11 = LayerNorm, SiLU and
+// exchange (two warps per TMEM quadrant).  TMEM: P, later O, 2 T columns; S double-buffered, T columns each.  The MMA warp issues S(0),
+// S(1), then per chunk O(c) followed by S(c+2): the tensor pipe executes in issue order, so S(c+2) complete also means that H(c) has
+// been read.
 #include "ffn_common.cuh"
 #include "kernels.cuh"
 
@@ -408,11 +409,17 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
 #pragma unroll
                 for (int k = 1; k < CS; ++k) { v.x += t[i][h][k].x; v.y += t[i][h][k].y; v.z += t[i][h][k].z; v.w += t[i][h][k].w; }
                 add_twice(own[i][h], v, obias2[h]);
-                asm volatile("" ::"f"(own[i][h].x), "f"(own[i][h].y), "f"(own[i][h].z), "f"(own[i][h].w));      // the peers' memory has been read
             }
     }
     __syncwarp();
-    tc::cluster_arrive_relaxed();                     // (nothing was written for the peers: a release would wait for nothing, 1100 clocks)
+    // The peers must not end before these reads are done, so the arrival has to release them.  A release costs a warp 1100 clocks,
+    // whatever it has to wait for, and the stores below would queue behind it: an idle warp makes it for the epilogue's, which hand their
+    // reads to it through a barrier of the CTA and arrive for themselves without an order (a ranking call of one user: 121.9 us without
+    // any release, 122.6 with this one).
+    if (warp >= 4) asm volatile("bar.arrive 2, %0;" ::"n"(kEpiThreads + 32) : "memory");
+    else if (warp == 3) asm volatile("bar.sync 2, %0;" ::"n"(kEpiThreads + 32) : "memory");
+    if (warp == 3) tc::cluster_arrive_release();
+    else tc::cluster_arrive_relaxed();
     if (finisher && o_ready && !stopped) {
         if (tail.kind != FFN_TAIL_SCORE) {
 #pragma unroll
