@@ -68,14 +68,16 @@ __device__ __forceinline__ void mid_group(uint32_t (&r)[32], const uint64_t (&x)
 }
 
 // The statistics of the whole row from its two halves (the two warps of a quadrant exchange them through `stat`): mean and 1 / std.
-__device__ __forceinline__ void row_stats(const RowStats &st, float2 *stat, int quad, int ch, int rr, float eps, float &mean, float &rstd)
+// ok: this warp's waits so far succeeded; returns whether both warps' did.
+__device__ __forceinline__ bool row_stats(const RowStats &st, float2 *stat, int quad, int ch, int rr, float eps, float &mean, float &rstd, bool ok)
 {
     stat[ch * kRows + rr] = make_float2(st.mean, st.m2);
-    asm volatile("bar.sync %0, 64;" ::"r"(1 + quad) : "memory");      // the two warps that share these 32 rows
+    ok = tc::pair_all(1 + quad, ok);                  // the two warps that share these 32 rows
     const float2 o = stat[(ch ^ 1) * kRows + rr];
     mean = 0.5f * (st.mean + o.x);
     const float diff = st.mean - o.x;
     rstd = rsqrtf((st.m2 + o.y + diff * diff * (0.25f * kD)) * (1.f / kD) + eps);
+    return ok;
 }
 
 // LN(mid) of this thread's half row, from O's columns, as bf16 into the K-major tile sA (rows of 128 bytes per K block).

@@ -342,30 +342,33 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
                 }
             };
             int gc = 0, n = 0;
-            for (int tile = tile0; tile < n_tiles && ok; tile += tile_step, ++n) {
+            // (a wait that ran out ends the loop at row_stats, for both warps of a quadrant: until there nothing more is waited for or stored)
+            for (int tile = tile0; tile < n_tiles; tile += tile_step, ++n) {
                 const bool more = tile + tile_step < n_tiles;
                 // The tile before is drained column group by column group, and mid = x + att Wo^T + bo takes the place of what was
                 // drained: the stores of one group are read while the next group's mid is computed.
-                if (n > 0 && !wait(&bars->o_full, (n - 1) & 1)) break;
-                tc::tc_fence_after();
+                if (ok && n > 0) wait(&bars->o_full, (n - 1) & 1);
                 RowStats st;
+                if (ok) {
+                    tc::tc_fence_after();
 #pragma unroll
-                for (int gi = 0; gi < 4; ++gi) {
-                    if (n > 0) drain(tile - tile_step, gi, patches + (gi & 1) * kPatch, gi > 1);
-                    if (gi == 0) {
-                        if (!wait(&bars->o1_full, n & 1)) break;
-                        tc::tc_fence_after();
+                    for (int gi = 0; gi < 4; ++gi) {
+                        if (n > 0) drain(tile - tile_step, gi, patches + (gi & 1) * kPatch, gi > 1);
+                        if (gi == 0) {
+                            if (!wait(&bars->o1_full, n & 1)) break;
+                            tc::tc_fence_after();
+                        }
+                        const int cc = ch * 128 + gi * 32;
+                        uint32_t r[32];
+                        tc::tmem_ld32(lane_addr + kColS + cc, r);
+                        tc::tmem_ld_wait();
+                        mid_group(r, xp[gi], bos + cc, gi, st);
+                        tc::tmem_st32(lane_addr + kColO + cc, r);
                     }
-                    const int cc = ch * 128 + gi * 32;
-                    uint32_t r[32];
-                    tc::tmem_ld32(lane_addr + kColS + cc, r);
-                    tc::tmem_ld_wait();
-                    mid_group(r, xp[gi], bos + cc, gi, st);
-                    tc::tmem_st32(lane_addr + kColO + cc, r);
                 }
-                if (!ok) break;
                 float mean, rstd;
-                row_stats(st, stat, quad, ch, rr, eps, mean, rstd);
+                ok = row_stats(st, stat, quad, ch, rr, eps, mean, rstd, ok);
+                if (!ok) break;
                 tc::tmem_st_wait();
                 normalise(lane_addr + kColO + ch * 128, gs, bs, mean, rstd, sA, ch, rr);
                 tc::fence_proxy_async();              // generic-proxy writes of the tile before the tensor core reads it
@@ -393,7 +396,6 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
                         take_x(Int<1>());
                     }
                 }
-                if (!ok) break;
                 gc += nc;
             }
             if (ok && n > 0 && wait(&bars->o_full, (n - 1) & 1)) {          // the last tile

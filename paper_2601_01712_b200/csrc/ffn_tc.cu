@@ -281,8 +281,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant
                 tc::tmem_st_wait();
             }
             // O = mid = x + att Wo^T + bo, then LN(mid) into the tile the attention rows came in
-            ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->o1_full, 0, err));
-            if (!ok) break;
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->o1_full, 0, err));      // (if not: out with the partner, at row_stats)
             tc::tc_fence_after();
             RowStats st;
 #pragma unroll 1
@@ -298,7 +297,8 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant
                 tc::tmem_st32(o_cols + gi * 32, r);
             }
             float mean, rstd;
-            row_stats(st, stat, quad, ch, rr, eps, mean, rstd);
+            ok = row_stats(st, stat, quad, ch, rr, eps, mean, rstd, ok);
+            if (!ok) break;
             tc::tmem_st_wait();
             normalise(o_cols, gs, bs, mean, rstd, sA, ch, rr);
             tc::fence_proxy_async();                  // generic-proxy writes of the tile before the tensor core reads it

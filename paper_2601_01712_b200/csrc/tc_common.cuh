@@ -61,6 +61,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, int *e
     return true;
 }
 
+// Named barrier of two warps, behind waits that each of them may have given up: whether neither did.  Both leave their common work on
+// this answer alone - a warp that left on its own account would not come to the next barrier, and the other would wait there for ever.
+__device__ __forceinline__ bool pair_all(int barrier, bool ok)
+{
+    uint32_t all;
+    asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.and.pred q, %2, 64, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+                 : "=r"(all) : "r"((uint32_t)ok), "r"(barrier) : "memory");
+    return all != 0;
+}
+
 // ---- TMA --------------------------------------------------------------------------------------------
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap *m)
 {
