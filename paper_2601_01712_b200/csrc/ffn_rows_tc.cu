@@ -468,6 +468,9 @@ cudaError_t launch_ffn_rows(const FfnMaps &w, float *x, const float *g, const fl
                             const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail, int *err, cudaStream_t stream, bool *taken)
 {
     *taken = false;
+    // This form reads the vectors 16 bytes at a time; the others read them value by value, as they may come at any multiple of 4 bytes.
+    auto aligned = [](const float *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+    if (!aligned(g) || !aligned(b) || !aligned(b2) || !aligned(bo)) return cudaSuccess;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;

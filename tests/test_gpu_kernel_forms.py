@@ -78,6 +78,23 @@ def _check_f32(shape, batch, seed, model_of=None, users=None):
     pool.close(); model.close()
 
 
+def _off_by_four(model, batch, names):
+    """Another slot of the model, the named weights of which start 4 bytes behind a multiple of 16."""
+    from paper_2601_01712_b200 import binding as B
+    weights = B.Weights()
+    for name in B.WEIGHT_FIELDS:
+        t = model._t[name]
+        if name in names:
+            raw = torch.empty(t.numel() + 1, dtype=t.dtype, device=t.device)
+            raw[1:].copy_(t.flatten())
+            model._t[name] = t = raw[1:].view(t.shape)
+        setattr(weights, name, t.data_ptr())
+    model._w = weights
+    other = model.new_slot()
+    other.reserve(int(batch.prefix_off[-1] + batch.short_off[-1] + batch.cand_off[-1]), batch.n_users, 64)
+    return other
+
+
 # fp32 model.  A call runs on the tensor cores from rows x d_model = 49152 on: ranking calls just below and at that, both head
 # widths, widths that are no multiple of the 64-column tiles, users whose rows start inside a group of 32, one user whose key
 # blocks are split over several CTAs (merge), pointwise attention; and calls of a few rows, where the CUDA-core tiles are lowest.
@@ -116,24 +133,30 @@ def test_f32_weights_off_16_bytes_stay_on_the_cuda_cores():
     shape = synth.ModelShape(2, 128, 2, 64, 256, 2000, synth.DTYPE_F32)
     batch = _tiny_batch(shape, 320, [600, 100], [3, 0], [300, 130])
 
-    def off_by_four(model, batch):
-        from paper_2601_01712_b200 import binding as B
-        weights = B.Weights()
-        for name in B.WEIGHT_FIELDS:
-            t = model._t[name]
-            if name not in ("w_qkv", "w_o", "w1", "w2"):
-                setattr(weights, name, t.data_ptr())
-                continue
-            raw = torch.empty(t.numel() + 1, dtype=t.dtype, device=t.device)
-            raw[1:].copy_(t.flatten())
-            model._t[name] = raw[1:].view(t.shape)
-            setattr(weights, name, model._t[name].data_ptr())
-        model._w = weights
-        other = model.new_slot()
-        other.reserve(int(batch.prefix_off[-1] + batch.short_off[-1] + batch.cand_off[-1]), batch.n_users, 64)
-        return other
+    _check_f32(shape, batch, 64, lambda model, batch: _off_by_four(model, batch, ("w_qkv", "w_o", "w1", "w2")))
 
-    _check_f32(shape, batch, 64, off_by_four)
+
+# The bf16 model's vectors that are only ever read value by value may start at any multiple of 4 bytes: with those off 16 bytes, the
+# feed-forward kernel for few rows, which reads them 16 bytes at a time, leaves the call to another form.
+@pytest.mark.parametrize("names", [("ln2_g", "ln2_b", "b_qkv", "b_o", "b1", "b2"), ("ln2_g",), ("ln2_b",), ("b_o",), ("b2",)])
+@pytest.mark.parametrize("ff", [128, 1024])
+def test_vectors_off_16_bytes(names, ff):
+    from paper_2601_01712_b200 import runtime as rt
+    shape = small_bf16_shape(vocab=3000, ff=ff)
+    batch = _tiny_batch(shape, 345, [200, 70], [3, 0], [60, 9])
+    w, model, pool, db = _setup(shape, 69, batch)
+    pool.close()
+    model = _off_by_four(model, batch, names)
+    pool = rt.KvPool(model, 8)
+    for i in range(batch.n_users):
+        pool.alloc(batch.users[i], batch.prefix_off[i + 1] - batch.prefix_off[i])
+    pool.preinfer(db)
+    scores = pool.rank(db).cpu().numpy()
+    assert model.device_status() == 0
+    want = oracle_scores(oracle_model(shape, w), batch)
+    max_bound, _, _ = bf16_noise_bounds(shape, w, batch, want)
+    assert max_abs_err(scores, batch, want) <= max_bound
+    pool.close(); model.close()
 
 
 # Full inference moves the candidates together for the end of the last layer when the other rows cost more than that (here from some
