@@ -160,7 +160,9 @@ WorkspaceLayout Forward::layout(int64_t rows, int64_t users, int64_t pages) cons
     l.partial = take(l.partial_bytes);
     const size_t n_items = (size_t)cfg.n_heads * ((size_t)rows / 128 + (size_t)users + 1) + 2 * (size_t)kMaxSplitTiles;
     // two descriptor arrays and two work lists: all rows, and the candidate rows of the last layer
-    l.meta_bytes = 4 * (((size_t)users + 1) * 5 + 2 * (size_t)users * (sizeof(SeqDesc) / 4) + (size_t)pages + 2 * n_items * (sizeof(AttnItem) / 4) + (size_t)rows / 32 + 1 + (size_t)cfg.n_layers + 64);
+    const size_t page_runs = pages > 0 ? (size_t)rows / 32 + 1 : 0;      // of a pre-infer call; a call without pages (full inference) has none
+    l.meta_bytes = 4 * (((size_t)users + 1) * 5 + 2 * (size_t)users * (sizeof(SeqDesc) / 4) + (size_t)pages + 2 * n_items * (sizeof(AttnItem) / 4) + page_runs +
+                        (size_t)cfg.n_layers + 64);
     l.meta = take(l.meta_bytes);
     l.total = at;
     return l;

@@ -53,6 +53,29 @@ def test_both_attention_kinds_are_accepted():
         B.relaygr_destroy(ctx)
 
 
+@pytest.mark.parametrize("dtype,L,d,H,F", [(B.DTYPE_BF16, 4, 256, 4, 1024), (B.DTYPE_F32, 2, 64, 2, 128)])
+def test_scratch_of_a_call_without_pages(dtype, L, d, H, F):
+    """What full inference needs, term by term: relaygr_rank_full_static accepts a batch by this number, so it must not grow with tables
+    that only calls with pages have."""
+    def up(v):
+        return (v + 1023) // 1024 * 1024
+
+    def need(rows, users):
+        es, r, split_tiles, seq, item = (2 if dtype == B.DTYPE_BF16 else 4), rows + 128, 1536, 13, 8
+        total = 1024 + up(r * d * 4) + 5 * up(r * d * es) + up(r * F * es) + up(r * d * 4) + up(r * d * es)
+        total += up(split_tiles * 128 * (d // H + 4) * 4)
+        items = H * (rows // 128 + users + 1) + 2 * split_tiles
+        return total + up(4 * ((users + 1) * 5 + 2 * users * seq + 2 * items * item + L + 64))
+
+    ctx = B.relaygr_create_host_only(_cfg(dtype, L, d, H, F))
+    rows = next(n for n in range(100_000, 0, -1) if need(n, 3) <= B.STATIC_SCRATCH_BYTES)      # the largest batch of three users that fits
+    for n in (1, 4000, rows - 1, rows, rows + 1):
+        assert B.relaygr_workspace_bytes(ctx, n, 3, 0) == need(n, 3)
+    assert B.relaygr_workspace_bytes(ctx, rows, 3, 0) <= B.STATIC_SCRATCH_BYTES < B.relaygr_workspace_bytes(ctx, rows + 1, 3, 0)
+    assert B.relaygr_workspace_bytes(ctx, rows, 3, 1000) >= need(rows, 3) + 4 * 1000
+    B.relaygr_destroy(ctx)
+
+
 def test_no_cpu_compute_path():
     ctx = B.relaygr_create_host_only(_cfg())
     slab = np.zeros(4 * B.relaygr_kv_page_bytes(ctx) + 1024, dtype=np.uint8)
