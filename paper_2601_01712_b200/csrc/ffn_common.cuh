@@ -126,12 +126,16 @@ __device__ __forceinline__ void silu_chunk(uint32_t s_cols, const float *b1_half
     }
 }
 
-// How many clusters of `cs` CTAs of a kernel with `smem` bytes can be resident at once on the current device (`dev`); asked once.
+// How many clusters of `cs` CTAs of a kernel with `smem` bytes can be resident at once on the current device (`dev`); asked once.  None
+// (a device or a part of one without that many SMs side by side) is an answer, not an error: the caller takes another form.
 template <typename K>
 cudaError_t resident_clusters(K kernel, int cs, size_t smem, PerDeviceValue &known, int dev, int *out)
 {
     *out = known.get(dev);
-    if (*out > 0) return cudaSuccess;
+    if (*out != 0) {
+        *out = *out > 0 ? *out : 0;                   // (-1: none)
+        return cudaSuccess;
+    }
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(cs * 16); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = smem;
@@ -141,8 +145,7 @@ cudaError_t resident_clusters(K kernel, int cs, size_t smem, PerDeviceValue &kno
     cfg.attrs = attr; cfg.numAttrs = 1;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(out, kernel, &cfg);
     if (e != cudaSuccess) return e;
-    if (*out < 1) return cudaErrorLaunchOutOfResources;
-    known.set(dev, *out);
+    known.set(dev, *out > 0 ? *out : -1);
     return cudaSuccess;
 }
 

@@ -1,0 +1,96 @@
+"""Which form of the fused feed-forward kernel a call takes, on the host: the launchers are compiled against stand-ins for the CUDA calls
+they make, so that a device's answers can be chosen and no GPU is needed."""
+import os
+import subprocess
+
+import pytest
+
+from paper_2601_01712_b200 import build
+
+FAKES = r"""
+#pragma once
+#include <cuda_runtime.h>
+extern int fake_resident[17], fake_queries;          // by cluster size
+extern int fake_grid, fake_cluster;                  // of the last launch
+inline cudaError_t fake_device(int *dev) { *dev = 0; return cudaSuccess; }
+template <typename K> cudaError_t fake_attribute(K, cudaFuncAttribute, int) { return cudaSuccess; }
+template <typename K> cudaError_t fake_attributes(cudaFuncAttributes *a, K) { a->numRegs = 168; return cudaSuccess; }
+template <typename K> cudaError_t fake_clusters(int *n, K, const cudaLaunchConfig_t *c)
+{ ++fake_queries; *n = fake_resident[c->attrs[0].val.clusterDim.x]; return cudaSuccess; }
+template <typename... P, typename... A> cudaError_t fake_launch(const cudaLaunchConfig_t *c, void (*)(P...), A &&...)
+{ fake_grid = (int)c->gridDim.x; fake_cluster = c->numAttrs > 1 ? (int)c->attrs[1].val.clusterDim.x : 1; return cudaSuccess; }
+#define cudaGetDevice fake_device
+#define cudaFuncSetAttribute fake_attribute
+#define cudaFuncGetAttributes fake_attributes
+#define cudaOccupancyMaxActiveClusters fake_clusters
+#define cudaLaunchKernelEx fake_launch
+"""
+
+MAIN = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "kernels.cuh"
+using namespace relaygr;
+int fake_resident[17], fake_queries, fake_grid, fake_cluster;
+int main(int argc, char **argv)                      // resident clusters of 8, 4, 2; then rows:d_ff ...
+{
+    fake_resident[8] = atoi(argv[1]); fake_resident[4] = atoi(argv[2]); fake_resident[2] = atoi(argv[3]);
+    FfnMaps w{};
+    CUtensorMap m{};
+    FfnTail tail{};
+    float *aligned = reinterpret_cast<float *>(1024);
+    for (int i = 4; i < argc; ++i) {
+        long rows = 0; int d_ff = 0, off = 0;
+        sscanf(argv[i], "%ld:%d:%d", &rows, &d_ff, &off);
+        const float *p[4] = {aligned, aligned, aligned, aligned};
+        if (off) p[off - 1] += 1;                    // one of the vectors 4 bytes off
+        bool tail_done = false;
+        int64_t launches = 0;
+        fake_grid = fake_cluster = 0;
+        const cudaError_t e = launch_ffn_fused(w, m, aligned, p[0], p[1], aligned, p[2], m, m, p[3], rows, d_ff, 1e-5f, tail, &tail_done, nullptr, 0, &launches);
+        printf("%d %d %d %d\n", (int)e, fake_grid, fake_cluster, (int)tail_done);
+    }
+    printf("%d\n", fake_queries);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def launcher(tmp_path_factory):
+    d = tmp_path_factory.mktemp("ffn")
+    (d / "fakes.h").write_text(FAKES)
+    (d / "main.cu").write_text(MAIN)
+    src = [os.path.join(build.CSRC, f) for f in ("ffn_tc.cu", "ffn_rows_tc.cu", "ffn_pair_tc.cu")]
+    cmd = ["nvcc", "-gencode", "arch=compute_100a,code=compute_100a", "-std=c++17", "--expt-relaxed-constexpr", "-t", "4", "-I", build.INCLUDE, "-I", build.CSRC,
+           "-include", str(d / "fakes.h"), "-o", str(d / "launcher"), str(d / "main.cu"), *src]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+
+    def run(resident, *calls):
+        out = subprocess.run([str(d / "launcher"), *map(str, resident), *calls], capture_output=True, text=True, check=True).stdout.split("\n")
+        return [tuple(map(int, line.split())) for line in out[:len(calls)]], int(out[len(calls)])
+    return run
+
+
+def test_forms_by_rows(launcher):
+    """(error, CTAs, cluster, whether the tail is in the kernel) with a B200's answers: the smallest tile, then the largest cluster, that runs at once."""
+    got, _ = launcher((17, 36, 74), "1:1024", "544:1024", "545:1024", "1152:1024", "1153:1024", "2368:1024", "2369:1024", "4736:1024", "4737:1024", "9472:1024",
+                      "9473:1024", "60000:1024", "100:512", "100:256", "100:128")
+    assert got == [(0, 8, 8, 1), (0, 136, 8, 1), (0, 72, 4, 1), (0, 144, 4, 1), (0, 74, 2, 1), (0, 148, 2, 1), (0, 76, 2, 1), (0, 148, 2, 1), (0, 76, 2, 1), (0, 148, 2, 1),
+                   (0, 76, 2, 0), (0, 148, 2, 0), (0, 16, 4, 1), (0, 8, 2, 1), (0, 2, 2, 0)]
+
+
+def test_a_cluster_size_that_does_not_fit_is_passed_over(launcher):
+    """No clusters of 8 (or of 4 either) side by side: the next form, not an error; the device is asked once."""
+    got, queries = launcher((0, 18, 74), "1:1024", "1:1024", "600:1024")
+    assert got == [(0, 4, 4, 1), (0, 4, 4, 1), (0, 38, 2, 1)] and queries == 3
+    got, queries = launcher((0, 0, 70), "1:1024", "1:1024")
+    assert got == [(0, 2, 2, 1), (0, 2, 2, 1)] and queries == 3
+    got, _ = launcher((0, 0, 0), "1:1024")
+    assert got[0][0] != 0                             # no form at all
+
+
+@pytest.mark.parametrize("off", [1, 2, 3, 4])
+def test_a_vector_off_16_bytes_takes_the_form_that_reads_it_by_value(launcher, off):
+    got, _ = launcher((17, 36, 74), "600:1024:%d" % off)
+    assert got == [(0, 10, 2, 1)]
