@@ -258,6 +258,8 @@ cudaError_t launch_gemm(const float *A, const float *W, int64_t M, int N, int K,
 // bound by it.  S = Q K^T takes two dimensions per fma.rn.f32x2, O += P V two output dimensions (P duplicated in registers),
 // so neither K nor V is transposed and both arrive by cp.async, V under S.  A row belongs to eight lanes of one warp: its maximum
 // and its weights, which overwrite the K tile, need no wider exchange.
+// Registers: tiles of 16 rows with one group come in such numbers that an SM should hold many; heads of 32 fit 128 registers without a
+// spill (1024 users of 8 rows, 8 heads: 496 us a call, 435 so), heads of 64 do not (128 users x 2048 keys: 1025 us, 1252 with 168).
 template <int DH, int RT, int G> struct AttnSmem {
     static constexpr int kLdq = DH + 4, kLdp = 64 + 4;
     static constexpr int kQ = 8 * RT * kLdq;                                              // floats
@@ -268,7 +270,7 @@ template <int DH, int RT, int G> struct AttnSmem {
 };
 
 template <int DH, int RT, int G, bool kPointwise>
-__global__ void __launch_bounds__(64 * G, RT == 8 ? 4 / G : 1)
+__global__ void __launch_bounds__(64 * G, RT == 8 ? 4 / G : G == 1 && DH == 32 ? 8 : 1)
 f32_attention_kernel(const float *__restrict__ q, const float *__restrict__ k_lin, const float *__restrict__ v_lin, PagedKV paged,
                      const SeqDesc *__restrict__ seqs, const F32Tile *__restrict__ tiles, int n_heads, float *__restrict__ out)
 {
@@ -551,30 +553,47 @@ cudaError_t launch_gemm_f32(const float *A, const float *W, int64_t M, int N, in
 
 int build_f32_tiles(const std::vector<SeqDesc> &seqs, int n_heads, int n_sms, std::vector<F32Tile> &tiles)
 {
-    int64_t n64 = 0, n32 = 0;
-    for (const SeqDesc &s : seqs) { n64 += (s.n_q + 63) / 64; n32 += (s.n_q + 31) / 32; }
-    const int rows = tile_rows_for(n64 * n_heads, n32 * n_heads, n_sms);
+    int64_t n64 = 0, n32 = 0, n16 = 0;
+    for (const SeqDesc &s : seqs) { n64 += (s.n_q + 63) / 64; n32 += (s.n_q + 31) / 32; n16 += (s.n_q + 15) / 16; }
+    // ... unless a lower tile leaves so many fewer rows empty that it costs less: a tile's time goes with its height + 16
+    int rows = tile_rows_for(n64 * n_heads, n32 * n_heads, n_sms);
+    if (rows == 64 && n32 * 48 < n64 * 80) rows = 32;
+    if (rows == 32 && n16 * 32 < n32 * 48) rows = 16;
     tiles.clear();
-    for (int u = 0; u < (int)seqs.size(); ++u)
-        for (int q0 = 0; q0 < seqs[(size_t)u].n_q; q0 += rows) tiles.push_back({u, q0});
+    tiles.reserve((size_t)(rows == 64 ? n64 : rows == 32 ? n32 : n16));
     // most keys first: the longest tiles of a causal pass would otherwise start last
     auto keys = [&](const F32Tile &t) {
         const SeqDesc &s = seqs[(size_t)t.seq];
         return std::min(s.causal_end, s.q_pos0 + std::min(s.n_q, t.q0 + rows));
     };
-    std::stable_sort(tiles.begin(), tiles.end(), [&](const F32Tile &a, const F32Tile &b) { return keys(a) > keys(b); });
+    bool in_order = true;
+    int before = INT32_MAX;
+    for (int u = 0; u < (int)seqs.size(); ++u)
+        for (int q0 = 0; q0 < seqs[(size_t)u].n_q; q0 += rows) {
+            const F32Tile t{u, q0};
+            const int k = keys(t);
+            in_order = in_order && k <= before;
+            before = k;
+            tiles.push_back(t);
+        }
+    if (!in_order) std::stable_sort(tiles.begin(), tiles.end(), [&](const F32Tile &a, const F32Tile &b) { return keys(a) > keys(b); });
     return rows;
 }
 
 cudaError_t launch_attention_f32(const float *q, const float *k_lin, const float *v_lin, PagedKV paged, const SeqDesc *seqs,
-                                 const F32Tile *tiles, int n_tiles, int tile_rows, int n_heads, int d_head, int attn_kind, float *out,
+                                 const F32Tile *tiles, int n_tiles, int tile_rows, int n_heads, int d_head, int attn_kind, int n_sms, float *out,
                                  cudaStream_t stream, int64_t *launches)
 {
     if (n_tiles == 0) return cudaSuccess;
     *launches += 1;
+    // 16 rows: the key blocks of a tile go to four groups as long as SMs would be idle otherwise; with three blocks for every SM a tile
+    // takes less of an SM (20 or 38 KB of shared memory instead of 72 or 140) and several run beside each other.  With four groups / one,
+    // 8 rows of 128 users x 2048 keys: 2 heads of 32 (256 blocks) 231 / 318 us a call, 4 heads of 64 (512 blocks) 1103 / 1024.
+    const bool many = (int64_t)n_tiles * n_heads >= 3 * (int64_t)n_sms;
 #define RELAYGR_ATTN(DH)                                                                                                              \
     return tile_rows == 64   ? launch_attention<DH, 8, 2>(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, out, stream) \
            : tile_rows == 32 ? launch_attention<DH, 4, 4>(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, out, stream) \
+           : many            ? launch_attention<DH, 2, 1>(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, out, stream) \
                              : launch_attention<DH, 2, 4>(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, out, stream)
     if (d_head == 32) RELAYGR_ATTN(32);
     if (d_head == 64) RELAYGR_ATTN(64);

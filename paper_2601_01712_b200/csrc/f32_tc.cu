@@ -772,6 +772,17 @@ cudaError_t launch_gemm_f32_tc(const CUtensorMap &tmA, const CUtensorMap &tmW, c
                             tmA, tmW, om, M, N, K, epi, err);
 }
 
+// A tile has 128 rows whoever fills them; with users of a few rows each the CUDA cores' tiles of 16 cost less.  A ranking call on the
+// tensor cores / the CUDA cores in us (width 256, 4 layers, 4 heads): 128 users x 512 keys, 8 rows each 588 / 469, 16 rows 637 / 523, 20
+// rows 674 / 717, 32 rows 742 / 796; x 2048 keys, 16 rows 1218 / 1079, 20 rows 1258 / 1468; 3000 users x 8 keys, 1 row 3356 / 1034.
+// (Heads of 32 gain up to 20 % from 17 to 32 rows too.)
+bool f32_attention_on_tensor_cores(const std::vector<SeqDesc> &seqs)
+{
+    int64_t rows = 0, tiles = 0;
+    for (const SeqDesc &s : seqs) { rows += s.n_q; tiles += (s.n_q + kQRows - 1) / kQRows; }
+    return rows > 16 * tiles;
+}
+
 cudaError_t launch_attention_f32_tc(const float *q, const float *k_lin, const float *v_lin, PagedKV paged, const SeqDesc *seqs, const AttnItem *items,
                                     int n_items, const AttnMerge *merges, int n_merges, int n_heads, int d_head, int attn_kind, float *out,
                                     float *partial, int *err, cudaStream_t stream, int64_t *launches)

@@ -235,11 +235,11 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     // made a launch of its own): worth it when the other rows' share of the linear maps (4 d^2 + 4 d F FLOPs a row at about
     // 0.6 PFLOP/s) costs more than two more launches (10 us) and the copy (12 d bytes a candidate at about 4 TB/s) - full
     // inference with its prefix rows, not a rank call with its few short-term rows.
-    const bool cand_last = !preinfer && n_scores > 0;
+    const bool cand_last = !preinfer && n_scores > 0 && n_scores < R;      // (a call of candidates alone: those are all its rows)
     const bool compact_last = cand_last && (double)(R - n_scores) * (4.0 * d * d + 4.0 * d * F) / 0.6e15 > 10e-6 + (double)n_scores * 12.0 * d / 4e12;
 
     // ---- metadata blob: row_off | seg_off x3 | score_off | SeqDesc[] | page table | attention items [| the same for the last layer]
-    std::vector<int32_t> blob;
+    blob.clear();
     auto put = [&](const int32_t *p, size_t n) { const size_t o = blob.size(); blob.insert(blob.end(), p, p + n); return o; };
     std::vector<int32_t> row_off((size_t)B + 1);
     for (int i = 0; i < B; ++i) row_off[(size_t)i] = call.seqs[(size_t)i].q_row0;
@@ -262,26 +262,31 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         }
         o_runs = put(runs.data(), runs.size());
     }
-    std::vector<AttnItem> items, items_c;
-    std::vector<AttnMerge> merges, merges_c;
     std::vector<SeqDesc> seqs_c;                  // the candidates of each user as rows of their own (last layer)
-    size_t o_items = 0, o_merges = 0, o_seq_c = 0, o_items_c = 0, o_merges_c = 0;
-    // the work of an attention launch over `seqs`: items and merges (tensor cores), or query tiles (CUDA cores)
-    std::vector<F32Tile> tiles, tiles_c;
-    int tile_rows = 0, tile_rows_c = 0;
-    auto put_work = [&](const std::vector<SeqDesc> &seqs, std::vector<AttnItem> &it, std::vector<AttnMerge> &mg, std::vector<F32Tile> &ti,
-                        size_t &o_it, size_t &o_mg, int &rows) {
-        if (kTensor || tensor32) {
+    size_t o_seq_c = 0;
+    // the work of an attention launch over some descriptors: items and merges (tensor cores), or query tiles (CUDA cores)
+    struct AttnWork { bool tensor = false; size_t o_items = 0, o_merges = 0; int n_items = 0, n_merges = 0, tile_rows = 0; };
+    AttnWork work, work_c;
+    auto put_work = [&](const std::vector<SeqDesc> &seqs) {
+        AttnWork wk;
+        wk.tensor = kTensor || (tensor32 && f32_attention_on_tensor_cores(seqs));
+        if (wk.tensor) {
+            std::vector<AttnItem> it;
+            std::vector<AttnMerge> mg;
             build_attention_worklist(seqs, H, kTensor ? attn_machine_bf16(n_sms) : attn_machine_f32(n_sms), kMaxSplitTiles, it, mg);
-            if (!it.empty()) o_it = put(reinterpret_cast<const int32_t *>(it.data()), it.size() * (sizeof(AttnItem) / 4));
-            if (!mg.empty()) o_mg = put(reinterpret_cast<const int32_t *>(mg.data()), mg.size() * (sizeof(AttnMerge) / 4));
+            if (!it.empty()) wk.o_items = put(reinterpret_cast<const int32_t *>(it.data()), it.size() * (sizeof(AttnItem) / 4));
+            if (!mg.empty()) wk.o_merges = put(reinterpret_cast<const int32_t *>(mg.data()), mg.size() * (sizeof(AttnMerge) / 4));
+            wk.n_items = (int)it.size(); wk.n_merges = (int)mg.size();
         } else {
-            rows = build_f32_tiles(seqs, H, n_sms, ti);
-            if (!ti.empty()) o_it = put(reinterpret_cast<const int32_t *>(ti.data()), ti.size() * (sizeof(F32Tile) / 4));
+            std::vector<F32Tile> ti;
+            wk.tile_rows = build_f32_tiles(seqs, H, n_sms, ti);
+            if (!ti.empty()) wk.o_items = put(reinterpret_cast<const int32_t *>(ti.data()), ti.size() * (sizeof(F32Tile) / 4));
+            wk.n_items = (int)ti.size();
         }
+        return wk;
     };
     {
-        put_work(call.seqs, items, merges, tiles, o_items, o_merges, tile_rows);
+        work = put_work(call.seqs);
         if (cand_last) {
             seqs_c = call.seqs;
             for (int u = 0; u < B; ++u) {
@@ -292,7 +297,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
                 c.q_pos0 = c.causal_end;              // every row is a candidate
             }
             o_seq_c = put(reinterpret_cast<const int32_t *>(seqs_c.data()), (size_t)B * (sizeof(SeqDesc) / 4));
-            put_work(seqs_c, items_c, merges_c, tiles_c, o_items_c, o_merges_c, tile_rows_c);
+            work_c = put_work(seqs_c);
         }
     }
     // one item counter per layer's attention launch (the persistent kernel draws its work from it), zeroed by this upload
@@ -407,10 +412,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     float *xm = x;
     const GemmOutMaps *om_xm = &om_x;
     const SeqDesc *seqs_m = d_seqs;
-    const AttnItem *items_m = reinterpret_cast<const AttnItem *>(meta + o_items);
-    const AttnMerge *merges_m = reinterpret_cast<const AttnMerge *>(meta + o_merges);
-    const F32Tile *tiles_m = reinterpret_cast<const F32Tile *>(meta + o_items);
-    int n_items_m = (int)(kTensor || tensor32 ? items.size() : tiles.size()), n_merges_m = (int)merges.size();
+    AttnWork work_m = work;
     bool dead_tail = false;                       // a call without candidates: nothing reads the last layer
     bool ln_done = false, scored = false;         // the fused kernel of the layer before has taken this layer's LayerNorm 1 / the scores
 
@@ -457,10 +459,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
 
         if (last && cand_last) {
             seqs_m = reinterpret_cast<const SeqDesc *>(meta + o_seq_c);
-            items_m = reinterpret_cast<const AttnItem *>(meta + o_items_c);
-            merges_m = reinterpret_cast<const AttnMerge *>(meta + o_merges_c);
-            tiles_m = reinterpret_cast<const F32Tile *>(meta + o_items_c); tile_rows = tile_rows_c;
-            n_items_m = (int)(kTensor || tensor32 ? items_c.size() : tiles_c.size()); n_merges_m = (int)merges_c.size();
+            work_m = work_c;
         }
         if (last && compact_last) {
             // move the candidates' rows of x and of LN1(x) together, then project their queries
@@ -482,15 +481,18 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
 
         {
             cudaEvent_t pe = prof_begin(stream);
+            const AttnItem *items_m = reinterpret_cast<const AttnItem *>(meta + work_m.o_items);
+            const AttnMerge *merges_m = reinterpret_cast<const AttnMerge *>(meta + work_m.o_merges);
             if constexpr (kTensor)
-                e = launch_attention_tc(tm_q, tm_k, tm_v, tm_pool, items_m, n_items_m, merges_m, n_merges_m, seqs_m, meta + o_pt, L,
+                e = launch_attention_tc(tm_q, tm_k, tm_v, tm_pool, items_m, work_m.n_items, merges_m, work_m.n_merges, seqs_m, meta + o_pt, L,
                                         l, d, cfg.attn_kind, call.mode == MODE_RANK, att, reinterpret_cast<float *>(ws + lay.partial),
                                         reinterpret_cast<int *>(ws + lay.meta) + o_ctr + l, n_sms, d_status, stream, &launches);
-            else if (tensor32)
-                e = launch_attention_f32_tc(q, kl, vl, paged, seqs_m, items_m, n_items_m, merges_m, n_merges_m, H, cfg.d_head, cfg.attn_kind, att,
-                                            reinterpret_cast<float *>(ws + lay.partial), d_status, stream, &launches);
+            else if (work_m.tensor)
+                e = launch_attention_f32_tc(q, kl, vl, paged, seqs_m, items_m, work_m.n_items, merges_m, work_m.n_merges, H, cfg.d_head, cfg.attn_kind,
+                                            att, reinterpret_cast<float *>(ws + lay.partial), d_status, stream, &launches);
             else
-                e = launch_attention_f32(q, kl, vl, paged, seqs_m, tiles_m, n_items_m, tile_rows, H, cfg.d_head, cfg.attn_kind, att, stream, &launches);
+                e = launch_attention_f32(q, kl, vl, paged, seqs_m, reinterpret_cast<const F32Tile *>(meta + work_m.o_items), work_m.n_items,
+                                         work_m.tile_rows, H, cfg.d_head, cfg.attn_kind, n_sms, att, stream, &launches);
             prof_end(KC_ATTENTION, pe, stream);
         }
         if (!ck("attention")) return RELAYGR_E_CUDA;

@@ -64,6 +64,7 @@ struct Forward {
         GemmOutMaps om_qkv, om_hid, om_x, om_x_c;
     } act;
 
+    std::vector<int32_t> blob;   // the metadata of a call being built (its memory is kept: thousands of users make half a megabyte)
     // pinned staging ring for the per-call metadata
     static constexpr int kSlots = 4;
     static constexpr size_t kSlotBytes = 2u << 20;

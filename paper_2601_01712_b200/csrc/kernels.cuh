@@ -85,7 +85,7 @@ cudaError_t launch_gemm_f32(const float *A, const float *W, int64_t M, int N, in
 // build_f32_tiles fills the tiles of a call (host) and returns their height, which the launcher takes with them (device).
 int build_f32_tiles(const std::vector<SeqDesc> &seqs, int n_heads, int n_sms, std::vector<F32Tile> &tiles);
 cudaError_t launch_attention_f32(const float *q, const float *k_lin, const float *v_lin, PagedKV paged, const SeqDesc *seqs,
-                                 const F32Tile *tiles, int n_tiles, int tile_rows, int n_heads, int d_head, int attn_kind, float *out,
+                                 const F32Tile *tiles, int n_tiles, int tile_rows, int n_heads, int d_head, int attn_kind, int n_sms, float *out,
                                  cudaStream_t stream, int64_t *launches);
 
 // Where a GEMM's epilogue stores: tensor maps with a 32-row box of 128 bytes and the 128-byte swizzle, in the model's type.
@@ -100,6 +100,7 @@ struct GemmOutMaps { CUtensorMap o[3]; CUtensorMap pool; };
 constexpr int kF32WeightBoxRows = 64;
 cudaError_t launch_gemm_f32_tc(const CUtensorMap &tmA, const CUtensorMap &tmW, const GemmOutMaps &om, int64_t M, int N, int K, const Epilogue &epi,
                                int n_sms, int *err, cudaStream_t stream, int64_t *launches);
+bool f32_attention_on_tensor_cores(const std::vector<SeqDesc> &seqs);
 cudaError_t launch_attention_f32_tc(const float *q, const float *k_lin, const float *v_lin, PagedKV paged, const SeqDesc *seqs, const AttnItem *items,
                                     int n_items, const AttnMerge *merges, int n_merges, int n_heads, int d_head, int attn_kind, float *out,
                                     float *partial, int *err, cudaStream_t stream, int64_t *launches);

@@ -1,0 +1,66 @@
+"""How the fp32 attention of a call is cut into tiles, on the host: the tiles' height follows the rows that fill them."""
+import os
+import subprocess
+
+import pytest
+
+from paper_2601_01712_b200 import build
+
+MAIN = r"""
+#include <algorithm>
+#include <cstdio>
+#include <cstdlib>
+#include "kernels.cuh"
+using namespace relaygr;
+int main(int argc, char **argv)                      // heads, then users of so many rows behind so long a prefix: rows:prefix:count ...
+{
+    std::vector<SeqDesc> seqs;
+    for (int i = 2; i < argc; ++i) {
+        int rows = 0, prefix = 0, count = 1;
+        sscanf(argv[i], "%d:%d:%d", &rows, &prefix, &count);
+        SeqDesc s{};
+        s.n_q = rows; s.q_pos0 = s.n_paged = prefix; s.causal_end = prefix;
+        seqs.insert(seqs.end(), count, s);
+    }
+    std::vector<F32Tile> tiles;
+    const int height = build_f32_tiles(seqs, atoi(argv[1]), 148, tiles);
+    bool in_order = true;
+    int64_t covered = 0;
+    for (size_t i = 0; i < tiles.size(); ++i) {
+        covered += std::min(height, seqs[tiles[i].seq].n_q - tiles[i].q0);
+        if (i && seqs[tiles[i].seq].n_paged > seqs[tiles[i - 1].seq].n_paged) in_order = false;
+    }
+    printf("%d %d %d %d %d\n", (int)f32_attention_on_tensor_cores(seqs), height, (int)tiles.size(), (int)covered, (int)in_order);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def plan(tmp_path_factory):
+    d = tmp_path_factory.mktemp("f32")
+    (d / "main.cu").write_text(MAIN)
+    src = [os.path.join(build.CSRC, f) for f in ("f32_kernels.cu", "f32_tc.cu")]
+    r = subprocess.run(["nvcc", "-gencode", "arch=compute_100a,code=compute_100a", "-std=c++17", "--expt-relaxed-constexpr", "-t", "4", "-I", build.INCLUDE, "-I",
+                        build.CSRC, "-o", str(d / "plan"), str(d / "main.cu"), *src], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return lambda heads, *users: tuple(map(int, subprocess.run([str(d / "plan"), str(heads), *users], capture_output=True, text=True, check=True).stdout.split()))
+
+
+@pytest.mark.parametrize("users,tensor,height,tiles", [
+    (("1:128:1024",), 0, 16, 1024),                  # one row each: no tile of 64, however many blocks there are
+    (("16:8:300",), 0, 16, 300),
+    (("17:8:300",), 1, 32, 300),
+    (("33:8:300",), 1, 64, 300),
+    (("512:2048:30",), 1, 64, 240),
+    (("1:100:150", "40:100:150"), 1, 16, 600),
+    (("3:2000:1",), 0, 16, 1),
+    (("129:64:500",), 1, 64, 1500),
+    (("16:64:500", "0:64:3"), 0, 16, 500),           # users without rows have no tile
+])
+def test_tiles_by_rows(plan, users, tensor, height, tiles):
+    rows = sum(int(u.split(":")[0]) * int(u.split(":")[2]) for u in users)
+    assert plan(4, *users) == (tensor, height, tiles, rows, 1)
+
+
+def test_longest_prefixes_first(plan):
+    assert plan(4, "1:10:50", "1:900:50", "1:64:50")[-1] == 1

@@ -108,6 +108,12 @@ F32 = [
     (128, 2, 260, 1, [900], [1], [400]),                                   # pointwise, d_head 64, split
     (64, 2, 128, 0, [1, 70], [0, 1], [1, 14]),
     (64, 2, 128, 0, [64, 200, 90], [7, 0, 1], [100, 33, 60]),
+    # users of a few rows: attention on the CUDA cores beside tensor-core GEMMs, tiles of 16 rows with one group (from 444 blocks on) and
+    # with four; in the last layer alone; pointwise
+    (256, 4, 512, 0, [1, 63, 64, 65, 200] * 26, [0] * 130, [1, 2, 8, 16, 15] * 26),
+    (256, 8, 512, 0, [1, 63, 64, 65, 200] * 8, [0] * 40, [16, 2, 8, 16, 15] * 8),
+    (256, 8, 512, 0, [70, 64] * 16, [30, 20] * 16, [2, 0] * 16),
+    (256, 8, 512, 1, [1, 63, 64, 65, 200] * 16, [0, 1] * 40, [1, 2, 8, 11, 15] * 16),
 ]
 
 
@@ -115,7 +121,7 @@ F32 = [
 def test_f32_forms(case):
     d, heads, ff, kind, p, s, c = F32[case]
     shape = synth.ModelShape(2, d, heads, d // heads, ff, 2000, synth.DTYPE_F32, attn_kind=kind)
-    _check_f32(shape, _tiny_batch(shape, 300 + case, p, s, c), 63)
+    _check_f32(shape, _tiny_batch(shape, 300 + case, p, s, c), 63, users=None if len(p) < 9 else range(0, len(p), 3))
 
 
 # Widths whose last 64-column tile holds 32 columns or fewer, with so many rows that a CTA goes on from such a tile to another one: the
