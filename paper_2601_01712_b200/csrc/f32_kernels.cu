@@ -8,6 +8,7 @@
 // (two wavefronts for 256 bytes, the minimum) and the two A rows of a warp are broadcasts in distinct banks: per four k a
 // warp spends RT + 8 wavefronts of shared-memory bandwidth on RT * 16 clocks of multiply-adds.
 #include <algorithm>
+#include <type_traits>
 
 #include "kernels.cuh"
 #include "tc_common.cuh"
@@ -408,27 +409,34 @@ f32_attention_kernel(const float *__restrict__ q, const float *__restrict__ k_li
             *reinterpret_cast<float4 *>(P + 32) = make_float4(s[i][4], s[i][5], s[i][6], s[i][7]);
         }
         __syncwarp();                                   // a row's weights come from, and go to, lanes of one warp
+        // kMasked: a key that a row does not see has weight 0 and must not reach it, whatever its V holds (0 x NaN is NaN)
+        auto add_pv = [&](auto kMasked) {
 #pragma unroll 2
-        for (int k = 0; k < 64; k += 4) {
-            float4 p[RT];
+            for (int k = 0; k < 64; k += 4) {
+                float4 p[RT];
 #pragma unroll
-            for (int i = 0; i < RT; ++i) p[i] = *reinterpret_cast<const float4 *>(Ks + (ty + 8 * i) * L::kLdp + k);
+                for (int i = 0; i < RT; ++i) p[i] = *reinterpret_cast<const float4 *>(Ks + (ty + 8 * i) * L::kLdp + k);
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                uint64_t v[CT / 2];
+                for (int kk = 0; kk < 4; ++kk) {
+                    uint64_t v[CT / 2];
 #pragma unroll
-                for (int c = 0; c < CT / 4; ++c) {
-                    const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(Vs + (k + kk) * DH + 4 * tx + 32 * c);
-                    v[2 * c] = w.x; v[2 * c + 1] = w.y;
-                }
+                    for (int c = 0; c < CT / 4; ++c) {
+                        const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(Vs + (k + kk) * DH + 4 * tx + 32 * c);
+                        v[2 * c] = w.x; v[2 * c + 1] = w.y;
+                    }
 #pragma unroll
-                for (int i = 0; i < RT; ++i) {
-                    const uint64_t pp = dup(kk == 0 ? p[i].x : kk == 1 ? p[i].y : kk == 2 ? p[i].z : p[i].w);
+                    for (int i = 0; i < RT; ++i) {
+                        const float pk = kk == 0 ? p[i].x : kk == 1 ? p[i].y : kk == 2 ? p[i].z : p[i].w;
+                        if (decltype(kMasked)::value && pk == 0.f) continue;
+                        const uint64_t pp = dup(pk);
 #pragma unroll
-                    for (int c = 0; c < CT / 2; ++c) o[i][c] = fma2(pp, v[c], o[i][c]);
+                        for (int c = 0; c < CT / 2; ++c) o[i][c] = fma2(pp, v[c], o[i][c]);
+                    }
                 }
             }
-        }
+        };
+        if (mask) add_pv(std::true_type{});
+        else add_pv(std::false_type{});
         group_sync();                                   // P and V have been read
         if (j + G < n_blocks) load_block(j + G);
     }

@@ -351,12 +351,51 @@ constexpr int kAttnSmem = kOffABars + 256 + 1024;
 static_assert(kAttnSmem <= 227 * 1024, "shared memory budget");
 constexpr uint32_t kColS = 0, kSP = 96, kColO = 192, kColQ = 320, kAttnCols = 512;      // S (64) / P (3 x 32) buffers, O buffers (64), Q (3 x 32)
 
+// Edge blocks: those with keys that some row of the tile does not see - at most 5 of the causal diagonal (128 rows against two grids of
+// 64 keys) and 2 of own keys.  Such a key has weight 0, but 0 x NaN is NaN: V that is not finite is replaced by zeros there, noted, and
+// put in at the end for the rows that do see its key.
+constexpr int kEdgeBlocks = 8;
+
 struct AttnBars {
     uint64_t q_full, q_tmem, k_full[2], v_full[2], k_empty[2], v_empty[2], s_full[2], p_full[2], o_full[2];
+    unsigned long long bad_v[kEdgeBlocks];             // per edge block: the keys whose V is not finite
     uint32_t tmem_slot;
-    int abort_flag;
+    int abort_flag, any_bad;
 };
 static_assert(sizeof(AttnBars) <= 256, "barrier block");
+
+// The first edge block of an item: positions grow from block to block, and every row sees the keys at positions < min_lim.
+__device__ __forceinline__ int first_edge_block(const AttnItem &it, const SeqDesc &sd)
+{
+    const int pos0 = sd.q_pos0 + it.q0, min_lim = pos0 >= sd.causal_end ? sd.causal_end : pos0 + 1, n_page_blocks = (sd.n_paged + 63) >> 6;
+    int clean = min(n_page_blocks, min_lim >> 6);
+    if (clean == n_page_blocks) clean += max(0, min_lim - sd.lin_pos0) >> 6;
+    return min(max(clean - it.blk0, 0), it.blk1 - it.blk0);
+}
+// Whether row r of this CTA's tile sees a key of an edge block that is in `bad`.  Not inlined: what it needs would have to outlive the
+// softmax loop in registers.  (With the checks, 8 ranked users of width 256: 1392 -> 1434 us a call, pre-inference of 4: 1492 -> 1468; the
+// compiler schedules the loops differently, there is nothing of them in a block that is no edge.)
+__device__ __noinline__ bool sees_bad_key(const AttnItem *items, const SeqDesc *seqs, const unsigned long long *bad, int r)
+{
+    const AttnItem it = items[blockIdx.x];
+    const SeqDesc sd = seqs[it.seq];
+    const int pos0 = sd.q_pos0 + it.q0, nb_keys = it.blk1 - it.blk0, n_page_blocks = (sd.n_paged + 63) >> 6, first_cand = max(0, sd.causal_end - pos0);
+    const bool is_cand = pos0 + r >= sd.causal_end;
+    const int lim = is_cand ? sd.causal_end : pos0 + r + 1;
+    int j = first_edge_block(it, sd), slot = 0;
+    bool seen = false;
+    auto look = [&](int lo, int hi) {                      // keys lo <= key < hi of the next edge block
+        const unsigned long long b = bad[min(slot++, kEdgeBlocks - 1)];
+        for (int k = max(lo, 0); k < min(hi, 64); ++k) seen = seen || (b >> k & 1) != 0;
+    };
+    for (; j < nb_keys; ++j) {
+        const int blk = it.blk0 + j;
+        look(0, lim - (blk < n_page_blocks ? blk * 64 : sd.lin_pos0 + (blk - n_page_blocks) * 64));
+    }
+    if (it.with_self && first_cand < it.n_q)
+        for (int r0 = first_cand & ~63; r0 < it.n_q; r0 += 64) look(r - r0, is_cand ? r - r0 + 1 : r - r0);
+    return seen;
+}
 
 template <int DH, bool kPointwise>
 __global__ void __launch_bounds__(kAttnThreads, 1)
@@ -372,6 +411,8 @@ f32_attention_tc_kernel(const float *__restrict__ q, const float *__restrict__ k
 
     if (tid == 0) {
         tc::mbar_init(&bars->q_full, kConvThreads / 32); tc::mbar_init(&bars->q_tmem, kSoftThreads / 32);
+        for (int i = 0; i < kEdgeBlocks; ++i) bars->bad_v[i] = 0;
+        bars->any_bad = 0;
         for (int i = 0; i < 2; ++i) {
             tc::mbar_init(&bars->k_full[i], kConvThreads / 32); tc::mbar_init(&bars->v_full[i], kConvThreads / 32);
             tc::mbar_init(&bars->k_empty[i], 1); tc::mbar_init(&bars->v_empty[i], 1);
@@ -516,6 +557,7 @@ f32_attention_tc_kernel(const float *__restrict__ q, const float *__restrict__ k
             store_planes(buffer(0), rk, &bars->k_full[0]);
             if (nb > 1) load_k(1);
         }
+        const int first_edge = first_edge_block(it, sd);
         for (int j = 0; j < nb; ++j) {
             bool ok = true;
             const float *v_next = v_src;                   // of block j + 1, if there is one
@@ -528,6 +570,16 @@ f32_attention_tc_kernel(const float *__restrict__ q, const float *__restrict__ k
             }
             ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->v_empty[j & 1], ((j >> 1) & 1) ^ 1, err));
             if (!ok) break;
+            if (j >= first_edge) {
+#pragma unroll
+                for (int i = 0; i < kPer; ++i) {
+                    const float4 v = rv[i];
+                    if (((v.x - v.x) + (v.y - v.y)) + ((v.z - v.z) + (v.w - v.w)) == 0.f) continue;      // all four finite
+                    bars->any_bad = 1;
+                    atomicOr(&bars->bad_v[min(j - first_edge, kEdgeBlocks - 1)], 1ull << (pr + i * kStep));
+                    rv[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+            }
             store_planes(buffer(j) + 3 * kKVPlane, rv, &bars->v_full[j & 1]);
             if (j + 1 < nb) load_rows(v_next, v_next_rows, rv);
         }
@@ -686,6 +738,7 @@ f32_attention_tc_kernel(const float *__restrict__ q, const float *__restrict__ k
                 if (half == 0) *reinterpret_cast<float4 *>(row) = make_float4(m, l, 0.f, 0.f);
                 dst = row + 4 + half * kOD;
             }
+            if (bars->any_bad != 0 && sees_bad_key(items, seqs, bars->bad_v, r)) inv = __int_as_float(0x7fffffff);
             const uint64_t inv2 = tc::pack2(inv, inv);
 #pragma unroll
             for (int i = 0; i < kOD / 2; i += 2)

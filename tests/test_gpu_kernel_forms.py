@@ -165,6 +165,46 @@ def test_vectors_off_16_bytes(names, ff):
     pool.close(); model.close()
 
 
+# A token whose table row is not a number (row 0 of the table here) reaches whoever sees it and nobody else: not the other candidates of
+# its tile, not the tokens before it in its block of keys.  The forms: tiles of 16, 32 and 64 rows, one group and four, 128-row tiles
+# whole and split over the keys, both head widths, pointwise.
+@pytest.mark.parametrize("d,heads,kind,users,p,s,c", [
+    (64, 2, 0, 2, 100, 7, 20), (64, 1, 1, 12, 100, 33, 20), (96, 3, 0, 4, 150, 70, 200), (256, 4, 0, 1, 1500, 20, 180), (256, 8, 1, 2, 700, 5, 150),
+    (256, 4, 0, 130, 70, 0, 8), (256, 8, 0, 60, 70, 3, 8), (64, 1, 0, 30, 200, 20, 5)])
+def test_f32_values_that_are_no_numbers_stay_where_they_are_seen(d, heads, kind, users, p, s, c):
+    shape = synth.ModelShape(2, d, heads, d // heads, 2 * d, 2000, synth.DTYPE_F32, attn_kind=kind)
+    batch = _tiny_batch(shape, 360 + d + users, [p] * users, [s] * users, [c] * users)
+    for ids in (batch.prefix_ids, batch.short_ids, batch.cand_ids):
+        ids[ids == 0] = 1
+    at = p - 40                                         # user 0: in its prefix; the last user: one of its short-term tokens; every user: a candidate
+    batch.prefix_ids[at] = 0
+    if s > 1:
+        batch.short_ids[-s // 2] = 0
+    batch.cand_ids[c // 2::c] = 0
+    w, model, pool, db = _setup(shape, 70, batch)
+    om = oracle_model(shape, w)
+    keep = model._t["emb"][0].clone()
+    model._t["emb"][0] = float("nan")
+    pool.preinfer(db)
+    scores, full = pool.rank(db).cpu().numpy(), model.rank_full(db).cpu().numpy()
+    for got in (scores, full):
+        for i in sorted({0, 1, users // 2, users - 1} & set(range(users))):
+            g = got[batch.cand_off[i]:batch.cand_off[i + 1]]
+            if i == 0 or (s > 1 and i == users - 1):
+                assert np.all(np.isnan(g))
+                continue
+            assert np.isnan(g[c // 2])
+            others = np.arange(c) != c // 2
+            ps, ss, cs = batch.user_slices(i)
+            assert np.max(np.abs(g[others] - om.full(ps, ss, cs[others]))) <= TOL_F32
+    K, V = om.preinfer(batch.user_slices(0)[0][:at])
+    gK, gV = pool.read_kv(batch.users[0], p)
+    assert np.max(np.abs(gK[:, :at].cpu().numpy() - K)) <= TOL_F32 and np.max(np.abs(gV[:, :at].cpu().numpy() - V)) <= TOL_F32
+    assert bool(torch.all(torch.isnan(gV[1, at:])))
+    model._t["emb"][0] = keep
+    pool.close(); model.close()
+
+
 # Full inference moves the candidates together for the end of the last layer when the other rows cost more than that (here from some
 # 4700 rows on); the ranking calls of the tests above never do.
 @pytest.mark.parametrize("dtype", [synth.DTYPE_BF16, synth.DTYPE_F32])
