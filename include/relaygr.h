@@ -81,7 +81,7 @@ typedef struct relaygr_kv_pool relaygr_kv_pool;
  * Model shape.  d_model = n_heads * d_head.  dtype is the storage type of the
  * embedding table, the matrices, the activations and the K/V pages; vectors
  * are always fp32 and accumulation is always fp32.
- *   F32 : any d_model multiple of 4, d_head in {32, 64}        (CUDA-core kernels)
+ *   F32 : d_head in {32, 64}, d_ff a multiple of 4             (three bf16 parts on tcgen05; few rows: CUDA cores)
  *   BF16: d_head = 64, d_model and d_ff multiples of 128       (tcgen05 kernels)
  * page_tokens must be 64.
  *
@@ -159,7 +159,7 @@ int32_t relaygr_set_workspace(relaygr_ctx *ctx, void *dev, size_t bytes);
  * wait that ran out (RELAYGR_DEVSTATUS_WAIT_TIMEOUT), a token id outside [0, vocab)
  * (RELAYGR_DEVSTATUS_BAD_INDEX; a row that exists is read instead, so no access leaves
  * the table).  The first code stays.  While the word is non-zero the tensor-core
- * kernels of later calls return at once (results undefined, K/V pages not written), so
+ * kernels of later calls store nothing (results undefined, K/V pages not written), so
  * an error cannot pile up.  This call SYNCHRONISES `stream`, then copies the word to
  * *out (0 = healthy).  relaygr_set_workspace clears the word (synchronously).
  */

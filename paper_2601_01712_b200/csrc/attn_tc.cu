@@ -38,17 +38,16 @@ namespace relaygr {
 namespace {
 
 using tc::add2;
+using tc::ex2;
 using tc::fma2;
+using tc::max3;
 using tc::pack2;
 using tc::unpack2;
 
 constexpr int kQTile = 128, kKeys = 64, kDh = 64;
 constexpr int kQBytes = kQTile * kDh * 2;           // 16 KB
 constexpr int kKVBytes = kKeys * kDh * 2;           // 8 KB per K or V tile
-#ifndef RELAYGR_OFFP
-#define RELAYGR_OFFP 4
-#endif
-constexpr int kOffloadPairs = RELAYGR_OFFP;         // of every 16 pairs of exponentials, evenly spread, run on the FMA pipe (exp2_fma_pipe)
+constexpr int kOffloadPairs = 4;                            // of every 16 pairs of exponentials, evenly spread, run on the FMA pipe (exp2_fma_pipe)
 constexpr bool offloaded(int pair) { return (pair + 1) * kOffloadPairs / 16 != pair * kOffloadPairs / 16; }
 constexpr int kStagesKV = 4;
 constexpr int kSmemBytes = kQBytes + 2 * kStagesKV * kKVBytes + 1024 + 512;
@@ -75,12 +74,6 @@ struct Bars {
     int abort_flag;
 };
 
-__device__ __forceinline__ float ex2(float x)
-{
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 // 2^x, x = s * c - mc, for a pair WITHOUT the XU pipe: x is rounded to the nearest integer n by adding 1.5 * 2^23 (n then sits
 // in the low mantissa bits), a cubic gives 2^(x - n) on [-0.5, 0.5] (relative error 7.5e-5, far below the bf16 rounding of P that
 // follows) and n is added to the exponent field as an integer.  x has to lie in [-126, 127]: below, the result is ~1e-38 instead
@@ -113,13 +106,6 @@ __device__ __forceinline__ uint32_t select_eq(int a, int b, uint32_t x, uint32_t
     uint32_t r;
     asm("{\n .reg .pred p;\n setp.eq.s32 p, %1, %2;\n selp.b32 %0, %3, %4, p;\n}\n" : "=r"(r) : "r"(a), "r"(b), "r"(x), "r"(y));
     return r;
-}
-
-__device__ __forceinline__ float max3(float a, float b, float c)
-{
-    float d;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
 }
 
 // The candidates' own keys.  A candidate sees the prefix, the short-term tokens and itself: its own K / V row is not among

@@ -16,6 +16,9 @@ namespace relaygr {
 
 namespace {
 
+using tc::ex2;
+using tc::max3;
+
 // the three parts of a pair, one bf16x2 word each: nine instructions
 __device__ __forceinline__ void split2(uint64_t x, uint32_t (&w)[3])
 {
@@ -38,20 +41,6 @@ __device__ __forceinline__ void split_store(uint8_t *dst, int plane, float4 v)
 
 // 16-byte chunk j of row r in a tile of 128-byte rows with the 128-byte swizzle
 __device__ __forceinline__ uint8_t *chunk_at(uint8_t *tile, int r, int j) { return tile + r * 128 + ((j ^ (r & 7)) << 4); }
-
-__device__ __forceinline__ float max3(float a, float b, float c)
-{
-    float d;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-// 2^x; results below 2^-126 are zero (exp2f scales around that, with the same error otherwise)
-__device__ __forceinline__ float ex2(float x)
-{
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 
 // ---- GEMM: C[m, n] = sum_k A[m, k] W[n, k] ---------------------------------------------------------------------------
 // Persistent CTAs, one per SM, 128 x 64 tiles, 64 columns of K at a time.  Warp 13 loads fp32 by TMA (three stages of 48 KB);

@@ -1,4 +1,5 @@
-// What the two forms of the fused out-proj + feed-forward kernel (ffn_tc.cu, ffn_pair_tc.cu) share: the steps their eight
+// What the forms of the fused out-proj + feed-forward kernel share: sizes and the query for resident clusters (all three: ffn_rows_tc.cu,
+// ffn_tc.cu, ffn_pair_tc.cu), and, for ffn_tc.cu and ffn_pair_tc.cu, the steps their eight
 // epilogue warps take on one row (half) per thread.  Warp (quad, ch) owns TMEM lanes 32 quad .. + 31 and half ch of the columns.
 // The row lives in TMEM and the steps walk it in rolled loops of 32 columns: a kernel of this kind runs a few microseconds per
 // layer, between others that evict its instructions, so code that is executed once per tile costs its fetch from L2 (with
@@ -25,11 +26,6 @@ __device__ __forceinline__ uint4 *patch_chunk(uint8_t *patch, int r, int j)
 }
 
 // 32 bytes of x per lane, one whole sector each (a lane owns a row, so the rows of a warp are 1 KB apart)
-__device__ __forceinline__ void load_x8(const float *p, uint32_t *v)
-{
-    asm volatile("ld.global.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "l"(p) : "memory");
-}
 __device__ __forceinline__ void load_x8(const float *p, uint64_t *v)
 {
     asm volatile("ld.global.L1::no_allocate.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3]) : "l"(p) : "memory");

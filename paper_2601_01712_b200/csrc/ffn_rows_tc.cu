@@ -56,12 +56,6 @@ struct RowBars {
 };
 static_assert(sizeof(RowBars<6>) <= 256, "barrier block");
 
-__device__ __forceinline__ float4 load_cluster4(uint32_t addr)
-{
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-    return v;
-}
 __device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 __device__ __forceinline__ float4 load4_or_zero(const float *p, int c)
 {
@@ -368,7 +362,7 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     obias2[h] = load4_or_zero(b2, c0 + 128 * h);
-                    if (tail.kind != FFN_TAIL_NONE) { tg[h] = load4_or_zero(tail.g, c0 + 128 * h); tb[h] = load4_or_zero(tail.b, c0 + 128 * h); }
+                    tg[h] = load4_or_zero(tail.g, c0 + 128 * h); tb[h] = load4_or_zero(tail.b, c0 + 128 * h);
                     if (tail.kind == FFN_TAIL_SCORE) tw[h] = load4_or_zero(tail.w, c0 + 128 * h);
                 }
                 const int64_t r = tile_row0 + row(j_end + lane);
@@ -399,7 +393,7 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
 #pragma unroll
                 for (int k = 0; k < CS; ++k) {
                     const float *p = turn + row(j_end + i) * kD + c0 + 128 * h;
-                    t[i][h][k] = k == 0 ? *reinterpret_cast<const float4 *>(p) : load_cluster4(tc::cluster_addr(p, (rank + k) & (CS - 1)));
+                    t[i][h][k] = k == 0 ? *reinterpret_cast<const float4 *>(p) : tc::load_cluster4(tc::cluster_addr(p, (rank + k) & (CS - 1)));
                 }
 #pragma unroll
         for (int i = 0; i < kEnd; ++i)
@@ -430,28 +424,26 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
                     for (int h = 0; h < 2; ++h) *reinterpret_cast<float4 *>(x + r * kD + c0 + 128 * h) = own[i][h];
             }
         }
-        if (tail.kind != FFN_TAIL_NONE) {
-            float mean[kEnd], rstd[kEnd];
-            rows_stats<kEnd>(own, eps, mean, rstd);
+        float mean[kEnd], rstd[kEnd];
+        rows_stats<kEnd>(own, eps, mean, rstd);
 #pragma unroll
-            for (int i = 0; i < kEnd; ++i) {
-                const int64_t r = tile_row0 + row(j_end + i);
-                float acc = 0.f;
+        for (int i = 0; i < kEnd; ++i) {
+            const int64_t r = tile_row0 + row(j_end + i);
+            float acc = 0.f;
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const float4 y = normalised(own[i][h], mean[i], rstd[i], tg[h], tb[h]);
-                    if (tail.kind == FFN_TAIL_LN) {
-                        if (r < M) *reinterpret_cast<uint2 *>(tail.a + r * kD + c0 + 128 * h) = make_uint2(tc::pack_bf16(y.x, y.y), tc::pack_bf16(y.z, y.w));
-                    } else {
-                        acc += y.x * tw[h].x + y.y * tw[h].y + y.z * tw[h].z + y.w * tw[h].w;
-                    }
+            for (int h = 0; h < 2; ++h) {
+                const float4 y = normalised(own[i][h], mean[i], rstd[i], tg[h], tb[h]);
+                if (tail.kind == FFN_TAIL_LN) {
+                    if (r < M) *reinterpret_cast<uint2 *>(tail.a + r * kD + c0 + 128 * h) = make_uint2(tc::pack_bf16(y.x, y.y), tc::pack_bf16(y.z, y.w));
+                } else {
+                    acc += y.x * tw[h].x + y.y * tw[h].y + y.z * tw[h].z + y.w * tw[h].w;
                 }
-                if (tail.kind == FFN_TAIL_SCORE) {
+            }
+            if (tail.kind == FFN_TAIL_SCORE) {
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                    const int at = __shfl_sync(0xffffffffu, score_at, i);
-                    if (lane == 0 && at >= 0) tail.scores[at] = acc + (tail.bias ? tail.bias[0] : 0.f);
-                }
+                for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                const int at = __shfl_sync(0xffffffffu, score_at, i);
+                if (lane == 0 && at >= 0) tail.scores[at] = acc + (tail.bias ? tail.bias[0] : 0.f);
             }
         }
     }

@@ -56,13 +56,6 @@ __device__ __forceinline__ float warp_sum(float v)
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
-__device__ __forceinline__ float4 load_cluster4(uint32_t addr)
-{
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-    return v;
-}
-
 constexpr int CS = 2;                                 // CTAs per tile
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -316,17 +309,15 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant
             if (!ok) break;
 
             // what the end of the block needs, while O is on its way
-            if (tail.kind != FFN_TAIL_NONE) {
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    tg[h] = *reinterpret_cast<const float4 *>(tail.g + c0 + 128 * h); tb[h] = *reinterpret_cast<const float4 *>(tail.b + c0 + 128 * h);
-                    if (tail.kind == FFN_TAIL_SCORE) tw[h] = *reinterpret_cast<const float4 *>(tail.w + c0 + 128 * h);
-                }
-                const int64_t row = (int64_t)tile * kRows + row_first + lane;
-                if (tail.kind == FFN_TAIL_SCORE && lane < kRowsPerWarp && row < M) {
-                    const int u = find_user(tail.row_off, tail.n_users, (int)row), i = (int)row - tail.seqs[u].score_row0;
-                    if (i >= 0 && i < tail.seqs[u].n_score) score_at = tail.score_off[u] + i;
-                }
+            for (int h = 0; h < 2; ++h) {
+                tg[h] = *reinterpret_cast<const float4 *>(tail.g + c0 + 128 * h); tb[h] = *reinterpret_cast<const float4 *>(tail.b + c0 + 128 * h);
+                if (tail.kind == FFN_TAIL_SCORE) tw[h] = *reinterpret_cast<const float4 *>(tail.w + c0 + 128 * h);
+            }
+            const int64_t end_row = (int64_t)tile * kRows + row_first + lane;
+            if (tail.kind == FFN_TAIL_SCORE && lane < kRowsPerWarp && end_row < M) {
+                const int u = find_user(tail.row_off, tail.n_users, (int)end_row), i = (int)end_row - tail.seqs[u].score_row0;
+                if (i >= 0 && i < tail.seqs[u].n_score) score_at = tail.score_off[u] + i;
             }
             ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->o_full, 0, err));
             if (!ok) break;
@@ -361,7 +352,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
 #pragma unroll
-                    for (int k = 0; k < CS; ++k) t[i][h][k] = load_cluster4(tc::cluster_addr(src + h * (4 * 4096), k));
+                    for (int k = 0; k < CS; ++k) t[i][h][k] = tc::load_cluster4(tc::cluster_addr(src + h * (4 * 4096), k));
             }
 #pragma unroll
             for (int i = 0; i < kBatch; ++i) {
@@ -381,7 +372,6 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant
 #pragma unroll
                     for (int h = 0; h < 2; ++h) *reinterpret_cast<float4 *>(x + row * kD + c0 + 128 * h) = v[h];
                 }
-                if (tail.kind == FFN_TAIL_NONE) continue;
                 const float mean = warp_sum(sum) * (1.f / kD);
                 float sq = 0.f;
 #pragma unroll

@@ -9,10 +9,13 @@
 namespace relaygr {
 
 namespace {
-// Whether a call of the fp32 model runs on the tensor cores or on the CUDA cores: by the values of an activation tensor.  The
-// tensor-core kernels have the longer start-up (tile loads, splits, turning accumulators around) and 128-row tiles where those have
-// 16-row ones.  Measured, a call on the CUDA cores / the tensor cores in us: rank, 384 rows x 64 columns 93 / 110, 768 x 64 117 / 110,
-// 1536 x 64 134 / 114, 100 x 256 1015 / 605; pre-infer, 700 x 64 62 / 69, 1400 x 64 79 / 75, 700 x 256 1307 / 575.
+// Whether a call of the fp32 model runs on the tensor cores or on the CUDA cores (its attention: f32_attention_on_tensor_cores as
+// well): by the values of an activation tensor.  The tensor-core kernels have the longer start-up (tile loads, splits, turning
+// accumulators around) and 128-row tiles where those have 16-row ones.  Measured, a call with its GEMMs on the CUDA cores / the tensor cores
+// in us (attention alike): width 128, 200 rows 189 / 250, 400 rows 267 / 255; width 256, 100 rows 241 / 303, 200 rows 371 / 307; width
+// 512, 64 rows 373 / 409, 100 rows 581 / 425; width 1024, 32 rows 304 / 306, 64 rows 502 / 307.  The line does not fit everywhere: at width
+// 64 the GEMMs gain only from some 2500 rows on (1600 rows 120 / 134, 4096 rows 192 / 125), and a few rows over a long
+// prefix would rank faster with their attention alone on the tensor cores (100 rows of width 256 over 2048 keys: 374 us, 241 so).
 constexpr int64_t kF32TensorValues = 49152;
 inline bool f32_on_tensor_cores(int64_t rows, int d) { return rows * d >= kF32TensorValues; }
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -234,7 +237,8 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     // their rows alone.  What follows may run on them alone too, once they have been moved together (and their query projection
     // made a launch of its own): worth it when the other rows' share of the linear maps (4 d^2 + 4 d F FLOPs a row at about
     // 0.6 PFLOP/s) costs more than two more launches (10 us) and the copy (12 d bytes a candidate at about 4 TB/s) - full
-    // inference with its prefix rows, not a rank call with its few short-term rows.
+    // inference with its prefix rows, not a rank call with its few short-term rows.  (The rate is the bf16 model's.  The fp32 GEMMs do
+    // about an eighth of it, so that an fp32 call moves its candidates together later than would pay.)
     const bool cand_last = !preinfer && n_scores > 0 && n_scores < R;      // (a call of candidates alone: those are all its rows)
     const bool compact_last = cand_last && (double)(R - n_scores) * (4.0 * d * d + 4.0 * d * F) / 0.6e15 > 10e-6 + (double)n_scores * 12.0 * d / 4e12;
 

@@ -132,9 +132,8 @@ struct FfnMaps {                                  // one layer's weights, boxes 
     CUtensorMap w1, w1_half;                      // W1 [d_ff, 256], boxes of 128 and of 64 rows
     CUtensorMap w2, w2_wide, wo, wo_wide;         // W2 [256, d_ff] and Wo [256, 256], boxes of 128 and (wide) of 256 rows
 };
-// What the kernel does with finished rows beside storing them to x: nothing; the next layer's a = LN(x; g, b); or, instead of storing
-// them, the scores of the candidates' rows, w . LN(x; g, b) + bias (users by row_off and seqs, as in launch_score).
-enum FfnTailKind : int { FFN_TAIL_NONE = 0, FFN_TAIL_LN, FFN_TAIL_SCORE };
+// What the kernel does with finished rows: stores them to x and the next layer's a = LN(x; g, b); or, instead of storing them, the scores of the candidates' rows, w . LN(x; g, b) + bias (users by row_off and seqs, as in launch_score).
+enum FfnTailKind : int { FFN_TAIL_LN = 0, FFN_TAIL_SCORE };
 struct FfnTail {
     int kind;
     const float *g, *b;
