@@ -1,0 +1,351 @@
+// The fp32 model with few rows and matrices that fit an SM: a call is two launches a layer instead of five.
+//     first:  x = E[id],  then what `tail` says with LN(x)
+//     block:  everything after a layer's attention, x <- mid + W2 SiLU(W1 LN(mid) + b1) + b2, mid = x + Wo att + bo, then `tail`
+// where the tail is the next layer's LayerNorm and QKV projection (into q and the call's K / V rows, or the users' pages), or the final
+// LayerNorm and the scoring head.
+// What bounds it: the launch chain.  A launch of such a call costs the host 4-5 us and the GPU 4-6 us whatever it computes, and all the
+// products of a layer of width 64 are 2 us of one SM's FMA pipes for four rows.  So a block takes four rows (eight where there are
+// more than four for every SM) through all of them, with every matrix of the layer in its shared memory, requested before the wait for the
+// attention.  Four rows of width 64: 206 KB of matrices are read from shared memory once (1600 clocks), the rows are broadcast
+// reads (800), the multiply-adds take 1540.  The 2-layer model of width 64, four users of 96 rows over 256 keys: 66 us a call with five
+// launches a layer, 44 so, of which the host's part is now 44.
+#include <algorithm>
+
+#include "kernels.cuh"
+#include "tc_common.cuh"
+
+namespace relaygr {
+
+namespace {
+
+constexpr int kThreads = 512;
+
+using tc::fma2;
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ float warp_sum(float v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Floats of shared memory.  Rows are 4 words longer than a multiple of 32: see dot().
+struct Layout {
+    int wo, w1, w2, wt, rows, total;                  // wt: the tail's matrix; rows: att / a, x / mid [d] and hidden values [F] of the block's rows
+};
+__host__ __device__ inline Layout layout_of(int d, int F, int tail_n, bool first, int BR)
+{
+    Layout l{};
+    int at = 0;
+    l.wo = at; at += first ? 0 : d * (d + 4);
+    l.w1 = at; at += first ? 0 : F * (d + 4);
+    l.w2 = at; at += first ? 0 : d * (F + 4);
+    l.wt = at; at += tail_n * (d + 4);
+    l.rows = at; at += BR * (2 * (d + 4) + (first ? 0 : F + 4));
+    l.total = at;
+    return l;
+}
+
+__device__ __forceinline__ void load_matrix(float *dst, const float *W, int n, int k)      // [n, k] row by row
+{
+    const int per_row = k / 4;
+    for (int i = threadIdx.x; i < n * per_row; i += kThreads) {
+        const int r = i / per_row, c = (i - r * per_row) * 4;
+        cp_async16(dst + r * (k + 4) + c, W + (size_t)r * k + c);
+    }
+}
+
+// sum[i][q] = sum_k a[4 q + (lane & 3)][k] W[n + i step][k] in the lanes that share (n, lane & 3): LANES lanes to an output take eight of
+// every 8 LANES columns each, all BR rows at a time, and are added up by a transposing butterfly.  A quarter of a warp reads
+// 16 bytes a lane from 32 distinct banks: 8 / LANES outputs whose rows lie 4 banks apart, LANES pieces 8 apart (with eight lanes the
+// upper four start with their second four columns).  n < n_end, K a multiple of 32.
+template <int BR, int NI, int LANES>
+__device__ __forceinline__ void dot(float (&sum)[NI][BR / 4], const float *W, int n, int step, int n_end, int K, const float *a, int lda)
+{
+    const int lane = threadIdx.x & 31, ks = lane & (LANES - 1), flip = LANES == 8 ? (ks & 4) : 0;
+    uint64_t acc[NI][BR] = {};
+    const float *w = W + (size_t)min(n, n_end - 1) * (K + 4);
+    const size_t w_step = (size_t)step * (K + 4);
+    const bool second = NI > 1 && n + step < n_end;
+    for (int k = ks * 8; k < K; k += 8 * LANES) {
+        ulonglong2 wv[NI][2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            wv[0][h] = *reinterpret_cast<const ulonglong2 *>(w + k + ((4 * h) ^ flip));
+            if (NI > 1) wv[NI - 1][h] = second ? *reinterpret_cast<const ulonglong2 *>(w + w_step + k + ((4 * h) ^ flip)) : make_ulonglong2(0, 0);
+        }
+#pragma unroll
+        for (int r = 0; r < BR; ++r)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const ulonglong2 av = *reinterpret_cast<const ulonglong2 *>(a + r * lda + k + ((4 * h) ^ flip));
+#pragma unroll
+                for (int i = 0; i < NI; ++i) acc[i][r] = fma2(av.y, wv[i][h].y, fma2(av.x, wv[i][h].x, acc[i][r]));
+            }
+    }
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+#pragma unroll
+        for (int q = 0; q < BR / 4; ++q) {
+            float v[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                float lo, hi;
+                tc::unpack2(acc[i][4 * q + r], lo, hi);
+                v[r] = lo + hi;
+                if (LANES == 8) v[r] += __shfl_xor_sync(0xffffffffu, v[r], 4);
+            }
+            const bool up = lane & 2, odd = lane & 1;
+            const float t0 = (up ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, up ? v[0] : v[2], 2);
+            const float t1 = (up ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, up ? v[1] : v[3], 2);
+            sum[i][q] = (odd ? t1 : t0) + __shfl_xor_sync(0xffffffffu, odd ? t0 : t1, 1);
+        }
+}
+
+// LayerNorm of a row in a warp's lanes (columns lane and lane + 32), biased variance
+__device__ __forceinline__ void ln_row(float (&v)[2], int d, float eps, const float (&g)[2], const float (&b)[2])
+{
+    const int lane = threadIdx.x & 31;
+    const float inv_d = 1.f / (float)d;
+    const bool in0 = lane < d, in1 = lane + 32 < d;
+    const float mean = warp_sum((in0 ? v[0] : 0.f) + (in1 ? v[1] : 0.f)) * inv_d;
+    const float c0 = in0 ? v[0] - mean : 0.f, c1 = in1 ? v[1] - mean : 0.f;
+    const float rstd = rsqrtf(warp_sum(c0 * c0 + c1 * c1) * inv_d + eps);
+    v[0] = in0 ? c0 * rstd * g[0] + b[0] : 0.f;
+    v[1] = in1 ? c1 * rstd * g[1] + b[1] : 0.f;
+}
+__device__ __forceinline__ void load_row2(float (&v)[2], const float *p, int d)
+{
+    const int lane = threadIdx.x & 31;
+    v[0] = lane < d ? p[lane] : 0.f;
+    v[1] = lane + 32 < d ? p[lane + 32] : 0.f;
+}
+
+template <int BR, bool kFirst>
+__global__ void __launch_bounds__(kThreads, 1)
+f32_block_kernel(F32First first, F32BlockWeights wt, F32BlockTail tail, float *__restrict__ x, const float *__restrict__ att, int64_t M, int d, int F, float eps,
+                 int *err)
+{
+    extern __shared__ __align__(16) float smem[];
+    __shared__ int64_t page_off[BR];
+    __shared__ int last_slot[BR];
+    const Layout L = layout_of(d, F, tail.kind == F32_TAIL_QKV ? tail.n : 0, kFirst, BR);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t m0 = (int64_t)blockIdx.x * BR;
+    const int lda = d + 4, ldh = F + 4;
+    float *a_s = smem + L.rows, *x_s = a_s + BR * lda, *h_s = x_s + BR * lda;
+
+    // parameters, requested while the kernel before is still running
+    if (!kFirst) {
+        grid_launch_dependents();
+        load_matrix(smem + L.wo, wt.wo, d, d);
+        load_matrix(smem + L.w1, wt.w1, F, d);
+        load_matrix(smem + L.w2, wt.w2, d, F);
+    }
+    if (tail.kind == F32_TAIL_QKV) load_matrix(smem + L.wt, tail.w, tail.n, d);
+    const int slot8 = warp * 4 + (lane >> 3), slot4 = warp * 8 + (lane >> 2), rq = lane & 3;      // output of eight / four lanes; row of a group of four
+    float g2[2] = {0.f, 0.f}, b2n[2] = {0.f, 0.f}, gt[2] = {0.f, 0.f}, bt[2] = {0.f, 0.f}, ws[2] = {0.f, 0.f};
+    if (warp < BR) {
+        if (!kFirst) { load_row2(g2, wt.ln_g, d); load_row2(b2n, wt.ln_b, d); }
+        if (tail.kind != F32_TAIL_NONE) { load_row2(gt, tail.g, d); load_row2(bt, tail.b, d); }
+        if (tail.kind == F32_TAIL_SCORE) load_row2(ws, tail.w, d);
+    }
+    const float bo = !kFirst && wt.bo && slot8 < d ? wt.bo[slot8] : 0.f, b2 = !kFirst && wt.b2 && slot8 < d ? wt.b2[slot8] : 0.f;
+    const float score_bias = tail.kind == F32_TAIL_SCORE && tail.bias ? tail.bias[0] : 0.f;
+    // Where the rows' results go: call metadata, on the device before the call's first kernel ran to its end
+    const bool paged = tail.kind == F32_TAIL_QKV && tail.e.paged.slab != nullptr;
+    const int64_t row = m0 + warp;                    // of a warp that takes LayerNorms
+    const bool has_row = warp < BR && row < M;
+    int score_at = -1;
+    auto look_up = [&] {
+        if (paged && tid >= 480 && tid < 480 + BR) {  // K / V rows in pages; of a user's last row, its slot
+            const int r = tid - 480;
+            int64_t off = 0;
+            int last = -1;
+            if (m0 + r < M) {
+                const int u = find_user(tail.e.row_off, tail.e.n_users, (int)(m0 + r));
+                const int t = (int)(m0 + r) - tail.e.row_off[u];
+                off = (int64_t)page_elem_offset(tail.e.paged, tail.e.paged.pt[tail.e.seqs[u].pt_base + (t >> 6)], 0, t & 63);
+                if (t == tail.e.seqs[u].n_q - 1) last = t & 63;
+            }
+            page_off[r] = off;
+            last_slot[r] = last;
+        }
+        if (tail.kind == F32_TAIL_SCORE && has_row) {
+            const int u = find_user(tail.e.row_off, tail.e.n_users, (int)row);
+            const int i = (int)row - tail.e.seqs[u].score_row0;
+            if (i >= 0 && i < tail.e.seqs[u].n_score) score_at = tail.score_off[u] + i;
+        }
+    };
+    // The first kernel of a call lets the next one start only after its own wait: see gather_ln_kernel.
+    if (!kFirst) look_up();
+    grid_dependency_wait();
+    if (kFirst) {
+        grid_launch_dependents();
+        look_up();
+    }
+
+    float v[2];                                       // a row's values, in the warps that take the LayerNorms
+    if constexpr (kFirst) {
+        if (warp < BR) {
+            long long id = 0;
+            if (has_row && lane == 0) {
+                id = row_token_id(first.src, row);
+                if (id < 0 || id >= first.vocab) {
+                    // an id outside the table: recorded in the status word, and a row that exists is read instead
+                    if (err) atomicCAS(err, (int)STATUS_OK, (int)STATUS_BAD_INDEX);
+                    id = id < 0 ? 0 : first.vocab - 1;
+                }
+            }
+            id = __shfl_sync(0xffffffffu, id, 0);
+            load_row2(v, first.emb + id * d, has_row ? d : 0);
+            if (has_row && lane < d) x[row * d + lane] = v[0];
+            if (has_row && lane + 32 < d) x[row * d + lane + 32] = v[1];
+        }
+    } else {
+        for (int i = tid; i < 2 * BR * (d / 4); i += kThreads) {
+            const int r = i / (d / 4), c = (i - r * (d / 4)) * 4, rr = r < BR ? r : r - BR;
+            float4 val = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (m0 + rr < M) val = *reinterpret_cast<const float4 *>((r < BR ? att : x) + (m0 + rr) * d + c);
+            *reinterpret_cast<float4 *>((r < BR ? a_s : x_s) + rr * lda + c) = val;
+        }
+        cp_async_wait();
+        __syncthreads();
+        {                                             // mid = x + Wo att + bo
+            float s[1][BR / 4];
+            dot<BR, 1, 8>(s, smem + L.wo, slot8, 0, d, d, a_s, lda);
+            if (slot8 < d && (lane & 4) == 0)
+#pragma unroll
+                for (int q = 0; q < BR / 4; ++q) x_s[(4 * q + rq) * lda + slot8] += s[0][q] + bo;
+        }
+        __syncthreads();
+        if (warp < BR) {
+            load_row2(v, x_s + warp * lda, d);
+            ln_row(v, d, eps, g2, b2n);
+            if (lane < d) a_s[warp * lda + lane] = v[0];
+            if (lane + 32 < d) a_s[warp * lda + lane + 32] = v[1];
+        }
+        __syncthreads();
+        for (int n = slot4; n - slot4 < F; n += 256) {      // hidden values (all lanes of a warp go round together)
+            float s[2][BR / 4];
+            dot<BR, 2, 4>(s, smem + L.w1, n, 128, F, d, a_s, lda);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int nn = n + 128 * i;
+                if (nn >= F) continue;
+                const float bias = wt.b1 ? wt.b1[nn] : 0.f;
+#pragma unroll
+                for (int q = 0; q < BR / 4; ++q) {
+                    const float z = s[i][q] + bias;
+                    h_s[(4 * q + rq) * ldh + nn] = z / (1.f + expf(-z));
+                }
+            }
+        }
+        __syncthreads();
+        {                                             // x = mid + W2 h + b2
+            float s[1][BR / 4];
+            dot<BR, 1, 8>(s, smem + L.w2, slot8, 0, d, F, h_s, ldh);
+            if (slot8 < d && (lane & 4) == 0)
+#pragma unroll
+                for (int q = 0; q < BR / 4; ++q) {
+                    const int r = 4 * q + rq;
+                    const float val = x_s[r * lda + slot8] + (s[0][q] + b2);
+                    x_s[r * lda + slot8] = val;
+                    if (tail.kind == F32_TAIL_QKV && m0 + r < M) x[(m0 + r) * d + slot8] = val;
+                }
+        }
+        if (tail.kind == F32_TAIL_NONE) return;
+        __syncthreads();
+        if (warp < BR) load_row2(v, x_s + warp * lda, d);
+    }
+    if (warp < BR) ln_row(v, d, eps, gt, bt);
+    if (tail.kind == F32_TAIL_SCORE) {
+        const float s = warp_sum(v[0] * ws[0] + v[1] * ws[1]);
+        if (score_at >= 0 && lane == 0) tail.scores[score_at] = s + score_bias;
+        return;
+    }
+    if (warp < BR) {
+        if (lane < d) a_s[warp * lda + lane] = v[0];
+        if (lane + 32 < d) a_s[warp * lda + lane + 32] = v[1];
+    }
+    if (kFirst) cp_async_wait();
+    __syncthreads();
+    const Epilogue &e = tail.e;
+    for (int n = slot4; n - slot4 < tail.n; n += 256) {
+        float s[2][BR / 4];
+        dot<BR, 2, 4>(s, smem + L.wt, n, 128, tail.n, d, a_s, lda);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int nn = n + 128 * i;
+            if (nn >= tail.n) continue;
+            const float bias = tail.bias ? tail.bias[nn] : 0.f;
+            const int col = e.col0 + nn, which = (col >= d) + (col >= 2 * d), c = col - which * d;
+#pragma unroll
+            for (int q = 0; q < BR / 4; ++q) {
+                const int r = 4 * q + rq;
+                const int64_t m = m0 + r;
+                if (m >= M) continue;
+                const float val = s[i][q] + bias;
+                if (which == 0 || !paged) {
+                    reinterpret_cast<float *>(which == 0 ? e.q : which == 1 ? e.k_lin : e.v_lin)[m * d + c] = val;
+                    continue;
+                }
+                float *p = reinterpret_cast<float *>(e.paged.slab) + page_off[r] + (int64_t)(which - 1) * 64 * d + c;
+                *p = val;
+                if (last_slot[r] >= 0)                // last row of the prefix: clear the unused slots of its page
+                    for (int z = 1; last_slot[r] + z < 64; ++z) p[(int64_t)z * d] = 0.f;
+            }
+        }
+    }
+}
+
+template <int BR, bool kFirst>
+cudaError_t launch(const F32First &first, const F32BlockWeights &wt, const F32BlockTail &tail, float *x, const float *att, int64_t M, int d, int F, float eps, int *err,
+                   cudaStream_t stream)
+{
+    static PerDeviceValue attr_set;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (!attr_set.get(dev)) {
+        e = cudaFuncSetAttribute(f32_block_kernel<BR, kFirst>, cudaFuncAttributeMaxDynamicSharedMemorySize, kF32BlockSmem);
+        if (e != cudaSuccess) return e;
+        attr_set.set(dev, 1);
+    }
+    const size_t smem = sizeof(float) * (size_t)layout_of(d, F, tail.kind == F32_TAIL_QKV ? tail.n : 0, kFirst, BR).total;
+    return launch_dependent(f32_block_kernel<BR, kFirst>, dim3((unsigned)((M + BR - 1) / BR)), dim3(kThreads), smem, stream, 1, first, wt, tail, x, att, M, d, F,
+                            eps, err);
+}
+
+}  // namespace
+
+bool f32_block_supported(int64_t M, int d, int F, int n_sms)
+{
+    return (d == 32 || d == 64) && F % 32 == 0 && layout_of(d, F, 3 * d, false, 8).total * (int64_t)sizeof(float) <= kF32BlockSmem && M <= 8 * (int64_t)n_sms;
+}
+
+// Four rows to a block as long as every block has an SM to itself, then eight.
+cudaError_t launch_f32_first(const F32First &first, const F32BlockTail &tail, float *x, int64_t M, int d, float eps, int n_sms, int *err, cudaStream_t stream,
+                             int64_t *launches)
+{
+    if (M == 0) return cudaSuccess;
+    *launches += 1;
+    return M <= 4 * (int64_t)n_sms ? launch<4, true>(first, F32BlockWeights{}, tail, x, nullptr, M, d, 0, eps, err, stream)
+                                   : launch<8, true>(first, F32BlockWeights{}, tail, x, nullptr, M, d, 0, eps, err, stream);
+}
+
+cudaError_t launch_f32_block(const F32BlockWeights &w, const F32BlockTail &tail, float *x, const float *att, int64_t M, int d, int F, float eps, int n_sms,
+                             cudaStream_t stream, int64_t *launches)
+{
+    if (M == 0) return cudaSuccess;
+    *launches += 1;
+    return M <= 4 * (int64_t)n_sms ? launch<4, false>(F32First{}, w, tail, x, att, M, d, F, eps, nullptr, stream)
+                                   : launch<8, false>(F32First{}, w, tail, x, att, M, d, F, eps, nullptr, stream);
+}
+
+}  // namespace relaygr

@@ -424,6 +424,31 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     auto ln_in_gemm = [&](int64_t M, int N) { return !kTensor && !tensor32 && gemm_f32_takes_ln(M, N, d, n_sms); };
     auto with_ln = [&](Epilogue &ep, const float *g, const float *b) { ep.ln_g = g; ep.ln_b = b; ep.ln_eps = cfg.ln_eps; };
 
+    // The launch chain is what such a call costs: as long as a block of eight rows has an SM to itself, two launches a layer instead of
+    // five (f32_block.cu; 384 rows of width 64: 44 us a call instead of 66)
+    const bool blocks32 = !kTensor && !tensor32 && !compact_last && f32_block_supported(R, d, F, n_sms) &&
+                          (((uintptr_t)w.w_qkv | (uintptr_t)w.w_o | (uintptr_t)w.w1 | (uintptr_t)w.w2) & 15) == 0;
+    // what follows layer l - 1 (l = 0: the gather; l = L: the scoring head) in the same kernel
+    auto tail_of = [&](int l) {
+        F32BlockTail t{};
+        if (l < L && !(l == L - 1 && !preinfer && n_scores == 0)) {
+            t.kind = F32_TAIL_QKV;
+            t.g = w.ln1_g + (size_t)l * d; t.b = w.ln1_b + (size_t)l * d;
+            t.e.col0 = preinfer && l == L - 1 ? d : 0;
+            t.n = 3 * d - t.e.col0;
+            t.w = (const float *)w.w_qkv + ((size_t)l * 3 * d + t.e.col0) * d;
+            t.bias = w.b_qkv ? w.b_qkv + (size_t)l * 3 * d + t.e.col0 : nullptr;
+            t.e.q = q; t.e.k_lin = kl; t.e.v_lin = vl;
+            if (preinfer) t.e.paged = PagedKV{call.pool_slab, meta + o_pt, L, d, l};
+        } else if (l == L) {
+            t.kind = F32_TAIL_SCORE;
+            t.g = w.lnf_g; t.b = w.lnf_b; t.w = w.w_score; t.bias = w.b_score;
+            t.score_off = meta + o_score; t.scores = scores;
+        }
+        t.e.seqs = d_seqs; t.e.row_off = d_row_off; t.e.n_users = B;
+        return t;
+    };
+
     for (int l = 0; l < L; ++l) {
         const bool last = l == L - 1;
         if (last && !preinfer && n_scores == 0) { dead_tail = true; break; }
@@ -431,6 +456,20 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         // K and V only in the last pre-infer layer (psi is K/V alone) and in the last layer of a call whose candidates are moved together
         // (their queries follow below, on their rows alone)
         const bool kv_only = last && (preinfer || compact_last);
+        PagedKV paged{};
+        if (call.pool_slab) {
+            paged.slab = call.pool_slab; paged.pt = meta + o_pt; paged.n_layers = L; paged.d_model = d; paged.layer = l;
+        }
+        lm = wmaps_ok ? &wmaps[(size_t)l] : nullptr;
+        if constexpr (!kTensor) {
+            if (blocks32 && l == 0) {
+                cudaEvent_t pe = prof_begin(stream);
+                e = launch_f32_first(F32First{(const float *)w.emb, cfg.vocab, src}, tail_of(0), x, R, d, cfg.ln_eps, n_sms, d_status, stream, &launches);
+                prof_end(KC_GATHER_LN, pe, stream);
+                if (!ck("gather, LayerNorm and QKV projection")) return RELAYGR_E_CUDA;
+            }
+        }
+        if (!blocks32) {
         const bool ln1_in_gemm = l > 0 && !(last && compact_last) && ln_in_gemm(R, kv_only ? 2 * d : 3 * d);
         if (l == 0) {
             cudaEvent_t pe = prof_begin(stream);
@@ -450,15 +489,11 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         ep.d_model = d;
         ep.q = q; ep.k_lin = kl; ep.v_lin = vl;
         ep.seqs = d_seqs; ep.row_off = d_row_off; ep.n_users = B;
-        PagedKV paged{};
-        if (call.pool_slab) {
-            paged.slab = call.pool_slab; paged.pt = meta + o_pt; paged.n_layers = L; paged.d_model = d; paged.layer = l;
-        }
         if (preinfer) { ep.paged = paged; ep.page_runs = meta + o_runs; }
         const T *Wqkv = (const T *)w.w_qkv + ((size_t)l * 3 * d + ep.col0) * d;
-        lm = wmaps_ok ? &wmaps[(size_t)l] : nullptr;
         e = gemm(R, ln1_in_gemm ? reinterpret_cast<const T *>(x) : a, tm_a, Wqkv, lm ? (kv_only ? &lm->kv : &lm->qkv) : nullptr, om_qkv, 3 * d - ep.col0, d, ep);
         if (!ck("QKV projection")) return RELAYGR_E_CUDA;
+        }
         if (preinfer && last) break;
 
         if (last && cand_last) {
@@ -524,6 +559,19 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
             prof_end(KC_GEMM, pe, stream);
             if (!ck("output projection + feed-forward")) return RELAYGR_E_CUDA;
             continue;
+        }
+        if constexpr (!kTensor) {
+            if (blocks32) {
+                cudaEvent_t pe = prof_begin(stream);
+                const F32BlockWeights bw{(const float *)w.w_o + (size_t)l * d * d, w.b_o ? w.b_o + (size_t)l * d : nullptr, w.ln2_g + (size_t)l * d, w.ln2_b + (size_t)l * d,
+                                         (const float *)w.w1 + (size_t)l * F * d, w.b1 ? w.b1 + (size_t)l * F : nullptr,
+                                         (const float *)w.w2 + (size_t)l * d * F, w.b2 ? w.b2 + (size_t)l * d : nullptr};
+                e = launch_f32_block(bw, tail_of(l + 1), x, att, R, d, F, cfg.ln_eps, n_sms, stream, &launches);
+                scored = last;
+                prof_end(KC_GEMM, pe, stream);
+                if (!ck("output projection + feed-forward")) return RELAYGR_E_CUDA;
+                continue;
+            }
         }
         Epilogue eo{};
         eo.mode = EPI_RESID; eo.bias = w.b_o ? w.b_o + (size_t)l * d : nullptr; eo.resid = xm; eo.out_f32 = xm;

@@ -111,6 +111,20 @@ __device__ __forceinline__ int find_user(const int32_t *row_off, int n_users, in
     return lo;
 }
 
+__device__ __forceinline__ int row_token_id(const RowSource &src, int64_t row)
+{
+    const int u = find_user(src.row_off, src.n_users, (int)row);
+    int i = (int)row - src.row_off[u];
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        if (!src.ids[s]) continue;
+        const int len = src.off[s][u + 1] - src.off[s][u];
+        if (i < len) return src.ids[s][src.off[s][u] + i];
+        i -= len;
+    }
+    return 0;
+}
+
 __device__ __forceinline__ size_t page_elem_offset(const PagedKV &p, int page, int kv, int slot)
 {
     return ((((size_t)page * p.n_layers + p.layer) * 2 + kv) * 64 + slot) * (size_t)p.d_model;

@@ -88,6 +88,28 @@ cudaError_t launch_attention_f32(const float *q, const float *k_lin, const float
                                  const F32Tile *tiles, int n_tiles, int tile_rows, int n_heads, int d_head, int attn_kind, int n_sms, float *out,
                                  cudaStream_t stream, int64_t *launches);
 
+// The fp32 model with few rows and matrices that fit an SM's shared memory (f32_block_supported; w_qkv, w_o, w1, w2 and the table 16-byte
+// aligned): a call's first kernel, x = E[id(r)], and everything of a layer after its attention, x <- mid + W2 SiLU(W1 LN(mid) + b1) + b2 with
+// mid = x + Wo att + bo; each goes on with `tail`.
+constexpr int kF32BlockSmem = 226 * 1024;
+enum F32TailKind : int { F32_TAIL_NONE = 0, F32_TAIL_QKV, F32_TAIL_SCORE };
+struct F32First { const float *emb; int64_t vocab; RowSource src; };
+struct F32BlockWeights { const float *wo, *bo, *ln_g, *ln_b, *w1, *b1, *w2, *b2; };      // of one layer; ln: LayerNorm 2
+struct F32BlockTail {
+    int kind;
+    const float *g, *b;           // the LayerNorm that follows
+    const float *w, *bias;        // F32_TAIL_QKV: [n, d] and [n]; F32_TAIL_SCORE: w_score and one value
+    int n;
+    Epilogue e;                   // F32_TAIL_QKV: as in EPI_QKV; F32_TAIL_SCORE: seqs, row_off, n_users of the rows
+    const int32_t *score_off;
+    float *scores;
+};
+bool f32_block_supported(int64_t M, int d, int F, int n_sms);
+cudaError_t launch_f32_first(const F32First &first, const F32BlockTail &tail, float *x, int64_t M, int d, float eps, int n_sms, int *err, cudaStream_t stream,
+                             int64_t *launches);
+cudaError_t launch_f32_block(const F32BlockWeights &w, const F32BlockTail &tail, float *x, const float *att, int64_t M, int d, int F, float eps, int n_sms,
+                             cudaStream_t stream, int64_t *launches);
+
 // Where a GEMM's epilogue stores: tensor maps with a 32-row box of 128 bytes and the 128-byte swizzle, in the model's type.
 // EPI_STORE: o[0] = out [M, N].  EPI_RESID: o[0] = the fp32 residual stream [M, N] (tile added in place).
 // EPI_QKV: o[0] = q, o[1] = k_lin, o[2] = v_lin, each [M, d] (o[1], o[2] are not used when K / V go to pages);

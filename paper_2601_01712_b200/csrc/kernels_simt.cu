@@ -33,20 +33,6 @@ __device__ __forceinline__ void store4(__nv_bfloat16 *p, float4 v)
     *reinterpret_cast<uint2 *>(p) = u;
 }
 
-__device__ __forceinline__ int row_token_id(const RowSource &src, int64_t row)
-{
-    const int u = find_user(src.row_off, src.n_users, (int)row);
-    int i = (int)row - src.row_off[u];
-#pragma unroll
-    for (int s = 0; s < 3; ++s) {
-        if (!src.ids[s]) continue;
-        const int len = src.off[s][u + 1] - src.off[s][u];
-        if (i < len) return src.ids[s][src.off[s][u] + i];
-        i -= len;
-    }
-    return 0;
-}
-
 template <typename T>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 gather_rows_kernel(const T *__restrict__ emb, int64_t vocab, int d, const int32_t *__restrict__ ids, int64_t n, T *__restrict__ out, int *err)

@@ -249,3 +249,15 @@ def test_preinfer_rows_in_and_across_pages():
 def test_f32_few_rows(d, heads, ff, cand):
     shape = synth.ModelShape(2, d, heads, d // heads, ff, 2000, synth.DTYPE_F32)
     _check_f32(shape, _tiny_batch(shape, 350 + d + ff, [20], [3], [cand]), 67)
+
+
+# Few rows of the fp32 model with matrices that fit an SM (widths 32 and 64): blocks of four rows, from 593 rows on of eight, the last one
+# ragged; one layer and three; pages that end inside, at and behind their last slot; the widest feed-forward that fits (256 at width
+# 64) and the next; a user without candidates.
+@pytest.mark.parametrize("layers,d,heads,ff,prefix,short,cand", [
+    (2, 64, 2, 256, [1], [0], [1]), (1, 64, 1, 256, [64, 65, 3], [2, 0, 1], [9, 4, 30]), (3, 32, 1, 128, [70, 128], [0, 33], [31, 62]),
+    (2, 64, 2, 256, [20], [0], [592]), (2, 64, 2, 256, [20], [0], [593]), (2, 64, 2, 288, [90, 20], [5, 3], [70, 31]), (3, 64, 2, 32, [300, 150], [5, 3], [60, 0]),
+    (2, 32, 1, 1024, [700], [5], [760]), (1, 32, 1, 96, [191], [0], [2])])
+def test_f32_blocks(layers, d, heads, ff, prefix, short, cand):
+    shape = synth.ModelShape(layers, d, heads, d // heads, ff, 2000, synth.DTYPE_F32)
+    _check_f32(shape, _tiny_batch(shape, 370 + d + ff, prefix, short, cand), 71)
