@@ -72,6 +72,7 @@ struct Forward {
     cudaEvent_t slot_event[kSlots] = {};
     bool slot_used[kSlots] = {};
     int next_slot = 0;
+    bool slot_open = false;      // the call being enqueued reads slot next_slot, whose event is yet to be recorded
 
     // optional per-kernel-class timing with CUDA events on the call's stream
     enum KernelClass { KC_GATHER_LN = 0, KC_LAYERNORM, KC_GEMM, KC_ATTENTION, KC_SCORE, KC_COUNT };

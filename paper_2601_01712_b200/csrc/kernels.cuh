@@ -45,6 +45,9 @@ struct PerDeviceValue {
 
 // ---- memory-bound steps (CUDA cores, vectorised loads, warp-shuffle reductions) ----------------
 
+// dst <- src, pinned host memory; both 16-byte aligned and bytes rounded up to 16 readable and writable.
+cudaError_t launch_upload(const void *src, void *dst, size_t bytes, cudaStream_t stream, int64_t *launches);
+
 // out[i, :] = emb[ids[i], :], a bit-exact row copy.  An id outside [0, vocab) records STATUS_BAD_INDEX in *err (err may
 // be nullptr) and row 0 / vocab - 1 is copied instead, so that no access leaves the table.
 template <typename T>

@@ -33,6 +33,21 @@ __device__ __forceinline__ void store4(__nv_bfloat16 *p, float4 v)
     *reinterpret_cast<uint2 *>(p) = u;
 }
 
+// The call's metadata from pinned host memory into the workspace.  A copy by the copy engine would keep the first kernel waiting for 6 us
+// behind it; from a kernel the first one goes on at once, and the bytes (a few KB) cross PCIe in one round trip.  One user's ranking call
+// 122 -> 116 us, its pre-inference 122 -> 117, a batch of 32 users 456 -> 443.
+constexpr int kUploadThreads = 256;
+__global__ void __launch_bounds__(kUploadThreads)
+upload_kernel(const int4 *__restrict__ src, int4 *__restrict__ dst, int n)
+{
+    grid_launch_dependents();
+    const int i = blockIdx.x * kUploadThreads + threadIdx.x;
+    int4 v{};
+    if (i < n) v = __ldcv(src + i);                   // (staged before the launch)
+    grid_dependency_wait();                           // the call before has read what was there
+    if (i < n) dst[i] = v;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 gather_rows_kernel(const T *__restrict__ emb, int64_t vocab, int d, const int32_t *__restrict__ ids, int64_t n, T *__restrict__ out, int *err)
@@ -255,6 +270,15 @@ score_kernel(const float *__restrict__ x, int d, const SeqDesc *__restrict__ seq
 inline unsigned blocks_for(int64_t warps) { return (unsigned)((warps + kWarpsPerBlock - 1) / kWarpsPerBlock); }
 
 }  // namespace
+
+cudaError_t launch_upload(const void *src, void *dst, size_t bytes, cudaStream_t stream, int64_t *launches)
+{
+    if (bytes == 0) return cudaSuccess;
+    *launches += 1;
+    const int n = (int)((bytes + 15) / 16);
+    return launch_dependent(upload_kernel, dim3((unsigned)((n + kUploadThreads - 1) / kUploadThreads)), dim3(kUploadThreads), 0, stream, 1,
+                            reinterpret_cast<const int4 *>(src), reinterpret_cast<int4 *>(dst), n);
+}
 
 template <typename T>
 cudaError_t launch_gather_rows(const T *emb, int64_t vocab, int d, const int32_t *ids, int64_t n, T *out, int *err,
