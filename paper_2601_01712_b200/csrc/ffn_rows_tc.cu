@@ -7,8 +7,10 @@
 //     mid, A = LN(mid)        P is turned around in shared memory, a warp then has T / 8 whole rows; A as bf16 where att was
 //     per chunk:              S^T = W1c A^T, H = SiLU(S + b1c) as bf16 into shared memory, O^T += W2c H^T
 // The partial O are turned around like P and added up through distributed shared memory, the CTA's own first, then in rank order - for
-// every row one fixed order of the fp32 sums, so results do not vary from run to run - and each CTA finishes its share of the tile's rows, the next layer's LayerNorm
-// (or the final one and the scoring head) included.
+// every row one fixed order of the fp32 sums, so results do not vary from run to run - and each CTA finishes its share of the tile's rows, the
+// next layer's LayerNorm (or the final one and the scoring head) included.  In clusters of four or eight the normalised rows go on to every CTA's
+// shared memory (st.async) and the next layer's QKV projection follows, its 128-column chunks dealt like the hidden units: a launch of
+// 5 us less in every layer.
 //
 // What bounds it: a serial chain of short steps, each with its own latency, and the exchange - distributed shared memory delivers
 // about 16 bytes per clock to an SM, and a CTA takes T KB of partial sums.  With 128-row tiles (rows on the lanes) that chain took
@@ -17,7 +19,7 @@
 //
 // Warp roles (384 threads): warp 0 = TMA producer (a ring of 32 KB stages: Wo in four K blocks, then half a W1 chunk or half a W2
 // chunk per stage, in the order the MMAs consume them; the whole ring is under way before the kernel waits for its predecessor),
-// warp 1 = TMEM owner + MMA issuer, warp 2 none, warp 3 = arrival at the last cluster barrier, warps 4-11 = LayerNorm, SiLU and
+// warp 1 = TMEM owner + MMA issuer, warp 2 = look-up of page rows, warp 3 = arrival at the last cluster barrier, warps 4-11 = LayerNorm, SiLU and
 // exchange (two warps per TMEM quadrant).  TMEM: P, later O, 2 T columns; S double-buffered, T columns each.  The MMA warp issues S(0),
 // S(1), then per chunk O(c) followed by S(c+2): the tensor pipe executes in issue order, so S(c+2) complete also means that H(c) has
 // been read.
@@ -39,11 +41,17 @@ struct Shape {
     static constexpr int kOffH = 4 * kKB;             // two buffers of two K blocks, behind A; A and H together: T rows x 256 fp32
     static constexpr int kOffW = 8 * kKB;
     static constexpr int kOffBars = kOffW + kStages * kStageBytes;
-    static constexpr int kSmemBytes = kOffBars + 256 + 1024;
+    static constexpr int kOffPages = kOffBars + 256;  // of the tile's rows that go to pages: offset of (page, K, slot); of a user's last row its slot
+    static constexpr int kSmemBytes = kOffPages + T * 12 + 1024;
     static constexpr int kColS = 2 * T;
     static constexpr uint32_t kTmemCols = 4 * T;
     static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
 };
+
+// Whether the kernel goes on to the next layer's QKV projection: where a CTA has two of its six 128-column chunks at most.  With three, in
+// clusters of two, 192 KB of weights and three trips through TMEM follow one another (the pre-inference of 2000 tokens 122 us, 112 with the
+// projection as a launch of its own; a ranking call of one user, clusters of four, 110 and 116).
+template <int CS> constexpr bool kProjects = CS >= 4;
 
 template <int kStages>
 struct RowBars {
@@ -52,6 +60,7 @@ struct RowBars {
     uint64_t s_full[2];                               // S complete in its buffer
     uint64_t h_full[2];                               // H in shared memory
     uint64_t o_full;                                  // O complete
+    uint64_t next_full;                               // the next layer's LN(x), all rows of the tile, in shared memory
     uint32_t tmem_slot;
 };
 static_assert(sizeof(RowBars<6>) <= 256, "barrier block");
@@ -103,7 +112,7 @@ __device__ __forceinline__ float4 normalised(const float4 &v, float mean, float 
 template <int T, int CS>
 __global__ void __launch_bounds__(kThreads, 1)
 ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2,
-                const __grid_constant__ CUtensorMap tmAtt, const __grid_constant__ CUtensorMap tmWo,
+                const __grid_constant__ CUtensorMap tmAtt, const __grid_constant__ CUtensorMap tmWo, const __grid_constant__ CUtensorMap tmQkv,
                 float *__restrict__ x, const float *__restrict__ g, const float *__restrict__ b, const float *__restrict__ b1,
                 const float *__restrict__ b2, const float *__restrict__ bo, int64_t M, int F, float eps, FfnTail tail, int *err)
 {
@@ -125,6 +134,9 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
     // this CTA's hidden chunks: rank, rank + CS, ...; there are at least CS
     const int nc = (F / kChunk - rank + CS - 1) / CS;
     auto chunk_at = [&](int i) { return rank + i * CS; };
+    // ... and of the next layer's QKV projection, 128 output columns each
+    const bool project = kProjects<CS> && tail.kind == FFN_TAIL_QKV;
+    const int nq = project ? max(0, (tail.n_qkv / kChunk - rank + CS - 1) / CS) : 0;
     const int ew = warp - 4, quad = warp & 3, ch = ew >> 2, c0 = 4 * lane;      // epilogue warps; c0 .. + 3 and 128 + c0 .. + 3: columns of a lane
     auto row = [&](int j) { return 16 * (j >> 1) + 2 * ew + (j & 1); };
     const int j_end = rank / kShare * kEnd;
@@ -140,12 +152,13 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
         if (ok) tc::mbar_expect_tx(&bars->w_full[s], kStageBytes);
         return s;
     };
-    auto load_w1 = [&](int c, int half) {             // rows c*128 .. +127 of W1 [F, 256], K blocks 2*half and 2*half + 1
+    auto load_rows = [&](const CUtensorMap *map, int c, int half) {      // rows c*128 .. +127 of a matrix [.., 256], K blocks 2*half and 2*half + 1
         const int s = acquire();
         if (!ok) return;
-        tc::tma_load_2d(sW + s * kStageBytes, &tmW1, (2 * half) * 64, c * kChunk, &bars->w_full[s]);
-        tc::tma_load_2d(sW + s * kStageBytes + kHalfStage, &tmW1, (2 * half + 1) * 64, c * kChunk, &bars->w_full[s]);
+        tc::tma_load_2d(sW + s * kStageBytes, map, (2 * half) * 64, c * kChunk, &bars->w_full[s]);
+        tc::tma_load_2d(sW + s * kStageBytes + kHalfStage, map, (2 * half + 1) * 64, c * kChunk, &bars->w_full[s]);
     };
+    auto load_w1 = [&](int c, int half) { load_rows(&tmW1, c, half); };
     auto load_w2 = [&](int c, int half) {             // all 256 rows of W2 [256, F], 64 hidden columns
         const int s = acquire();
         if (ok) tc::tma_load_2d(sW + s * kStageBytes, &tmW2, c * kChunk + half * 64, 0, &bars->w_full[s]);
@@ -158,8 +171,9 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
         for (int s = 0; s < kStages; ++s) { tc::mbar_init(&bars->w_full[s], 1); tc::mbar_init(&bars->w_empty[s], 1); }
         for (int i = 0; i < 2; ++i) { tc::mbar_init(&bars->s_full[i], 1); tc::mbar_init(&bars->h_full[i], kEpiWarps); }
         tc::mbar_init(&bars->att_full, 1); tc::mbar_init(&bars->p_full, 1); tc::mbar_init(&bars->a_ready, kEpiWarps);
-        tc::mbar_init(&bars->o_full, 1);
+        tc::mbar_init(&bars->o_full, 1); tc::mbar_init(&bars->next_full, 1);
         tc::fence_mbar_init();
+        if (project) tc::mbar_expect_tx(&bars->next_full, T * kD * 2);
         for (int kb = 0; kb < 4; ++kb) {
             const int s = acquire();
             tc::tma_load_2d(sW + s * kStageBytes, &tmWo, kb * 64, 0, &bars->w_full[s]);
@@ -167,6 +181,23 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
         for (int h = 0; h < kEarlyHalves; ++h) load_w1(chunk_at(0), h);
         tc::tma_prefetch_desc(&tmW1); tc::tma_prefetch_desc(&tmW2); tc::tma_prefetch_desc(&tmAtt);
     }
+    // K / V rows that go to pages (call metadata, on the device before the call's first kernel ran to its end)
+    int64_t *page_off = reinterpret_cast<int64_t *>(smem + L::kOffPages);
+    int *last_slot = reinterpret_cast<int *>(page_off + T);
+    const bool paged = project && tail.paged.slab != nullptr;
+    if (paged && warp == 2)
+        for (int i = lane; i < T; i += 32) {
+            const int64_t r = tile_row0 + i;
+            int64_t off = 0;
+            int last = -1;
+            if (r < M) {
+                const int u = find_user(tail.row_off, tail.n_users, (int)r), t = (int)r - tail.row_off[u];
+                off = (int64_t)page_elem_offset(tail.paged, tail.paged.pt[tail.seqs[u].pt_base + (t >> 6)], 0, t & 63);
+                if (t == tail.seqs[u].n_q - 1) last = t & 63;
+            }
+            page_off[i] = off;
+            last_slot[i] = last;
+        }
     if (warp == 1) {
         tc::tmem_alloc(&bars->tmem_slot, L::kTmemCols);
         tc::tmem_relinquish();
@@ -206,6 +237,40 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
     float4 own[kEnd][2];                              // mid of the rows this CTA finishes
     float4 obias2[2], tg[2], tb[2], tw[2];            // of the end of the block
     int score_at = -1;                                // lane i < kEnd: where the score of the warp's row i goes (-1: not a candidate's)
+    int next_half = 0;                                // of the next layer's projection: stages requested so far
+    // MMA issuer.
+            // The chain's pace: an MMA of 128 x T x 16 takes some 50 clocks, what surrounds a stage's eight must not take as long again
+            // (it did, 350 clocks, with one loop for all kinds of stage and divisions for the ring position).
+            constexpr uint32_t idesc = tc::make_idesc(kRows, T, 0, 0);             // weights x rows, both K-major
+            const uint64_t adesc0 = tc::smem_desc_sw128(tc::smem_u32(sA)), hdesc0 = tc::smem_desc_sw128(tc::smem_u32(sH)), wdesc0 = tc::smem_desc_sw128(tc::smem_u32(sW));
+            uint32_t s = 0, phase = 0;                    // of the ring
+            auto stage = [&] {
+                ok = ok && tc::mbar_wait(&bars->w_full[s], phase, err);
+                tc::tc_fence_after();
+                return ok;
+            };
+            auto next_stage = [&] {
+                if (++s == kStages) { s = 0; phase ^= 1; }
+            };
+            auto issue_s = [&](int i) {                   // S^T = W1c A^T (or the next projection's): two stages, each two K blocks of 64
+                const uint32_t d = tmem_base + L::kColS + (i & 1) * T;
+    #pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    if (!stage()) return;
+                    const uint64_t wdesc = wdesc0 + s * (kStageBytes / 16);
+                    if (tc::elect_one()) {
+    #pragma unroll
+                        for (int kb = 0; kb < 2; ++kb)
+    #pragma unroll
+                            for (int k = 0; k < 4; ++k)
+                                tc::mma_ss(d, wdesc + kb * (kHalfStage / 16) + 2 * k, adesc0 + (2 * half + kb) * (kKB / 16) + 2 * k, idesc, (half | kb | k) != 0);
+                        tc::mma_commit(&bars->w_empty[s]);
+                        if (half == 1) tc::mma_commit(&bars->s_full[i & 1]);
+                    }
+                    __syncwarp();
+                    next_stage();
+                }
+            };
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer
         if (lane == 0) {
@@ -215,41 +280,10 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
                 load_w2(chunk_at(i), 0); load_w2(chunk_at(i), 1);
                 if (i + 2 < nc) { load_w1(chunk_at(i + 2), 0); load_w1(chunk_at(i + 2), 1); }
             }
+            for (; next_half < min(2 * nq, kStages) && ok; ++next_half) load_rows(&tmQkv, chunk_at(next_half >> 1), next_half & 1);
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer (convergent warp, one elected lane issues)
-        // The chain's pace: an MMA of 128 x T x 16 takes some 50 clocks, what surrounds a stage's eight must not take as long again
-        // (it did, 350 clocks, with one loop for all kinds of stage and divisions for the ring position).
-        constexpr uint32_t idesc = tc::make_idesc(kRows, T, 0, 0);             // weights x rows, both K-major
-        const uint64_t adesc0 = tc::smem_desc_sw128(tc::smem_u32(sA)), hdesc0 = tc::smem_desc_sw128(tc::smem_u32(sH)), wdesc0 = tc::smem_desc_sw128(tc::smem_u32(sW));
-        uint32_t s = 0, phase = 0;                    // of the ring
-        auto stage = [&] {
-            ok = ok && tc::mbar_wait(&bars->w_full[s], phase, err);
-            tc::tc_fence_after();
-            return ok;
-        };
-        auto next_stage = [&] {
-            if (++s == kStages) { s = 0; phase ^= 1; }
-        };
-        auto issue_s = [&](int i) {                   // S^T = W1c A^T: two stages, each two K blocks of 64
-            const uint32_t d = tmem_base + L::kColS + (i & 1) * T;
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                if (!stage()) return;
-                const uint64_t wdesc = wdesc0 + s * (kStageBytes / 16);
-                if (tc::elect_one()) {
-#pragma unroll
-                    for (int kb = 0; kb < 2; ++kb)
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            tc::mma_ss(d, wdesc + kb * (kHalfStage / 16) + 2 * k, adesc0 + (2 * half + kb) * (kKB / 16) + 2 * k, idesc, (half | kb | k) != 0);
-                    tc::mma_commit(&bars->w_empty[s]);
-                    if (half == 1) tc::mma_commit(&bars->s_full[i & 1]);
-                }
-                __syncwarp();
-                next_stage();
-            }
-        };
         // one K block of 64 into both halves of P or O: 256 weight rows (output columns) x the tile's rows
         auto issue_wide = [&](uint64_t rdesc, bool fresh, uint64_t *done) {
             if (!stage()) return;
@@ -414,8 +448,40 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
     else if (warp == 3) asm volatile("bar.sync 2, %0;" ::"n"(kEpiThreads + 32) : "memory");
     if (warp == 3) tc::cluster_arrive_release();
     else tc::cluster_arrive_relaxed();
-    if (finisher && o_ready && !stopped) {
-        if (tail.kind != FFN_TAIL_SCORE) {
+    if (finisher && o_ready) {
+        float mean[kEnd], rstd[kEnd];
+        rows_stats<kEnd>(own, eps, mean, rstd);
+        if (project) tc::cluster_wait();              // nobody reads `turn` any more: the tile of the next projection's rows takes its place
+#pragma unroll
+        for (int i = 0; i < kEnd; ++i) {
+            const int rt = row(j_end + i);
+            const int64_t r = tile_row0 + rt;
+            const bool store = r < M && !stopped;
+            float acc = 0.f;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float4 y = normalised(own[i][h], mean[i], rstd[i], tg[h], tb[h]);
+                if (tail.kind == FFN_TAIL_SCORE) {
+                    acc += y.x * tw[h].x + y.y * tw[h].y + y.z * tw[h].z + y.w * tw[h].w;
+                    continue;
+                }
+                const uint2 y2 = make_uint2(tc::pack_bf16(y.x, y.y), tc::pack_bf16(y.z, y.w));
+                if (project) {                        // to every CTA of the cluster
+                    const uint8_t *dst = sA + (lane >> 4) * kKB + rt * 128 + ((((lane & 15) >> 1) ^ (rt & 7)) << 4) + (lane & 1) * 8 + 2 * h * kKB;
+#pragma unroll
+                    for (int k = 0; k < CS; ++k) tc::st_async8(tc::cluster_addr(dst, k), y2, tc::cluster_addr(&bars->next_full, k));
+                } else if (store) {
+                    *reinterpret_cast<uint2 *>(tail.a + r * kD + c0 + 128 * h) = y2;
+                }
+            }
+            if (tail.kind == FFN_TAIL_SCORE) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                const int at = __shfl_sync(0xffffffffu, score_at, i);
+                if (lane == 0 && at >= 0 && !stopped) tail.scores[at] = acc + (tail.bias ? tail.bias[0] : 0.f);
+            }
+        }
+        if (tail.kind != FFN_TAIL_SCORE && !stopped) {
 #pragma unroll
             for (int i = 0; i < kEnd; ++i) {
                 const int64_t r = tile_row0 + row(j_end + i);
@@ -424,28 +490,61 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
                     for (int h = 0; h < 2; ++h) *reinterpret_cast<float4 *>(x + r * kD + c0 + 128 * h) = own[i][h];
             }
         }
-        float mean[kEnd], rstd[kEnd];
-        rows_stats<kEnd>(own, eps, mean, rstd);
+    } else if (project) {
+        tc::cluster_wait();
+    }
+    __syncwarp();
+    if (project) {
+        // The next layer's QKV projection of the tile, its 128-column chunks dealt to the CTAs like the hidden units: S buffers, stages
+        // and barriers go on where the feed-forward left them.
+        tc::cluster_arrive_relaxed();                 // nobody ends before everybody has sent its rows
+        if (warp == 0) {
+            if (lane == 0)
+                for (; next_half < 2 * nq && ok; ++next_half) load_rows(&tmQkv, chunk_at(next_half >> 1), next_half & 1);
+        } else if (warp == 1) {
+            ok = ok && tc::mbar_wait(&bars->next_full, 0, err);      // (CTAs without a chunk as well: what is sent to them lands before they end)
+            tc::fence_proxy_async();
+            tc::tc_fence_after();
+            for (int i = 0; i < nq && ok; ++i) {
+                if (i >= 2) {                         // the buffer's S before is in registers
+                    ok = tc::mbar_wait(&bars->h_full[(nc + i) & 1], ((nc + i - 2) >> 1) & 1, err);
+                    tc::tc_fence_after();
+                }
+                if (ok) issue_s(nc + i);
+            }
+        } else if (warp >= 4 && o_ready) {
+            const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
+#pragma unroll 1
+            for (int i = 0; i < nq; ++i) {
+                const int hb = (nc + i) & 1, n = chunk_at(i) * kChunk + quad * 32 + lane;      // this lane's output column
+                const int which = (tail.col0 + n) >> 8, c = (tail.col0 + n) & (kD - 1);
+                const float scale = which == 0 ? tail.q_scale : 1.f, bias = tail.bias ? tail.bias[n] * scale : 0.f;
+                ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->s_full[hb], ((nc + i) >> 1) & 1, err));
+                if (!ok) break;
+                tc::tc_fence_after();
+                uint32_t r[T / 2];
+                if constexpr (T == 64) tc::tmem_ld32(lane_addr + L::kColS + hb * T + ch * (T / 2), r);
+                else tc::tmem_ld16(lane_addr + L::kColS + hb * T + ch * (T / 2), r);
+                tc::tmem_ld_wait();
+                tc::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&bars->h_full[hb]);
+                if (stopped) continue;
+                const bool to_page = paged && which > 0;
+                __nv_bfloat16 *base = to_page ? reinterpret_cast<__nv_bfloat16 *>(tail.paged.slab) + (which - 1) * 64 * kD + c
+                                              : (which == 0 ? tail.q : which == 1 ? tail.k : tail.v) + tile_row0 * kD + c;
 #pragma unroll
-        for (int i = 0; i < kEnd; ++i) {
-            const int64_t r = tile_row0 + row(j_end + i);
-            float acc = 0.f;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const float4 y = normalised(own[i][h], mean[i], rstd[i], tg[h], tb[h]);
-                if (tail.kind == FFN_TAIL_LN) {
-                    if (r < M) *reinterpret_cast<uint2 *>(tail.a + r * kD + c0 + 128 * h) = make_uint2(tc::pack_bf16(y.x, y.y), tc::pack_bf16(y.z, y.w));
-                } else {
-                    acc += y.x * tw[h].x + y.y * tw[h].y + y.z * tw[h].z + y.w * tw[h].w;
+                for (int e = 0; e < T / 2; ++e) {
+                    const int rt = ch * (T / 2) + e;
+                    if (tile_row0 + rt >= M) break;
+                    __nv_bfloat16 *p = base + (to_page ? page_off[rt] : (int64_t)rt * kD);
+                    *p = __float2bfloat16_rn(fmaf(__uint_as_float(r[e]), scale, bias));
+                    if (to_page && last_slot[rt] >= 0)      // last row of the prefix: clear the unused slots of its page
+                        for (int z = 1; last_slot[rt] + z < 64; ++z) p[z * kD] = __float2bfloat16_rn(0.f);
                 }
             }
-            if (tail.kind == FFN_TAIL_SCORE) {
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                const int at = __shfl_sync(0xffffffffu, score_at, i);
-                if (lane == 0 && at >= 0) tail.scores[at] = acc + (tail.bias ? tail.bias[0] : 0.f);
-            }
         }
+        __syncwarp();
     }
     __syncwarp();
     tc::cluster_wait();
@@ -457,9 +556,9 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
 }  // namespace
 
 cudaError_t launch_ffn_rows(const FfnMaps &w, float *x, const float *g, const float *b, const float *b1, const float *b2, const CUtensorMap &tmAtt32,
-                            const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail, int *err, cudaStream_t stream, bool *taken)
+                            const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail, int *err, cudaStream_t stream, bool *taken, bool *projected)
 {
-    *taken = false;
+    *taken = *projected = false;
     // This form reads the vectors 16 bytes at a time; the others read them value by value, as they may come at any multiple of 4 bytes.
     auto aligned = [](const float *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
     if (!aligned(g) || !aligned(b) || !aligned(b2) || !aligned(bo)) return cudaSuccess;
@@ -467,25 +566,29 @@ cudaError_t launch_ffn_rows(const FfnMaps &w, float *x, const float *g, const fl
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     const int chunks = d_ff / kChunk;
-    auto attempt = [&](auto kernel, int T, int cs, size_t smem, PerDeviceValue &known) {
+    const CUtensorMap &qkv_map = tail.kind == FFN_TAIL_QKV ? *tail.qkv_map : w.w1;
+    FfnTail no_projection = tail;
+    if (tail.kind == FFN_TAIL_QKV) no_projection.kind = FFN_TAIL_LN;
+    auto attempt = [&](auto kernel, int T, int cs, bool projects, size_t smem, PerDeviceValue &known) {
         if (*taken || e != cudaSuccess || chunks < cs) return;
         int resident = 0;
         e = resident_clusters(kernel, cs, smem, known, dev, &resident);
         const int64_t tiles = (M + T - 1) / T;
         if (e != cudaSuccess || tiles > resident) return;
         *taken = true;
-        e = launch_dependent(kernel, dim3((unsigned)(tiles * cs)), dim3(kThreads), smem, stream, cs, w.w1, w.w2_wide, tmAtt32, w.wo_wide, x, g, b, b1, b2, bo,
-                             M, d_ff, eps, tail, err);
+        *projected = projects && tail.kind == FFN_TAIL_QKV;
+        e = launch_dependent(kernel, dim3((unsigned)(tiles * cs)), dim3(kThreads), smem, stream, cs, w.w1, w.w2_wide, tmAtt32, w.wo_wide, qkv_map, x, g, b, b1, b2, bo,
+                             M, d_ff, eps, projects ? tail : no_projection, err);
     };
     static PerDeviceValue known[4];
     // The smallest tile, then the largest cluster with which all tiles still run at once (and every CTA has a chunk): both shorten the
     // chain of a tile, a smaller tile the exchange too.  64 rows only from where two CTAs per 32 rows no longer fit (2400 rows); in
     // clusters of 4 or 8 they lose to 32 rows in half as large clusters (640 rows: 26 us for 32 x 4, 30 us for 64 x 8), and one CTA per
     // tile loses to the clusters of 128-row tiles (5000 rows), weights going through every SM.
-    attempt(ffn_rows_kernel<32, 8>, 32, 8, Shape<32>::kSmemBytes, known[0]);
-    attempt(ffn_rows_kernel<32, 4>, 32, 4, Shape<32>::kSmemBytes, known[1]);
-    attempt(ffn_rows_kernel<32, 2>, 32, 2, Shape<32>::kSmemBytes, known[2]);
-    attempt(ffn_rows_kernel<64, 2>, 64, 2, Shape<64>::kSmemBytes, known[3]);
+    attempt(ffn_rows_kernel<32, 8>, 32, 8, kProjects<8>, Shape<32>::kSmemBytes, known[0]);
+    attempt(ffn_rows_kernel<32, 4>, 32, 4, kProjects<4>, Shape<32>::kSmemBytes, known[1]);
+    attempt(ffn_rows_kernel<32, 2>, 32, 2, kProjects<2>, Shape<32>::kSmemBytes, known[2]);
+    attempt(ffn_rows_kernel<64, 2>, 64, 2, kProjects<2>, Shape<64>::kSmemBytes, known[3]);
     return e;
 }
 

@@ -385,7 +385,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant
                 for (int h = 0; h < 2; ++h) {
                     const float4 y = make_float4(v[h].x * rstd * tg[h].x + tb[h].x, v[h].y * rstd * tg[h].y + tb[h].y,
                                                  v[h].z * rstd * tg[h].z + tb[h].z, v[h].w * rstd * tg[h].w + tb[h].w);
-                    if (tail.kind == FFN_TAIL_LN) {
+                    if (tail.kind != FFN_TAIL_SCORE) {
                         if (row < M && !stopped) *reinterpret_cast<uint2 *>(tail.a + row * kD + c0 + 128 * h) = make_uint2(tc::pack_bf16(y.x, y.y), tc::pack_bf16(y.z, y.w));
                     } else {
                         acc += y.x * tw[h].x + y.y * tw[h].y + y.z * tw[h].z + y.w * tw[h].w;
@@ -412,13 +412,15 @@ bool ffn_fused_supported(int d_model, int d_ff) { return d_model == kD && d_ff %
 
 cudaError_t launch_ffn_fused(const FfnMaps &w, const CUtensorMap &tmX, float *x, const float *g, const float *b, const float *b1,
                              const float *b2, const CUtensorMap &tmAtt, const CUtensorMap &tmAtt32, const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail,
-                             bool *tail_done, int *err, cudaStream_t stream, int64_t *launches)
+                             FfnTailDone *done, int *err, cudaStream_t stream, int64_t *launches)
 {
-    *tail_done = false;
+    *done = FFN_DONE_NOTHING;
     if (M == 0) return cudaSuccess;
     *launches += 1;
-    cudaError_t e = launch_ffn_rows(w, x, g, b, b1, b2, tmAtt32, bo, M, d_ff, eps, tail, err, stream, tail_done);
-    if (e != cudaSuccess || *tail_done) return e;
+    bool taken = false, projected = false;
+    cudaError_t e = launch_ffn_rows(w, x, g, b, b1, b2, tmAtt32, bo, M, d_ff, eps, tail, err, stream, &taken, &projected);
+    if (taken) *done = projected ? FFN_DONE_QKV : FFN_DONE_TAIL;
+    if (e != cudaSuccess || taken) return e;
     int dev = 0, resident = 0;
     e = cudaGetDevice(&dev);
     static PerDeviceValue known;
@@ -428,7 +430,7 @@ cudaError_t launch_ffn_fused(const FfnMaps &w, const CUtensorMap &tmX, float *x,
     // GPU in pairs with 256 rows each.
     const int64_t tiles = (M + kRows - 1) / kRows;
     if (tiles <= resident && d_ff / kChunk >= CS) {
-        *tail_done = true;
+        *done = FFN_DONE_TAIL;
         return launch_dependent(ffn_fused_kernel, dim3((unsigned)(tiles * CS)), dim3(kThreads), (size_t)kSmemBytes, stream, CS, w.w1, w.w2_wide, tmAtt,
                                 w.wo_wide, x, g, b, b1, b2, bo, M, d_ff, eps, tail, err);
     }

@@ -426,7 +426,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     const SeqDesc *seqs_m = d_seqs;
     AttnWork work_m = work;
     bool dead_tail = false;                       // a call without candidates: nothing reads the last layer
-    bool ln_done = false, scored = false;         // the fused kernel of the layer before has taken this layer's LayerNorm 1 / the scores
+    bool ln_done = false, qkv_done = false, scored = false;      // the fused kernel of the layer before has taken this layer's LayerNorm 1 / QKV projection / the scores
 
     // fp32 model, few rows: the GEMM behind a LayerNorm normalises its rows itself
     auto ln_in_gemm = [&](int64_t M, int N) { return !kTensor && !tensor32 && gemm_f32_takes_ln(M, N, d, n_sms); };
@@ -477,7 +477,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
                 if (!ck("gather, LayerNorm and QKV projection")) return RELAYGR_E_CUDA;
             }
         }
-        if (!blocks32) {
+        if (!blocks32 && !qkv_done) {
         const bool ln1_in_gemm = l > 0 && !(last && compact_last) && ln_in_gemm(R, kv_only ? 2 * d : 3 * d);
         if (l == 0) {
             cudaEvent_t pe = prof_begin(stream);
@@ -551,7 +551,16 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
             cudaEvent_t pe = prof_begin(stream);
             FfnTail tail{};
             if (!last) {
-                tail.kind = FFN_TAIL_LN;
+                // (a layer whose candidates are moved together has a projection of its own; a layer that nothing reads has none)
+                const bool next_last = l + 1 == L - 1, next_kv = next_last && preinfer;
+                tail.kind = next_last && (compact_last || (!preinfer && n_scores == 0)) ? FFN_TAIL_LN : FFN_TAIL_QKV;
+                tail.qkv_map = next_kv ? &wmaps[(size_t)l + 1].kv : &wmaps[(size_t)l + 1].qkv;
+                tail.col0 = next_kv ? d : 0; tail.n_qkv = 3 * d - tail.col0;
+                tail.bias = w.b_qkv ? w.b_qkv + (size_t)(l + 1) * 3 * d + tail.col0 : nullptr;
+                tail.q_scale = q_scale;
+                tail.q = reinterpret_cast<__nv_bfloat16 *>(q); tail.k = reinterpret_cast<__nv_bfloat16 *>(kl); tail.v = reinterpret_cast<__nv_bfloat16 *>(vl);
+                if (preinfer) tail.paged = PagedKV{call.pool_slab, meta + o_pt, L, d, l + 1};
+                tail.row_off = d_row_off; tail.seqs = d_seqs; tail.n_users = B;
                 tail.g = w.ln1_g + (size_t)(l + 1) * d; tail.b = w.ln1_b + (size_t)(l + 1) * d; tail.a = reinterpret_cast<__nv_bfloat16 *>(a);
             } else {
                 tail.kind = FFN_TAIL_SCORE;
@@ -559,13 +568,14 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
                 tail.row_off = compact_last ? meta + o_score : d_row_off; tail.seqs = compact_last ? seqs_m : d_seqs;
                 tail.score_off = meta + o_score; tail.n_users = B;
             }
-            bool tail_done = false;
+            FfnTailDone done = FFN_DONE_NOTHING;
             e = launch_ffn_fused(lm->ffn, om_xm->o[0], xm, w.ln2_g + (size_t)l * d, w.ln2_b + (size_t)l * d, w.b1 ? w.b1 + (size_t)l * F : nullptr,
                                  w.b2 ? w.b2 + (size_t)l * d : nullptr, tm_att, tm_att32,
                                  w.b_o ? w.b_o + (size_t)l * d : nullptr, M, (int)F, cfg.ln_eps,
-                                 tail, &tail_done, d_status, stream, &launches);
-            ln_done = tail_done && !last;
-            scored = tail_done && last;
+                                 tail, &done, d_status, stream, &launches);
+            ln_done = done == FFN_DONE_TAIL && !last;
+            qkv_done = done == FFN_DONE_QKV;
+            scored = done == FFN_DONE_TAIL && last;
             prof_end(KC_GEMM, pe, stream);
             if (!ck("output projection + feed-forward")) return RELAYGR_E_CUDA;
             continue;

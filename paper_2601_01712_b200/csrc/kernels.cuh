@@ -158,7 +158,9 @@ struct FfnMaps {                                  // one layer's weights, boxes 
     CUtensorMap w2, w2_wide, wo, wo_wide;         // W2 [256, d_ff] and Wo [256, 256], boxes of 128 and (wide) of 256 rows
 };
 // What the kernel does with finished rows: stores them to x and the next layer's a = LN(x; g, b); or, instead of storing them, the scores of the candidates' rows, w . LN(x; g, b) + bias (users by row_off and seqs, as in launch_score).
-enum FfnTailKind : int { FFN_TAIL_LN = 0, FFN_TAIL_SCORE };
+// FFN_TAIL_QKV: the forms for the fewest rows also make the next layer's QKV projection of LN(x) instead of storing it (others: as FFN_TAIL_LN).
+enum FfnTailKind : int { FFN_TAIL_LN = 0, FFN_TAIL_SCORE, FFN_TAIL_QKV };
+enum FfnTailDone : int { FFN_DONE_NOTHING = 0, FFN_DONE_TAIL, FFN_DONE_QKV };
 struct FfnTail {
     int kind;
     const float *g, *b;
@@ -169,15 +171,22 @@ struct FfnTail {
     const SeqDesc *seqs;          // score_row0, n_score: rows of this launch
     const int32_t *score_off;
     int n_users;
+    // FFN_TAIL_QKV (with row_off, seqs, n_users): columns col0 .. col0 + n_qkv - 1 of [q | k | v] = LN(x) W^T + bias, q times q_scale; k and v
+    // into pages where paged.slab is set.  qkv_map: rows col0 .. of W in boxes of 128 rows x 64 columns.
+    const CUtensorMap *qkv_map;
+    int n_qkv, col0;
+    float q_scale;
+    __nv_bfloat16 *q, *k, *v;
+    PagedKV paged;
 };
 bool ffn_fused_supported(int d_model, int d_ff);
 cudaError_t launch_ffn_fused(const FfnMaps &w, const CUtensorMap &tmX, float *x, const float *g, const float *b, const float *b1,
                              const float *b2, const CUtensorMap &tmAtt, const CUtensorMap &tmAtt32, const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail,
-                             bool *tail_done, int *err, cudaStream_t stream, int64_t *launches);
-// (the form for the fewest rows: *taken tells whether there was one)
+                             FfnTailDone *done, int *err, cudaStream_t stream, int64_t *launches);
+// (the form for the fewest rows: *taken tells whether there was one, *projected whether it made the next projection)
 cudaError_t launch_ffn_rows(const FfnMaps &w, float *x, const float *g, const float *b, const float *b1, const float *b2, const CUtensorMap &tmAtt32,
-                            const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail, int *err, cudaStream_t stream, bool *taken);
-// (the form for many rows, called by the launcher above: it leaves the tail to the caller, *tail_done = false)
+                            const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail, int *err, cudaStream_t stream, bool *taken, bool *projected);
+// (the form for many rows, called by the launcher above: it leaves the tail to the caller)
 cudaError_t launch_ffn_pair(const FfnMaps &w, const CUtensorMap &tmX, const float *x, const float *g, const float *b, const float *b1, const float *b2,
                             const CUtensorMap &tmAtt, const float *bo, int64_t M, int d_ff, float eps, int *err, cudaStream_t stream);
 

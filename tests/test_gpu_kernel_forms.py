@@ -261,3 +261,34 @@ def test_f32_few_rows(d, heads, ff, cand):
 def test_f32_blocks(layers, d, heads, ff, prefix, short, cand):
     shape = synth.ModelShape(layers, d, heads, d // heads, ff, 2000, synth.DTYPE_F32)
     _check_f32(shape, _tiny_batch(shape, 370 + d + ff, prefix, short, cand), 71)
+
+
+# The feed-forward kernel for few rows goes on to the next layer's QKV projection: three layers, so that one projection is followed by
+# another and one by the last layer's (K and V alone in a pre-inference), in each of its forms (clusters of 8 / 4 / 2, 64-row tiles); rows that go to
+# pages ending inside, at and behind a page's last slot; a ragged last tile.
+@pytest.mark.parametrize("prefix,cand", [([1], [1]), ([33, 64, 130, 63], [40, 9, 100, 3]), ([512, 128], [450, 30]), ([700, 301], [590, 333]),
+                                         ([1500, 900], [1100, 700])])
+def test_feed_forward_into_the_next_projection(prefix, cand):
+    shape = synth.ModelShape(3, 256, 4, 64, 1024, 3000, synth.DTYPE_BF16)
+    batch = _tiny_batch(shape, 380 + len(prefix), prefix, [3] * len(prefix), cand)
+    w, model, pool, db = _setup(shape, 72, batch)
+    pool.preinfer(db)
+    scores, full = pool.rank(db).cpu().numpy(), model.rank_full(db).cpu().numpy()
+    assert model.device_status() == 0
+    users = sorted({0, len(prefix) - 1})
+    om = oracle_model(shape, w)
+    want = oracle_scores(om, batch, users=users)
+    max_bound, _, _ = bf16_noise_bounds(shape, w, batch, want)
+    assert max_abs_err(scores, batch, want) <= max_bound
+    assert max_abs_err(full, batch, want) <= max_bound
+    for i in users:
+        p = batch.user_slices(i)[0]
+        K, V = om.preinfer(p)
+        gK, gV = pool.read_kv(batch.users[i], len(p))
+        assert np.max(np.abs(gK.float().cpu().numpy() - K)) <= 5e-2      # as in test_preinfer_rows_in_and_across_pages
+        assert np.max(np.abs(gV.float().cpu().numpy() - V)) <= 5e-2
+        used = len(p) % 64                              # the unused slots of the last page are cleared
+        if used:
+            last = pool.slab.view(torch.bfloat16).view(-1, 3, 2, 64, 256)[int(pool.pages(batch.users[i])[-1])]
+            assert bool(torch.all(last[:, :, used:] == 0))
+    pool.close(); model.close()
