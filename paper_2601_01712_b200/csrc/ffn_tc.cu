@@ -412,15 +412,16 @@ bool ffn_fused_supported(int d_model, int d_ff) { return d_model == kD && d_ff %
 
 cudaError_t launch_ffn_fused(const FfnMaps &w, const CUtensorMap &tmX, float *x, const float *g, const float *b, const float *b1,
                              const float *b2, const CUtensorMap &tmAtt, const CUtensorMap &tmAtt32, const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail,
-                             FfnTailDone *done, int *err, cudaStream_t stream, int64_t *launches)
+                             bool *tail_done, int *err, cudaStream_t stream, int64_t *launches, bool *projected)
 {
-    *done = FFN_DONE_NOTHING;
+    *tail_done = false;
+    if (projected) *projected = false;
     if (M == 0) return cudaSuccess;
     *launches += 1;
-    bool taken = false, projected = false;
-    cudaError_t e = launch_ffn_rows(w, x, g, b, b1, b2, tmAtt32, bo, M, d_ff, eps, tail, err, stream, &taken, &projected);
-    if (taken) *done = projected ? FFN_DONE_QKV : FFN_DONE_TAIL;
-    if (e != cudaSuccess || taken) return e;
+    bool with_projection = false;
+    cudaError_t e = launch_ffn_rows(w, x, g, b, b1, b2, tmAtt32, bo, M, d_ff, eps, tail, err, stream, tail_done, &with_projection);
+    if (projected) *projected = with_projection;
+    if (e != cudaSuccess || *tail_done) return e;
     int dev = 0, resident = 0;
     e = cudaGetDevice(&dev);
     static PerDeviceValue known;
@@ -430,7 +431,7 @@ cudaError_t launch_ffn_fused(const FfnMaps &w, const CUtensorMap &tmX, float *x,
     // GPU in pairs with 256 rows each.
     const int64_t tiles = (M + kRows - 1) / kRows;
     if (tiles <= resident && d_ff / kChunk >= CS) {
-        *done = FFN_DONE_TAIL;
+        *tail_done = true;
         return launch_dependent(ffn_fused_kernel, dim3((unsigned)(tiles * CS)), dim3(kThreads), (size_t)kSmemBytes, stream, CS, w.w1, w.w2_wide, tmAtt,
                                 w.wo_wide, x, g, b, b1, b2, bo, M, d_ff, eps, tail, err);
     }

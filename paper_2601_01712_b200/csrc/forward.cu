@@ -568,14 +568,14 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
                 tail.row_off = compact_last ? meta + o_score : d_row_off; tail.seqs = compact_last ? seqs_m : d_seqs;
                 tail.score_off = meta + o_score; tail.n_users = B;
             }
-            FfnTailDone done = FFN_DONE_NOTHING;
+            bool tail_done = false, projected = false;
             e = launch_ffn_fused(lm->ffn, om_xm->o[0], xm, w.ln2_g + (size_t)l * d, w.ln2_b + (size_t)l * d, w.b1 ? w.b1 + (size_t)l * F : nullptr,
                                  w.b2 ? w.b2 + (size_t)l * d : nullptr, tm_att, tm_att32,
                                  w.b_o ? w.b_o + (size_t)l * d : nullptr, M, (int)F, cfg.ln_eps,
-                                 tail, &done, d_status, stream, &launches);
-            ln_done = done == FFN_DONE_TAIL && !last;
-            qkv_done = done == FFN_DONE_QKV;
-            scored = done == FFN_DONE_TAIL && last;
+                                 tail, &tail_done, d_status, stream, &launches, &projected);
+            ln_done = tail_done && !last;
+            qkv_done = projected;
+            scored = tail_done && last;
             prof_end(KC_GEMM, pe, stream);
             if (!ck("output projection + feed-forward")) return RELAYGR_E_CUDA;
             continue;

@@ -158,9 +158,8 @@ struct FfnMaps {                                  // one layer's weights, boxes 
     CUtensorMap w2, w2_wide, wo, wo_wide;         // W2 [256, d_ff] and Wo [256, 256], boxes of 128 and (wide) of 256 rows
 };
 // What the kernel does with finished rows: stores them to x and the next layer's a = LN(x; g, b); or, instead of storing them, the scores of the candidates' rows, w . LN(x; g, b) + bias (users by row_off and seqs, as in launch_score).
-// FFN_TAIL_QKV: the forms for the fewest rows also make the next layer's QKV projection of LN(x) instead of storing it (others: as FFN_TAIL_LN).
+// FFN_TAIL_QKV: the forms for the fewest rows also make the next layer's QKV projection of LN(x) instead of storing it (*projected; others: as FFN_TAIL_LN).
 enum FfnTailKind : int { FFN_TAIL_LN = 0, FFN_TAIL_SCORE, FFN_TAIL_QKV };
-enum FfnTailDone : int { FFN_DONE_NOTHING = 0, FFN_DONE_TAIL, FFN_DONE_QKV };
 struct FfnTail {
     int kind;
     const float *g, *b;
@@ -182,11 +181,11 @@ struct FfnTail {
 bool ffn_fused_supported(int d_model, int d_ff);
 cudaError_t launch_ffn_fused(const FfnMaps &w, const CUtensorMap &tmX, float *x, const float *g, const float *b, const float *b1,
                              const float *b2, const CUtensorMap &tmAtt, const CUtensorMap &tmAtt32, const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail,
-                             FfnTailDone *done, int *err, cudaStream_t stream, int64_t *launches);
+                             bool *tail_done, int *err, cudaStream_t stream, int64_t *launches, bool *projected = nullptr);
 // (the form for the fewest rows: *taken tells whether there was one, *projected whether it made the next projection)
 cudaError_t launch_ffn_rows(const FfnMaps &w, float *x, const float *g, const float *b, const float *b1, const float *b2, const CUtensorMap &tmAtt32,
                             const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail, int *err, cudaStream_t stream, bool *taken, bool *projected);
-// (the form for many rows, called by the launcher above: it leaves the tail to the caller)
+// (the form for many rows, called by the launcher above: it leaves the tail to the caller, *tail_done = false)
 cudaError_t launch_ffn_pair(const FfnMaps &w, const CUtensorMap &tmX, const float *x, const float *g, const float *b, const float *b1, const float *b2,
                             const CUtensorMap &tmAtt, const float *bo, int64_t M, int d_ff, float eps, int *err, cudaStream_t stream);
 
