@@ -7,25 +7,13 @@
 
 namespace relaygr {
 
-// ---- tensor-core attention work items: one per (user, head, 128-row tile[, KV split]) of the rows in `seqs` ------------------
-// Items are taken in list order by whichever of the machine's slots is free (bf16: two CTAs per SM; fp32: one).  The list is therefore
-// ordered costliest first, and the plan decides how finely to split the key ranges so that the last wave is not a few
-// whole items running on an otherwise idle GPU.  Cost model, in units of one 64-key block of one tile (about 0.7 us):
-// an item costs item_fixed (launch, Q and first K loads, first S, epilogue) plus its key blocks; `slots` items run at a
-// time.  Every item is split `ns` ways; the items left over after the last full wave (the cheapest ones, at the end of
-// the list) are split `nst` times finer still, so that their pieces spread over all slots.  ns is the value with the
-// smallest estimated makespan; a split piece keeps at least kMinSplitBlocks key blocks.
-void build_attention_worklist(const std::vector<SeqDesc> &seqs, int n_heads, const AttnMachine &machine, int64_t max_split_tiles,
-                              std::vector<AttnItem> &items, std::vector<AttnMerge> &merges)
+namespace {
+struct Tile { int seq, q0, n_q, nb; };      // 128 rows of a user; key blocks that any of them sees
+
+std::vector<Tile> tiles_of(const std::vector<SeqDesc> &seqs, int64_t &sum_nb)
 {
-    constexpr double kMergeCost = 5.0;
-    const double item_fixed = machine.item_fixed;
-    constexpr int kMinSplitBlocks = 4, kMaxSplit = 16;
-    items.clear();
-    merges.clear();
-    struct Tile { int seq, q0, n_q, nb; };
     std::vector<Tile> tiles;
-    int64_t sum_nb = 0;
+    sum_nb = 0;
     for (int u = 0; u < (int)seqs.size(); ++u) {
         const SeqDesc &sd = seqs[(size_t)u];
         const int nPB = (sd.n_paged + 63) / 64, nLB = (sd.n_lin + 63) / 64;      // key blocks of 64 (one page each)
@@ -44,6 +32,28 @@ void build_attention_worklist(const std::vector<SeqDesc> &seqs, int n_heads, con
             sum_nb += nb;
         }
     }
+    return tiles;
+}
+}  // namespace
+
+// ---- tensor-core attention work items: one per (user, head, 128-row tile[, KV split]) of the rows in `seqs` ------------------
+// Items are taken in list order by whichever of the machine's slots is free (bf16: two CTAs per SM; fp32: one).  The list is therefore
+// ordered costliest first, and the plan decides how finely to split the key ranges so that the last wave is not a few
+// whole items running on an otherwise idle GPU.  Cost model, in units of one 64-key block of one tile (about 0.7 us):
+// an item costs item_fixed (launch, Q and first K loads, first S, epilogue) plus its key blocks; `slots` items run at a
+// time.  Every item is split `ns` ways; the items left over after the last full wave (the cheapest ones, at the end of
+// the list) are split `nst` times finer still, so that their pieces spread over all slots.  ns is the value with the
+// smallest estimated makespan; a split piece keeps at least kMinSplitBlocks key blocks.
+void build_attention_worklist(const std::vector<SeqDesc> &seqs, int n_heads, const AttnMachine &machine, int64_t max_split_tiles,
+                              std::vector<AttnItem> &items, std::vector<AttnMerge> &merges)
+{
+    constexpr double kMergeCost = 5.0;
+    const double item_fixed = machine.item_fixed;
+    constexpr int kMinSplitBlocks = 4, kMaxSplit = 16;
+    items.clear();
+    merges.clear();
+    int64_t sum_nb = 0;
+    std::vector<Tile> tiles = tiles_of(seqs, sum_nb);
     if (tiles.empty()) return;
     // costliest first (key blocks x softmax warps with live rows); ties keep a user's tiles together (they share K / V through L2)
     std::sort(tiles.begin(), tiles.end(), [](const Tile &x, const Tile &y) {
@@ -105,6 +115,51 @@ void build_attention_worklist(const std::vector<SeqDesc> &seqs, int n_heads, con
             }
         }
     }
+}
+
+// A few tiles, as of a call of one user: pieces that a cluster takes put their results together inside the launch, which saves the merge and its
+// launch, but they are equal in number for every tile, at most eight, and a cluster's CTAs share SMs.  What the longest piece costs decides, in
+// key blocks (about 0.7 us where two CTAs share an SM, 0.7 of that for a CTA alone): the exchange four, merge and launch five.  The longest
+// tile has to have 8 + 2 blocks per piece.  Measured, general plan / clusters in us a call: one user's 512 + 64 rows over 2048 keys 110 /
+// 106 (clusters of 8), over 8000 keys 129 / 136 (14 pieces against 8: not taken), 5 users x 2000 keys 142 / 140, a pre-inference of
+// 2000 tokens 117 / 114, of 2 x 900 115 / 118 (not taken).
+int build_attention_clusters(const std::vector<SeqDesc> &seqs, int n_heads, const AttnMachine &machine, const int (&resident)[3], const std::vector<AttnItem> &general,
+                             bool merges, std::vector<AttnItem> &items)
+{
+    constexpr double kExchangeCost = 4.0, kMergeCost = 5.0, kAlone = 0.7;
+    const int64_t slots = machine.slots, n_sms = slots / 2;
+    if (general.empty() || (int64_t)general.size() > slots) return 1;
+    auto own_blocks = [&](int seq, int q0, int n_q) {
+        const SeqDesc &sd = seqs[(size_t)seq];
+        const int first_cand = std::max(0, sd.causal_end - (sd.q_pos0 + q0));
+        return first_cand < n_q ? (n_q + 63) / 64 - first_cand / 64 : 0;
+    };
+    int longest = 0;
+    for (const AttnItem &it : general) longest = std::max(longest, it.blk1 - it.blk0 + (it.with_self ? own_blocks(it.seq, it.q0, it.n_q) : 0));
+    double best = longest * ((int64_t)general.size() <= n_sms ? kAlone : 1.0) + (merges ? kMergeCost : 0.0);
+    int64_t sum_nb = 0;
+    const std::vector<Tile> tiles = tiles_of(seqs, sum_nb);
+    const int64_t base = (int64_t)tiles.size() * n_heads;
+    int most = 0;
+    for (const Tile &t : tiles) most = std::max(most, t.nb);
+    int best_cs = 1;
+    for (int i = 0; i < 3; ++i) {
+        const int cs = 2 << i;
+        if (base > resident[i] || base * cs > slots || most < 8 + 2 * cs) continue;
+        int piece = 0;
+        for (const Tile &t : tiles) piece = std::max(piece, (t.nb + own_blocks(t.seq, t.q0, t.n_q) + cs - 1) / cs);
+        const double cost = piece * (base * cs <= n_sms / 2 ? kAlone : 1.0) + kExchangeCost;
+        if (cost < best) { best = cost; best_cs = cs; }
+    }
+    if (best_cs == 1) return 1;
+    items.clear();
+    for (const Tile &t : tiles) {
+        const int n_diag = own_blocks(t.seq, t.q0, t.n_q);      // of the first piece
+        auto cut = [&](int i) { return i == best_cs ? t.nb : (int)std::max<int64_t>(0, (int64_t)(t.nb + n_diag) * i / best_cs - n_diag); };
+        for (int h = 0; h < n_heads; ++h)
+            for (int i = 0; i < best_cs; ++i) items.push_back({t.seq, h, t.q0, t.n_q, cut(i), cut(i + 1), 0, i == 0 && n_diag > 0 ? 1 : 0});
+    }
+    return best_cs;
 }
 
 }  // namespace relaygr

@@ -51,8 +51,7 @@ constexpr int kQBytes = kQTile * kDh * 2;           // 16 KB
 constexpr int kKVBytes = kKeys * kDh * 2;           // 8 KB per K or V tile
 constexpr int kOffloadPairs = 4;                            // of every 16 pairs of exponentials, evenly spread, run on the FMA pipe (exp2_fma_pipe)
 constexpr bool offloaded(int pair) { return (pair + 1) * kOffloadPairs / 16 != pair * kOffloadPairs / 16; }
-constexpr int kStagesKV = 4;
-constexpr int kSmemBytes = kQBytes + 2 * kStagesKV * kKVBytes + 1024 + 512;
+constexpr int kMaxStagesKV = 4;
 constexpr uint32_t kTmemCols = 256;                 // S[2]: 0..127, P[2]: 128..191, O: 192..255
 constexpr uint32_t kColS = 0, kColP = 128, kColO = 192;
 constexpr int kPartStride = kDh + 4;                // floats per row of a split partial: m, l, two unused, then O (16-byte aligned rows)
@@ -62,6 +61,16 @@ constexpr int kPartStride = kDh + 4;                // floats per row of a split
 constexpr float kZeroRef = 32.f;
 constexpr float kRaise = 54.f;                      // a score this far above the reference raises it ...
 constexpr float kRowSumLimit = 0x1p60f;             // ... which a block's row sum shows: 64 weights
+
+// CS > 1: the CS pieces of a tile's key range are the CTAs of a cluster, which put their results together themselves (merge_rows): a
+// ring stage less makes room for them.
+template <int CS> struct Shape {
+    static constexpr int kStagesKV = CS > 1 ? 3 : kMaxStagesKV;
+    static constexpr int kOffMerge = kQBytes + 2 * kStagesKV * kKVBytes, kMergeBytes = CS > 1 ? kQTile * kPartStride * 4 : 0;
+    static constexpr int kOffBars = kOffMerge + kMergeBytes;
+    static constexpr int kSmemBytes = kOffBars + 1024 + 512;
+    static_assert(2 * (kSmemBytes + 1024) <= 228 * 1024, "two CTAs per SM");
+};
 
 // A work item as the producer hands it to the other warps (nb_keys < 0: no more).
 struct ItemInfo {
@@ -73,7 +82,8 @@ struct ItemInfo {
 
 struct Bars {
     uint64_t q_full, q_empty;
-    uint64_t k_full[kStagesKV], k_empty[kStagesKV], v_full[kStagesKV], v_empty[kStagesKV];
+    uint64_t k_full[kMaxStagesKV], k_empty[kMaxStagesKV], v_full[kMaxStagesKV], v_empty[kMaxStagesKV];
+    uint64_t merge_full;         // clusters: all partial results of this CTA's rows are here
     uint64_t s_full[2], p_full[2], p_free[2];
     uint64_t item_full[2], item_empty[2];
     ItemInfo ring[2];            // items on their way from the producer to the other warps
@@ -130,9 +140,43 @@ __device__ __forceinline__ void own_key_blocks(const AttnItem &it, const SeqDesc
     }
 }
 
+// O = sum_i 2^(m_i - M) O_i / sum_i 2^(m_i - M) l_i of the 128 / CS rows that this CTA finishes, from `parts` [CS][rows][kPartStride]: CS threads
+// a row, each 64 / CS columns, the partial results in rank order.  Called by the softmax warps.
+template <int CS>
+__device__ __forceinline__ void merge_rows(const float *parts, int64_t row0, int n_q, int col, int d_model, __nv_bfloat16 *out)
+{
+    constexpr int kRows = kQTile / CS, kCols = kDh / CS;
+    const int t = threadIdx.x - 64, row = t / CS, c0 = (t % CS) * kCols, r = (int)tc::cluster_ctarank() * kRows + row;
+    if (r >= n_q) return;
+    const float *p = parts + row * kPartStride;
+    float2 ml[CS];
+    float M = -INFINITY, l = 0.f, o[kCols] = {};
+#pragma unroll
+    for (int i = 0; i < CS; ++i) {
+        ml[i] = *reinterpret_cast<const float2 *>(p + i * (kRows * kPartStride));
+        M = fmaxf(M, ml[i].x);
+    }
+#pragma unroll
+    for (int i = 0; i < CS; ++i) {
+        const float w = ml[i].x == -INFINITY ? 0.f : ex2(ml[i].x - M);
+        l = fmaf(ml[i].y, w, l);
+#pragma unroll
+        for (int c = 0; c < kCols; c += 4) {
+            const float4 v = *reinterpret_cast<const float4 *>(p + i * (kRows * kPartStride) + 4 + c0 + c);
+            o[c] = fmaf(v.x, w, o[c]); o[c + 1] = fmaf(v.y, w, o[c + 1]); o[c + 2] = fmaf(v.z, w, o[c + 2]); o[c + 3] = fmaf(v.w, w, o[c + 3]);
+        }
+    }
+    const float inv = 1.f / l;
+    __nv_bfloat16 *dst = out + (row0 + r) * d_model + col + c0;
+#pragma unroll
+    for (int c = 0; c < kCols; c += 8)
+        *reinterpret_cast<uint4 *>(dst + c) = make_uint4(tc::pack_bf16(o[c] * inv, o[c + 1] * inv), tc::pack_bf16(o[c + 2] * inv, o[c + 3] * inv),
+                                                         tc::pack_bf16(o[c + 4] * inv, o[c + 5] * inv), tc::pack_bf16(o[c + 6] * inv, o[c + 7] * inv));
+}
+
 // kPointwise: pointwise aggregated attention (HSTU style) - the weight of a visible key is SiLU(q.k / sqrt(d_h)) and the
 // sum is divided by the number of visible keys; no running maximum, no row sum, no rescaling of O.
-template <bool kPointwise>
+template <bool kPointwise, int CS>
 __global__ void __launch_bounds__(192, 2)
 attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKlin,
                     const __grid_constant__ CUtensorMap tmVlin, const __grid_constant__ CUtensorMap tmPool,
@@ -140,12 +184,13 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     const int32_t *__restrict__ pt, int n_layers, int layer, int d_model, bool early_pages, __nv_bfloat16 *__restrict__ out,
                     float *__restrict__ partial, int *err)
 {
+    constexpr int kStagesKV = Shape<CS>::kStagesKV;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t *sQ = smem;
     uint8_t *sK = smem + kQBytes;
     uint8_t *sV = sK + kStagesKV * kKVBytes;
-    Bars *bars = reinterpret_cast<Bars *>(sV + kStagesKV * kKVBytes);
+    Bars *bars = reinterpret_cast<Bars *>(smem + Shape<CS>::kOffBars);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // set-up that touches nothing earlier kernels wrote; it may run while the previous kernel is still finishing
@@ -160,7 +205,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             tc::mbar_init(&bars->p_full[b], 4); tc::mbar_init(&bars->p_free[b], 1);
             tc::mbar_init(&bars->item_full[b], 1); tc::mbar_init(&bars->item_empty[b], 5);     // MMA warp + four softmax warps
         }
+        tc::mbar_init(&bars->merge_full, 1);
         tc::fence_mbar_init();
+        if constexpr (CS > 1) tc::mbar_expect_tx(&bars->merge_full, Shape<CS>::kMergeBytes);
         tc::tma_prefetch_desc(&tmQ); tc::tma_prefetch_desc(&tmKlin); tc::tma_prefetch_desc(&tmVlin); tc::tma_prefetch_desc(&tmPool);
     }
     if (warp == 1) {
@@ -175,7 +222,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     int nb = 0, d0 = 0, n_diag = 0, n_page_blocks = 0, g = 0, j0 = 0;      // of the item: key blocks in all, its own-key blocks, the user's pages
     auto draw_item = [&](int n) {                     // this CTA's n-th item into ring slot n & 1; false: no more
         const int slot = n & 1;
-        const int idx = n == 0 ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(next_item, 1);
+        // (the CTAs of a cluster have one item each)
+        const int idx = n == 0 ? (int)blockIdx.x : CS > 1 ? n_items : (int)gridDim.x + atomicAdd(next_item, 1);
         ItemInfo &info = bars->ring[slot];
         const bool more = idx < n_items;
         if (more) {
@@ -228,6 +276,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     if (threadIdx.x == 64) bars->abort_flag = *reinterpret_cast<volatile int *>(err);
     tc::tc_fence_before();
     __syncthreads();
+    if constexpr (CS > 1) tc::cluster_sync();                     // the peers' barriers exist before anything is sent
     tc::tc_fence_after();
     const uint32_t tmem_base = bars->tmem_slot;
     const bool live = bars->abort_flag == 0;
@@ -249,6 +298,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         return info;
     };
 
+    int64_t merge_row0 = 0;                                       // clusters: of the item, once this thread has sent its row
+    int merge_n_q = 0, merge_col = 0;
     if (!live) {
         if (threadIdx.x == 0)                                     // what was requested above lands before the CTA ends
             for (int s = 0; s < j0; ++s) { tc::mbar_wait(&bars->k_full[s], 0, err); tc::mbar_wait(&bars->v_full[s], 0, err); }
@@ -327,6 +378,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         }
     } else {
         // ---------------------------------------------------------------- softmax / correction / epilogue
+        float *merge = reinterpret_cast<float *>(smem + Shape<CS>::kOffMerge);
         const int quad = warp & 3;
         const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
         bool ok = true;
@@ -542,7 +594,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         if (nb > 0) ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->p_free[(g + nb - 1) & 1], ((g + nb - 1) >> 1) & 1, err));
         if (!ok) break;
         tc::tc_fence_after();
-        if (ok && warp_live) {
+        if (ok && (CS > 1 || warp_live)) {                    // (rows past the tile's last one are sent as well: the receiver counts bytes)
             float o[kDh];
             if (nb > 0) {
                 uint32_t ov[2][32];
@@ -562,7 +614,21 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 // a candidate); a split item hands it over as l with m = 0, so that the merge of partials needs no change
                 const float n_seen = (float)(is_cand ? it.causal_end + 1 : tpos + 1);
                 m = 0.f;
-                l = (it.partial_slot < 0 || it.blk0 == 0) ? n_seen : 0.f;
+                l = (CS > 1 ? tc::cluster_ctarank() == 0 : it.partial_slot < 0 || it.blk0 == 0) ? n_seen : 0.f;
+            }
+            if constexpr (CS > 1) {
+                // row r goes to the CTA that finishes it, r / (128 / CS), behind the rows of the ranks below this one
+                constexpr int kRows = kQTile / CS;
+                const int to = r / kRows;
+                const float *slot = merge + (tc::cluster_ctarank() * kRows + r % kRows) * kPartStride;
+                const uint32_t dst = tc::cluster_addr(slot, to), bar = tc::cluster_addr(&bars->merge_full, to);
+                tc::st_async16(dst, make_float4(m, l, 0.f, 0.f), bar);
+#pragma unroll
+                for (int i = 0; i < kDh / 4; ++i) tc::st_async16(dst + 16 * (i + 1), make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]), bar);
+                merge_row0 = it.row0;
+                merge_n_q = it.n_q;
+                merge_col = it.head * kDh;
+                continue;
             }
             if (row_ok) {
                 if (it.partial_slot < 0) {
@@ -587,6 +653,14 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         }
         g += nb;
         }   // items
+    }
+    if constexpr (CS > 1) {
+        __syncwarp();
+        tc::cluster_arrive_relaxed();                             // nobody ends before everybody has sent its rows
+        if (warp >= 2 && merge_n_q > 0 && __all_sync(0xffffffffu, tc::mbar_wait(&bars->merge_full, 0, err)))
+            merge_rows<CS>(reinterpret_cast<const float *>(smem + Shape<CS>::kOffMerge), merge_row0, merge_n_q, merge_col, d_model, out);
+        __syncwarp();
+        tc::cluster_wait();
     }
     tc::tc_fence_before();
     __syncthreads();
@@ -650,27 +724,69 @@ attention_merge_kernel(const AttnMerge *__restrict__ merges, const SeqDesc *__re
 
 }  // namespace
 
+namespace {
+
+template <int CS>
+cudaError_t launch_cs(const CUtensorMap &tmQ, const CUtensorMap &tmK, const CUtensorMap &tmV, const CUtensorMap &tmPool, const AttnItem *items, int n_items,
+                      const SeqDesc *seqs, const int32_t *pt, int n_layers, int layer, int d_model, int attn_kind, bool early_pages, __nv_bfloat16 *out,
+                      float *partial, int *next_item, int n_sms, int *err, cudaStream_t stream)
+{
+    static PerDeviceValue attr_set;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (!attr_set.get(dev)) {
+        e = cudaFuncSetAttribute(attention_tc_kernel<false, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<CS>::kSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(attention_tc_kernel<true, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<CS>::kSmemBytes);
+        if (e != cudaSuccess) return e;
+        attr_set.set(dev, 1);
+    }
+    auto kernel = attn_kind == ATTN_POINTWISE ? attention_tc_kernel<true, CS> : attention_tc_kernel<false, CS>;
+    // two CTAs per SM, each drawing items until none is left; or one item to a CTA
+    const int grid = CS > 1 ? n_items : std::min(n_items, 2 * std::max(1, n_sms));
+    return launch_dependent(kernel, dim3(grid), dim3(192), (size_t)Shape<CS>::kSmemBytes, stream, CS, tmQ, tmK, tmV, tmPool, items,
+                            n_items, next_item, seqs, pt, n_layers, layer, d_model, early_pages, out, partial, err);
+}
+
+// How many clusters run at once.  The occupancy query answers for one CTA per SM (74, 33 and 15 clusters of 2, 4 and 8 on a B200); two fit an SM,
+// clusters of one beside those of another: a launch of 20 of 8 or 64 of 4 runs in one round, one of 36 of 8 takes a second.
+template <int CS>
+int resident_clusters(int n_sms)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(CS * 64); cfg.blockDim = dim3(192); cfg.dynamicSmemBytes = Shape<CS>::kSmemBytes;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = CS; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    auto count = [&](auto kernel) {
+        int n = 0, per_sm = 0;
+        const bool ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<CS>::kSmemBytes) == cudaSuccess &&
+                        cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess &&
+                        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 192, Shape<CS>::kSmemBytes) == cudaSuccess;
+        return !ok ? 0 : n * CS <= n_sms ? n * std::max(1, per_sm) : n;
+    };
+    return std::min(count(attention_tc_kernel<false, CS>), count(attention_tc_kernel<true, CS>));
+}
+
+}  // namespace
+
+void attention_clusters(int n_sms, int (&resident)[3])
+{
+    resident[0] = resident_clusters<2>(n_sms); resident[1] = resident_clusters<4>(n_sms); resident[2] = resident_clusters<8>(n_sms);
+    cudaGetLastError();                               // (a size that the device does not have is an answer, not an error)
+}
+
 cudaError_t launch_attention_tc(const CUtensorMap &tmQ, const CUtensorMap &tmK, const CUtensorMap &tmV, const CUtensorMap &tmPool,
-                                const AttnItem *items, int n_items, const AttnMerge *merges, int n_merges, const SeqDesc *seqs,
+                                const AttnItem *items, int n_items, int cluster, const AttnMerge *merges, int n_merges, const SeqDesc *seqs,
                                 const int32_t *pt, int n_layers, int layer, int d_model, int attn_kind, bool early_pages, __nv_bfloat16 *out,
                                 float *partial, int *next_item, int n_sms, int *err, cudaStream_t stream, int64_t *launches)
 {
     if (n_items == 0) return cudaSuccess;
-    static PerDeviceValue attr_set;
-    int dev = 0;
-    cudaError_t e0 = cudaGetDevice(&dev);
-    if (e0 != cudaSuccess) return e0;
-    if (!attr_set.get(dev)) {
-        cudaError_t e = cudaFuncSetAttribute(attention_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(attention_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e != cudaSuccess) return e;
-        attr_set.set(dev, 1);
-    }
     *launches += 1;
-    auto kernel = attn_kind == ATTN_POINTWISE ? attention_tc_kernel<true> : attention_tc_kernel<false>;
-    const int grid = std::min(n_items, 2 * std::max(1, n_sms));       // two CTAs per SM, each drawing items until none is left
-    cudaError_t e = launch_dependent(kernel, dim3(grid), dim3(192), (size_t)kSmemBytes, stream, 1, tmQ, tmK, tmV, tmPool, items,
-                                     n_items, next_item, seqs, pt, n_layers, layer, d_model, early_pages, out, partial, err);
+    auto launch = cluster == 8 ? launch_cs<8> : cluster == 4 ? launch_cs<4> : cluster == 2 ? launch_cs<2> : launch_cs<1>;
+    cudaError_t e = launch(tmQ, tmK, tmV, tmPool, items, n_items, seqs, pt, n_layers, layer, d_model, attn_kind, early_pages, out, partial, next_item,
+                           n_sms, err, stream);
     if (e != cudaSuccess || n_merges == 0) return e;
     *launches += 1;
     // few rows to merge have many partials each, and registers for all of them; with many rows the occupancy counts

@@ -100,6 +100,7 @@ int Forward::init_device(int dev, std::string &err)
             if (rc != 0) { err = "tensor-map encoding of the weights failed (pointers must be 16-byte aligned)"; return RELAYGR_E_CUDA; }
         }
         wmaps_ok = true;
+        attention_clusters(n_sms, attn_clusters);
     } else if (cfg.d_model >= 32 && cfg.d_ff >= 32) {
         const uint64_t d = (uint64_t)cfg.d_model, F = (uint64_t)cfg.d_ff;
         wmaps.resize((size_t)cfg.n_layers);
@@ -276,7 +277,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
     std::vector<SeqDesc> seqs_c;                  // the candidates of each user as rows of their own (last layer)
     size_t o_seq_c = 0;
     // the work of an attention launch over some descriptors: items and merges (tensor cores), or query tiles (CUDA cores)
-    struct AttnWork { bool tensor = false; size_t o_items = 0, o_merges = 0; int n_items = 0, n_merges = 0, tile_rows = 0; };
+    struct AttnWork { bool tensor = false; size_t o_items = 0, o_merges = 0; int n_items = 0, n_merges = 0, tile_rows = 0, cluster = 1; };
     AttnWork work, work_c;
     auto put_work = [&](const std::vector<SeqDesc> &seqs) {
         AttnWork wk;
@@ -285,6 +286,9 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
             std::vector<AttnItem> it;
             std::vector<AttnMerge> mg;
             build_attention_worklist(seqs, H, kTensor ? attn_machine_bf16(n_sms) : attn_machine_f32(n_sms), kMaxSplitTiles, it, mg);
+            std::vector<AttnItem> pieces;
+            if (kTensor) wk.cluster = build_attention_clusters(seqs, H, attn_machine_bf16(n_sms), attn_clusters, it, !mg.empty(), pieces);
+            if (wk.cluster > 1) { it.swap(pieces); mg.clear(); }
             if (!it.empty()) wk.o_items = put(reinterpret_cast<const int32_t *>(it.data()), it.size() * (sizeof(AttnItem) / 4));
             if (!mg.empty()) wk.o_merges = put(reinterpret_cast<const int32_t *>(mg.data()), mg.size() * (sizeof(AttnMerge) / 4));
             wk.n_items = (int)it.size(); wk.n_merges = (int)mg.size();
@@ -533,7 +537,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
             const AttnItem *items_m = reinterpret_cast<const AttnItem *>(meta + work_m.o_items);
             const AttnMerge *merges_m = reinterpret_cast<const AttnMerge *>(meta + work_m.o_merges);
             if constexpr (kTensor)
-                e = launch_attention_tc(tm_q, tm_k, tm_v, tm_pool, items_m, work_m.n_items, merges_m, work_m.n_merges, seqs_m, meta + o_pt, L,
+                e = launch_attention_tc(tm_q, tm_k, tm_v, tm_pool, items_m, work_m.n_items, work_m.cluster, merges_m, work_m.n_merges, seqs_m, meta + o_pt, L,
                                         l, d, cfg.attn_kind, call.mode == MODE_RANK, att, reinterpret_cast<float *>(ws + lay.partial),
                                         reinterpret_cast<int *>(ws + lay.meta) + o_ctr + l, n_sms, d_status, stream, &launches);
             else if (work_m.tensor)

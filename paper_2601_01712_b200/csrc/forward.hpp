@@ -24,6 +24,10 @@ inline AttnMachine attn_machine_bf16(int n_sms) { return {2 * (int64_t)(n_sms < 
 inline AttnMachine attn_machine_f32(int n_sms) { return {(int64_t)(n_sms < 1 ? 1 : n_sms), 4.0}; }           // one CTA per SM, blocks of about 1.5 us
 void build_attention_worklist(const std::vector<SeqDesc> &seqs, int n_heads, const AttnMachine &machine, int64_t max_split_tiles,
                               std::vector<AttnItem> &items, std::vector<AttnMerge> &merges);
+// The same launch in clusters, where that is better than its general plan (`general`, with merges or without): every tile in as many pieces, which
+// the CTAs of a cluster take together.  resident: how many clusters of 2, 4 and 8 can run at once.  Returns the size, or 1 (items is not touched).
+int build_attention_clusters(const std::vector<SeqDesc> &seqs, int n_heads, const AttnMachine &machine, const int (&resident)[3], const std::vector<AttnItem> &general,
+                             bool merges, std::vector<AttnItem> &items);
 
 struct CallDesc {
     int mode = MODE_RANK;
@@ -50,6 +54,7 @@ struct Forward {
     int64_t launches = 0;
     int device = 0;
     int n_sms = 148;
+    int attn_clusters[3] = {0, 0, 0};      // how many clusters of 2, 4 and 8 CTAs of the attention kernel the device holds at once (bf16 model)
 
     // tensor maps of the weights, one set per layer
     struct LayerMaps { CUtensorMap qkv, kv, wq; FfnMaps ffn; };

@@ -197,8 +197,11 @@ cudaError_t launch_ffn_pair(const FfnMaps &w, const CUtensorMap &tmX, const floa
 // a device counter that must be zero when the kernel starts and belongs to this launch alone (the kernel leaves it non-zero).
 // items, seqs, pt and the counter must be in place when the kernel BEFORE this one on the stream starts; early_pages: so are the
 // pages (the call does not write them).
+// cluster > 1 (2, 4 or 8, of which attention_clusters() says how many the current device holds at once): every `cluster` consecutive items are the pieces of one tile in rank order,
+// put together inside the launch; no merges.
+void attention_clusters(int n_sms, int (&resident)[3]);
 cudaError_t launch_attention_tc(const CUtensorMap &tmQ, const CUtensorMap &tmK, const CUtensorMap &tmV, const CUtensorMap &tmPool,
-                                const AttnItem *items, int n_items, const AttnMerge *merges, int n_merges, const SeqDesc *seqs,
+                                const AttnItem *items, int n_items, int cluster, const AttnMerge *merges, int n_merges, const SeqDesc *seqs,
                                 const int32_t *pt, int n_layers, int layer, int d_model, int attn_kind, bool early_pages, __nv_bfloat16 *out,
                                 float *partial, int *next_item, int n_sms, int *err, cudaStream_t stream, int64_t *launches);
 

@@ -170,6 +170,11 @@ __device__ __forceinline__ void st_async8(uint32_t addr, uint2 v, uint32_t bar)
 {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(bar) : "memory");
 }
+__device__ __forceinline__ void st_async16(uint32_t addr, float4 v, uint32_t bar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar) : "memory");
+}
 // 2-D tile load into this CTA's shared memory whose bytes are counted on a barrier of either CTA of the pair.
 __device__ __forceinline__ void tma_load_2d_pair(void *smem_dst, const CUtensorMap *m, int x, int y, uint32_t bar_cluster_addr)
 {

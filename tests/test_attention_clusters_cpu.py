@@ -1,0 +1,92 @@
+"""The plan of an attention launch in clusters, on the host: its pieces against the tiles of the general plan."""
+import os
+import random
+import subprocess
+
+import pytest
+
+from paper_2601_01712_b200 import build
+
+MAIN = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "forward.hpp"
+using namespace relaygr;
+int main(int argc, char **argv)                      // heads, resident clusters of 2, 4, 8, then P:S:C of every user (C < 0: a pre-inference)
+{
+    const int heads = atoi(argv[1]), resident[3] = {atoi(argv[2]), atoi(argv[3]), atoi(argv[4])};
+    std::vector<SeqDesc> seqs;
+    for (int i = 5; i < argc; ++i) {
+        int p = 0, s = 0, c = 0;
+        sscanf(argv[i], "%d:%d:%d", &p, &s, &c);
+        SeqDesc d{};
+        d.n_paged = p;
+        if (c < 0) { d.n_q = d.causal_end = d.lin_pos0 = p; }
+        else { d.n_q = s + c; d.q_pos0 = d.lin_pos0 = p; d.n_lin = s; d.causal_end = p + s; }
+        seqs.push_back(d);
+    }
+    std::vector<AttnItem> general, items;
+    std::vector<AttnMerge> merges;
+    build_attention_worklist(seqs, heads, attn_machine_bf16(148), 1536, general, merges);
+    const int cs = build_attention_clusters(seqs, heads, attn_machine_bf16(148), resident, general, !merges.empty(), items);
+    printf("%d\n", cs);
+    for (const AttnItem &it : general) printf("g %d %d %d %d %d %d %d\n", it.seq, it.head, it.q0, it.n_q, it.blk0, it.blk1, it.with_self);
+    for (const AttnItem &it : items) printf("c %d %d %d %d %d %d %d\n", it.seq, it.head, it.q0, it.n_q, it.blk0, it.blk1, it.with_self);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def plan(tmp_path_factory):
+    d = tmp_path_factory.mktemp("clusters")
+    (d / "main.cu").write_text(MAIN)
+    r = subprocess.run(["nvcc", "-gencode", "arch=compute_100a,code=compute_100a", "-std=c++17", "--expt-relaxed-constexpr", "-I", build.INCLUDE, "-I", build.CSRC,
+                        "-o", str(d / "plan"), str(d / "main.cu"), "-x", "cu", os.path.join(build.CSRC, "attn_plan.cpp")], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+
+    def run(heads, users, resident=(148, 74, 30)):
+        out = subprocess.run([str(d / "plan"), str(heads), *map(str, resident), *("%d:%d:%d" % u for u in users)], capture_output=True, text=True,
+                             check=True).stdout.split("\n")
+        rows = [line.split() for line in out[1:] if line]
+        return int(out[0]), [tuple(map(int, r[1:])) for r in rows if r[0] == "g"], [tuple(map(int, r[1:])) for r in rows if r[0] == "c"]
+    return run
+
+
+def _tiles(items):
+    """(user, head, first row, rows) -> key blocks covered, items with the own keys."""
+    out = {}
+    for seq, head, q0, n_q, b0, b1, own in items:
+        blocks, owns = out.setdefault((seq, head, q0, n_q), ([], []))
+        blocks.extend(range(b0, b1))
+        owns.append(own)
+    return {k: (sorted(v[0]), sum(v[1])) for k, v in out.items()}
+
+
+def test_pieces_cover_what_the_general_plan_covers(plan):
+    rng = random.Random(5)
+    sizes = set()
+    for _ in range(150):
+        heads = rng.choice([1, 2, 4, 8])
+        users = [(rng.randint(1, 3000), rng.randint(0, 100), rng.choice([-1, 0, 1, 60, 300, 600])) for _ in range(rng.choice([1, 1, 2, 3, 6]))]
+        if any(c < 0 for _, _, c in users):
+            users = [(p, 0, -1) for p, _, _ in users]
+        cs, general, pieces = plan(heads, users)
+        sizes.add(cs)
+        if cs == 1:
+            assert not pieces
+            continue
+        assert len(pieces) % cs == 0 and len(pieces) <= 296 and len(pieces) // cs <= {2: 148, 4: 74, 8: 30}[cs]
+        assert _tiles(pieces) == _tiles(general)
+        for i in range(0, len(pieces), cs):               # a cluster: one tile, its key blocks in rank order, its own keys with the first rank
+            group = pieces[i:i + cs]
+            assert len({g[:4] for g in group}) == 1
+            assert group[0][4] == 0 and all(a[5] == b[4] for a, b in zip(group, group[1:])) and all(g[4] <= g[5] for g in group)
+            assert not any(g[6] for g in group[1:])
+    assert sizes == {1, 2, 4, 8}
+
+
+def test_a_device_without_room_for_the_clusters_keeps_the_general_plan(plan):
+    assert plan(4, [(2048, 64, 512)])[0] == 8
+    assert plan(4, [(2048, 64, 512)], (148, 74, 19))[0] < 8      # 20 tiles
+    assert plan(4, [(2048, 64, 512)], (0, 0, 0))[0] == 1
+    assert plan(4, [(2048, 64, 512)] * 32)[0] == 1                # more items than run at once

@@ -292,3 +292,27 @@ def test_feed_forward_into_the_next_projection(prefix, cand):
             last = pool.slab.view(torch.bfloat16).view(-1, 3, 2, 64, 256)[int(pool.pages(batch.users[i])[-1])]
             assert bool(torch.all(last[:, :, used:] == 0))
     pool.close(); model.close()
+
+
+# Few tiles: the pieces of a tile's keys are a cluster that puts its results together (2, 4 and 8 CTAs; pieces without a key block, which the
+# first tiles of a causal pass have; tiles with a few rows, candidates' own keys in the first piece; both attention kinds), and just too
+# many tiles or too few keys for it.
+@pytest.mark.parametrize("prefix,short,cand", [([700], [5], [1]), ([1100], [0], [130]), ([1600], [64], [600]), ([2100], [64], [512]), ([1990, 800], [3, 0], [20, 200]),
+                                               ([800] * 9, [3] * 9, [200] * 9), ([640], [3], [40]), ([768], [0], [60])])
+@pytest.mark.parametrize("kind", [0, 1])
+def test_attention_clusters(prefix, short, cand, kind):
+    shape = small_bf16_shape(vocab=3000, attn_kind=kind)
+    batch = _tiny_batch(shape, 390 + len(prefix), prefix, short, cand)
+    w, model, pool, db = _setup(shape, 73, batch)
+    pool.preinfer(db)
+    scores, full = pool.rank(db).cpu().numpy(), model.rank_full(db).cpu().numpy()
+    again = pool.rank(db).cpu().numpy()
+    assert model.device_status() == 0
+    assert np.array_equal(scores, again)
+    users = sorted({0, len(prefix) - 1})
+    om = oracle_model(shape, w)
+    want = oracle_scores(om, batch, users=users)
+    max_bound, _, _ = bf16_noise_bounds(shape, w, batch, want)
+    assert max_abs_err(scores, batch, want) <= max_bound
+    assert max_abs_err(full, batch, want) <= max_bound
+    pool.close(); model.close()
