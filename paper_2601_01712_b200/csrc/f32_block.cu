@@ -54,6 +54,7 @@ __host__ __device__ inline Layout layout_of(int d, int F, int tail_n, bool first
 __device__ __forceinline__ void load_matrix(float *dst, const float *W, int n, int k)      // [n, k] row by row
 {
     const int per_row = k / 4;
+#pragma unroll 1
     for (int i = threadIdx.x; i < n * per_row; i += kThreads) {
         const int r = i / per_row, c = (i - r * per_row) * 4;
         cp_async16(dst + r * (k + 4) + c, W + (size_t)r * k + c);
@@ -72,6 +73,7 @@ __device__ __forceinline__ void dot(float (&sum)[NI][BR / 4], const float *W, in
     const float *w = W + (size_t)min(n, n_end - 1) * (K + 4);
     const size_t w_step = (size_t)step * (K + 4);
     const bool second = NI > 1 && n + step < n_end;
+#pragma unroll 1
     for (int k = ks * 8; k < K; k += 8 * LANES) {
         ulonglong2 wv[NI][2];
 #pragma unroll
@@ -231,6 +233,7 @@ f32_block_kernel(F32First first, F32BlockWeights wt, F32BlockTail tail, float *_
             if (lane + 32 < d) a_s[warp * lda + lane + 32] = v[1];
         }
         __syncthreads();
+#pragma unroll 1
         for (int n = slot4; n - slot4 < F; n += 256) {      // hidden values (all lanes of a warp go round together)
             float s[2][BR / 4];
             dot<BR, 2, 4>(s, smem + L.w1, n, 128, F, d, a_s, lda);
@@ -276,6 +279,7 @@ f32_block_kernel(F32First first, F32BlockWeights wt, F32BlockTail tail, float *_
     if (kFirst) cp_async_wait();
     __syncthreads();
     const Epilogue &e = tail.e;
+#pragma unroll 1
     for (int n = slot4; n - slot4 < tail.n; n += 256) {
         float s[2][BR / 4];
         dot<BR, 2, 4>(s, smem + L.wt, n, 128, tail.n, d, a_s, lda);

@@ -273,7 +273,7 @@ template <int DH, int RT, int G> struct AttnSmem {
 template <int DH, int RT, int G, bool kPointwise>
 __global__ void __launch_bounds__(64 * G, RT == 8 ? 4 / G : G == 1 && DH == 32 ? 8 : 1)
 f32_attention_kernel(const float *__restrict__ q, const float *__restrict__ k_lin, const float *__restrict__ v_lin, PagedKV paged,
-                     const SeqDesc *__restrict__ seqs, const F32Tile *__restrict__ tiles, int n_heads, float *__restrict__ out)
+                     const SeqDesc *__restrict__ seqs, const F32Tile *__restrict__ tiles, int n_heads, bool early_pages, float *__restrict__ out)
 {
     using L = AttnSmem<DH, RT, G>;
     constexpr int CT = DH / 8, BQ = 8 * RT;             // CT: output dimensions per thread
@@ -296,7 +296,6 @@ f32_attention_kernel(const float *__restrict__ q, const float *__restrict__ k_li
     const int n_page_blocks = (n_page_keys + 63) >> 6, n_blocks = n_page_blocks + ((n_lin_keys + 63) >> 6);
     auto group_sync = [&] { asm volatile("bar.sync %0, 64;" ::"r"(1 + grp) : "memory"); };
     const int page_first = grp < n_page_blocks ? paged.pt[sd.pt_base + grp] : 0;      // of the group's first block
-    grid_dependency_wait();
     int b_pos = 0, b_valid = 0;                         // the current block: position of its first key, number of keys
     auto load_block = [&](int j) {                      // K and V rows; those past the last key are zeros
         const float *k, *v;
@@ -330,7 +329,11 @@ f32_attention_kernel(const float *__restrict__ q, const float *__restrict__ k_li
         }
         cp_commit();
     };
-    if (grp < n_blocks) load_block(grp);
+    // a rank call only reads its pages: the groups' first blocks are on their way while the previous kernel finishes
+    const bool early = early_pages && grp < n_page_blocks;
+    if (early) load_block(grp);
+    grid_dependency_wait();
+    if (!early && grp < n_blocks) load_block(grp);
 
     // logits in units of log2(e) (softmax), so that a weight is 2^x
     const float scale = rsqrtf((float)DH) * (kPointwise ? 1.f : 1.4426950408889634f);
@@ -343,6 +346,18 @@ f32_attention_kernel(const float *__restrict__ q, const float *__restrict__ k_li
     __syncthreads();
     const int min_lim = pos0 >= sd.causal_end ? sd.causal_end : pos0 + 1;
     auto lim_of = [&](int r) { return pos0 + r >= sd.causal_end ? sd.causal_end : pos0 + r + 1; };   // row r sees keys at positions < this
+
+    // a candidate's own key and value, long before they are wanted (one row per thread in the low tiles: there are registers for it)
+    constexpr bool kEarlyOwn = RT == 1;
+    ulonglong2 own_k[kEarlyOwn ? CT / 4 : 1] = {}, own_v[kEarlyOwn ? CT / 4 : 1] = {};
+    if (kEarlyOwn && grp == 0 && ty < n_q && pos0 + ty >= sd.causal_end) {
+        const int64_t self = (int64_t)(sd.self_row0 + tile.q0 + ty) * d + h * DH + 4 * tx;
+#pragma unroll
+        for (int c = 0; c < CT / 4; ++c) {
+            own_k[kEarlyOwn ? c : 0] = *reinterpret_cast<const ulonglong2 *>(k_lin + self + 32 * c);
+            own_v[kEarlyOwn ? c : 0] = *reinterpret_cast<const ulonglong2 *>(v_lin + self + 32 * c);
+        }
+    }
 
     uint64_t o[RT][CT / 2] = {};
     float m[RT], l[RT];
@@ -458,7 +473,9 @@ f32_attention_kernel(const float *__restrict__ q, const float *__restrict__ k_li
 #pragma unroll
             for (int c = 0; c < CT / 4; ++c) {
                 const float4 a = *reinterpret_cast<const float4 *>(Qs + r * L::kLdq + 4 * tx + 32 * c);
-                const float4 b = *reinterpret_cast<const float4 *>(k_lin + self + 32 * c);
+                float4 b;
+                if constexpr (kEarlyOwn) { tc::unpack2(own_k[c].x, b.x, b.y); tc::unpack2(own_k[c].y, b.z, b.w); }
+                else b = *reinterpret_cast<const float4 *>(k_lin + self + 32 * c);
                 dot += (a.x * b.x + a.y * b.y) + (a.z * b.z + a.w * b.w);
             }
 #pragma unroll
@@ -477,7 +494,7 @@ f32_attention_kernel(const float *__restrict__ q, const float *__restrict__ k_li
             }
 #pragma unroll
             for (int c = 0; c < CT / 4; ++c) {
-                const ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(v_lin + self + 32 * c);
+                const ulonglong2 b = kEarlyOwn ? own_v[kEarlyOwn ? c : 0] : *reinterpret_cast<const ulonglong2 *>(v_lin + self + 32 * c);
                 o[i][2 * c] = fma2(dup(p), b.x, mul2(o[i][2 * c], dup(corr)));
                 o[i][2 * c + 1] = fma2(dup(p), b.y, mul2(o[i][2 * c + 1], dup(corr)));
             }
@@ -509,7 +526,7 @@ f32_attention_kernel(const float *__restrict__ q, const float *__restrict__ k_li
 
 template <int DH, int RT, int G>
 cudaError_t launch_attention(const float *q, const float *k_lin, const float *v_lin, PagedKV paged, const SeqDesc *seqs,
-                             const F32Tile *tiles, int n_tiles, int n_heads, int attn_kind, float *out, cudaStream_t stream)
+                             const F32Tile *tiles, int n_tiles, int n_heads, int attn_kind, bool early_pages, float *out, cudaStream_t stream)
 {
     constexpr int kBytes = AttnSmem<DH, RT, G>::kBytes;
     static PerDeviceValue attr_set;
@@ -524,7 +541,7 @@ cudaError_t launch_attention(const float *q, const float *k_lin, const float *v_
     }
     auto kernel = attn_kind == ATTN_POINTWISE ? f32_attention_kernel<DH, RT, G, true> : f32_attention_kernel<DH, RT, G, false>;
     return launch_dependent(kernel, dim3((unsigned)n_tiles * (unsigned)n_heads), dim3(64 * G), (size_t)kBytes, stream, 1, q, k_lin, v_lin,
-                            paged, seqs, tiles, n_heads, out);
+                            paged, seqs, tiles, n_heads, early_pages, out);
 }
 
 }  // namespace
@@ -588,8 +605,26 @@ int build_f32_tiles(const std::vector<SeqDesc> &seqs, int n_heads, int n_sms, st
     return rows;
 }
 
+// With an SM to every tile of eight rows the chain of a tile counts alone: half the rows, and as many groups of threads for the key blocks as fit
+// (with the pages of a rank call and a candidate's own key requested early: 4 users of 96 rows over 256 keys, two heads of 32, 9.5 -> 7 us
+// a launch, 42.9 -> 38 us a call with the loops of f32_block.cu rolled up as well).
+int halve_f32_tiles(const std::vector<SeqDesc> &seqs, int n_heads, int n_sms, int rows, std::vector<F32Tile> &tiles)
+{
+    int64_t n8 = 0;
+    for (const F32Tile &t : tiles) n8 += seqs[(size_t)t.seq].n_q - t.q0 > 8 ? 2 : 1;
+    if (rows != 16 || n8 * n_heads > n_sms) return rows;
+    std::vector<F32Tile> halves;
+    halves.reserve((size_t)n8);
+    for (const F32Tile &t : tiles) {
+        halves.push_back(t);
+        if (seqs[(size_t)t.seq].n_q - t.q0 > 8) halves.push_back({t.seq, t.q0 + 8});
+    }
+    tiles.swap(halves);
+    return 8;
+}
+
 cudaError_t launch_attention_f32(const float *q, const float *k_lin, const float *v_lin, PagedKV paged, const SeqDesc *seqs,
-                                 const F32Tile *tiles, int n_tiles, int tile_rows, int n_heads, int d_head, int attn_kind, int n_sms, float *out,
+                                 const F32Tile *tiles, int n_tiles, int tile_rows, int n_heads, int d_head, int attn_kind, bool early_pages, int n_sms, float *out,
                                  cudaStream_t stream, int64_t *launches)
 {
     if (n_tiles == 0) return cudaSuccess;
@@ -599,12 +634,11 @@ cudaError_t launch_attention_f32(const float *q, const float *k_lin, const float
     // 8 rows of 128 users x 2048 keys: 2 heads of 32 (256 blocks) 231 / 318 us a call, 4 heads of 64 (512 blocks) 1103 / 1024.
     const bool many = (int64_t)n_tiles * n_heads >= 3 * (int64_t)n_sms;
 #define RELAYGR_ATTN(DH)                                                                                                              \
-    return tile_rows == 64   ? launch_attention<DH, 8, 2>(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, out, stream) \
-           : tile_rows == 32 ? launch_attention<DH, 4, 4>(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, out, stream) \
-           : many            ? launch_attention<DH, 2, 1>(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, out, stream) \
-                             : launch_attention<DH, 2, 4>(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, out, stream)
-    if (d_head == 32) RELAYGR_ATTN(32);
-    if (d_head == 64) RELAYGR_ATTN(64);
+    auto launch = tile_rows == 64 ? launch_attention<DH, 8, 2> : tile_rows == 32 ? launch_attention<DH, 4, 4> : tile_rows == 8 ? launch_attention<DH, 1, DH == 32 ? 8 : 4> \
+                  : many ? launch_attention<DH, 2, 1> : launch_attention<DH, 2, 4>;                                                    \
+    return launch(q, k_lin, v_lin, paged, seqs, tiles, n_tiles, n_heads, attn_kind, early_pages, out, stream)
+    if (d_head == 32) { RELAYGR_ATTN(32); }
+    if (d_head == 64) { RELAYGR_ATTN(64); }
 #undef RELAYGR_ATTN
     return cudaErrorInvalidValue;
 }

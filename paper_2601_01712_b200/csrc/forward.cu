@@ -294,7 +294,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
             wk.n_items = (int)it.size(); wk.n_merges = (int)mg.size();
         } else {
             std::vector<F32Tile> ti;
-            wk.tile_rows = build_f32_tiles(seqs, H, n_sms, ti);
+            wk.tile_rows = halve_f32_tiles(seqs, H, n_sms, build_f32_tiles(seqs, H, n_sms, ti), ti);
             if (!ti.empty()) wk.o_items = put(reinterpret_cast<const int32_t *>(ti.data()), ti.size() * (sizeof(F32Tile) / 4));
             wk.n_items = (int)ti.size();
         }
@@ -545,7 +545,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
                                             att, reinterpret_cast<float *>(ws + lay.partial), d_status, stream, &launches);
             else
                 e = launch_attention_f32(q, kl, vl, paged, seqs_m, reinterpret_cast<const F32Tile *>(meta + work_m.o_items), work_m.n_items,
-                                         work_m.tile_rows, H, cfg.d_head, cfg.attn_kind, n_sms, att, stream, &launches);
+                                         work_m.tile_rows, H, cfg.d_head, cfg.attn_kind, call.mode == MODE_RANK, n_sms, att, stream, &launches);
             prof_end(KC_ATTENTION, pe, stream);
         }
         if (!ck("attention")) return RELAYGR_E_CUDA;

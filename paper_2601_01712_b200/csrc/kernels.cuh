@@ -87,8 +87,10 @@ cudaError_t launch_gemm_f32(const float *A, const float *W, int64_t M, int N, in
 // One block per (query tile, head): attention (softmax, or pointwise SiLU for ATTN_POINTWISE) under the SeqDesc mask.
 // build_f32_tiles fills the tiles of a call (host) and returns their height, which the launcher takes with them (device).
 int build_f32_tiles(const std::vector<SeqDesc> &seqs, int n_heads, int n_sms, std::vector<F32Tile> &tiles);
+// Tiles of 16 rows into tiles of 8 where there are SMs for all of them; returns the height.
+int halve_f32_tiles(const std::vector<SeqDesc> &seqs, int n_heads, int n_sms, int rows, std::vector<F32Tile> &tiles);
 cudaError_t launch_attention_f32(const float *q, const float *k_lin, const float *v_lin, PagedKV paged, const SeqDesc *seqs,
-                                 const F32Tile *tiles, int n_tiles, int tile_rows, int n_heads, int d_head, int attn_kind, int n_sms, float *out,
+                                 const F32Tile *tiles, int n_tiles, int tile_rows, int n_heads, int d_head, int attn_kind, bool early_pages, int n_sms, float *out,
                                  cudaStream_t stream, int64_t *launches);
 
 // The fp32 model with few rows and matrices that fit an SM's shared memory (f32_block_supported; w_qkv, w_o, w1, w2 and the table 16-byte

@@ -316,3 +316,13 @@ def test_attention_clusters(prefix, short, cand, kind):
     assert max_abs_err(scores, batch, want) <= max_bound
     assert max_abs_err(full, batch, want) <= max_bound
     pool.close(); model.close()
+
+
+# fp32 attention in tiles of eight rows, one to an SM (148 tiles and heads, then one more row), with eight groups of threads for heads of 32 and four for
+# heads of 64: fewer key blocks than groups, more, none in pages; rows of short-term tokens and candidates in one tile; pointwise.
+@pytest.mark.parametrize("d,heads,kind,prefix,short,cand", [(64, 2, 0, [1], [0], [8]), (64, 2, 0, [700, 65], [9, 4], [200, 80]), (64, 1, 0, [500], [60], [61]),
+                                                            (64, 2, 0, [64], [0], [592]), (64, 2, 0, [64], [0], [593]), (64, 1, 1, [300, 20], [3, 0], [7, 30]),
+                                                            (96, 3, 1, [130], [70], [9])])
+def test_f32_tiles_of_eight_rows(d, heads, kind, prefix, short, cand):
+    shape = synth.ModelShape(2, d, heads, d // heads, 4 * d, 2000, synth.DTYPE_F32, attn_kind=kind)
+    _check_f32(shape, _tiny_batch(shape, 410 + d + heads, prefix, short, cand), 75)
