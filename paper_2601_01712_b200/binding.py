@@ -131,7 +131,7 @@ def _ptr(x):
         return x
     if isinstance(x, np.ndarray):
         assert x.flags["C_CONTIGUOUS"]
-        return x.ctypes.data
+        return x.__array_interface__["data"][0]      # (x.ctypes builds an object for it: 1 us)
     return x.data_ptr()
 
 
