@@ -11,12 +11,12 @@
 // with one bulk tensor store where a warp's 32 rows are 32 consecutive slots of one page,
 // with plain stores after a page-table walk per row otherwise.
 //
-// Two shapes (Cfg below): single CTAs with 128 x 128 tiles, and CTA pairs (a cluster of two,
-// tcgen05 cta_group::2) with 256 x 256 tiles, where each CTA loads its 128 rows of A and half
-// of W and the even CTA issues the MMAs for both.
+// The shapes (Cfg below): single CTAs with 128 x 128 tiles, and CTA pairs (a cluster of two,
+// tcgen05 cta_group::2) with 256 x 256 tiles - 256 x 128 where those would leave every other pair
+// idle -, where each CTA loads its 128 rows of A and half of W and the even CTA issues the MMAs for both.
 //
 // Warp roles (320 threads per CTA): warp 0 = TMA producer (128 x 64 tiles of A and W, 128-byte
-// swizzle, five-stage ring), warp 1 = TMEM owner + MMA issuer (tcgen05.mma K16), warps 2-9 =
+// swizzle, a ring of five stages or seven), warp 1 = TMEM owner + MMA issuer (tcgen05.mma K16), warps 2-9 =
 // epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 (its hardware quadrant), columns
 // (BN / 2) ((w - 2) / 4) .. + BN / 2 - 1, 64 at a time, applies bias / SiLU in the
 // row-per-thread layout tcgen05.ld delivers and stages the result for the store.
@@ -27,7 +27,7 @@ namespace relaygr {
 
 namespace {
 
-constexpr int BM = 128, BK = 64, kMaxStages = 5;
+constexpr int BM = 128, BK = 64, kMaxStages = 7;
 constexpr int kEpiWarps = 8;
 constexpr int kThreads = 32 * (2 + kEpiWarps);
 constexpr int kABytes = BM * BK * 2;
@@ -43,7 +43,7 @@ constexpr int kMaxBias = 4096;                                       // output c
 template <int BN, int CTAS> struct Cfg {
     static constexpr int kBBytes = (BN / CTAS) * BK * 2;
     static constexpr int kStage = kABytes + kBBytes;
-    static constexpr int kStages = (CTAS == 1 && BN == 256) ? 3 : 5;
+    static constexpr int kStages = CTAS == 2 && BN == 128 ? 7 : 5;
     static constexpr int kOffPatch = kStages * kStage;                                    // 1024-byte aligned: stages are
     static constexpr int kOffBias = kOffPatch + kEpiWarps * kPatches * kPatchBytes;       // kMaxBias floats
     static constexpr int kOffRowOff = kOffBias + kMaxBias * 4;                            // per warp 32 x int64
@@ -51,7 +51,6 @@ template <int BN, int CTAS> struct Cfg {
     static constexpr int kSmemBytes = kOffBars + 256 /*barriers*/ + 1024 /*alignment slack*/;
     static constexpr uint32_t kTmemCols = 2 * BN;
     static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
-    static_assert(CTAS == 1 || BN == 256, "a CTA pair works on 256 x 256");
 };
 
 struct GemmBars {
@@ -398,7 +397,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 }  // namespace
 
 template <int BN, int CTAS>
-static cudaError_t launch_cfg(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmOutMaps &om, int64_t M, int N, int K,
+static cudaError_t launch_cfg(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmB64, const GemmOutMaps &om, int64_t M, int N, int K,
                               const Epilogue &epi, int *err, cudaStream_t stream)
 {
     using C = Cfg<BN, CTAS>;
@@ -428,19 +427,23 @@ static cudaError_t launch_cfg(const CUtensorMap &tmA, const CUtensorMap &tmB, co
         n_workers_max = n;
         workers_of.set(dev, n);
     }
+    // Pairs with half-wide tiles where at least every other pair would be idle otherwise: such a tile takes three quarters of a whole one's time
+    // (24 KB of operands a K block instead of 32 KB through the same 64 B / clk).  Ranking calls of one user, 576 rows: d_model 512 512 -> 452 us,
+    // 1024 339 -> 305; the candidates' GEMMs of the widest model's full inference, 36 tiles, 10 us of 865.
     const int64_t tiles = ((M + BM * CTAS - 1) / (BM * CTAS)) * (N / BN);
+    if (CTAS == 2 && BN == 256 && 2 * tiles <= n_workers_max) return launch_cfg<128, 2>(tmA, tmB, tmB64, om, M, N, K, epi, err, stream);
     const unsigned workers = (unsigned)(tiles < n_workers_max ? tiles : n_workers_max);
-    return launch_dependent(gemm_tc_kernel<BN, CTAS>, dim3(workers * CTAS), dim3(kThreads), (size_t)C::kSmemBytes, stream, CTAS, tmA, tmB, om,
+    return launch_dependent(gemm_tc_kernel<BN, CTAS>, dim3(workers * CTAS), dim3(kThreads), (size_t)C::kSmemBytes, stream, CTAS, tmA, BN / CTAS == 64 ? tmB64 : tmB, om,
                             M, N, K, epi, err);
 }
 
-cudaError_t launch_gemm_tc(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmOutMaps &om, int64_t M, int N, int K,
+cudaError_t launch_gemm_tc(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmB64, const GemmOutMaps &om, int64_t M, int N, int K,
                            const Epilogue &epi, int *err, cudaStream_t stream, int64_t *launches)
 {
     if (M == 0 || N == 0) return cudaSuccess;
     *launches += 1;
-    return gemm_pair(M, N, K) ? launch_cfg<256, 2>(tmA, tmB, om, M, N, K, epi, err, stream)
-                        : launch_cfg<128, 1>(tmA, tmB, om, M, N, K, epi, err, stream);
+    return gemm_pair(M, N, K) ? launch_cfg<256, 2>(tmA, tmB, tmB64, om, M, N, K, epi, err, stream)
+                        : launch_cfg<128, 1>(tmA, tmB, tmB64, om, M, N, K, epi, err, stream);
 }
 
 }  // namespace relaygr

@@ -326,3 +326,27 @@ def test_attention_clusters(prefix, short, cand, kind):
 def test_f32_tiles_of_eight_rows(d, heads, kind, prefix, short, cand):
     shape = synth.ModelShape(2, d, heads, d // heads, 4 * d, 2000, synth.DTYPE_F32, attn_kind=kind)
     _check_f32(shape, _tiny_batch(shape, 410 + d + heads, prefix, short, cand), 75)
+
+
+# GEMMs of a wider model in half-wide tiles of CTA pairs: as long as two of them go to every pair (d_model 512: the QKV projection up to 1536 rows, the
+# others up to 2304 and 4608), ragged last rows, pages, the candidates' own GEMMs of a full inference.
+@pytest.mark.parametrize("prefix,short,cand", [([1], [0], [1]), ([257], [3], [254]), ([70, 64], [0, 5], [1036, 495]), ([70, 64], [0, 5], [1036, 496]), ([1537], [1], [60])])
+def test_half_wide_tiles(prefix, short, cand):
+    shape = synth.ModelShape(2, 512, 8, 64, 1024, 2000, synth.DTYPE_BF16)
+    batch = _tiny_batch(shape, 420 + len(prefix) + cand[-1], prefix, short, cand)
+    w, model, pool, db = _setup(shape, 76, batch)
+    pool.preinfer(db)
+    scores, full = pool.rank(db).cpu().numpy(), model.rank_full(db).cpu().numpy()
+    assert model.device_status() == 0
+    users = [len(prefix) - 1]
+    om = oracle_model(shape, w)
+    want = oracle_scores(om, batch, users=users)
+    max_bound, _, _ = bf16_noise_bounds(shape, w, batch, want)
+    assert max_abs_err(scores, batch, want) <= max_bound
+    assert max_abs_err(full, batch, want) <= max_bound
+    p = batch.user_slices(users[0])[0]
+    K, V = om.preinfer(p)
+    gK, gV = pool.read_kv(batch.users[users[0]], len(p))
+    assert np.max(np.abs(gK.float().cpu().numpy() - K)) <= 5e-2      # as in test_preinfer_rows_in_and_across_pages
+    assert np.max(np.abs(gV.float().cpu().numpy() - V)) <= 5e-2
+    pool.close(); model.close()
