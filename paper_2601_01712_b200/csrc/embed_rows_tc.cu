@@ -1,0 +1,184 @@
+// The first kernel of a bf16 call with few rows, for d_model = 256: x = E[id] widened to fp32, and the first layer's QKV projection of LN(x).
+// A CTA takes 32 rows and one 128-column chunk of the projection: it gathers and normalises its rows itself (16 KB of the table, what another CTA
+// of the same rows does too), and the product is computed transposed, 128 rows of W_qkv x the 32 rows, as in ffn_rows_tc.cu.  The weights (64 KB) are on
+// their way before the wait for the metadata.
+// What bounds it: latency - look-ups, table rows, 16 MMAs, stores, one after the other.  As gather and GEMM it was two launches, of 4.3 and
+// 5.4 us in a ranking call of one user.
+#include "ffn_common.cuh"
+#include "kernels.cuh"
+
+namespace relaygr {
+
+namespace {
+
+using namespace ffn;
+
+constexpr int kT = 32, kEmbedThreads = 256, kRowsPerWarp = kT / (kEmbedThreads / 32);
+constexpr int kKB = kT * 128;                         // one K block (64 bf16) of the rows
+constexpr int kOffW = 4 * kKB, kOffEmbedBars = kOffW + 4 * kKBlock, kEmbedSmem = kOffEmbedBars + 64 + kT * 12 + 1024;
+constexpr uint32_t kEmbedCols = 32;
+
+struct EmbedBars {
+    uint64_t w_full, s_full;
+    uint32_t tmem_slot;
+};
+
+__global__ void __launch_bounds__(kEmbedThreads, 2)
+embed_rows_kernel(const __grid_constant__ CUtensorMap tmQkv, const __nv_bfloat16 *__restrict__ emb, int64_t vocab, RowSource src, int64_t M, const float *__restrict__ g,
+                  const float *__restrict__ b, float eps, float *__restrict__ x, FfnTail to, int *err)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t *sA = smem, *sW = smem + kOffW;
+    EmbedBars *bars = reinterpret_cast<EmbedBars *>(smem + kOffEmbedBars);
+    int64_t *page_off = reinterpret_cast<int64_t *>(smem + kOffEmbedBars + 64);      // of rows that go to pages: offset of (page, K, slot) ...
+    int *last_slot = reinterpret_cast<int *>(page_off + kT);                         // ... and of a user's last row its slot
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quad = warp & 3, half = warp >> 2;
+    const int64_t tile_row0 = (int64_t)blockIdx.x * kT;
+    const int chunk = blockIdx.y;
+
+    // set-up and parameters, while the kernel before is still running
+    if (threadIdx.x == 0) {
+        tc::mbar_init(&bars->w_full, 1); tc::mbar_init(&bars->s_full, 1);
+        tc::fence_mbar_init();
+        tc::mbar_expect_tx(&bars->w_full, 4 * kKBlock);
+        for (int kb = 0; kb < 4; ++kb) tc::tma_load_2d(sW + kb * kKBlock, &tmQkv, kb * 64, chunk * kChunk, &bars->w_full);
+    }
+    if (warp == 1) {
+        tc::tmem_alloc(&bars->tmem_slot, kEmbedCols);
+        tc::tmem_relinquish();
+    }
+    const int n = chunk * kChunk + quad * 32 + lane, which = (to.col0 + n) >> 8, c = (to.col0 + n) & (kD - 1);      // this lane's output column
+    const float scale = which == 0 ? to.q_scale : 1.f, bias = to.bias ? to.bias[n] * scale : 0.f;
+    const bool to_page = to.paged.slab != nullptr && which > 0;
+    float4 gain[2], shift[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        gain[h] = *reinterpret_cast<const float4 *>(g + 8 * lane + 4 * h); shift[h] = *reinterpret_cast<const float4 *>(b + 8 * lane + 4 * h);
+    }
+    // The first kernel of a call lets the next one start only after its own wait: see gather_ln_kernel.
+    grid_dependency_wait();
+    grid_launch_dependents();
+    const bool stopped = *reinterpret_cast<volatile int *>(err) != 0;      // an earlier call gave up: everything runs as ever, but nothing is stored
+
+    // a warp takes four rows, the look-ups side by side in its first lanes
+    const int rt0 = warp * kRowsPerWarp;
+    const int64_t row0 = tile_row0 + rt0;
+    long long id = 0;
+    if (lane < kRowsPerWarp && row0 + lane < M) {
+        id = row_token_id(src, row0 + lane);
+        if (id < 0 || id >= vocab) {
+            // an id outside the table: recorded in the status word, and a row that exists is read instead
+            atomicCAS(err, (int)STATUS_OK, (int)STATUS_BAD_INDEX);
+            id = id < 0 ? 0 : vocab - 1;
+        }
+    }
+    if (to_page && lane >= 8 && lane < 8 + kRowsPerWarp) {
+        const int i = lane - 8;
+        const int64_t r = row0 + i;
+        int64_t off = 0;
+        int last = -1;
+        if (r < M) {
+            const int u = find_user(to.row_off, to.n_users, (int)r), t = (int)r - to.row_off[u];
+            off = (int64_t)page_elem_offset(to.paged, to.paged.pt[to.seqs[u].pt_base + (t >> 6)], 0, t & 63);
+            if (t == to.seqs[u].n_q - 1) last = t & 63;
+        }
+        page_off[rt0 + i] = off;
+        last_slot[rt0 + i] = last;
+    }
+    __syncwarp();
+    float4 v[kRowsPerWarp][2];                        // columns 8 lane .. + 7
+#pragma unroll
+    for (int j = 0; j < kRowsPerWarp; ++j) {
+        const uint4 w = *reinterpret_cast<const uint4 *>(emb + __shfl_sync(0xffffffffu, id, j) * kD + 8 * lane);      // (rows past the last: row 0)
+        v[j][0] = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u));
+        v[j][1] = make_float4(__uint_as_float(w.z << 16), __uint_as_float(w.z & 0xffff0000u), __uint_as_float(w.w << 16), __uint_as_float(w.w & 0xffff0000u));
+    }
+    float mean[kRowsPerWarp], rstd[kRowsPerWarp];
+    rows_stats<kRowsPerWarp>(v, eps, mean, rstd);
+#pragma unroll
+    for (int j = 0; j < kRowsPerWarp; ++j) {
+        const int rt = rt0 + j;
+        uint32_t y[4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float4 o = normalised(v[j][h], mean[j], rstd[j], gain[h], shift[h]);
+            y[2 * h] = tc::pack_bf16(o.x, o.y); y[2 * h + 1] = tc::pack_bf16(o.z, o.w);
+        }
+        *reinterpret_cast<uint4 *>(sA + (lane >> 3) * kKB + rt * 128 + (((lane & 7) ^ (rt & 7)) << 4)) = make_uint4(y[0], y[1], y[2], y[3]);
+    }
+    tc::fence_proxy_async();
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    const uint32_t tmem_base = bars->tmem_slot;
+    bool ok = true;
+    if (warp == 0) {
+        constexpr uint32_t idesc = tc::make_idesc(kRows, kT, 0, 0);                // weights x rows, both K-major
+        ok = tc::mbar_wait(&bars->w_full, 0, err);
+        tc::tc_fence_after();
+        if (ok && tc::elect_one()) {
+            const uint64_t wdesc = tc::smem_desc_sw128(tc::smem_u32(sW)), adesc = tc::smem_desc_sw128(tc::smem_u32(sA));
+#pragma unroll
+            for (int kb = 0; kb < 4; ++kb)
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    tc::mma_ss(tmem_base, wdesc + kb * (kKBlock / 16) + 2 * k, adesc + kb * (kKB / 16) + 2 * k, idesc, (kb | k) != 0);
+            tc::mma_commit(&bars->s_full);
+        }
+        __syncwarp();
+    }
+    if (chunk == 0 && !stopped)                       // the residual stream, under the products
+#pragma unroll
+        for (int j = 0; j < kRowsPerWarp; ++j)
+            if (row0 + j < M)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) *reinterpret_cast<float4 *>(x + (row0 + j) * kD + 8 * lane + 4 * h) = v[j][h];
+    ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->s_full, 0, err));
+    tc::tc_fence_after();
+    if (ok) {
+        uint32_t r[16];
+        tc::tmem_ld16(tmem_base + ((uint32_t)(quad * 32) << 16) + half * 16, r);
+        tc::tmem_ld_wait();
+        __nv_bfloat16 *base = to_page ? reinterpret_cast<__nv_bfloat16 *>(to.paged.slab) + (which - 1) * 64 * kD + c
+                                      : (which == 0 ? to.q : which == 1 ? to.k : to.v) + tile_row0 * kD + c;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const int rt = half * 16 + e;
+            if (tile_row0 + rt >= M || stopped) break;
+            __nv_bfloat16 *p = base + (to_page ? page_off[rt] : (int64_t)rt * kD);
+            *p = __float2bfloat16_rn(fmaf(__uint_as_float(r[e]), scale, bias));
+            if (to_page && last_slot[rt] >= 0)        // last row of the prefix: clear the unused slots of its page
+                for (int z = 1; last_slot[rt] + z < 64; ++z) p[z * kD] = __float2bfloat16_rn(0.f);
+        }
+    }
+    tc::tc_fence_before();
+    __syncthreads();
+    if (warp == 1) tc::tmem_dealloc(tmem_base, kEmbedCols);
+}
+
+}  // namespace
+
+// Two CTAs to an SM at most, all of them at once: with more rows the weights, read once for every 32 of them, cost more than the second launch (a call in us,
+// two kernels / this one: 576 rows 109.4 / 106.7, 1300 rows 112.6 / 111.0, 2000 rows 116.8 / 118.0).
+bool embed_rows_supported(int64_t M, int d_model, int n_sms) { return d_model == kD && (M + kT - 1) / kT * 6 <= 2 * (int64_t)n_sms; }
+
+cudaError_t launch_embed_rows(const __nv_bfloat16 *emb, int64_t vocab, const RowSource &src, int64_t M, const float *g, const float *b, float eps, float *x, const FfnTail &to,
+                              int *err, cudaStream_t stream, int64_t *launches)
+{
+    if (M == 0) return cudaSuccess;
+    static PerDeviceValue attr_set;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (!attr_set.get(dev)) {
+        e = cudaFuncSetAttribute(embed_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kEmbedSmem);
+        if (e != cudaSuccess) return e;
+        attr_set.set(dev, 1);
+    }
+    *launches += 1;
+    return launch_dependent(embed_rows_kernel, dim3((unsigned)((M + kT - 1) / kT), (unsigned)(to.n_qkv / kChunk)), dim3(kEmbedThreads), (size_t)kEmbedSmem, stream, 1,
+                            *to.qkv_map, emb, vocab, src, M, g, b, eps, x, to, err);
+}
+
+}  // namespace relaygr

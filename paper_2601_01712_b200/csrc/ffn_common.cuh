@@ -1,5 +1,5 @@
 // What the forms of the fused out-proj + feed-forward kernel share: sizes and the query for resident clusters (all three: ffn_rows_tc.cu,
-// ffn_tc.cu, ffn_pair_tc.cu), and, for ffn_tc.cu and ffn_pair_tc.cu, the steps their eight
+// ffn_tc.cu, ffn_pair_tc.cu), LayerNorm of whole rows in a warp (ffn_rows_tc.cu, embed_rows_tc.cu), and, for ffn_tc.cu and ffn_pair_tc.cu, the steps their eight
 // epilogue warps take on one row (half) per thread.  Warp (quad, ch) owns TMEM lanes 32 quad .. + 31 and half ch of the columns.
 // The row lives in TMEM and the steps walk it in rolled loops of 32 columns: a kernel of this kind runs a few microseconds per
 // layer, between others that evict its instructions, so code that is executed once per tile costs its fetch from L2 (with
@@ -120,6 +120,40 @@ __device__ __forceinline__ void silu_chunk(uint32_t s_cols, const float *b1_half
         }
         tc::tmem_st16(s_cols + 16 * p, pk);
     }
+}
+
+__device__ __forceinline__ float sum8(const float4 (&v)[2]) { return ((v[0].x + v[0].y) + (v[0].z + v[0].w)) + ((v[1].x + v[1].y) + (v[1].z + v[1].w)); }
+// Mean and 1 / std of N rows, eight columns of each per lane.  Two passes; the rows' shuffles overlap.
+template <int N>
+__device__ __forceinline__ void rows_stats(const float4 (&v)[N][2], float eps, float (&mean)[N], float (&rstd)[N])
+{
+#pragma unroll
+    for (int i = 0; i < N; ++i) mean[i] = sum8(v[i]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < N; ++i) mean[i] += __shfl_xor_sync(0xffffffffu, mean[i], o);
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        mean[i] *= 1.f / kD;
+        float sq = 0.f;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float dx = v[i][h].x - mean[i], dy = v[i][h].y - mean[i], dz = v[i][h].z - mean[i], dw = v[i][h].w - mean[i];
+            sq += (dx * dx + dy * dy) + (dz * dz + dw * dw);
+        }
+        rstd[i] = sq;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < N; ++i) rstd[i] += __shfl_xor_sync(0xffffffffu, rstd[i], o);
+#pragma unroll
+    for (int i = 0; i < N; ++i) rstd[i] = rsqrtf(rstd[i] * (1.f / kD) + eps);
+}
+__device__ __forceinline__ float4 normalised(const float4 &v, float mean, float rstd, const float4 &g, const float4 &b)
+{
+    return make_float4((v.x - mean) * rstd * g.x + b.x, (v.y - mean) * rstd * g.y + b.y, (v.z - mean) * rstd * g.z + b.z, (v.w - mean) * rstd * g.w + b.w);
 }
 
 // How many clusters of `cs` CTAs of a kernel with `smem` bytes can be resident at once on the current device (`dev`); asked once.  None

@@ -70,45 +70,11 @@ __device__ __forceinline__ float4 load4_or_zero(const float *p, int c)
 {
     return p ? *reinterpret_cast<const float4 *>(p + c) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
-__device__ __forceinline__ float sum8(const float4 (&v)[2]) { return ((v[0].x + v[0].y) + (v[0].z + v[0].w)) + ((v[1].x + v[1].y) + (v[1].z + v[1].w)); }
 // v = (v + p) + q
 __device__ __forceinline__ void add_twice(float4 &v, const float4 &p, const float4 &q)
 {
     v.x = (v.x + p.x) + q.x; v.y = (v.y + p.y) + q.y; v.z = (v.z + p.z) + q.z; v.w = (v.w + p.w) + q.w;
 }
-// Mean and 1 / std of N rows, eight columns of each per lane.  Two passes; the rows' shuffles overlap.
-template <int N>
-__device__ __forceinline__ void rows_stats(const float4 (&v)[N][2], float eps, float (&mean)[N], float (&rstd)[N])
-{
-#pragma unroll
-    for (int i = 0; i < N; ++i) mean[i] = sum8(v[i]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int i = 0; i < N; ++i) mean[i] += __shfl_xor_sync(0xffffffffu, mean[i], o);
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-        mean[i] *= 1.f / kD;
-        float sq = 0.f;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const float dx = v[i][h].x - mean[i], dy = v[i][h].y - mean[i], dz = v[i][h].z - mean[i], dw = v[i][h].w - mean[i];
-            sq += (dx * dx + dy * dy) + (dz * dz + dw * dw);
-        }
-        rstd[i] = sq;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int i = 0; i < N; ++i) rstd[i] += __shfl_xor_sync(0xffffffffu, rstd[i], o);
-#pragma unroll
-    for (int i = 0; i < N; ++i) rstd[i] = rsqrtf(rstd[i] * (1.f / kD) + eps);
-}
-__device__ __forceinline__ float4 normalised(const float4 &v, float mean, float rstd, const float4 &g, const float4 &b)
-{
-    return make_float4((v.x - mean) * rstd * g.x + b.x, (v.y - mean) * rstd * g.y + b.y, (v.z - mean) * rstd * g.z + b.z, (v.w - mean) * rstd * g.w + b.w);
-}
-
 template <int T, int CS>
 __global__ void __launch_bounds__(kThreads, 1)
 ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2,

@@ -467,6 +467,20 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         return t;
     };
 
+    // Layer l's QKV projection as part of the kernel before it (bf16 model; a last layer whose candidates are moved together has one of its own, one
+    // that nothing reads has none)
+    auto projects = [&](int l) { return !(l == L - 1 && (compact_last || (!preinfer && n_scores == 0))); };
+    auto projection_of = [&](int l, FfnTail &t) {
+        const bool kv = preinfer && l == L - 1;
+        t.qkv_map = kv ? &wmaps[(size_t)l].kv : &wmaps[(size_t)l].qkv;
+        t.col0 = kv ? d : 0; t.n_qkv = 3 * d - t.col0;
+        t.bias = w.b_qkv ? w.b_qkv + (size_t)l * 3 * d + t.col0 : nullptr;
+        t.q_scale = q_scale;
+        t.q = reinterpret_cast<__nv_bfloat16 *>(q); t.k = reinterpret_cast<__nv_bfloat16 *>(kl); t.v = reinterpret_cast<__nv_bfloat16 *>(vl);
+        if (preinfer) t.paged = PagedKV{call.pool_slab, meta + o_pt, L, d, l};
+        t.row_off = d_row_off; t.seqs = d_seqs; t.n_users = B;
+    };
+
     for (int l = 0; l < L; ++l) {
         const bool last = l == L - 1;
         if (last && !preinfer && n_scores == 0) { dead_tail = true; break; }
@@ -485,6 +499,17 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
                 e = launch_f32_first(F32First{(const float *)w.emb, cfg.vocab, src}, tail_of(0), x, R, d, cfg.ln_eps, n_sms, d_status, stream, &launches);
                 prof_end(KC_GATHER_LN, pe, stream);
                 if (!ck("gather, LayerNorm and QKV projection")) return RELAYGR_E_CUDA;
+            }
+        }
+        if constexpr (kTensor) {
+            if (l == 0 && projects(0) && embed_rows_supported(R, d, n_sms)) {
+                FfnTail to{};
+                projection_of(0, to);
+                cudaEvent_t pe = prof_begin(stream);
+                e = launch_embed_rows((const __nv_bfloat16 *)w.emb, cfg.vocab, src, R, g1, b1n, cfg.ln_eps, x, to, d_status, stream, &launches);
+                prof_end(KC_GATHER_LN, pe, stream);
+                if (!ck("gather, LayerNorm and QKV projection")) return RELAYGR_E_CUDA;
+                qkv_done = true;
             }
         }
         if (!blocks32 && !qkv_done) {
@@ -513,6 +538,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         e = gemm(R, ln1_in_gemm ? reinterpret_cast<const T *>(x) : a, tm_a, Wqkv, lm ? (kv_only ? &lm->kv : &lm->qkv) : nullptr, lm ? (kv_only ? &lm->kv64 : &lm->qkv64) : nullptr, om_qkv, 3 * d - ep.col0, d, ep);
         if (!ck("QKV projection")) return RELAYGR_E_CUDA;
         }
+        qkv_done = false;
         if (preinfer && last) break;
 
         if (last && cand_last) {
@@ -561,16 +587,8 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
             cudaEvent_t pe = prof_begin(stream);
             FfnTail tail{};
             if (!last) {
-                // (a layer whose candidates are moved together has a projection of its own; a layer that nothing reads has none)
-                const bool next_last = l + 1 == L - 1, next_kv = next_last && preinfer;
-                tail.kind = next_last && (compact_last || (!preinfer && n_scores == 0)) ? FFN_TAIL_LN : FFN_TAIL_QKV;
-                tail.qkv_map = next_kv ? &wmaps[(size_t)l + 1].kv : &wmaps[(size_t)l + 1].qkv;
-                tail.col0 = next_kv ? d : 0; tail.n_qkv = 3 * d - tail.col0;
-                tail.bias = w.b_qkv ? w.b_qkv + (size_t)(l + 1) * 3 * d + tail.col0 : nullptr;
-                tail.q_scale = q_scale;
-                tail.q = reinterpret_cast<__nv_bfloat16 *>(q); tail.k = reinterpret_cast<__nv_bfloat16 *>(kl); tail.v = reinterpret_cast<__nv_bfloat16 *>(vl);
-                if (preinfer) tail.paged = PagedKV{call.pool_slab, meta + o_pt, L, d, l + 1};
-                tail.row_off = d_row_off; tail.seqs = d_seqs; tail.n_users = B;
+                tail.kind = projects(l + 1) ? FFN_TAIL_QKV : FFN_TAIL_LN;
+                projection_of(l + 1, tail);
                 tail.g = w.ln1_g + (size_t)(l + 1) * d; tail.b = w.ln1_b + (size_t)(l + 1) * d; tail.a = reinterpret_cast<__nv_bfloat16 *>(a);
             } else {
                 tail.kind = FFN_TAIL_SCORE;

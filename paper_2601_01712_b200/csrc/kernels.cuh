@@ -180,6 +180,11 @@ struct FfnTail {
     __nv_bfloat16 *q, *k, *v;
     PagedKV paged;
 };
+// The first kernel of a bf16 call with few rows of d_model = 256: x[r, :] = E[id(r), :] in fp32, and the QKV projection of LN(x; g, b) (`to`: its
+// FFN_TAIL_QKV fields).
+bool embed_rows_supported(int64_t M, int d_model, int n_sms);
+cudaError_t launch_embed_rows(const __nv_bfloat16 *emb, int64_t vocab, const RowSource &src, int64_t M, const float *g, const float *b, float eps, float *x, const FfnTail &to,
+                              int *err, cudaStream_t stream, int64_t *launches);
 bool ffn_fused_supported(int d_model, int d_ff);
 cudaError_t launch_ffn_fused(const FfnMaps &w, const CUtensorMap &tmX, float *x, const float *g, const float *b, const float *b1,
                              const float *b2, const CUtensorMap &tmAtt, const CUtensorMap &tmAtt32, const float *bo, int64_t M, int d_ff, float eps, const FfnTail &tail,

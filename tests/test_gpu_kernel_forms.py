@@ -350,3 +350,28 @@ def test_half_wide_tiles(prefix, short, cand):
     assert np.max(np.abs(gK.float().cpu().numpy() - K)) <= 5e-2      # as in test_preinfer_rows_in_and_across_pages
     assert np.max(np.abs(gV.float().cpu().numpy() - V)) <= 5e-2
     pool.close(); model.close()
+
+
+# The first kernel of a bf16 call with few rows (gather, LayerNorm and QKV projection in tiles of 32 rows, from 1569 rows on two kernels): ragged
+# tiles, users that start inside a tile, one layer (whose pre-inference projects K and V alone), a feed-forward too wide for the fused kernels.
+@pytest.mark.parametrize("layers,ff,prefix,short,cand", [(2, 512, [1], [0], [1]), (1, 512, [31, 33, 64], [2, 0, 5], [29, 1, 33]), (2, 2304, [90, 40], [7, 0], [100, 60]),
+                                                         (2, 512, [700] * 4, [40] * 4, [352] * 4), (2, 512, [392, 393, 392, 392], [40] * 4, [352, 352, 352, 353])])
+def test_first_kernel_forms(layers, ff, prefix, short, cand):
+    shape = synth.ModelShape(layers, 256, 4, 64, ff, 3000, synth.DTYPE_BF16)
+    batch = _tiny_batch(shape, 400 + len(prefix) + ff, prefix, short, cand)
+    w, model, pool, db = _setup(shape, 74, batch)
+    pool.preinfer(db)
+    scores = pool.rank(db).cpu().numpy()
+    assert model.device_status() == 0
+    users = sorted({0, len(prefix) - 1})
+    om = oracle_model(shape, w)
+    want = oracle_scores(om, batch, users=users)
+    max_bound, _, _ = bf16_noise_bounds(shape, w, batch, want)
+    assert max_abs_err(scores, batch, want) <= max_bound
+    for i in users:
+        p = batch.user_slices(i)[0]
+        K, V = om.preinfer(p)
+        gK, gV = pool.read_kv(batch.users[i], len(p))
+        assert np.max(np.abs(gK.float().cpu().numpy() - K)) <= 5e-2      # as in test_preinfer_rows_in_and_across_pages
+        assert np.max(np.abs(gV.float().cpu().numpy() - V)) <= 5e-2
+    pool.close(); model.close()
