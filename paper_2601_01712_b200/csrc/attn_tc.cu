@@ -748,8 +748,9 @@ cudaError_t launch_cs(const CUtensorMap &tmQ, const CUtensorMap &tmK, const CUte
                             n_items, next_item, seqs, pt, n_layers, layer, d_model, early_pages, out, partial, err);
 }
 
-// How many clusters run at once.  The occupancy query answers for one CTA per SM (74, 33 and 15 clusters of 2, 4 and 8 on a B200); two fit an SM,
-// clusters of one beside those of another: a launch of 20 of 8 or 64 of 4 runs in one round, one of 36 of 8 takes a second.
+// How many clusters run at once.  The occupancy query answers as if an SM held one CTA (74, 33 and 15 clusters of 2, 4 and 8 on a B200); the kernel is
+// built for two (launch bounds, shared memory, TMEM): launches of 20 clusters of 8 and of 64 of 4 run in one round (with one CTA to an SM
+// they would take two, and lose to the general plan), one of 36 of 8 takes a second.
 template <int CS>
 int resident_clusters(int n_sms)
 {
@@ -760,11 +761,10 @@ int resident_clusters(int n_sms)
     attr[0].val.clusterDim.x = CS; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
     auto count = [&](auto kernel) {
-        int n = 0, per_sm = 0;
+        int n = 0;
         const bool ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<CS>::kSmemBytes) == cudaSuccess &&
-                        cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess &&
-                        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 192, Shape<CS>::kSmemBytes) == cudaSuccess;
-        return !ok ? 0 : n * CS <= n_sms ? n * std::max(1, per_sm) : n;
+                        cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess;
+        return !ok ? 0 : n * CS <= n_sms ? 2 * n : n;
     };
     return std::min(count(attention_tc_kernel<false, CS>), count(attention_tc_kernel<true, CS>));
 }
@@ -773,7 +773,18 @@ int resident_clusters(int n_sms)
 
 void attention_clusters(int n_sms, int (&resident)[3])
 {
-    resident[0] = resident_clusters<2>(n_sms); resident[1] = resident_clusters<4>(n_sms); resident[2] = resident_clusters<8>(n_sms);
+    static PerDeviceValue known[3];                   // the answer + 1, asked once per device
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+    int (*const ask[3])(int) = {resident_clusters<2>, resident_clusters<4>, resident_clusters<8>};
+    for (int i = 0; i < 3; ++i) {
+        if (known[i].get(dev) == 0) {
+            resident[i] = ask[i](n_sms);
+            known[i].set(dev, resident[i] + 1);
+        } else {
+            resident[i] = known[i].get(dev) - 1;
+        }
+    }
     cudaGetLastError();                               // (a size that the device does not have is an answer, not an error)
 }
 
