@@ -93,11 +93,14 @@ int Forward::init_device(int dev, std::string &err)
             rc |= make_tmap_2d_bf16(&wmaps[(size_t)l].ffn.w1, (const __nv_bfloat16 *)w.w1 + (size_t)l * F * d, F, d, d, (uint32_t)kGemmWeightBoxRows, 64);
             rc |= make_tmap_2d_bf16(&wmaps[(size_t)l].ffn.w2, (const __nv_bfloat16 *)w.w2 + (size_t)l * d * F, d, F, F, (uint32_t)kGemmWeightBoxRows, 64);
             LayerMaps &m = wmaps[(size_t)l];
-            auto map64 = [&](CUtensorMap &out, const __nv_bfloat16 *base, uint64_t rows, uint64_t cols) { rc |= make_tmap_2d_bf16(&out, base, rows, cols, cols, 64, 64); };
-            map64(m.qkv64, wq, 3 * d, d); map64(m.kv64, wq + d * d, 2 * d, d); map64(m.wq64, wq, d, d);
-            map64(m.wo64, (const __nv_bfloat16 *)w.w_o + (size_t)l * d * d, d, d);
-            map64(m.w1_64, (const __nv_bfloat16 *)w.w1 + (size_t)l * F * d, F, d);
-            map64(m.w2_64, (const __nv_bfloat16 *)w.w2 + (size_t)l * d * F, d, F);
+            auto narrow = [&](LayerMaps::Narrow &out, const __nv_bfloat16 *base, uint64_t rows, uint64_t cols) {
+                rc |= make_tmap_2d_bf16(&out.rows64, base, rows, cols, cols, 64, 64);
+                rc |= make_tmap_2d_bf16(&out.rows32, base, rows, cols, cols, 32, 64);
+            };
+            narrow(m.qkv_n, wq, 3 * d, d); narrow(m.kv_n, wq + d * d, 2 * d, d); narrow(m.wq_n, wq, d, d);
+            narrow(m.wo_n, (const __nv_bfloat16 *)w.w_o + (size_t)l * d * d, d, d);
+            narrow(m.w1_n, (const __nv_bfloat16 *)w.w1 + (size_t)l * F * d, F, d);
+            narrow(m.w2_n, (const __nv_bfloat16 *)w.w2 + (size_t)l * d * F, d, F);
             if (ffn_fused_supported((int)d, (int)F)) {
                 rc |= make_tmap_2d_bf16(&wmaps[(size_t)l].ffn.w1_half, (const __nv_bfloat16 *)w.w1 + (size_t)l * F * d, F, d, d, 64, 64);
                 rc |= make_tmap_2d_bf16(&wmaps[(size_t)l].ffn.w2_wide, (const __nv_bfloat16 *)w.w2 + (size_t)l * d * F, d, F, F, 256, 64);
@@ -410,11 +413,11 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         if (trc != 0) { err = "tensor-map encoding of the activations failed"; return RELAYGR_E_CUDA; }
         act.ws = ws; act.rows = R; act.cand_rows = cand_rows; act.slab = call.pool_slab; act.pages = call.pool_pages;
     }
-    auto gemm = [&](int64_t M, const T *A, const CUtensorMap &tmA, const T *W, const CUtensorMap *tmW, const CUtensorMap *tmW64, const GemmOutMaps &om, int N, int K,
+    auto gemm = [&](int64_t M, const T *A, const CUtensorMap &tmA, const T *W, const CUtensorMap *tmW, const LayerMaps::Narrow *tmWn, const GemmOutMaps &om, int N, int K,
                     const Epilogue &ep) {
         cudaEvent_t pe = prof_begin(stream);
         cudaError_t r;
-        if constexpr (kTensor) r = launch_gemm_tc(tmA, *tmW, *tmW64, om, M, N, K, ep, d_status, stream, &launches);
+        if constexpr (kTensor) r = launch_gemm_tc(tmA, GemmWeightMaps{*tmW, tmWn->rows64, tmWn->rows32}, om, M, N, K, ep, d_status, stream, &launches);
         else if (tensor32) r = launch_gemm_f32_tc(tmA, *tmW, om, M, N, K, ep, n_sms, d_status, stream, &launches);
         else r = launch_gemm_f32(A, W, M, N, K, ep, n_sms, stream, &launches);
         prof_end(KC_GEMM, pe, stream);
@@ -535,7 +538,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         ep.seqs = d_seqs; ep.row_off = d_row_off; ep.n_users = B;
         if (preinfer) { ep.paged = paged; ep.page_runs = meta + o_runs; }
         const T *Wqkv = (const T *)w.w_qkv + ((size_t)l * 3 * d + ep.col0) * d;
-        e = gemm(R, ln1_in_gemm ? reinterpret_cast<const T *>(x) : a, tm_a, Wqkv, lm ? (kv_only ? &lm->kv : &lm->qkv) : nullptr, lm ? (kv_only ? &lm->kv64 : &lm->qkv64) : nullptr, om_qkv, 3 * d - ep.col0, d, ep);
+        e = gemm(R, ln1_in_gemm ? reinterpret_cast<const T *>(x) : a, tm_a, Wqkv, lm ? (kv_only ? &lm->kv : &lm->qkv) : nullptr, lm ? (kv_only ? &lm->kv_n : &lm->qkv_n) : nullptr, om_qkv, 3 * d - ep.col0, d, ep);
         if (!ck("QKV projection")) return RELAYGR_E_CUDA;
         }
         qkv_done = false;
@@ -560,7 +563,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
             eq.q_scale = q_scale;
             eq.q = q; eq.k_lin = kl; eq.v_lin = vl;
             eq.seqs = seqs_m; eq.row_off = meta + o_score; eq.n_users = B;
-            e = gemm(M, a_c, tm_a_c, (const T *)w.w_qkv + (size_t)l * 3 * d * d, lm ? &lm->wq : nullptr, lm ? &lm->wq64 : nullptr, om_qkv, d, d, eq);
+            e = gemm(M, a_c, tm_a_c, (const T *)w.w_qkv + (size_t)l * 3 * d * d, lm ? &lm->wq : nullptr, lm ? &lm->wq_n : nullptr, om_qkv, d, d, eq);
             if (!ck("query projection")) return RELAYGR_E_CUDA;
         }
 
@@ -623,7 +626,7 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         }
         Epilogue eo{};
         eo.mode = EPI_RESID; eo.bias = w.b_o ? w.b_o + (size_t)l * d : nullptr; eo.resid = xm; eo.out_f32 = xm;
-        e = gemm(M, att, tm_att, (const T *)w.w_o + (size_t)l * d * d, lm ? &lm->ffn.wo : nullptr, lm ? &lm->wo64 : nullptr, *om_xm, d, d, eo);
+        e = gemm(M, att, tm_att, (const T *)w.w_o + (size_t)l * d * d, lm ? &lm->ffn.wo : nullptr, lm ? &lm->wo_n : nullptr, *om_xm, d, d, eo);
         if (!ck("output projection")) return RELAYGR_E_CUDA;
 
         const float *g2 = w.ln2_g + (size_t)l * d, *b2n = w.ln2_b + (size_t)l * d;
@@ -634,12 +637,12 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         Epilogue e1{};
         if (ln2_in_gemm) with_ln(e1, g2, b2n);
         e1.mode = EPI_STORE; e1.silu = 1; e1.bias = w.b1 ? w.b1 + (size_t)l * F : nullptr; e1.out = hid;
-        e = gemm(M, ln2_in_gemm ? reinterpret_cast<const T *>(xm) : a, tm_a, (const T *)w.w1 + (size_t)l * F * d, lm ? &lm->ffn.w1 : nullptr, lm ? &lm->w1_64 : nullptr, om_hid, F, d, e1);
+        e = gemm(M, ln2_in_gemm ? reinterpret_cast<const T *>(xm) : a, tm_a, (const T *)w.w1 + (size_t)l * F * d, lm ? &lm->ffn.w1 : nullptr, lm ? &lm->w1_n : nullptr, om_hid, F, d, e1);
         if (!ck("FFN 1")) return RELAYGR_E_CUDA;
 
         Epilogue e2{};
         e2.mode = EPI_RESID; e2.bias = w.b2 ? w.b2 + (size_t)l * d : nullptr; e2.resid = xm; e2.out_f32 = xm;
-        e = gemm(M, hid, tm_hid, (const T *)w.w2 + (size_t)l * d * F, lm ? &lm->ffn.w2 : nullptr, lm ? &lm->w2_64 : nullptr, *om_xm, d, F, e2);
+        e = gemm(M, hid, tm_hid, (const T *)w.w2 + (size_t)l * d * F, lm ? &lm->ffn.w2 : nullptr, lm ? &lm->w2_n : nullptr, *om_xm, d, F, e2);
         if (!ck("FFN 2")) return RELAYGR_E_CUDA;
     }
 

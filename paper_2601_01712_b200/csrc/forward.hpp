@@ -57,7 +57,7 @@ struct Forward {
     int attn_clusters[3] = {0, 0, 0};      // how many clusters of 2, 4 and 8 CTAs of the attention kernel the device holds at once (bf16 model)
 
     // tensor maps of the weights, one set per layer
-    struct LayerMaps { CUtensorMap qkv, kv, wq; FfnMaps ffn; CUtensorMap qkv64, kv64, wq64, wo64, w1_64, w2_64; };      // (..64: boxes of 64 rows, bf16 model)
+    struct LayerMaps { CUtensorMap qkv, kv, wq; FfnMaps ffn; struct Narrow { CUtensorMap rows64, rows32; } qkv_n, kv_n, wq_n, wo_n, w1_n, w2_n; };      // (.._n: lower boxes, bf16 model)
     std::vector<LayerMaps> wmaps;
     bool wmaps_ok = false;       // false (fp32 model only): a weight pointer is not 16-byte aligned and cannot have a map
 

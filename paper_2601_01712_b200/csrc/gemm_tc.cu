@@ -12,13 +12,13 @@
 // with plain stores after a page-table walk per row otherwise.
 //
 // The shapes (Cfg below): single CTAs with 128 x 128 tiles, and CTA pairs (a cluster of two,
-// tcgen05 cta_group::2) with 256 x 256 tiles - 256 x 128 where those would leave every other pair
+// tcgen05 cta_group::2) with 256 x 256 tiles - 256 x 128 or 256 x 64 where those would leave pairs
 // idle -, where each CTA loads its 128 rows of A and half of W and the even CTA issues the MMAs for both.
 //
 // Warp roles (320 threads per CTA): warp 0 = TMA producer (128 x 64 tiles of A and W, 128-byte
-// swizzle, a ring of five stages or seven), warp 1 = TMEM owner + MMA issuer (tcgen05.mma K16), warps 2-9 =
+// swizzle, a ring of five to eight stages), warp 1 = TMEM owner + MMA issuer (tcgen05.mma K16), warps 2-9 =
 // epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 (its hardware quadrant), columns
-// (BN / 2) ((w - 2) / 4) .. + BN / 2 - 1, 64 at a time, applies bias / SiLU in the
+// (BN / 2) ((w - 2) / 4) .. + BN / 2 - 1 (all 64 of the narrowest tile: warps 2-5 alone), 64 at a time, applies bias / SiLU in the
 // row-per-thread layout tcgen05.ld delivers and stages the result for the store.
 #include "kernels.cuh"
 #include "tc_common.cuh"
@@ -27,7 +27,7 @@ namespace relaygr {
 
 namespace {
 
-constexpr int BM = 128, BK = 64, kMaxStages = 7;
+constexpr int BM = 128, BK = 64, kMaxStages = 8;
 constexpr int kEpiWarps = 8;
 constexpr int kThreads = 32 * (2 + kEpiWarps);
 constexpr int kABytes = BM * BK * 2;
@@ -43,7 +43,8 @@ constexpr int kMaxBias = 4096;                                       // output c
 template <int BN, int CTAS> struct Cfg {
     static constexpr int kBBytes = (BN / CTAS) * BK * 2;
     static constexpr int kStage = kABytes + kBBytes;
-    static constexpr int kStages = CTAS == 2 && BN == 128 ? 7 : 5;
+    static constexpr int kStages = CTAS == 1 || BN == 256 ? 5 : BN == 128 ? 7 : 8;
+    static constexpr int kHalves = BN >= 128 ? 2 : 1;                                     // warps to a TMEM quadrant in the epilogue, 64 columns or more each
     static constexpr int kOffPatch = kStages * kStage;                                    // 1024-byte aligned: stages are
     static constexpr int kOffBias = kOffPatch + kEpiWarps * kPatches * kPatchBytes;       // kMaxBias floats
     static constexpr int kOffRowOff = kOffBias + kMaxBias * 4;                            // per warp 32 x int64
@@ -100,7 +101,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // set-up that touches nothing earlier kernels wrote; it may run while the previous kernel is still finishing
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { tc::mbar_init(&bars->full[s], 1); tc::mbar_init(&bars->empty[s], 1); }
-        for (int s = 0; s < 2; ++s) { tc::mbar_init(&bars->acc_full[s], 1); tc::mbar_init(&bars->acc_empty[s], kEpiWarps * CTAS); }
+        for (int s = 0; s < 2; ++s) { tc::mbar_init(&bars->acc_full[s], 1); tc::mbar_init(&bars->acc_empty[s], 4 * C::kHalves * CTAS); }
         tc::fence_mbar_init();
         tc::tma_prefetch_desc(&tmA);
         tc::tma_prefetch_desc(&tmB);
@@ -189,7 +190,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int ew = warp - 2;
         const int quad = warp & 3;                          // TMEM lanes this warp may touch: 32*quad .. 32*quad+31
         const int half = ew >> 2;                           // columns (BN/2)*half .. +BN/2-1 of the tile, 64 at a time
-        constexpr int kColsPerWarp = BN / 2;
+        constexpr int kColsPerWarp = BN / C::kHalves;
         uint8_t *patches = smem + C::kOffPatch + ew * (kPatches * kPatchBytes);
         // An earlier kernel gave up: nothing is stored.  (The loads and products go on as ever: to wait for this word before them would
         // put a trip to L2 and a block-wide barrier, 1000 clocks, between the predecessor's end and the first load.)
@@ -226,7 +227,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         uint32_t ti = 0;
         bool ok = true;
         const uint32_t acc_empty_bar = CTAS == 2 ? tc::cluster_addr(&bars->acc_empty[0], 0) : tc::smem_u32(&bars->acc_empty[0]);
-        for (int t = worker; t < n_tiles && ok; t += n_workers, ++ti) {
+        for (int t = half < C::kHalves ? worker : n_tiles; t < n_tiles && ok; t += n_workers, ++ti) {
             const int64_t m0 = (int64_t)(t / n_tiles_n) * (BM * CTAS) + rank * BM;
             const int n_w = (t % n_tiles_n) * BN + half * kColsPerWarp;      // first column of this warp's part
             const uint32_t as = ti & 1;
@@ -397,7 +398,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 }  // namespace
 
 template <int BN, int CTAS>
-static cudaError_t launch_cfg(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmB64, const GemmOutMaps &om, int64_t M, int N, int K,
+static cudaError_t launch_cfg(const CUtensorMap &tmA, const GemmWeightMaps &tmB, const GemmOutMaps &om, int64_t M, int N, int K,
                               const Epilogue &epi, int *err, cudaStream_t stream)
 {
     using C = Cfg<BN, CTAS>;
@@ -427,23 +428,26 @@ static cudaError_t launch_cfg(const CUtensorMap &tmA, const CUtensorMap &tmB, co
         n_workers_max = n;
         workers_of.set(dev, n);
     }
-    // Pairs with half-wide tiles where at least every other pair would be idle otherwise: such a tile takes three quarters of a whole one's time
-    // (24 KB of operands a K block instead of 32 KB through the same 64 B / clk).  Ranking calls of one user, 576 rows: d_model 512 512 -> 452 us,
-    // 1024 339 -> 305; the candidates' GEMMs of the widest model's full inference, 36 tiles, 10 us of 865.
+    // Pairs with half-wide tiles where at least every other pair would be idle otherwise, and with quarter-wide ones where at least three of four would:
+    // such a tile takes three quarters (five eighths) of a whole one's time, 24 KB (20 KB) of operands a K block instead of 32 KB through
+    // the same 64 B / clk.  A call in us with whole / half / quarter-wide tiles: ranking of 576 rows, d_model 512 512 / 451 / 449, d_model 1024
+    // 339 / 304 / 301; pre-inference of 1500 rows, d_model 512 506 / 451 / 428; the candidates' GEMMs of the widest model's full inference, 36
+    // tiles, take 10 us less of 865 in half-wide ones.
     const int64_t tiles = ((M + BM * CTAS - 1) / (BM * CTAS)) * (N / BN);
-    if (CTAS == 2 && BN == 256 && 2 * tiles <= n_workers_max) return launch_cfg<128, 2>(tmA, tmB, tmB64, om, M, N, K, epi, err, stream);
+    if constexpr (CTAS == 2 && BN > 64)
+        if (2 * tiles <= n_workers_max) return launch_cfg<BN / 2, 2>(tmA, tmB, om, M, N, K, epi, err, stream);
     const unsigned workers = (unsigned)(tiles < n_workers_max ? tiles : n_workers_max);
-    return launch_dependent(gemm_tc_kernel<BN, CTAS>, dim3(workers * CTAS), dim3(kThreads), (size_t)C::kSmemBytes, stream, CTAS, tmA, BN / CTAS == 64 ? tmB64 : tmB, om,
+    return launch_dependent(gemm_tc_kernel<BN, CTAS>, dim3(workers * CTAS), dim3(kThreads), (size_t)C::kSmemBytes, stream, CTAS, tmA, BN / CTAS == 128 ? tmB.rows128 : BN / CTAS == 64 ? tmB.rows64 : tmB.rows32, om,
                             M, N, K, epi, err);
 }
 
-cudaError_t launch_gemm_tc(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmB64, const GemmOutMaps &om, int64_t M, int N, int K,
+cudaError_t launch_gemm_tc(const CUtensorMap &tmA, const GemmWeightMaps &tmB, const GemmOutMaps &om, int64_t M, int N, int K,
                            const Epilogue &epi, int *err, cudaStream_t stream, int64_t *launches)
 {
     if (M == 0 || N == 0) return cudaSuccess;
     *launches += 1;
-    return gemm_pair(M, N, K) ? launch_cfg<256, 2>(tmA, tmB, tmB64, om, M, N, K, epi, err, stream)
-                        : launch_cfg<128, 1>(tmA, tmB, tmB64, om, M, N, K, epi, err, stream);
+    return gemm_pair(M, N, K) ? launch_cfg<256, 2>(tmA, tmB, om, M, N, K, epi, err, stream)
+                        : launch_cfg<128, 1>(tmA, tmB, om, M, N, K, epi, err, stream);
 }
 
 }  // namespace relaygr

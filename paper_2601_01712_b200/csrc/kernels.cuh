@@ -145,9 +145,10 @@ inline bool gemm_pair(int64_t M, int N, int K)
 constexpr int kGemmWeightBoxRows = 128;
 
 // C[m, n] = sum_k A[m, k] W[n, k] on tcgen05; tmA covers A [M, K] with a 128-row box, tmB covers W [N, K]
-// with a box of kGemmWeightBoxRows rows, tmB64 with one of 64 rows, all 64 columns wide with the 128-byte swizzle.  N % 128 == 0, K % 64 == 0.
+// with boxes of kGemmWeightBoxRows, 64 and 32 rows, all 64 columns wide with the 128-byte swizzle.  N % 128 == 0, K % 64 == 0.
 // err is a device status word: kernels record a code there instead of hanging or trapping.
-cudaError_t launch_gemm_tc(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmB64, const GemmOutMaps &om, int64_t M, int N, int K,
+struct GemmWeightMaps { const CUtensorMap &rows128, &rows64, &rows32; };
+cudaError_t launch_gemm_tc(const CUtensorMap &tmA, const GemmWeightMaps &tmB, const GemmOutMaps &om, int64_t M, int N, int K,
                            const Epilogue &epi, int *err, cudaStream_t stream, int64_t *launches);
 
 // Everything of a block after the attention in one kernel, for the shapes ffn_fused_supported() accepts (d_model = 256, d_ff a

@@ -328,10 +328,12 @@ def test_f32_tiles_of_eight_rows(d, heads, kind, prefix, short, cand):
     _check_f32(shape, _tiny_batch(shape, 410 + d + heads, prefix, short, cand), 75)
 
 
-# GEMMs of a wider model in half-wide tiles of CTA pairs: as long as two of them go to every pair (d_model 512: the QKV projection up to 1536 rows, the
-# others up to 2304 and 4608), ragged last rows, pages, the candidates' own GEMMs of a full inference.
-@pytest.mark.parametrize("prefix,short,cand", [([1], [0], [1]), ([257], [3], [254]), ([70, 64], [0, 5], [1036, 495]), ([70, 64], [0, 5], [1036, 496]), ([1537], [1], [60])])
-def test_half_wide_tiles(prefix, short, cand):
+# GEMMs of a wider model in half- and quarter-wide tiles of CTA pairs: as long as they do not outnumber the pairs (d_model 512: half-wide ones of the QKV
+# projection up to 1536 rows, quarter-wide ones up to 768; the others up to 2304 and 4608), ragged last rows, pages, the candidates' own GEMMs of a
+# full inference.
+@pytest.mark.parametrize("prefix,short,cand", [([1], [0], [1]), ([257], [3], [254]), ([769], [3], [765]), ([70, 64], [0, 5], [1036, 495]),
+                                               ([70, 64], [0, 5], [1036, 496]), ([1537], [1], [60])])
+def test_narrow_tiles(prefix, short, cand):
     shape = synth.ModelShape(2, 512, 8, 64, 1024, 2000, synth.DTYPE_BF16)
     batch = _tiny_batch(shape, 420 + len(prefix) + cand[-1], prefix, short, cand)
     w, model, pool, db = _setup(shape, 76, batch)
