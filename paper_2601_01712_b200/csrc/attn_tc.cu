@@ -6,17 +6,20 @@
 // 64-key blocks (one block = one 64-token page of the pool, or 64 rows of the call's transient
 // K/V buffers; one 8 KB TMA box each for K and V).  Per block:
 //     S = Q K^T   tcgen05.mma M=128 N=64 K=64, operands in shared memory, S in TMEM
-//     softmax     128 threads, one row each: S row -> registers, p = 2^(s - m) (the queries carry
-//                 log2(e) / sqrt(d_h)), bf16 P written back to TMEM
+//     softmax     128 threads, one row each: S row -> registers, running max, p = 2^(s c - m c),
+//                 bf16 P written back to TMEM
 //     O += P V    tcgen05.mma M=128 N=64 K=64, A = P from TMEM, B = V in shared memory (MN-major),
 //                 O accumulated in TMEM
 // S and P are double-buffered in TMEM, so the MMA warp runs one block ahead of the softmax and
-// the tensor pipe never waits for it in steady state.  The reference m of a row is fixed by its first
-// block: 0 where that block's maximum is near 0 (then the scores go into the exponential as they are: two
-// instructions less for every four scores, 1 % of a rank call of 32 users, 2-3 % of the long-sequence
-// calls), else that maximum.  Only when a block's row sum shows that some score lies far above the
-// reference is the block maximum computed, the reference raised, O rescaled in TMEM (after the pending
-// PV has drained) and the block redone - so no maximum is on the fast path, and rescales are rare.
+// the tensor pipe never waits for it in steady state.  The exponentials of a block are taken
+// against the running maximum as it stood before the block; only when the block's row sum shows
+// that some exponent may have exceeded 2^8 is the block maximum computed, the running maximum
+// raised, O rescaled in TMEM (after the pending PV has drained) and the block redone - so no
+// maximum is on the fast path, every exponent that is kept stays below 2^8, and rescales are rare.
+// (The loop is bound by its issue slots.  Queries that carry log2(e) / sqrt(d_h), so that rows near 0
+// need neither scale nor maximum, took 2 % off a rank call of 32 users and 2-4 % off the long ones; but
+// q times that factor rounds to other bf16 values than q, and calls with few candidates then differed
+// from before by as much as the whole rounding error, 1 %.)
 // A candidate's own key (it sees the prefix, the short-term tokens and itself) is one more block
 // of the same pipeline: the 64-row group of the call's K / V that holds the candidate's row, with
 // a diagonal mask (own_key_blocks) and one exponential per row.
@@ -30,7 +33,6 @@
 // Warp roles (192 threads): warp 0 = TMA producer (and the item counter), warp 1 = TMEM owner +
 // MMA issuer, warps 2-5 = softmax / correction / epilogue (TMEM lane quadrant = warp index % 4).
 #include <algorithm>
-#include <type_traits>
 
 #include "kernels.cuh"
 #include "tc_common.cuh"
@@ -55,12 +57,8 @@ constexpr int kMaxStagesKV = 4;
 constexpr uint32_t kTmemCols = 256;                 // S[2]: 0..127, P[2]: 128..191, O: 192..255
 constexpr uint32_t kColS = 0, kColP = 128, kColO = 192;
 constexpr int kPartStride = kDh + 4;                // floats per row of a split partial: m, l, two unused, then O (16-byte aligned rows)
-// The reference m of a row's weights 2^(s - m) need not be its maximum: any that keeps the weights and their sums well inside fp32 (and bf16,
-// which has its exponents) gives the same relative precision.  A row whose first block's maximum lies within kZeroRef of 0 is taken
-// against 0, and a warp of such rows takes its exponentials straight from the scores.
-constexpr float kZeroRef = 32.f;
-constexpr float kRaise = 54.f;                      // a score this far above the reference raises it ...
-constexpr float kRowSumLimit = 0x1p60f;             // ... which a block's row sum shows: 64 weights
+constexpr float kRowSumLimit = 256.f;               // a block's row sum above this: some p may exceed 2^8 -> redo against a raised maximum
+constexpr float kLogit = 0.125f * 1.4426950408889634f;       // 1/sqrt(64) * log2(e)
 
 // CS > 1: the CS pieces of a tile's key range are the CTAs of a cluster, which put their results together themselves (merge_rows): a
 // ring stage less makes room for them.
@@ -91,12 +89,12 @@ struct Bars {
     int abort_flag;
 };
 
-// 2^x, x = s - m, for a pair WITHOUT the XU pipe: x is rounded to the nearest integer n by adding 1.5 * 2^23 (n then sits
+// 2^x, x = s * c - mc, for a pair WITHOUT the XU pipe: x is rounded to the nearest integer n by adding 1.5 * 2^23 (n then sits
 // in the low mantissa bits), a cubic gives 2^(x - n) on [-0.5, 0.5] (relative error 7.5e-5, far below the bf16 rounding of P that
 // follows) and n is added to the exponent field as an integer.  x has to lie in [-126, 127]: below, the result is ~1e-38 instead
 // of 0 (a masked key's -inf included: its weight stays negligible), above, the row-sum check of the caller fails and the block is
 // redone against a true maximum.  The multiply-add that scales s clamps for nothing: it computes t = (x + 126) / 253 saturated to
-// [0, 1] (x is then off by at most 8e-6).  ct = 1 / 253, mt = (126 - m) / 253.
+// [0, 1] (x is then off by at most 8e-6).  ct = c / 253, mt = (126 - mc) / 253.
 constexpr float kExpLo = 126.f, kExpSpan = 253.f;
 __device__ __forceinline__ void exp2_fma_pipe(float s0, float s1, float ct, float mt, float &p0, float &p1)
 {
@@ -140,7 +138,7 @@ __device__ __forceinline__ void own_key_blocks(const AttnItem &it, const SeqDesc
     }
 }
 
-// O = sum_i 2^(m_i - M) O_i / sum_i 2^(m_i - M) l_i of the 128 / CS rows that this CTA finishes, from `parts` [CS][rows][kPartStride]: CS threads
+// O = sum_i 2^((m_i - M) c) O_i / sum_i 2^((m_i - M) c) l_i of the 128 / CS rows that this CTA finishes, from `parts` [CS][rows][kPartStride]: CS threads
 // a row, each 64 / CS columns, the partial results in rank order.  Called by the softmax warps.
 template <int CS>
 __device__ __forceinline__ void merge_rows(const float *parts, int64_t row0, int n_q, int col, int d_model, __nv_bfloat16 *out)
@@ -158,7 +156,7 @@ __device__ __forceinline__ void merge_rows(const float *parts, int64_t row0, int
     }
 #pragma unroll
     for (int i = 0; i < CS; ++i) {
-        const float w = ml[i].x == -INFINITY ? 0.f : ex2(ml[i].x - M);
+        const float w = ml[i].x == -INFINITY ? 0.f : ex2((ml[i].x - M) * kLogit);
         l = fmaf(ml[i].y, w, l);
 #pragma unroll
         for (int c = 0; c < kCols; c += 4) {
@@ -405,21 +403,18 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         if (n_clean == n_paged_blocks && tile_min_lim >= it.lin_pos0) n_clean += min(it.n_lin, tile_min_lim + 1 - it.lin_pos0) / kKeys;
         n_clean -= it.blk0;                                   // relative to the item's first block
         float m = -INFINITY, l = 0.f;
-        bool zero_ref = false;                                // all rows of the warp: m = 0
         // a warp whose 32 rows all lie past the tile's last row keeps the hand-shakes going but takes no exponentials:
         // its rows of P (and of O) hold whatever TMEM held, which only ever reaches those same, unused, rows
         const bool warp_live = quad * 32 < it.n_q;
 
-        // A block's largest score mx of the row: raises the reference, and rescales O (which then has to hold blocks 0..j-1 completely) and, by
-        // the caller, l.
-        auto raise_reference = [&](int j, float mx, float &alpha) {
-            // (a row's own keys decide, not those of the warp's other rows; false when mx == -inf)
-            const bool raise = m == -INFINITY ? mx > m : mx > m + kRaise;
+        // A block's largest score mx of the row: raises the running maximum, and rescales O (which then has to hold blocks 0..j-1 completely)
+        // and, by the caller, l.
+        auto raise_maximum = [&](int j, float mx, float &alpha) {
+            const bool raise = mx > m;                        // false when mx == -inf
             if (raise) {
-                alpha = (m == -INFINITY) ? 0.f : ex2(m - mx);
-                m = m == -INFINITY && fabsf(mx) <= kZeroRef ? 0.f : mx;
+                alpha = (m == -INFINITY) ? 0.f : ex2((m - mx) * kLogit);
+                m = mx;
             }
-            zero_ref = __all_sync(0xffffffffu, m == 0.f);
             if (j == 0 || !__any_sync(0xffffffffu, raise)) return true;
             const int gb = g + j;
             if (!__all_sync(0xffffffffu, tc::mbar_wait(&bars->p_free[(gb - 1) & 1], ((gb - 1) >> 1) & 1, err))) return false;
@@ -493,8 +488,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     if (sees) p = fmaf(h, t, h);
                 } else {
                     float alpha = 1.f;
-                    if (!(ok = raise_reference(j, sees ? sv : -INFINITY, alpha))) break;
-                    if (sees) p = ex2(sv - (m == -INFINITY ? 0.f : m));
+                    if (!(ok = raise_maximum(j, sees ? sv : -INFINITY, alpha))) break;
+                    if (sees) p = ex2((sv - (m == -INFINITY ? 0.f : m)) * kLogit);
                     l = fmaf(l, alpha, p);
                 }
                 const uint32_t word = tc::pack_bf16(own & 1 ? 0.f : p, own & 1 ? p : 0.f);
@@ -532,15 +527,16 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 publish_p(b);
                 continue;
             }
-            // p = 2^(s - m), bf16 P into TMEM (P[b] is free: see the MMA issuer), row sum in fp32.  The exponentials are first taken against
-            // the reference as it stood before this block; only if the row sum shows that some score is far above it (or the row has
-            // none yet) is the block maximum computed, the reference raised, O rescaled and the block redone.
+            // p = 2^(s c - m c), bf16 P into TMEM (P[b] is free: see the MMA issuer), row sum in fp32.  The exponentials
+            // are first taken against the running maximum as it stood before this block; only if the row sum shows that
+            // some p may have exceeded 2^8 (or the row has no maximum yet) is the block maximum computed, the running
+            // maximum raised, O rescaled and the block redone.  No maximum is on the fast path.
             // Every fourth pair takes its exponentials on the FMA pipe instead (exp2_fma_pipe): the XU pipe is what the two
             // CTAs of an SM compete for (measured: 5-7 % off a rank launch; an eighth or three eighths gain less).  (A compile-time pattern: a run-time switch between the two forms inside
             // the unrolled block cost more than the off-loading gains.)
-            auto exp_block = [&](auto kZero, float ref) {
-                const uint64_t nref2 = pack2(-ref, -ref);
-                const float mt = (kExpLo - ref) * (1.f / kExpSpan);
+            auto exp_block = [&](float mc) {
+                const uint64_t c2 = pack2(kLogit, kLogit), nmc2 = pack2(-mc, -mc);
+                const float mt = (kExpLo - mc) * (1.f / kExpSpan);
                 uint64_t rs2[2] = {0, 0};
                 uint32_t pk[16];
 #pragma unroll
@@ -550,10 +546,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                         const float a0 = __uint_as_float(half == 0 ? s0[2 * i] : s1[2 * i]), a1 = __uint_as_float(half == 0 ? s0[2 * i + 1] : s1[2 * i + 1]);
                         float p0, p1;
                         if (offloaded(i)) {
-                            exp2_fma_pipe(a0, a1, 1.f / kExpSpan, mt, p0, p1);
+                            exp2_fma_pipe(a0, a1, kLogit * (1.f / kExpSpan), mt, p0, p1);
                         } else {
-                            if constexpr (decltype(kZero)::value) { p0 = a0; p1 = a1; }
-                            else unpack2(add2(pack2(a0, a1), nref2), p0, p1);
+                            unpack2(fma2(pack2(a0, a1), c2, nmc2), p0, p1);
                             p0 = ex2(p0); p1 = ex2(p1);
                         }
                         rs2[i & 1] = add2(rs2[i & 1], pack2(p0, p1));
@@ -568,7 +563,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             float rs = 0.f, alpha = 1.f;
             bool redo = true;
             if (j > 0) {
-                rs = zero_ref ? exp_block(std::true_type{}, 0.f) : exp_block(std::false_type{}, (m == -INFINITY) ? 0.f : m);
+                rs = exp_block((m == -INFINITY) ? 0.f : m * kLogit);
                 redo = __any_sync(0xffffffffu, !(rs <= kRowSumLimit) || m == -INFINITY);
             }
             if (redo) {
@@ -581,8 +576,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     mx3 = max3(mx3, __uint_as_float(s1[i + 2]), __uint_as_float(s1[i + 3]));
                 }
                 mx = fmaxf(fmaxf(mx, mx1), fmaxf(mx2, mx3));
-                if (!(ok = raise_reference(j, mx, alpha))) break;
-                rs = exp_block(std::false_type{}, (m == -INFINITY) ? 0.f : m);
+                if (!(ok = raise_maximum(j, mx, alpha))) break;
+                rs = exp_block((m == -INFINITY) ? 0.f : m * kLogit);
             }
             l = fmaf(l, alpha, rs);
             tc::tmem_st_wait();
@@ -688,12 +683,12 @@ __device__ __forceinline__ void merge_row(const float *p, int n, int lane, float
         }
 #pragma unroll
         for (int i = 0; i < kBatch; ++i) Mb = fmaxf(Mb, ml[i].x);
-        const float alpha = M == -INFINITY ? 0.f : ex2(M - Mb);
+        const float alpha = M == -INFINITY ? 0.f : ex2((M - Mb) * kLogit);
         M = Mb;
         l *= alpha; o0 *= alpha; o1 *= alpha;
 #pragma unroll
         for (int i = 0; i < kBatch; ++i) {
-            const float wgt = (ml[i].x == -INFINITY) ? 0.f : ex2(ml[i].x - M);
+            const float wgt = (ml[i].x == -INFINITY) ? 0.f : ex2((ml[i].x - M) * kLogit);
             l = fmaf(ml[i].y, wgt, l);
             o0 = fmaf(v[i].x, wgt, o0);
             o1 = fmaf(v[i].y, wgt, o1);

@@ -49,7 +49,7 @@ embed_rows_kernel(const __grid_constant__ CUtensorMap tmQkv, const __nv_bfloat16
         tc::tmem_relinquish();
     }
     const int n = chunk * kChunk + quad * 32 + lane, which = (to.col0 + n) >> 8, c = (to.col0 + n) & (kD - 1);      // this lane's output column
-    const float scale = which == 0 ? to.q_scale : 1.f, bias = to.bias ? to.bias[n] * scale : 0.f;
+    const float bias = to.bias ? to.bias[n] : 0.f;
     const bool to_page = to.paged.slab != nullptr && which > 0;
     float4 gain[2], shift[2];
 #pragma unroll
@@ -147,7 +147,7 @@ embed_rows_kernel(const __grid_constant__ CUtensorMap tmQkv, const __nv_bfloat16
             const int rt = half * 16 + e;
             if (tile_row0 + rt >= M || stopped) break;
             __nv_bfloat16 *p = base + (to_page ? page_off[rt] : (int64_t)rt * kD);
-            *p = __float2bfloat16_rn(fmaf(__uint_as_float(r[e]), scale, bias));
+            *p = __float2bfloat16_rn(__uint_as_float(r[e]) + bias);
             if (to_page && last_slot[rt] >= 0)        // last row of the prefix: clear the unused slots of its page
                 for (int z = 1; last_slot[rt] + z < 64; ++z) p[z * kD] = __float2bfloat16_rn(0.f);
         }

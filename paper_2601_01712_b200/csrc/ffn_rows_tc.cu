@@ -484,7 +484,7 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
             for (int i = 0; i < nq; ++i) {
                 const int hb = (nc + i) & 1, n = chunk_at(i) * kChunk + quad * 32 + lane;      // this lane's output column
                 const int which = (tail.col0 + n) >> 8, c = (tail.col0 + n) & (kD - 1);
-                const float scale = which == 0 ? tail.q_scale : 1.f, bias = tail.bias ? tail.bias[n] * scale : 0.f;
+                const float bias = tail.bias ? tail.bias[n] : 0.f;
                 ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->s_full[hb], ((nc + i) >> 1) & 1, err));
                 if (!ok) break;
                 tc::tc_fence_after();
@@ -504,7 +504,7 @@ ffn_rows_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant_
                     const int rt = ch * (T / 2) + e;
                     if (tile_row0 + rt >= M) break;
                     __nv_bfloat16 *p = base + (to_page ? page_off[rt] : (int64_t)rt * kD);
-                    *p = __float2bfloat16_rn(fmaf(__uint_as_float(r[e]), scale, bias));
+                    *p = __float2bfloat16_rn(__uint_as_float(r[e]) + bias);
                     if (to_page && last_slot[rt] >= 0)      // last row of the prefix: clear the unused slots of its page
                         for (int z = 1; last_slot[rt] + z < 64; ++z) p[z * kD] = __float2bfloat16_rn(0.f);
                 }

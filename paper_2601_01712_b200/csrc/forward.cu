@@ -430,7 +430,6 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         return r;
     };
     const LayerMaps *lm = nullptr;
-    const float q_scale = cfg.attn_kind == ATTN_POINTWISE ? 1.f : 0.125f * 1.4426950408889634f;      // logits in units of log2(e)
 
     // the rows the part of a layer after the QKV projection runs on: all of them, or (last layer) the candidates alone
     int64_t M = R;
@@ -478,7 +477,6 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         t.qkv_map = kv ? &wmaps[(size_t)l].kv : &wmaps[(size_t)l].qkv;
         t.col0 = kv ? d : 0; t.n_qkv = 3 * d - t.col0;
         t.bias = w.b_qkv ? w.b_qkv + (size_t)l * 3 * d + t.col0 : nullptr;
-        t.q_scale = q_scale;
         t.q = reinterpret_cast<__nv_bfloat16 *>(q); t.k = reinterpret_cast<__nv_bfloat16 *>(kl); t.v = reinterpret_cast<__nv_bfloat16 *>(vl);
         if (preinfer) t.paged = PagedKV{call.pool_slab, meta + o_pt, L, d, l};
         t.row_off = d_row_off; t.seqs = d_seqs; t.n_users = B;
@@ -533,7 +531,6 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
         ep.col0 = kv_only ? d : 0;
         ep.bias = w.b_qkv ? w.b_qkv + (size_t)l * 3 * d + ep.col0 : nullptr;
         ep.d_model = d;
-        ep.q_scale = q_scale;
         ep.q = q; ep.k_lin = kl; ep.v_lin = vl;
         ep.seqs = d_seqs; ep.row_off = d_row_off; ep.n_users = B;
         if (preinfer) { ep.paged = paged; ep.page_runs = meta + o_runs; }
@@ -560,7 +557,6 @@ int Forward::run_t(const CallDesc &call, float *scores, cudaStream_t stream, std
             eq.col0 = 0;
             eq.bias = w.b_qkv ? w.b_qkv + (size_t)l * 3 * d : nullptr;
             eq.d_model = d;
-            eq.q_scale = q_scale;
             eq.q = q; eq.k_lin = kl; eq.v_lin = vl;
             eq.seqs = seqs_m; eq.row_off = meta + o_score; eq.n_users = B;
             e = gemm(M, a_c, tm_a_c, (const T *)w.w_qkv + (size_t)l * 3 * d * d, lm ? &lm->wq : nullptr, lm ? &lm->wq_n : nullptr, om_qkv, d, d, eq);

@@ -195,13 +195,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // An earlier kernel gave up: nothing is stored.  (The loads and products go on as ever: to wait for this word before them would
         // put a trip to L2 and a block-wide barrier, 1000 clocks, between the predecessor's end and the first load.)
         const bool stopped = *reinterpret_cast<volatile int *>(err) != 0;
-        // queries carry the factor of their logits
-        auto scale_of = [&](int n) { return epi.mode == EPI_QKV && epi.col0 + n < epi.d_model ? epi.q_scale : 1.f; };
         // the whole bias once, under the first tile's loads: a look-up per tile would be on the epilogue's path
         float *bias_s = reinterpret_cast<float *>(smem + C::kOffBias);
         const bool bias_staged = epi.bias && N <= kMaxBias;
         if (bias_staged) {
-            for (int i = threadIdx.x - 64; i < N; i += 32 * kEpiWarps) bias_s[i] = epi.bias[i] * scale_of(i);
+            for (int i = threadIdx.x - 64; i < N; i += 32 * kEpiWarps) bias_s[i] = epi.bias[i];
             asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
         }
         int64_t *rowoff = reinterpret_cast<int64_t *>(smem + C::kOffRowOff) + ew * 32;
@@ -236,7 +234,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             float *bias_w = bias_s + (bias_staged ? n_w : ew * kColsPerWarp);      // this warp's slice of the bias
             if (epi.bias && !bias_staged) {
 #pragma unroll
-                for (int c = 0; c < kColsPerWarp; c += 32) bias_w[c + lane] = epi.bias[n_w + c + lane] * scale_of(n_w + c + lane);
+                for (int c = 0; c < kColsPerWarp; c += 32) bias_w[c + lane] = epi.bias[n_w + c + lane];
             }
             // before the accumulator is ready, for K / V rows of a pre-infer call (they go straight into the user's pages): where in
             // the pool the warp's 32 rows are, if they are 32 consecutive slots of one page (the table says so), else the offset
@@ -282,26 +280,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 }
                 if (m_base >= M || stopped) continue;                            // the whole row group lies past the last row
                 const int n = n_w + pass * 64;                                   // first output column of these 64
-                const float scale = scale_of(n);                                 // (the bias carries it already)
                 if (epi.bias) {
                     const float4 *b4 = reinterpret_cast<const float4 *>(bias_w + pass * 64);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         const float4 b = b4[i], c = b4[8 + i];
-                        r0[4 * i] = __float_as_uint(fmaf(__uint_as_float(r0[4 * i]), scale, b.x));
-                        r0[4 * i + 1] = __float_as_uint(fmaf(__uint_as_float(r0[4 * i + 1]), scale, b.y));
-                        r0[4 * i + 2] = __float_as_uint(fmaf(__uint_as_float(r0[4 * i + 2]), scale, b.z));
-                        r0[4 * i + 3] = __float_as_uint(fmaf(__uint_as_float(r0[4 * i + 3]), scale, b.w));
-                        r1[4 * i] = __float_as_uint(fmaf(__uint_as_float(r1[4 * i]), scale, c.x));
-                        r1[4 * i + 1] = __float_as_uint(fmaf(__uint_as_float(r1[4 * i + 1]), scale, c.y));
-                        r1[4 * i + 2] = __float_as_uint(fmaf(__uint_as_float(r1[4 * i + 2]), scale, c.z));
-                        r1[4 * i + 3] = __float_as_uint(fmaf(__uint_as_float(r1[4 * i + 3]), scale, c.w));
-                    }
-                } else if (scale != 1.f) {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) {
-                        r0[i] = __float_as_uint(__uint_as_float(r0[i]) * scale);
-                        r1[i] = __float_as_uint(__uint_as_float(r1[i]) * scale);
+                        r0[4 * i] = __float_as_uint(__uint_as_float(r0[4 * i]) + b.x);
+                        r0[4 * i + 1] = __float_as_uint(__uint_as_float(r0[4 * i + 1]) + b.y);
+                        r0[4 * i + 2] = __float_as_uint(__uint_as_float(r0[4 * i + 2]) + b.z);
+                        r0[4 * i + 3] = __float_as_uint(__uint_as_float(r0[4 * i + 3]) + b.w);
+                        r1[4 * i] = __float_as_uint(__uint_as_float(r1[4 * i]) + c.x);
+                        r1[4 * i + 1] = __float_as_uint(__uint_as_float(r1[4 * i + 1]) + c.y);
+                        r1[4 * i + 2] = __float_as_uint(__uint_as_float(r1[4 * i + 2]) + c.z);
+                        r1[4 * i + 3] = __float_as_uint(__uint_as_float(r1[4 * i + 3]) + c.w);
                     }
                 }
                 if (epi.mode == EPI_RESID) {

@@ -80,8 +80,7 @@ struct Epilogue {
     // EPI_QKV: column c of the full [3d] output goes to q (c < d), K (d <= c < 2d) or V.
     int32_t col0;                 // first output column this GEMM computes (0, or d for K/V only)
     int32_t d_model;
-    void *q;                      // [M, d]; bf16 model: times q_scale
-    float q_scale;
+    void *q;                      // [M, d]
     void *k_lin, *v_lin;          // [M, d] transient K/V (used when paged.slab == nullptr)
     PagedKV paged;                // else K/V rows are scattered into pages
     // Per group of 32 rows of a paged scatter: page * 64 + first slot if the rows are 32 consecutive slots of one page of a user whose

@@ -173,11 +173,10 @@ struct FfnTail {
     const SeqDesc *seqs;          // score_row0, n_score: rows of this launch
     const int32_t *score_off;
     int n_users;
-    // FFN_TAIL_QKV (with row_off, seqs, n_users): columns col0 .. col0 + n_qkv - 1 of [q | k | v] = LN(x) W^T + bias, q times q_scale; k and v
+    // FFN_TAIL_QKV (with row_off, seqs, n_users): columns col0 .. col0 + n_qkv - 1 of [q | k | v] = LN(x) W^T + bias; k and v
     // into pages where paged.slab is set.  qkv_map: rows col0 .. of W in boxes of 128 rows x 64 columns.
     const CUtensorMap *qkv_map;
     int n_qkv, col0;
-    float q_scale;
     __nv_bfloat16 *q, *k, *v;
     PagedKV paged;
 };
